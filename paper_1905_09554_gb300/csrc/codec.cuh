@@ -123,7 +123,7 @@ struct CodecLocal16 {
     __device__ __forceinline__ static S from_f(float v) { return Half16<S16>::from_f(v); }
     template <int q>
     __device__ __forceinline__ static R decode_ref(S v, float ref, const DevParams& d) {
-        return float(wq(q)) * ref + to_f(v) * d.inv_scale;
+        return __fmaf_rn(to_f(v), d.inv_scale, __fmul_rn(float(wq(q)), ref));
     }
     template <int q>
     __device__ __forceinline__ static R load_ref(const S* p, float ref, const DevParams& d) {
@@ -132,7 +132,7 @@ struct CodecLocal16 {
     // the deviation before its rounding to S
     template <int q>
     __device__ __forceinline__ static float deviation_ref(R v, float ref, const DevParams& d) {
-        return (v - float(wq(q)) * ref) * d.scale;
+        return __fmul_rn(__fmaf_rn(-float(wq(q)), ref, v), d.scale);
     }
     template <int q>
     __device__ __forceinline__ static S encode_ref(R v, float ref, const DevParams& d) {
@@ -143,10 +143,10 @@ struct CodecLocal16 {
         *p = encode_ref<q>(v, ref, d);
     }
     __device__ __forceinline__ static double decode_rt(const S* p, float w, float ref, const DevParams& d) {
-        return double(w * ref + to_f(*p) * d.inv_scale);
+        return double(__fmaf_rn(to_f(*p), d.inv_scale, __fmul_rn(w, ref)));
     }
     __device__ __forceinline__ static void encode_rt(S* p, float w, double v, float ref, const DevParams& d) {
-        *p = from_f((float(v) - w * ref) * d.scale);
+        *p = from_f(__fmul_rn(__fmaf_rn(-w, ref, float(v)), d.scale));
     }
 };
 using CodecF16Local = CodecLocal16<__half>;

@@ -1,0 +1,490 @@
+// Moments, force and collision of one cell, shared by every step kernel.
+//
+// Every operation below is written as a single rounded add, subtract,
+// multiply or fused multiply-add, in one fixed order, so that a kernel that
+// holds a cell's 19 populations and a kernel that holds only its moments
+// (step_moment.cuh) give the same bits, whatever the compiler contracts.
+//
+// V is float, double, or F2 (two cells of float in one 64-bit register: GB300
+// issues a packed add / multiply / fma for both cells at once, each rounded
+// as the scalar operation).
+#pragma once
+#include "lattice.cuh"
+#include "step_args.h"
+
+namespace lbm {
+
+struct F2 {
+    unsigned long long v;
+};
+
+template <class V> struct VecTraits { using R = V; static constexpr int N = 1; };
+template <> struct VecTraits<F2> { using R = float; static constexpr int N = 2; };
+
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vfnma(float a, float b, float c) { return __fmaf_rn(-a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double vfnma(double a, double b, double c) { return __fma_rn(-a, b, c); }
+
+__device__ __forceinline__ F2 pack2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 vadd(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vsub(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vmul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfnma(F2 a, F2 b, F2 c) {
+    a.v ^= 0x8000000080000000ull;
+    return vfma(a, b, c);
+}
+
+// The scalar s in every cell of a V.
+template <class V, class S>
+__device__ __forceinline__ V vset(S s) {
+    if constexpr (VecTraits<V>::N == 2) return pack2(float(s), float(s));
+    else return V(s);
+}
+// Element-wise scalar function.
+template <class V, class F>
+__device__ __forceinline__ V vmap(V a, F&& f) {
+    if constexpr (VecTraits<V>::N == 2) {
+        float lo, hi;
+        unpack2(a, lo, hi);
+        return pack2(f(lo), f(hi));
+    } else {
+        return f(a);
+    }
+}
+
+// c a and c a + b for a number c, the same for every cell: two scalar
+// instructions for a pair, whose c is an immediate or a constant-bank operand
+// (a packed one would need c twice in a register pair).
+template <class V, class S>
+__device__ __forceinline__ V vmulc(S c, V a) {
+    using R = typename VecTraits<V>::R;
+    return vmap(a, [&](R x) { return vmul(x, R(c)); });
+}
+__device__ __forceinline__ float vmul1(float a, float b) { return vmul(a, b); }
+__device__ __forceinline__ double vmul1(double a, double b) { return vmul(a, b); }
+__device__ __forceinline__ F2 vmul1(F2 a, F2 b) {
+    float al, ah, bl, bh;
+    unpack2(a, al, ah);
+    unpack2(b, bl, bh);
+    return pack2(vmul(al, bl), vmul(ah, bh));
+}
+template <class V, class S>
+__device__ __forceinline__ V vfmac(S c, V a, V b) {
+    if constexpr (VecTraits<V>::N == 2) {
+        float al, ah, bl, bh;
+        unpack2(a, al, ah);
+        unpack2(b, bl, bh);
+        return pack2(vfma(al, float(c), bl), vfma(ah, float(c), bh));
+    } else {
+        return vfma(a, V(c), b);
+    }
+}
+template <class V, class S, class T>
+__device__ __forceinline__ V vfmac(S c, V a, T b) {  // b a number, too
+    using R = typename VecTraits<V>::R;
+    return vmap(a, [&](R x) { return vfma(x, R(c), R(b)); });
+}
+
+// psi = rho0 (1 - exp(-rho/rho0)).  Float arithmetic uses the hardware's base-2
+// exponential (2 ulp, and the rounding of its argument: a few ulp for the
+// densities of a two-phase state, |rho/rho0| < 4) instead of the correctly
+// rounded expf, whose range reduction costs about eight more instructions per
+// call.  Subnormal arguments and results are flushed (psi rounds to the same
+// value), which saves the scaling around them.
+template <class R>
+__device__ __forceinline__ R psi_of(R rho, R rho0, R inv_rho0);
+template <>
+__device__ __forceinline__ double psi_of<double>(double rho, double rho0, double inv_rho0) {
+    return rho0 * (1.0 - exp(-rho * inv_rho0));
+}
+template <>
+__device__ __forceinline__ float psi_of<float>(float rho, float rho0, float inv_rho0) {
+    float e;  // inv_rho0 times -log2(e): the same for every cell, formed once
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(rho, __fmul_rn(inv_rho0, -1.4426950408889634f))));
+    return __fmul_rn(rho0, __fsub_rn(1.0f, e));
+}
+
+// 1/rho.  Float arithmetic uses the hardware reciprocal (within 1 ulp) instead
+// of the IEEE division, whose special-case check adds a branch per cell.
+template <class R>
+__device__ __forceinline__ R recip(R x);
+template <>
+__device__ __forceinline__ double recip<double>(double x) {
+    return 1.0 / x;
+}
+template <>
+__device__ __forceinline__ float recip<float>(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// ------------------------------------------------------------------ moments
+// The populations that move up (c_z = +1), stay in the plane (c_z = 0) and
+// move down (c_z = -1) are summed apart, because a kernel that marches along
+// z receives them from three different planes.
+
+template <class V>
+struct SumUp {  // one of the two groups with c_z != 0
+    V r;        // its density
+    V dx, dy;   // x and y momentum
+    V sx, sy;   // sums of its two x-moving and its two y-moving populations
+};
+
+template <class V>
+struct Opp {  // two opposite populations: their sum and difference
+    V s, d;
+};
+template <class V>
+__device__ __forceinline__ Opp<V> opp(V p, V m) {
+    return {vadd(p, m), vsub(p, m)};
+}
+
+// f0: straight along z; x, y: the two with c_x (c_y) = +1, -1.
+template <class V>
+__device__ __forceinline__ SumUp<V> sum_vertical(V f0, const Opp<V>& x, const Opp<V>& y) {
+    SumUp<V> s;
+    s.sx = x.s;
+    s.sy = y.s;
+    s.r = vadd(f0, vadd(x.s, y.s));
+    s.dx = x.d;
+    s.dy = y.d;
+    return s;
+}
+
+template <class V>
+struct SumFlat {  // the nine populations with c_z = 0
+    V r, jx, jy;
+    V xx, yy, xy;  // second moments
+};
+
+// f0 and the opposite pairs (1, 2), (3, 4), (7, 8), (9, 10) of the library's velocity order.
+template <class V>
+__device__ __forceinline__ SumFlat<V> sum_flat(V f0, const Opp<V>& a, const Opp<V>& b, const Opp<V>& c,
+                                               const Opp<V>& d) {
+    SumFlat<V> s;
+    const V sdiag = vadd(c.s, d.s);
+    s.r = vadd(f0, vadd(vadd(a.s, b.s), sdiag));
+    s.jx = vadd(a.d, vadd(c.d, d.d));
+    s.jy = vadd(b.d, vsub(c.d, d.d));
+    s.xx = vadd(a.s, sdiag);
+    s.yy = vadd(b.s, sdiag);
+    s.xy = vsub(c.s, d.s);
+    return s;
+}
+
+// Moments that an operator reads before the collision: rho, jx, jy, jz, then
+// the second moments whose rates differ from 1.
+//   SRT at tau = 1, MRT with every rate 1:      4
+//   MRT, shear rule: 2 xx - yy - zz, yy - zz, xy, yz, xz:  9
+//   MRT, paper's rule: xx, yy, zz, xy, yz, xz:  10
+// (SRT at another tau and MRT with general rates need all 19 populations.)
+template <int COLL>
+constexpr int kMoments = COLL == COLL_MRT_SHEAR ? 9 : (COLL == COLL_MRT_SPARSE ? 10 : 4);
+
+template <int COLL, class V>
+__device__ __forceinline__ void moments_from(const SumUp<V>& up, const V& rho_uf, const V& jx_uf, const V& jy_uf,
+                                             const V& xx_uf, const V& yy_uf, const V& xy, const SumUp<V>& dn,
+                                             V (&m)[kMoments<COLL>]) {
+    // rho_uf etc.: the sums of the up and flat groups
+    m[0] = vadd(rho_uf, dn.r);
+    m[1] = vadd(jx_uf, dn.dx);
+    m[2] = vadd(jy_uf, dn.dy);
+    m[3] = vsub(up.r, dn.r);
+    if constexpr (COLL == COLL_MRT_SHEAR || COLL == COLL_MRT_SPARSE) {
+        const V xx = vadd(xx_uf, dn.sx), yy = vadd(yy_uf, dn.sy), zz = vadd(up.r, dn.r);
+        const V yz = vsub(up.dy, dn.dy), xz = vsub(up.dx, dn.dx);
+        if constexpr (COLL == COLL_MRT_SHEAR) {
+            m[4] = vsub(vadd(xx, xx), vadd(yy, zz));
+            m[5] = vsub(yy, zz);
+            m[6] = xy;
+            m[7] = yz;
+            m[8] = xz;
+        } else {
+            m[4] = xx;
+            m[5] = yy;
+            m[6] = zz;
+            m[7] = xy;
+            m[8] = yz;
+            m[9] = xz;
+        }
+    }
+}
+
+// Moments of 19 populations in registers.
+template <int COLL, class V>
+__device__ __forceinline__ void moments_of(const V (&f)[Q], V (&m)[kMoments<COLL>]) {
+    const SumUp<V> up = sum_vertical(f[5], opp(f[11], f[14]), opp(f[15], f[18]));
+    const SumUp<V> dn = sum_vertical(f[6], opp(f[13], f[12]), opp(f[17], f[16]));
+    const SumFlat<V> fl = sum_flat(f[0], opp(f[1], f[2]), opp(f[3], f[4]), opp(f[7], f[8]), opp(f[9], f[10]));
+    moments_from<COLL, V>(up, vadd(up.r, fl.r), vadd(up.dx, fl.jx), vadd(up.dy, fl.jy), vadd(up.sx, fl.xx),
+                          vadd(up.sy, fl.yy), fl.xy, dn, m);
+}
+
+// Density of a cell alone, from a getter of population q: the rho of
+// moments_of.
+template <class V, class Get>
+__device__ __forceinline__ V density_of(Get&& f) {
+    auto at = [&](auto qc) { return f(qc); };
+#define LBM_AT(q) at(std::integral_constant<int, q>{})
+    const V up = vadd(LBM_AT(5), vadd(vadd(LBM_AT(11), LBM_AT(14)), vadd(LBM_AT(15), LBM_AT(18))));
+    const V fl = vadd(LBM_AT(0), vadd(vadd(vadd(LBM_AT(1), LBM_AT(2)), vadd(LBM_AT(3), LBM_AT(4))),
+                                      vadd(vadd(LBM_AT(7), LBM_AT(8)), vadd(LBM_AT(9), LBM_AT(10)))));
+    const V dn = vadd(LBM_AT(6), vadd(vadd(LBM_AT(13), LBM_AT(12)), vadd(LBM_AT(17), LBM_AT(16))));
+#undef LBM_AT
+    return vadd(vadd(up, fl), dn);
+}
+
+// -------------------------------------------------------------------- force
+// Eq. SC_force, F = -G psi sum_a w_a psi(x + c_a) c_a, from what a cell sees
+// of each of three planes.  36 w_a = 2 on the axes and 1 on the edges, so
+//   36 S_x = 2 ex(z) + dx(z) + ex(z-1) + ex(z+1),
+//   36 S_z = 2 (c(z+1) - c(z-1)) + s4(z+1) - s4(z-1).
+template <class V>
+struct PsiView {
+    V c;       // psi of the cell
+    V s4;      // sum over its four axis neighbours in the plane
+    V ex, ey;  // differences along x and y
+    V dx, dy;  // the same from the four diagonal neighbours
+};
+
+// psi at an offset in a plane of row pitch PX.
+template <class R, int PX>
+struct PsiAt {
+    const R* p;
+    template <class DX, class DY>
+    __device__ __forceinline__ R operator()(DX, DY) const {
+        return p[DX::value + DY::value * PX];
+    }
+};
+
+// p(dx, dy): psi of the neighbour in the plane (compile-time offsets).
+template <class V, class P>
+__device__ __forceinline__ void psi_axis(PsiView<V>& w, P&& p) {
+    const V xp = p(std::integral_constant<int, 1>{}, std::integral_constant<int, 0>{});
+    const V xm = p(std::integral_constant<int, -1>{}, std::integral_constant<int, 0>{});
+    const V yp = p(std::integral_constant<int, 0>{}, std::integral_constant<int, 1>{});
+    const V ym = p(std::integral_constant<int, 0>{}, std::integral_constant<int, -1>{});
+    w.ex = vsub(xp, xm);
+    w.ey = vsub(yp, ym);
+    w.s4 = vadd(vadd(xp, xm), vadd(yp, ym));
+}
+template <class V, class P>
+__device__ __forceinline__ void psi_diag(PsiView<V>& w, P&& p) {
+    const V a = vsub(p(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{}),
+                     p(std::integral_constant<int, -1>{}, std::integral_constant<int, -1>{}));
+    const V b = vsub(p(std::integral_constant<int, 1>{}, std::integral_constant<int, -1>{}),
+                     p(std::integral_constant<int, -1>{}, std::integral_constant<int, 1>{}));
+    w.dx = vadd(a, b);
+    w.dy = vsub(a, b);
+}
+
+// F = g (sx, sy, sz), kept as factors: every use multiplies and adds.
+template <class V>
+struct Force {
+    V g, sx, sy, sz;
+};
+// gw = -G/36.
+template <class V, class R>
+__device__ __forceinline__ Force<V> force_of(const PsiView<V>& lo, const PsiView<V>& mid, const PsiView<V>& hi,
+                                             R gw) {
+    Force<V> F;
+    F.g = vmulc(gw, mid.c);
+    const V dc = vsub(hi.c, lo.c);
+    F.sx = vadd(vadd(mid.ex, mid.ex), vadd(mid.dx, vadd(lo.ex, hi.ex)));
+    F.sy = vadd(vadd(mid.ey, mid.ey), vadd(mid.dy, vadd(lo.ey, hi.ey)));
+    F.sz = vadd(vadd(dc, dc), vsub(hi.s4, lo.s4));
+    return F;
+}
+
+// ---------------------------------------------------------------- collision
+// With a = 3 u' and h = w rho / 2, the equilibrium is
+//   f_eq = h (b + (c.a)^2) +/- 2 h c.a,   b = 2 - a.a/3,
+// an even and an odd part for each pair of opposite velocities.
+//
+// SRT (Eq. vel_shift): u' = (j + tau F)/rho, f* = f + omega (f_eq - f).
+//
+// MRT with Guo-like forcing (Eq. barycentric) at u_b = (j + F/2)/rho, rates 1
+// outside K = {e, 3pxx, pww, pxy, pyz, pxz}: writing
+// m* = m_eq + S/2 + (1 - s)(m - m_eq + S/2), the conserved rows vanish (rho:
+// m = m_eq, S = 0; j: m - m_eq = -F/2, S = F), rows with s = 1 vanish, and
+//   f* = f_eq(rho, u_b) + S_pop/2 + sum_{k in K} M_k^T (1 - s_k)(m_k - m_eq_k + S_k/2)/norm_k.
+// With phi = 1.5 F/rho and a = 3 (j + F)/rho the first two terms are
+//   h (b + (c.a)^2 - (c.phi)^2) +/- 2 h c.a,   b = 2 - (a.a - phi.phi)/3,
+// and with g = a - 2 phi the second moments entering the rows of K are
+//   N_ij = Pi_ij - rho delta_ij/3 - (rho/9)(g_i g_j - phi_i phi_j).
+// The energy row is left out under the shear rule, where its rate is 1.
+//
+// w_a rho per speed shell, the rest one from sum_a w_a = 1: the rounded
+// weights float(1/3) + 6 float(1/18) + 12 float(1/36) sum to 1 + 3e-8, which
+// made FP32 runs gain ~3e-8 of their mass every step.
+
+// put(q, value) receives f*_q (for SRT at tau != 1: omega f_eq_q, to which
+// the caller adds (1 - omega) f_q).  TAU1: SRT at tau = 1, known when compiled
+// (multiplications by 1 are left out; the values are the same).
+template <int COLL, class V, bool TAU1 = false, class Put>
+__device__ __forceinline__ void collide_moments(const V (&m)[kMoments<COLL>], const Force<V>& F, const StepArgs& a,
+                                                Put&& put) {
+    using R = typename VecTraits<V>::R;
+    constexpr bool SRT = COLL == COLL_SRT;
+    constexpr bool ROWS = COLL == COLL_MRT_SHEAR || COLL == COLL_MRT_SPARSE;
+    const V rho = m[0];
+    const V inv = vmap(rho, [](R r) { return recip(r); });
+    const V inv3 = vmulc(R(3), inv);
+    V ax, ay, az, px, py, pz;
+    V b;
+    V gt = F.g;  // a = 3 (j + tau F)/rho (SRT), 3 (j + F)/rho (MRT)
+    if constexpr (SRT && !TAU1) gt = vmulc(par<R>(a.tau, a.tauf), F.g);
+    ax = vmul(inv3, vfma(gt, F.sx, m[1]));
+    ay = vmul(inv3, vfma(gt, F.sy, m[2]));
+    az = vmul(inv3, vfma(gt, F.sz, m[3]));
+    const V aa = vfma(az, az, vfma(ay, ay, vmul(ax, ax)));
+    if constexpr (SRT) {
+        px = py = pz = aa;  // not used
+        b = vfmac(R(-1.0 / 3.0), aa, R(2));
+    } else {
+        const V i15 = vmul(vmulc(R(1.5), inv), F.g);
+        px = vmul(i15, F.sx);
+        py = vmul(i15, F.sy);
+        pz = vmul(i15, F.sz);
+        b = vfmac(R(-1.0 / 3.0), vfnma(pz, pz, vfnma(py, py, vfnma(px, px, aa))), R(2));
+    }
+    // 2 h per speed shell: w rho on the axes (r1) and edges (r2 = rho/36, and r1 = 2 r2)
+    V r2 = vmulc(R(1.0 / 36.0), rho);
+    V r0 = vfmac(R(-24), r2, rho);
+
+    // corrections of the even part: rest, axis x / y / z, edges xy / xz / yz (+/- for the two pairs of an edge)
+    V k0, kx, ky, kz, kxy, kxz, kyz, cxy, cxz, cyz;
+    if constexpr (ROWS) {
+        const V gx = vfmac(R(-2), px, ax), gy = vfmac(R(-2), py, ay), gz = vfmac(R(-2), pz, az);
+        const V r9 = vmulc(R(1.0 / 9.0), rho);
+        auto flow = [&](V g1, V g2, V p1, V p2) { return vfnma(p1, p2, vmul(g1, g2)); };
+        const V xx = flow(gx, gx, px, px), yy = flow(gy, gy, py, py), zz = flow(gz, gz, pz, pz);
+        const R(&kk)[6] = row_rates<R>(a);
+        V d1, d2, pxy, pyz, pxz;
+        if constexpr (COLL == COLL_MRT_SHEAR) {
+            d1 = m[4];
+            d2 = m[5];
+            pxy = m[6];
+            pyz = m[7];
+            pxz = m[8];
+        } else {
+            d1 = vsub(vadd(m[4], m[4]), vadd(m[5], m[6]));
+            d2 = vsub(m[5], m[6]);
+            pxy = m[7];
+            pyz = m[8];
+            pxz = m[9];
+        }
+        const V A = vmulc(kk[1], vfnma(r9, vsub(vadd(xx, xx), vadd(yy, zz)), d1));
+        const V B = vmulc(kk[2], vfnma(r9, vsub(yy, zz), d2));
+        cxy = vmulc(kk[3], vfnma(r9, flow(gx, gy, px, py), pxy));
+        cyz = vmulc(kk[4], vfnma(r9, flow(gy, gz, py, pz), pyz));
+        cxz = vmulc(kk[5], vfnma(r9, flow(gx, gz, px, pz), pxz));
+        kx = vadd(A, A);
+        ky = vsub(B, A);
+        kxy = vadd(A, B);
+        kxz = vsub(A, B);
+        kz = vmulc(R(-1), kxy);
+        kyz = vmulc(R(-1), kx);
+        if constexpr (COLL == COLL_MRT_SPARSE) {
+            // e = 19 tr N; coefficients -30, -11, 8 at rest, axis and edge velocities
+            const V tr = vsub(vadd(vadd(m[4], m[5]), m[6]), rho);
+            const V E = vmulc(kk[0], vfnma(r9, vadd(vadd(xx, yy), zz), tr));
+            k0 = vmulc(R(-30), E);
+            kx = vfmac(R(-11), E, kx);
+            ky = vfmac(R(-11), E, ky);
+            kz = vfmac(R(-11), E, kz);
+            kxy = vfmac(R(8), E, kxy);
+            kxz = vfmac(R(8), E, kxz);
+            kyz = vfmac(R(8), E, kyz);
+        }
+    }
+    if constexpr (SRT && !TAU1) {
+        const R om = par<R>(a.omega, a.omegaf);
+        r0 = vmulc(om, r0);
+        r2 = vmulc(om, r2);
+    }
+    const V r1 = vadd(r2, r2), h2 = vmulc(R(0.5), r2), n2 = vmulc(R(-1), r2), n1 = vadd(n2, n2);
+    const V& h1 = r2;
+
+    {
+        // (the product cell by cell: a packed one may be contracted with the sum it enters later)
+        const V e0 = vmulc(R(0.5), r0);
+        if constexpr (COLL == COLL_MRT_SPARSE) put(std::integral_constant<int, 0>{}, vfma(e0, b, k0));
+        else put(std::integral_constant<int, 0>{}, vmul1(e0, b));
+    }
+    static_for<0, 9>([&](auto pc) {
+        constexpr int q = 2 * decltype(pc)::value + 1;
+        constexpr bool axis = q < 7;
+        // c.a and c.phi (one or two components)
+        auto dot = [&](V x, V y, V z) {
+            if constexpr (q == 1) return x;
+            else if constexpr (q == 3) return y;
+            else if constexpr (q == 5) return z;
+            else if constexpr (q == 7) return vadd(x, y);
+            else if constexpr (q == 9) return vsub(x, y);
+            else if constexpr (q == 11) return vadd(x, z);
+            else if constexpr (q == 13) return vsub(x, z);
+            else if constexpr (q == 15) return vadd(y, z);
+            else return vsub(y, z);
+        };
+        const V ca = dot(ax, ay, az);
+        V T = vfma(ca, ca, b);
+        if constexpr (!SRT) {
+            const V cp = dot(px, py, pz);
+            T = vfnma(cp, cp, T);
+        }
+        const V h = axis ? h1 : h2;
+        V e;
+        if constexpr (ROWS) {
+            V k;
+            if constexpr (q == 1) k = kx;
+            else if constexpr (q == 3) k = ky;
+            else if constexpr (q == 5) k = kz;
+            else if constexpr (q == 7) k = vadd(kxy, cxy);
+            else if constexpr (q == 9) k = vsub(kxy, cxy);
+            else if constexpr (q == 11) k = vadd(kxz, cxz);
+            else if constexpr (q == 13) k = vsub(kxz, cxz);
+            else if constexpr (q == 15) k = vadd(kyz, cyz);
+            else k = vsub(kyz, cyz);
+            e = vfma(h, T, k);
+        } else {
+            e = vmul(h, T);
+        }
+        put(std::integral_constant<int, q>{}, vfma(axis ? r1 : r2, ca, e));
+        put(std::integral_constant<int, q + 1>{}, vfma(axis ? n1 : n2, ca, e));
+    });
+}
+
+}  // namespace lbm

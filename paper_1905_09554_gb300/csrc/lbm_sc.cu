@@ -39,6 +39,7 @@ struct lbm_ctx {
     double* scratch = nullptr;        // staging / moments scratch (lazily grown)
     size_t scratch_bytes = 0;
     double* diag = nullptr;           // per-slice diagnostic partials (8 * nz)
+    void* psi_ws = nullptr;           // two-belt force: psi of the state being stepped
     int* dev_err = nullptr;           // device error word of the bounded waits
     std::vector<double> diag_host;
     long long own_bytes = 0;
@@ -786,6 +787,16 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     round_params(a);
     c->coll = collision_kernel(*p, a.s);
+    if (p->G2 != 0.0) {  // psi of the whole box; the step runs without it, slower, where there is no room
+        const size_t pbytes = (size_t)n * (p->storage == LBM_F64 ? 8 : 4);
+        if (cudaMalloc(&c->psi_ws, pbytes) == cudaSuccess) {
+            c->own_bytes += (long long)pbytes;
+        } else {
+            c->psi_ws = nullptr;
+            cudaGetLastError();
+        }
+        a.psi_ws = c->psi_ws;
+    }
     a.err = c->dev_err;
     a.test_stall = p->test_stall ? 1 : 0;
     a.dev = make_dev_params(p->rho_ref, p->dev_scale);
@@ -818,6 +829,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->ref[0]);
     cudaFree(c->ref[1]);
     cudaFree(c->scratch);
+    cudaFree(c->psi_ws);
     cudaFree(c->diag);
     cudaFree(c->dev_err);
     cudaFree(c->adj.cp);

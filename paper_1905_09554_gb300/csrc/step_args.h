@@ -26,11 +26,15 @@ struct StepArgs {
     double tau, omega;    // SRT relaxation time and 1/tau
     double rho0, inv_rho0;
     double s[Q];          // MRT rates, moment order
+    double gw;            // -G/36: the force's strength per edge weight
+    // (1 - s_k)/norm_k of the rows e (times 19), 3pxx, pww, pxy, pyz, pxz
+    double kk[6];
     // The same parameters rounded to float once on the host, for the float
     // arithmetic of the 32- and 16-bit formats: a double-to-float conversion
     // inside the cell loop would occupy the FP64 pipe (2 lanes per SM clock).
     float Gf, tauf, omegaf, rho0f, inv_rho0f;
     float sf[Q];
+    float gwf, kkf[6];
     DevParams dev;
     int* err;             // device error word (bit 0: a bounded wait timed out)
     const float* ref_src; // local-reference storage: density field of the source copy
@@ -40,6 +44,7 @@ struct StepArgs {
     // in the arithmetic type (the adjoint's recomputation keeps it for the
     // reverse step); nullptr normally.
     void* psi_out;
+    void* psi_ws;         // kernel 6: field of psi in the arithmetic type, or nullptr
 };
 
 // MRT rates in the arithmetic type R (see par() in lattice.cuh).
@@ -48,8 +53,20 @@ __host__ __device__ __forceinline__ const R (&rates(const StepArgs& a))[Q] {
     if constexpr (sizeof(R) == sizeof(double)) return a.s;
     else return a.sf;
 }
-// Fill the float copies from the double fields.
+template <class R>
+__host__ __device__ __forceinline__ const R (&row_rates(const StepArgs& a))[6] {
+    if constexpr (sizeof(R) == sizeof(double)) return a.kk;
+    else return a.kkf;
+}
+// Fill the derived parameters and the float copies from the double fields.
 inline void round_params(StepArgs& a) {
+    constexpr int rows[6] = {1, 9, 11, 13, 14, 15};
+    a.gw = -a.G / 36.0;
+    a.gwf = float(a.gw);
+    for (int i = 0; i < 6; ++i) {
+        a.kk[i] = (1.0 - a.s[rows[i]]) / mrt_norm(rows[i]) * (i == 0 ? 19.0 : 1.0);
+        a.kkf[i] = float(a.kk[i]);
+    }
     a.Gf = float(a.G);
     a.tauf = float(a.tau);
     a.omegaf = float(a.omega);

@@ -16,6 +16,11 @@ cudaError_t launch_step_t(const StepLaunch& c, const void* src, void* dst) {
     if constexpr ((std::is_same_v<Codec, CodecF32> || std::is_same_v<Codec, CodecF64>) && TY >= 8) {
         if (c.kernel == 6) {
             dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + a.zchunk - 1) / a.zchunk);
+            if (a.psi_ws) {
+                const long long blocks = (a.n + 255) / 256;
+                sc_psi_kernel<Codec><<<unsigned(blocks < 152 * 32 ? blocks : 152 * 32), 256, 0, c.stream>>>(
+                    static_cast<const typename Codec::S*>(src), static_cast<typename Codec::R*>(a.psi_ws), a);
+            }
             sc_step_mr_kernel<Codec, COLL, TX, TY><<<grid, TX * TY, 0, c.stream>>>(
                 static_cast<const typename Codec::S*>(src), static_cast<typename Codec::S*>(dst), a);
             return cudaGetLastError();

@@ -25,34 +25,11 @@
 #include <cstring>
 
 #include "codec.cuh"
+#include "collide.cuh"
 #include "lattice.cuh"
 #include "step_args.h"
 
 namespace lbm {
-
-// psi = rho0 (1 - exp(-rho/rho0)).  Float arithmetic uses the hardware
-// exponential (__expf, a few ulp for the densities of a two-phase state,
-// |rho/rho0| < 4) instead of the correctly rounded expf, whose range
-// reduction costs about eight more instructions per call.
-template <class R>
-__device__ __forceinline__ R psi_of(R rho, R rho0, R inv_rho0);
-template <>
-__device__ __forceinline__ double psi_of<double>(double rho, double rho0, double inv_rho0) {
-    return rho0 * (1.0 - exp(-rho * inv_rho0));
-}
-template <>
-__device__ __forceinline__ float psi_of<float>(float rho, float rho0, float inv_rho0) {
-    return rho0 * (1.0f - __expf(-rho * inv_rho0));
-}
-
-// 1/rho.  Float arithmetic uses the hardware reciprocal with one rounding
-// step (__fdividef, within 2 ulp) instead of the IEEE division, whose
-// special-case check adds a branch per cell.
-template <class R>
-__device__ __forceinline__ R recip(R x) {
-    if constexpr (sizeof(R) == sizeof(double)) return 1.0 / x;
-    else return __fdividef(1.0f, x);
-}
 
 // Population q of the field starting at p (population stride n elements).
 // The 64-bit product comes from kernel parameters only, so with 32-bit cell
@@ -66,50 +43,6 @@ __device__ __forceinline__ S* pop_at(S* p, int q, I n) {
 __device__ __forceinline__ int wrap_index(int i, int n) {
     i %= n;
     return i < 0 ? i + n : i;
-}
-
-// SRT with shifted equilibrium (Eq. vel_shift): u' = (j + tau F)/rho,
-// f* = f + (f_eq(rho, u') - f)/tau.  Velocities come in +/- pairs (q, q+1),
-// whose equilibria share the even part A and differ by the sign of the odd
-// part B: f_eq = A +/- B.
-template <class R>
-__device__ __forceinline__ void collide_srt(R (&f)[Q], R Fx, R Fy, R Fz, R tau, R omega) {
-    R rho = f[0], jx = R(0), jy = R(0), jz = R(0);
-    static_for<0, 9>([&](auto pc) {
-        constexpr int q = 2 * decltype(pc)::value + 1;
-        const R sum = f[q] + f[q + 1], dif = f[q] - f[q + 1];
-        rho += sum;
-        if constexpr (cx(q) != 0) jx += R(cx(q)) * dif;
-        if constexpr (cy(q) != 0) jy += R(cy(q)) * dif;
-        if constexpr (cz(q) != 0) jz += R(cz(q)) * dif;
-    });
-    const R inv_rho = recip(rho);
-    const R ux = (jx + tau * Fx) * inv_rho;
-    const R uy = (jy + tau * Fy) * inv_rho;
-    const R uz = (jz + tau * Fz) * inv_rho;
-    const R usq = R(1.5) * (ux * ux + uy * uy + uz * uz);
-    const R base = R(1) - usq;
-    // w_a rho per speed shell, the rest one from sum_a w_a = 1: the rounded
-    // weights float(1/3) + 6 float(1/18) + 12 float(1/36) sum to 1 + 3e-8,
-    // which made FP32 runs gain ~3e-8 of their mass every step.
-    const R r1 = R(wq(1)) * rho, r2 = R(wq(7)) * rho;
-    const R r0 = rho - R(6) * r1 - R(12) * r2;
-    // f* = (1 - omega) f + omega (A +/- B): omega w rho per shell once
-    const R keep = R(1) - omega;
-    const R o1 = omega * r1, o2 = omega * r2, o1b = R(3) * o1, o2b = R(3) * o2;
-    f[0] = keep * f[0] + omega * (r0 * base);
-    static_for<0, 9>([&](auto pc) {
-        constexpr int q = 2 * decltype(pc)::value + 1;
-        R cu = R(0);
-        if constexpr (cx(q) != 0) cu += R(cx(q)) * ux;
-        if constexpr (cy(q) != 0) cu += R(cy(q)) * uy;
-        if constexpr (cz(q) != 0) cu += R(cz(q)) * uz;
-        constexpr bool axis = wq(q) == wq(1);
-        const R oA = (axis ? o1 : o2) * (base + R(4.5) * cu * cu);
-        const R oB = (axis ? o1b : o2b) * cu;
-        f[q] = keep * f[q] + (oA + oB);
-        f[q + 1] = keep * f[q + 1] + (oA - oB);
-    });
 }
 
 // MRT with Guo-like forcing (Eq. barycentric), d'Humieres D3Q19 basis:
@@ -223,114 +156,41 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
     });
 }
 
-// MRT with Guo-like forcing when every rate outside K = {e, 3pxx, pww, pxy,
-// pyz, pxz} equals 1 (the paper's rule, and the shear rule), or when every
-// rate equals 1 (UNIT).  Writing m* = m_eq + S/2 + (1 - s)(m - m_eq + S/2),
-// the conserved rows vanish (rho: m = m_eq, S = 0; j: m - m_eq = -F/2,
-// S = F), rows with s = 1 vanish, and
-//   f* = f_eq(rho, u_b) + S_pop/2 + sum_{k in K} M_k^T (1 - s_k)(m_k - m_eq_k + S_k/2)/norm_k.
-// Algebraically identical to collide_mrt for such rates, with far fewer
-// operations (only the even rows of K are transformed).  WITH_E = false is
-// the shear rule's form: the energy row relaxes at 1 there, its correction
-// is exactly zero and the row is left out (a separate instantiation, chosen
-// on the host, so no kernel carries both forms).
-template <class R, bool UNIT, bool WITH_E = true>
-__device__ __forceinline__ void collide_mrt_sparse(R (&f)[Q], R Fx, R Fy, R Fz, const R (&s)[Q]) {
-    constexpr int K0 = WITH_E ? 0 : 1;  // first row of K transformed
-    R ps[9], rho = f[0], jx = R(0), jy = R(0), jz = R(0);
-    static_for<0, 9>([&](auto pc) {
-        constexpr int p = decltype(pc)::value, q = 2 * p + 1;
-        ps[p] = f[q] + f[q + 1];
-        const R dif = f[q] - f[q + 1];
-        rho += ps[p];
-        if constexpr (cx(q) != 0) jx += R(cx(q)) * dif;
-        if constexpr (cy(q) != 0) jy += R(cy(q)) * dif;
-        if constexpr (cz(q) != 0) jz += R(cz(q)) * dif;
-    });
-    const R inv_rho = recip(rho);
-    const R ux = (jx + R(0.5) * Fx) * inv_rho;
-    const R uy = (jy + R(0.5) * Fy) * inv_rho;
-    const R uz = (jz + R(0.5) * Fz) * inv_rho;
-    const R ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
-    const R u2 = ux2 + uy2 + uz2;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-
-    // correction per even row of K, already divided by the row norm
-    constexpr int KS[6] = {1, 9, 11, 13, 14, 15};
-    R dk[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-    if constexpr (!UNIT) {
-        const R pxx = R(2) * ux2 - uy2 - uz2, pww = uy2 - uz2;
-        const R gxx = R(2) * ux * Fx - uy * Fy - uz * Fz, gww = uy * Fy - uz * Fz;
-        const R meq[6] = {rho * (R(-11) + R(19) * u2), rho * pxx, rho * pww, rho * ux * uy, rho * uy * uz,
-                          rho * ux * uz};
-        const R sg[6] = {R(38) * uF, R(2) * gxx, R(2) * gww, ux * Fy + uy * Fx, uy * Fz + uz * Fy, ux * Fz + uz * Fx};
-        static_for<K0, 6>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int k = KS[i];
-            R m = R(0);
-            constexpr int c0 = mrt_coef(k, 0);
-            if constexpr (c0 != 0) m = R(c0) * f[0];
-            static_for<0, 9>([&](auto pc) {
-                constexpr int p = decltype(pc)::value;
-                constexpr int c = mrt_coef(k, 2 * p + 1);
-                if constexpr (c == 1) m += ps[p];
-                else if constexpr (c == -1) m -= ps[p];
-                else if constexpr (c != 0) m += R(c) * ps[p];
-            });
-            dk[i] = (R(1) - s[k]) * (m - meq[i] + R(0.5) * sg[i]) * R(1.0 / mrt_norm(k));
+// Collision of a cell's 19 populations (collide.cuh; general MRT rates above).
+template <int COLL, class R>
+__device__ __forceinline__ void collide(R (&f)[Q], const Force<R>& F, const StepArgs& a) {
+    if constexpr (COLL == COLL_MRT) {
+        collide_mrt<R>(f, vmul(F.g, F.sx), vmul(F.g, F.sy), vmul(F.g, F.sz), rates<R>(a));
+    } else {
+        R m[kMoments<COLL>];
+        moments_of<COLL, R>(f, m);
+        const R keep = R(1) - par<R>(a.omega, a.omegaf);
+        collide_moments<COLL, R>(m, F, a, [&](auto qc, R v) {
+            constexpr int q = decltype(qc)::value;
+            if constexpr (COLL == COLL_SRT) f[q] = vfma(keep, f[q], v);
+            else f[q] = v;
         });
     }
-    auto corr = [&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        R acc = R(0);
-        if constexpr (!UNIT) {
-            static_for<K0, 6>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                constexpr int c = mrt_coef(KS[i], q);
-                if constexpr (c == 1) acc += dk[i];
-                else if constexpr (c == -1) acc -= dk[i];
-                else if constexpr (c != 0) acc += R(c) * dk[i];
-            });
-        }
-        return acc;
-    };
-    const R base = R(1) - R(1.5) * u2;
-    // w_a rho per speed shell, the rest one from sum_a w_a = 1 (as in
-    // collide_srt: no systematic mass from the rounded weights)
-    const R r1 = R(wq(1)) * rho, r2 = R(wq(7)) * rho;
-    const R r0 = rho - R(6) * r1 - R(12) * r2;
-    const R r1b = R(3) * r1, r2b = R(3) * r2, uF15 = R(1.5) * uF;
-    f[0] = r0 * base - R(wq(0)) * uF15 + corr(std::integral_constant<int, 0>{});
-    static_for<0, 9>([&](auto pc) {
-        constexpr int q = 2 * decltype(pc)::value + 1;
-        R cu = R(0), cF = R(0);
-        if constexpr (cx(q) != 0) { cu += R(cx(q)) * ux; cF += R(cx(q)) * Fx; }
-        if constexpr (cy(q) != 0) { cu += R(cy(q)) * uy; cF += R(cy(q)) * Fy; }
-        if constexpr (cz(q) != 0) { cu += R(cz(q)) * uz; cF += R(cz(q)) * Fz; }
-        constexpr bool axis = wq(q) == wq(1);
-        // f_eq = A +/- B and the Guo source S/2 = E +/- O, as the even part
-        // A + E = w rho (base + 4.5 cu^2) + w (4.5 cu cF - 1.5 u.F) and the
-        // odd part B + O = 3 w rho cu + 1.5 w cF of the velocity pair
-        const R cu45 = R(4.5) * cu;
-        const R even = (axis ? r1 : r2) * (base + cu45 * cu) + R(wq(q)) * (cu45 * cF - uF15);
-        const R odd = (axis ? r1b : r2b) * cu + R(1.5 * wq(q)) * cF;
-        const R e = even + corr(std::integral_constant<int, q>{});  // even rows: equal on both members
-        f[q] = e + odd;
-        f[q + 1] = e - odd;
-    });
 }
+
+// Population q of a cell in a shared-memory stage of PITCH values each.
+template <int PITCH>
+struct StridedAt {
+    const float* p;
+    template <class QC>
+    __device__ __forceinline__ float operator()(QC) const {
+        return p[QC::value * PITCH];
+    }
+};
 
 template <class Codec>
 __device__ __forceinline__ typename Codec::R cell_density(const typename Codec::S* __restrict__ p,
                                                           long long n, const DevParams& dev, float ref = 0.0f) {
-    using R = typename Codec::R;
-    R r = R(0);
-    static_for<0, Q>([&](auto qc) {
+    return density_of<typename Codec::R>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        if constexpr (Codec::kLocal) r += Codec::template load_ref<q>(p + q * n, ref, dev);
-        else r += Codec::template load<q>(p + q * n, dev);
+        if constexpr (Codec::kLocal) return Codec::template load_ref<q>(p + q * n, ref, dev);
+        else return Codec::template load<q>(p + q * n, dev);
     });
-    return r;
 }
 
 // Force from the psi ring (planes z-1, z, z+1 of the tile + ring), collision
@@ -343,24 +203,15 @@ __device__ __forceinline__ void update_cell(typename Codec::R (&fc)[Q], const ty
                                             const int (&xidx)[3], const StepArgs& a,
                                             const float* const* rho_pl = nullptr) {
     using R = typename Codec::R;
-    const R* pl[3] = {pm, p0, pp};
-    // Eq. SC_force: F = -G psi(x) sum_a w_a psi(x + c_a) c_a.
-    R sx = R(0), sy = R(0), sz = R(0);
-    static_for<1, Q>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const R v = pl[cz(q) + 1][slot + cx(q) + cy(q) * PX];
-        if constexpr (cx(q) != 0) sx += R(wq(q) * cx(q)) * v;
-        if constexpr (cy(q) != 0) sy += R(wq(q) * cy(q)) * v;
-        if constexpr (cz(q) != 0) sz += R(wq(q) * cz(q)) * v;
-    });
-    const R gpsi = -par<R>(a.G, a.Gf) * p0[slot];
-    const R Fx = gpsi * sx, Fy = gpsi * sy, Fz = gpsi * sz;
-
-    if constexpr (COLL == COLL_SRT) collide_srt<R>(fc, Fx, Fy, Fz, par<R>(a.tau, a.tauf), par<R>(a.omega, a.omegaf));
-    else if constexpr (COLL == COLL_MRT) collide_mrt<R>(fc, Fx, Fy, Fz, rates<R>(a));
-    else if constexpr (COLL == COLL_MRT_SPARSE) collide_mrt_sparse<R, false>(fc, Fx, Fy, Fz, rates<R>(a));
-    else if constexpr (COLL == COLL_MRT_SHEAR) collide_mrt_sparse<R, false, false>(fc, Fx, Fy, Fz, rates<R>(a));
-    else collide_mrt_sparse<R, true>(fc, Fx, Fy, Fz, rates<R>(a));
+    PsiView<R> lo, mid, hi;
+    lo.c = pm[slot];
+    mid.c = p0[slot];
+    hi.c = pp[slot];
+    psi_axis(lo, PsiAt<R, PX>{pm + slot});
+    psi_axis(mid, PsiAt<R, PX>{p0 + slot});
+    psi_axis(hi, PsiAt<R, PX>{pp + slot});
+    psi_diag(mid, PsiAt<R, PX>{p0 + slot});
+    collide<COLL, R>(fc, force_of(lo, mid, hi, par<R>(a.gw, a.gwf)), a);
 
     // Eq. LBE streaming: f_a(x + c_a, t + 1) = f*_a(x, t).
     static_for<0, Q>([&](auto qc) {
@@ -457,12 +308,11 @@ sc_step_kernel(const typename Codec::S* __restrict__ src, typename Codec::S* __r
     {
         const long long zo = (long long)zs * plane;
         const float ref = ref_at(zo + my_xy);
-        R r = R(0);
         static_for<0, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             fc[q] = load_q(qc, src + q * n + zo + my_xy, ref);
-            r += fc[q];
         });
+        const R r = density_of<R>([&](auto qc) { return fc[decltype(qc)::value]; });
         psi_s[slot_of(zs)][my_slot] = psi_of<R>(r, rho0, inv_rho0);
         if (a.psi_out && active) static_cast<R*>(a.psi_out)[zo + my_xy] = psi_s[slot_of(zs)][my_slot];
         put_rho(slot_of(zs), my_slot, r);
@@ -480,12 +330,11 @@ sc_step_kernel(const typename Codec::S* __restrict__ src, typename Codec::S* __r
         {
             const long long zo = (long long)zn * plane;
             const float ref = ref_at(zo + my_xy);
-            R r = R(0);
             static_for<0, Q>([&](auto qc) {
                 constexpr int q = decltype(qc)::value;
                 fn[q] = load_q(qc, src + q * n + zo + my_xy, ref);
-                r += fn[q];
             });
+            const R r = density_of<R>([&](auto qc) { return fn[decltype(qc)::value]; });
             psi_s[zp_slot][my_slot] = psi_of<R>(r, rho0, inv_rho0);
             if (a.psi_out && active && z + 1 < ze) static_cast<R*>(a.psi_out)[zo + my_xy] = psi_s[zp_slot][my_slot];
             put_rho(zp_slot, my_slot, r);
@@ -536,9 +385,12 @@ template <int N>
 __device__ __forceinline__ void wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 template <int BYTES>
 __device__ __forceinline__ void copy(void* smem, const void* gmem) {
-    static_assert(BYTES == 4 || BYTES == 8, "cp.async element size");
+    static_assert(BYTES == 4 || BYTES == 8 || BYTES == 16, "cp.async element size");
     const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+    if constexpr (BYTES == 16)  // past L1
+        asm volatile("cp.async.cg.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
 }
 }  // namespace async_copy
 
@@ -624,17 +476,15 @@ sc_step_async_kernel(const typename Codec::S* __restrict__ src, typename Codec::
         };
         auto psi_from_stage = [&](int z) {
             const S* st = stage + stage_of(z) * (Q * SLOTS);
-            R r = R(0);
-            static_for<0, Q>([&](auto qc) {
+            const R r = density_of<R>([&](auto qc) {
                 constexpr int q = decltype(qc)::value;
-                r += Codec::template decode<q>(st[q * SLOTS + tid], dev);
+                return Codec::template decode<q>(st[q * SLOTS + tid], dev);
             });
             ring[slot_of(z) * PLANE + my_slot] = psi_of<R>(r, rho0, inv_rho0);
             if (h_slot >= 0) {
-                R rh = R(0);
-                static_for<0, Q>([&](auto qc) {
+                const R rh = density_of<R>([&](auto qc) {
                     constexpr int q = decltype(qc)::value;
-                    rh += Codec::template decode<q>(st[q * SLOTS + NT + tid], dev);
+                    return Codec::template decode<q>(st[q * SLOTS + NT + tid], dev);
                 });
                 ring[slot_of(z) * PLANE + h_slot] = psi_of<R>(rh, rho0, inv_rho0);
             }
@@ -831,23 +681,18 @@ sc_step_pipe_kernel(const typename Codec::S* __restrict__ src_all, typename Code
         auto halo_psi = [&](int z) {
             if (h_slot >= 0) {
                 const HS* st = hstage + stage_of(z) * (Q * NH);
-                R r = R(0);
-                if constexpr (LOCAL) {
-                    const float ref = rstage[stage_of(z) * NH + h];
-                    static_for<0, Q>([&](auto qc) {
-                        constexpr int q = decltype(qc)::value;
-                        r += Codec::template decode_ref<q>(half_of<S>(st[q * NH + h], hpar), ref, dev);
-                    });
-                    rring[slot_of(z) * PLANE + h_slot] = r;
-                } else {
-                    static_for<0, Q>([&](auto qc) {
-                        constexpr int q = decltype(qc)::value;
-                        if constexpr (L::kWord)
-                            r += Codec::template decode<q>(half_of<S>(st[q * NH + h], hpar), dev);
-                        else
-                            r += Codec::template decode<q>(st[q * NH + h], dev);
-                    });
-                }
+                float ref = 0.0f;
+                if constexpr (LOCAL) ref = rstage[stage_of(z) * NH + h];
+                const R r = density_of<R>([&](auto qc) {
+                    constexpr int q = decltype(qc)::value;
+                    if constexpr (LOCAL)
+                        return Codec::template decode_ref<q>(half_of<S>(st[q * NH + h], hpar), ref, dev);
+                    else if constexpr (L::kWord)
+                        return Codec::template decode<q>(half_of<S>(st[q * NH + h], hpar), dev);
+                    else
+                        return Codec::template decode<q>(st[q * NH + h], dev);
+                });
+                if constexpr (LOCAL) rring[slot_of(z) * PLANE + h_slot] = r;
                 ring[slot_of(z) * PLANE + h_slot] = psi_of<R>(r, rho0, inv_rho0);
             }
         };
@@ -867,11 +712,7 @@ sc_step_pipe_kernel(const typename Codec::S* __restrict__ src_all, typename Code
             }
         };
         auto own_psi = [&](const R (&f)[Q], int z) {
-            R r = R(0);
-            static_for<0, Q>([&](auto qc) {
-                constexpr int q = decltype(qc)::value;
-                r += f[q];
-            });
+            const R r = density_of<R>([&](auto qc) { return f[decltype(qc)::value]; });
             const R p = psi_of<R>(r, rho0, inv_rho0);
             ring[slot_of(z) * PLANE + my_slot] = p;
             if constexpr (LOCAL) rring[slot_of(z) * PLANE + my_slot] = r;
@@ -1177,18 +1018,10 @@ sc_step_bulk_kernel(const float* __restrict__ src, float* __restrict__ dst, cons
         auto slot_of = [&](int z) { return (z - zs + 1) & 3; };
         auto psi_from = [&](unsigned gi, int z) {
             const float* st = st_of(gi);
-            R r = R(0);
-            static_for<0, Q>([&](auto qc) {
-                constexpr int q = decltype(qc)::value;
-                r += st[q * ROWS * COLS + my_st];
-            });
+            const R r = density_of<R>(StridedAt<ROWS * COLS>{st + my_st});
             ring[slot_of(z) * PLANE + my_slot] = psi_of<R>(r, rho0, inv_rho0);
             if (h_slot >= 0) {
-                R rh = R(0);
-                static_for<0, Q>([&](auto qc) {
-                    constexpr int q = decltype(qc)::value;
-                    rh += st[q * ROWS * COLS + h_st];
-                });
+                const R rh = density_of<R>(StridedAt<ROWS * COLS>{st + h_st});
                 ring[slot_of(z) * PLANE + h_slot] = psi_of<R>(rh, rho0, inv_rho0);
             }
         };
@@ -1347,19 +1180,11 @@ sc_step_tma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __rest
         auto psi_from = [&](int p) {
             const int s = gi_of(p) % NS;
             const float* st = istage + s * L::stage_floats;
-            R r = R(0);
-            static_for<0, Q>([&](auto qc) {
-                constexpr int q = decltype(qc)::value;
-                r += st[q * NT + my_st];
-            });
+            const R r = density_of<R>(StridedAt<NT>{st + my_st});
             ring[slot_of(p) * PLANE + my_slot] = psi_of<R>(r, rho0, inv_rho0);
             if (h_slot >= 0) {
                 const float* hs = hstage + s * (Q * NH);
-                R rh = R(0);
-                static_for<0, Q>([&](auto qc) {
-                    constexpr int q = decltype(qc)::value;
-                    rh += hs[q * NH + h];
-                });
+                const R rh = density_of<R>(StridedAt<NH>{hs + h});
                 ring[slot_of(p) * PLANE + h_slot] = psi_of<R>(rh, rho0, inv_rho0);
             }
         };

@@ -12,27 +12,42 @@
 // second moment cs2, so the bulk equation of state is
 // P = rho cs2 + cs2 (G1 + G2) psi^2 / 2 whatever the split of G1 + G2.
 //
-// Register-staged like sc_step_kernel, with a two-cell psi halo: a ring of
-// eight planes of (TX + 4) x (TY + 4) psi values in shared memory (TY = 8 or
-// 16: both 17.6 GLUPS for FP32 at 256 x 256 x 575 on GB300; summing the
-// neighbours per shell before the coefficients measured 16.2 / 13.6); each
-// iteration fills plane z + 2 (every slot from its cell's 19 populations),
-// loads the populations of plane z, and after one barrier computes the force
-// from the 92 neighbours of planes z - 2 .. z + 2, collides and pushes (the
-// streaming itself is the D3Q19 one).
+// Two kernels per step.  sc_psi_kernel turns the populations into a field of
+// psi (80 B a cell); sc_step_mr_kernel then reads one value per cell and
+// two-cell halo instead of summing 19 populations 1.7 times a cell.  It
+// marches along z with two planes of (TX + 4) x (TY + 4) psi values in shared
+// memory.  What plane p contributes to the force at distance 0, 1 and 2 along
+// z differs only in the coefficients of the same five in-plane sums (by
+// a^2 + b^2 of the offset (a, b)), so each thread reads its 5 x 5 patch of a
+// plane once and adds to the forces of planes p - 2 .. p + 2: 25 shared loads
+// and ~110 operations per cell where the 92 neighbours one by one took 92 and
+// ~260.  Plane p - 2 then has its force, is collided and pushed (the streaming
+// itself is the D3Q19 one).
+//
+// Without the psi field (no memory for it) the halo planes are summed from
+// the populations as before.
 #pragma once
 #include "e8.cuh"
 #include "step_kernel.cuh"
 
 namespace lbm {
 
+template <class Codec>
+__global__ void __launch_bounds__(256)
+sc_psi_kernel(const typename Codec::S* __restrict__ f, typename Codec::R* __restrict__ psi, const StepArgs a) {
+    using R = typename Codec::R;
+    const R rho0 = par<R>(a.rho0, a.rho0f), inv_rho0 = par<R>(a.inv_rho0, a.inv_rho0f);
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < a.n; i += gridDim.x * 256LL)
+        psi[i] = psi_of<R>(cell_density<Codec>(f + i, a.n, a.dev), rho0, inv_rho0);
+}
+
 template <class Codec, int COLL, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY)
+__global__ void __launch_bounds__(TX * TY, sizeof(typename Codec::R) == 4 ? 512 / (TX * TY) : 1)
 sc_step_mr_kernel(const typename Codec::S* __restrict__ src, typename Codec::S* __restrict__ dst, const StepArgs a) {
     using R = typename Codec::R;
     static_assert(!Codec::kLocal, "the multirange kernel stores populations directly");
-    constexpr int NT = TX * TY, PX = TX + 4, PY = TY + 4, PLANE = PX * PY, NSLOT = 8;
-    __shared__ R psi_s[NSLOT][PLANE];
+    constexpr int NT = TX * TY, PX = TX + 4, PY = TY + 4, PLANE = PX * PY, NS = (PLANE + NT - 1) / NT;
+    __shared__ R psi_s[2][PLANE];
 
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
@@ -55,55 +70,86 @@ sc_step_mr_kernel(const typename Codec::S* __restrict__ src, typename Codec::S* 
 
     const R rho0 = par<R>(a.rho0, a.rho0f), inv_rho0 = par<R>(a.inv_rho0, a.inv_rho0f);
     const DevParams dev = a.dev;
+    const R* const psi_ws = static_cast<const R*>(a.psi_ws);
     // G1 w(s) + G2 p(s) / 3 per shell s = |e|^2
-    R coef[9];
+    R c[9];
 #pragma unroll
-    for (int s = 0; s < 9; ++s) coef[s] = R(a.G * mr::w_d3q19(s) + a.G2 * mr::p_e8(s) / 3.0);
+    for (int s = 0; s < 9; ++s) c[s] = R(a.G * mr::w_d3q19(s) + a.G2 * mr::p_e8(s) / 3.0);
 
-    auto wrapz = [&](int z) { return wrap_index(z, nz); };
-    auto slot_of = [&](int z) { return (z - zs + 2) & (NSLOT - 1); };
-    // psi of every slot (tile and two-cell halo) of plane z
-    auto fill = [&](int z) {
-        const long long zo = (long long)wrapz(z) * plane;
-        R* ps = psi_s[slot_of(z)];
-        for (int s = tid; s < PLANE; s += NT) {
-            const int sx = s % PX - 2, sy = s / PX - 2;
-            const long long cell = (long long)wrap_index(y0 + sy, ny) * nx + wrap_index(x0 + sx, nx);
-            ps[s] = psi_of<R>(cell_density<Codec>(src + zo + cell, n, dev), rho0, inv_rho0);
-        }
+    // cells of the psi plane that this thread fills
+    long long cell[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        const int s = min(tid + k * NT, PLANE - 1);
+        cell[k] = (long long)wrap_index(y0 + s / PX - 2, ny) * nx + wrap_index(x0 + s % PX - 2, nx);
+    }
+    R v[NS];  // psi of the next plane, on its way
+    auto fetch = [&](int z) {
+        const long long zo = (long long)wrap_index(z, nz) * plane;
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            v[k] = psi_ws ? __ldg(psi_ws + zo + cell[k])
+                          : psi_of<R>(cell_density<Codec>(src + zo + cell[k], n, dev), rho0, inv_rho0);
     };
 
-    for (int z = zs - 2; z <= zs + 1; ++z) fill(z);
-    for (int z = zs; z < ze; ++z) {
-        fill(z + 2);
-        R fc[Q];
-        const long long zo = (long long)z * plane;
-        static_for<0, Q>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            fc[q] = Codec::template load<q>(src + q * n + zo + my_xy, dev);
-        });
+    // Force sums of planes p - 2 .. p + 1 so far (ax[0]: p - 2), and psi of planes p - 1, p - 2.
+    R ax[4] = {}, ay[4] = {}, az[4] = {}, c1 = R(0), c2 = R(0);
+    fetch(zs - 2);
+    // One plane: fc holds the populations of plane p - 2; those of plane p - 1 are loaded into fl meanwhile.
+    auto turn = [&](R (&fc)[Q], R (&fl)[Q], int p) {
+        R* const buf = psi_s[p & 1];
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            if (tid + k * NT < PLANE) buf[tid + k * NT] = v[k];
         __syncthreads();
-        if (active) {
-            const R* pl[5] = {psi_s[slot_of(z - 2)], psi_s[slot_of(z - 1)], psi_s[slot_of(z)],
-                              psi_s[slot_of(z + 1)], psi_s[slot_of(z + 2)]};
-            R sx = R(0), sy = R(0), sz = R(0);
-            static_for<0, mr::kNE>([&](auto kc) {
-                constexpr mr::Vec e = mr::e8(decltype(kc)::value);
-                constexpr int s = e.x * e.x + e.y * e.y + e.z * e.z;
-                const R v = coef[s] * pl[e.z + 2][my_slot + e.x + e.y * PX];
-                if constexpr (e.x != 0) sx += R(e.x) * v;
-                if constexpr (e.y != 0) sy += R(e.y) * v;
-                if constexpr (e.z != 0) sz += R(e.z) * v;
+        if (p <= ze) fetch(p + 1);
+        const int z = p - 2;
+        const bool go = z >= zs && active;
+        const long long zo = (long long)z * plane;
+        if (z + 1 >= zs && z + 1 < ze) {
+            const typename Codec::S* const s1 = src + (zo + plane + my_xy);
+            static_for<0, Q>([&](auto qc) {
+                constexpr int q = decltype(qc)::value;
+                fl[q] = Codec::template load<q>(s1 + q * n, dev);
             });
-            const R mpsi = -pl[2][my_slot];
-            const R Fx = mpsi * sx, Fy = mpsi * sy, Fz = mpsi * sz;
-            if constexpr (COLL == COLL_SRT)
-                collide_srt<R>(fc, Fx, Fy, Fz, par<R>(a.tau, a.tauf), par<R>(a.omega, a.omegaf));
-            else if constexpr (COLL == COLL_MRT) collide_mrt<R>(fc, Fx, Fy, Fz, rates<R>(a));
-            else if constexpr (COLL == COLL_MRT_SPARSE) collide_mrt_sparse<R, false>(fc, Fx, Fy, Fz, rates<R>(a));
-            else if constexpr (COLL == COLL_MRT_SHEAR)
-                collide_mrt_sparse<R, false, false>(fc, Fx, Fy, Fz, rates<R>(a));
-            else collide_mrt_sparse<R, true>(fc, Fx, Fy, Fz, rates<R>(a));
+        }
+        const R* const b = buf + my_slot;
+        auto at = [&](int dx, int dy) { return b[dx + dy * PX]; };
+        const R v00 = at(0, 0);
+        // opposite neighbours along x (u) and y (w), by shell: differences and sums
+        const R d1x = at(1, 0) - at(-1, 0), d1y = at(0, 1) - at(0, -1);
+        const R S1 = (at(1, 0) + at(-1, 0)) + (at(0, 1) + at(0, -1));
+        const R e1 = at(1, 1) - at(-1, -1), e2 = at(1, -1) - at(-1, 1);
+        const R g2x = e1 + e2, g2y = e1 - e2;
+        const R S2 = (at(1, 1) + at(-1, -1)) + (at(1, -1) + at(-1, 1));
+        const R d4x = R(2) * (at(2, 0) - at(-2, 0)), d4y = R(2) * (at(0, 2) - at(0, -2));
+        const R S4 = (at(2, 0) + at(-2, 0)) + (at(0, 2) + at(0, -2));
+        const R h1 = at(2, 1) - at(-2, -1), h2 = at(2, -1) - at(-2, 1);
+        const R i1 = at(1, 2) - at(-1, -2), i2 = at(1, -2) - at(-1, 2);
+        const R g5x = R(2) * (h1 + h2) + (i1 + i2), g5y = (h1 - h2) + R(2) * (i1 - i2);
+        const R S5 = ((at(2, 1) + at(-2, -1)) + (at(2, -1) + at(-2, 1))) +
+                     ((at(1, 2) + at(-1, -2)) + (at(1, -2) + at(-1, 2)));
+        const R k1 = at(2, 2) - at(-2, -2), k2 = at(2, -2) - at(-2, 2);
+        const R g8x = R(2) * (k1 + k2), g8y = R(2) * (k1 - k2);
+
+        const R X2 = c[5] * d1x + c[6] * g2x + c[8] * d4x, Y2 = c[5] * d1y + c[6] * g2y + c[8] * d4y;
+        const R X1 = c[2] * d1x + c[3] * g2x + c[5] * d4x + c[6] * g5x;
+        const R Y1 = c[2] * d1y + c[3] * g2y + c[5] * d4y + c[6] * g5y;
+        const R X0 = c[1] * d1x + c[2] * g2x + c[4] * d4x + c[5] * g5x + c[8] * g8x;
+        const R Y0 = c[1] * d1y + c[2] * g2y + c[4] * d4y + c[5] * g5y + c[8] * g8y;
+        const R Z1 = c[1] * v00 + c[2] * S1 + c[3] * S2 + c[5] * S4 + c[6] * S5;
+        const R Z2 = R(2) * (c[4] * v00 + c[5] * S1 + c[6] * S2 + c[8] * S4);
+
+        const Force<R> F{-c2, ax[0] + X2, ay[0] + Y2, az[0] + Z2};
+        ax[0] = ax[1] + X1; ay[0] = ay[1] + Y1; az[0] = az[1] + Z1;
+        ax[1] = ax[2] + X0; ay[1] = ay[2] + Y0; az[1] = az[2];
+        ax[2] = ax[3] + X1; ay[2] = ay[3] + Y1; az[2] = az[3] - Z1;
+        ax[3] = X2;         ay[3] = Y2;         az[3] = -Z2;
+        c2 = c1;
+        c1 = v00;
+
+        if (go) {
+            collide<COLL, R>(fc, F, a);
             // Eq. LBE streaming: f_a(x + c_a, t + 1) = f*_a(x, t).
             const int zm = (z == 0) ? nz - 1 : z - 1, zn = (z + 1 == nz) ? 0 : z + 1;
             const long long zoff[3] = {(long long)zm * plane, zo, (long long)zn * plane};
@@ -113,6 +159,11 @@ sc_step_mr_kernel(const typename Codec::S* __restrict__ src, typename Codec::S* 
                 Codec::template store<q>(dst + (q * n + idx), fc[q], a.dev);
             });
         }
+    };
+    R fa[Q], fb[Q];
+    for (int p = zs - 2; p <= ze + 1; p += 2) {
+        turn(fa, fb, p);
+        if (p + 1 <= ze + 1) turn(fb, fa, p + 1);
     }
 }
 

@@ -162,16 +162,14 @@ sc_step_pair16_kernel(const typename Codec::S* __restrict__ src, typename Codec:
         };
         // density of one half of a raw word, summed in population order
         auto dens = [&](const uint32_t (&w)[Q], int hi, float ref) {
-            R r = R(0);
-            static_for<0, Q>([&](auto qc) {
+            return density_of<R>([&](auto qc) {
                 constexpr int q = decltype(qc)::value;
                 S v0, v1;
                 pair16::halves(w[q], v0, v1);
                 const S v = hi ? v1 : v0;
-                if constexpr (LOCAL) r += Codec::template decode_ref<q>(v, ref, dev);
-                else r += Codec::template decode<q>(v, dev);
+                if constexpr (LOCAL) return Codec::template decode_ref<q>(v, ref, dev);
+                else return Codec::template decode<q>(v, dev);
             });
-            return r;
         };
         auto halo_psi = [&](int z) {
             if (h_on) {
@@ -243,22 +241,17 @@ sc_step_pair16_kernel(const typename Codec::S* __restrict__ src, typename Codec:
                     (void)r.y;
                 }
             });
-            R F[2][3];
+            Force<R> F[2];
             static_for<0, 2>([&](auto cc) {
                 constexpr int c = decltype(cc)::value;
-                // Eq. SC_force, in the order of update_cell
-                R sx = R(0), sy = R(0), sz = R(0);
-                static_for<1, Q>([&](auto qc) {
-                    constexpr int q = decltype(qc)::value;
-                    const R vq = v[cz(q) + 1][cy(q) + 1][2 + c + cx(q)];
-                    if constexpr (cx(q) != 0) sx += R(wq(q) * cx(q)) * vq;
-                    if constexpr (cy(q) != 0) sy += R(wq(q) * cy(q)) * vq;
-                    if constexpr (cz(q) != 0) sz += R(wq(q) * cz(q)) * vq;
+                PsiView<R> w3[3];
+                static_for<0, 3>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    w3[k].c = v[k][1][2 + c];
+                    psi_axis(w3[k], PsiAt<R, 6>{&v[k][1][2 + c]});
+                    if constexpr (k == 1) psi_diag(w3[k], PsiAt<R, 6>{&v[k][1][2 + c]});
                 });
-                const R gpsi = -a.Gf * v[1][1][2 + c];
-                F[c][0] = gpsi * sx;
-                F[c][1] = gpsi * sy;
-                F[c][2] = gpsi * sz;
+                F[c] = force_of(w3[0], w3[1], w3[2], a.gwf);
             });
 
             const int zm = (z == 0) ? nz - 1 : z - 1;
@@ -279,13 +272,7 @@ sc_step_pair16_kernel(const typename Codec::S* __restrict__ src, typename Codec:
                     if constexpr (LOCAL) f[q] = Codec::template decode_ref<q>(sv, rf, dev);
                     else f[q] = Codec::template decode<q>(sv, dev);
                 });
-                if constexpr (COLL == COLL_SRT) collide_srt<R>(f, F[c][0], F[c][1], F[c][2], a.tauf, a.omegaf);
-                else if constexpr (COLL == COLL_MRT) collide_mrt<R>(f, F[c][0], F[c][1], F[c][2], a.sf);
-                else if constexpr (COLL == COLL_MRT_SPARSE)
-                    collide_mrt_sparse<R, false>(f, F[c][0], F[c][1], F[c][2], a.sf);
-                else if constexpr (COLL == COLL_MRT_SHEAR)
-                    collide_mrt_sparse<R, false, false>(f, F[c][0], F[c][1], F[c][2], a.sf);
-                else collide_mrt_sparse<R, true>(f, F[c][0], F[c][1], F[c][2], a.sf);
+                collide<COLL, R>(f, F[c], a);
                 static_for<0, Q>([&](auto qc) {
                     constexpr int q = decltype(qc)::value;
                     if constexpr (LOCAL) {
