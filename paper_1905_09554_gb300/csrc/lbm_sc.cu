@@ -50,6 +50,12 @@ struct lbm_ctx {
     int grid3 = 0;                    // kernel 5: grid of the pipelined kernel used for other buffers
     int coll = COLL_SRT;              // collision kernel (COLL_*)
     int grid = 0;                     // persistent grid size (kernels 2, 3)
+    // Calls of several steps through the moment fields (step_moment.cuh):
+    // launch shape, or mom == nullptr where only populations will do.
+    const MomentKernels* mom = nullptr;
+    MomentLaunch mom_launch{};
+    size_t mom_bytes = 0;             // one set of moment fields
+    bool mom_twice = false;           // two sets fit into one population copy
     char err[512] = {0};
     lbm_batch* batch = nullptr;       // set when the context is a view of a batch box
     // discrete adjoint (allocated by lbm_adjoint_forward)
@@ -443,10 +449,10 @@ lbm_status check_device_error(lbm_ctx* c) {
     return LBM_OK;
 }
 
-// Planes (plus one per work item for the two halo planes it reads first)
+// Planes (plus `extra` per work item for the halo planes it goes through first)
 // on the busiest block when `grid` persistent blocks take the work items
 // (tile, chunk of z planes), numbered chunk-major, round-robin.
-long long busiest_block_planes(long long nz, long long tiles, long long grid, long long zc) {
+long long busiest_block_planes(long long nz, long long tiles, long long grid, long long zc, long long extra = 1) {
     if (grid < 1 || tiles < 1 || zc < 1) return 0;
     const long long chunks = (nz + zc - 1) / zc, last = nz - (chunks - 1) * zc;
     const long long items = tiles * chunks;
@@ -455,7 +461,7 @@ long long busiest_block_planes(long long nz, long long tiles, long long grid, lo
     long long worst = 0;
     for (long long b = 0; b < grid; ++b) {
         const long long n = items / grid + (b < items % grid ? 1 : 0);
-        const long long load = n * (zc + 1) - (zc - last) * in_last[b];
+        const long long load = n * (zc + extra) - (zc - last) * in_last[b];
         if (load > worst) worst = load;
     }
     return worst;
@@ -612,6 +618,88 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
     if (c->kernel >= 2 && c->grid > a.n_items) c->grid = a.n_items;
     if (c->grid3 > a.n_items) c->grid3 = a.n_items;
 
+    return LBM_OK;
+}
+
+// Launch shape of the moment kernels (step_moment.cuh), where the collision
+// has a moment form and its fields fit into a population copy.  A context
+// created for one particular step kernel keeps to it.
+void configure_moments(lbm_ctx* c) {
+    const lbm_params& p = c->p;
+    c->mom = nullptr;
+    if (p.kernel != 0 || p.G2 != 0.0 || p.nx < 4) return;
+    if (c->coll == COLL_SRT && p.tau != 1.0) return;  // keeps (1 - omega) f: all 19 populations
+    const MomentKernels* k = moment_kernels(p.storage, c->coll);
+    if (!k) return;
+    const long long pitch = ((p.nx + 3) & ~3) + 4, cells = pitch * p.ny * p.nz;  // moment_pitch
+    c->mom_bytes = (size_t)k->fields * (size_t)cells * sizeof(float);
+    const size_t copy = (size_t)Q * (size_t)c->n * c->elem;
+    if (cells > 0xffffffffLL || c->mom_bytes > copy) return;
+    c->mom_twice = 2 * c->mom_bytes <= copy;
+    MomentLaunch& l = c->mom_launch;
+    l = MomentLaunch{};
+    const int per_sm = k->prepare(false);
+    if (per_sm < 1) {
+        cudaGetLastError();
+        return;
+    }
+    l.args = c->args;
+    l.args.tiles_x = (p.nx + k->tile_x - 1) / k->tile_x;
+    l.args.n_tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
+    const long long grid = (long long)per_sm * c->num_sms;
+    long long best = -1;
+    for (int z = p.nz < 128 ? p.nz : 128; z >= 1; --z) {
+        const long long load = busiest_block_planes(p.nz, l.args.n_tiles, grid, z, 4);
+        if (best < 0 || load < best) {
+            best = load;
+            l.args.zchunk = z;
+        }
+    }
+    l.args.n_items = l.args.n_tiles * ((p.nz + l.args.zchunk - 1) / l.args.zchunk);
+    l.grid = int(grid < l.args.n_items ? grid : l.args.n_items);
+    const long long rows = ((long long)p.ny * p.nz + 7) / 8;
+    l.gather_grid = int(rows < 8LL * c->num_sms ? rows : 8LL * c->num_sms);
+    c->mom = k;
+}
+
+// n >= 2 steps through the moment fields.  The state ends in the copy that n
+// single steps would leave it in, so that a call captured into a graph can be
+// replayed as before.
+lbm_status step_moments(lbm_ctx* c, long nsteps) {
+    MomentLaunch l = c->mom_launch;
+    l.stream = c->stream;
+    const int from = c->cur, to = c->cur ^ int(nsteps & 1);
+    l.args.ref_src = c->ref[from];
+    l.args.ref_dst = c->ref[to];
+    void* const src = c->f[from];
+    void* const other = c->f[from ^ 1];
+    LBM_CUDA(c, c->mom->gather(l, src, other));
+    // the fields end in the copy that does not receive the populations
+    void* at = other;
+    int hi = 0;
+    if (!c->mom_twice) {  // one set per copy: the sets alternate between the copies, starting in the first
+        LBM_CUDA(c, cudaMemcpyAsync(src, other, c->mom_bytes, cudaMemcpyDeviceToDevice, c->stream));
+        at = src;
+    }
+    for (long k = 1; k < nsteps; ++k) {
+        void* nxt = at;
+        l.src_hi = hi;
+        if (!c->mom_twice) {
+            nxt = at == src ? other : src;
+        } else if (k + 1 == nsteps && (nsteps & 1)) {
+            nxt = src;
+            hi = 0;
+        } else {
+            hi ^= 1;
+        }
+        l.dst_hi = hi;
+        LBM_CUDA(c, c->mom->step(l, at, nxt));
+        at = nxt;
+    }
+    l.src_hi = hi;
+    LBM_CUDA(c, c->mom->emit(l, at, c->f[to]));
+    c->cur = to;
+    c->t += nsteps;
     return LBM_OK;
 }
 
@@ -808,6 +896,8 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
             return st;
         }
     }
+
+    configure_moments(c);
 
     e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1091,6 +1181,7 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (!c) return LBM_EINVAL;
     if (nsteps < 0) return c->fail(LBM_EINVAL, "lbm_step: n must be >= 0");
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_step: this context is a box of a batch; use lbm_batch_step");
+    if (nsteps >= 2 && c->mom) return step_moments(c, nsteps);
     for (long k = 0; k < nsteps; ++k) {
         cudaError_t e = launch_step(c, c->f[c->cur], c->f[c->cur ^ 1]);
         if (e != cudaSuccess) return c->fail(LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));

@@ -118,4 +118,30 @@ struct StepKernels {
 // storage: LBM_F64 .. LBM_BF16_LOCAL (0..5); coll: COLL_SRT .. COLL_MRT_SHEAR.
 const StepKernels& step_kernels(int storage, int coll);
 
+// Launch description of the moment kernels (step_moment.cuh).  args.tiles_x,
+// n_tiles, n_items and zchunk are those of the moment kernel's tiles; boxes:
+// the batch's box table (nbox > 0) with work items of the same tiles.
+struct MomentLaunch {
+    StepArgs args;
+    BatchArgs batch;
+    int grid;             // persistent grid of the step
+    int gather_grid;      // blocks (per box) of the populations -> moments pass
+    int src_hi, dst_hi;   // which of a copy's two sets of moment fields
+    cudaStream_t stream;
+};
+
+struct MomentKernels {
+    // opts the step kernels in to their shared memory and returns their
+    // resident blocks per SM (0 or less: cannot run)
+    int (*prepare)(bool batch);
+    cudaError_t (*gather)(const MomentLaunch& l, const void* pops, void* moments);
+    cudaError_t (*step)(const MomentLaunch& l, const void* moments, void* out);
+    cudaError_t (*emit)(const MomentLaunch& l, const void* moments, void* pops);
+    int fields;           // moment fields of the collision
+    int tile_x, tile_y;   // an output tile
+};
+
+// nullptr where the collision (or the storage) has no moment form.
+const MomentKernels* moment_kernels(int storage, int coll);
+
 }  // namespace lbm

@@ -34,6 +34,17 @@ extern const StepKernels kStep_bf16l_mrts;
 extern const StepKernels kStep_bf16l_mrtu;
 extern const StepKernels kStep_bf16l_mrtsh;
 
+extern const MomentKernels kMoment_f32_srt;
+extern const MomentKernels kMoment_f32_mrts;
+extern const MomentKernels kMoment_f32_mrtu;
+extern const MomentKernels kMoment_f32_mrtsh;
+
+const MomentKernels* moment_kernels(int storage, int coll) {
+    static const MomentKernels* f32[COLL_COUNT] = {&kMoment_f32_srt, nullptr, &kMoment_f32_mrts, &kMoment_f32_mrtu,
+                                                   &kMoment_f32_mrtsh};
+    return storage == 1 ? f32[coll] : nullptr;
+}
+
 const StepKernels& step_kernels(int storage, int coll) {
     static const StepKernels* table[6][COLL_COUNT] = {
         {&kStep_f64_srt, &kStep_f64_mrt, &kStep_f64_mrts, &kStep_f64_mrtu, &kStep_f64_mrtsh},

@@ -1,0 +1,46 @@
+"""Calls of several steps go through the moment fields where the collision
+forgets the other populations (SRT at tau = 1; MRT whose rates outside
+{e, 3pxx, pww, pxy, pyz, pxz} are 1).  They must leave exactly the populations
+that single steps of the register-staged population kernel leave.
+
+Boxes: smaller than a tile, odd and ragged sides, one past a tile, a box whose
+rows are shorter than two tiles apart, nz from 1 up; even and odd numbers of
+steps (the state ends in the copy that single steps would use)."""
+
+import numpy as np
+import pytest
+
+from oracle import lbm_oracle as o
+from paper_1905_09554_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - CUDA device only
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1905_09554_gb300 import lbm  # noqa: E402
+
+OPS = {"srt": dict(collision="srt", tau=1.0), "unit": dict(collision="mrt", tau=1.0),
+       "paper": dict(collision="mrt", tau=0.8), "shear": dict(collision="mrt", tau=0.8, rates=o.mrt_rates(0.8, rule="shear"))}
+BOXES = [(4, 1, 1), (5, 3, 2), (6, 14, 9), (33, 13, 5), (32, 26, 33), (65, 15, 7), (97, 31, 21), (128, 40, 130)]
+
+
+def _state(box, kernel, calls, storage="f32", **op):
+    nx, ny, nz = box
+    rho = inputs.random_density(nx, ny, nz, seed=7, lo=0.3, hi=1.9)
+    with lbm.Lattice(nx, ny, nz, G=-5.5, storage=storage, kernel=kernel, **op) as L:
+        L.set_density(rho)
+        for n in calls:
+            L.step(n)
+        return L.get_populations(), lbm.lbm_current_copy(L.ctx), L.time
+
+
+@pytest.mark.parametrize("op", list(OPS))
+@pytest.mark.parametrize("box", BOXES)
+def test_many_steps_at_once_equal_single_steps(box, op):
+    for calls in ((2,), (3,), (1, 6, 3)):
+        want, copy, t = _state(box, 1, [1] * sum(calls), **OPS[op])
+        got, copy2, t2 = _state(box, 0, calls, **OPS[op])
+        assert (copy, t) == (copy2, t2)
+        assert np.array_equal(got, want), (calls, np.abs(got - want).max())
