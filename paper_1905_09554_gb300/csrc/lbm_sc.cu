@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdarg>
@@ -631,7 +632,7 @@ void configure_moments(lbm_ctx* c) {
     if (c->coll == COLL_SRT && p.tau != 1.0) return;  // keeps (1 - omega) f: all 19 populations
     const MomentKernels* k = moment_kernels(p.storage, c->coll);
     if (!k) return;
-    const long long pitch = ((p.nx + 3) & ~3) + 4, cells = pitch * p.ny * p.nz;  // moment_pitch
+    const long long cells = moment_cells(p.nx, p.ny, p.nz);
     c->mom_bytes = (size_t)k->fields * (size_t)cells * sizeof(float);
     const size_t copy = (size_t)Q * (size_t)c->n * c->elem;
     if (cells > 0xffffffffLL || c->mom_bytes > copy) return;
@@ -662,42 +663,49 @@ void configure_moments(lbm_ctx* c) {
     c->mom = k;
 }
 
-// n >= 2 steps through the moment fields.  The state ends in the copy that n
-// single steps would leave it in, so that a call captured into a graph can be
-// replayed as before.
-lbm_status step_moments(lbm_ctx* c, long nsteps) {
-    MomentLaunch l = c->mom_launch;
-    l.stream = c->stream;
-    const int from = c->cur, to = c->cur ^ int(nsteps & 1);
-    l.args.ref_src = c->ref[from];
-    l.args.ref_dst = c->ref[to];
-    void* const src = c->f[from];
-    void* const other = c->f[from ^ 1];
-    LBM_CUDA(c, c->mom->gather(l, src, other));
-    // the fields end in the copy that does not receive the populations
+// n >= 2 steps from the populations in f[from] through the moment fields.  The
+// state ends in the copy that n single steps would leave it in (returned in
+// *to), so that a call captured into a graph can be replayed as before.
+// bytes: of one set of moment fields; twice: two sets fit into a copy.
+cudaError_t run_moments(const MomentKernels& k, MomentLaunch l, void* const (&f)[2], int from, long nsteps,
+                        size_t bytes, bool twice, int* to) {
+    *to = from ^ int(nsteps & 1);
+    void* const src = f[from];
+    void* const other = f[from ^ 1];
+    cudaError_t e = k.gather(l, src, other);
+    // the fields have to end in the copy that does not receive the populations
     void* at = other;
     int hi = 0;
-    if (!c->mom_twice) {  // one set per copy: the sets alternate between the copies, starting in the first
-        LBM_CUDA(c, cudaMemcpyAsync(src, other, c->mom_bytes, cudaMemcpyDeviceToDevice, c->stream));
+    if (e == cudaSuccess && !twice) {  // one set a copy: they alternate between the copies, starting in the first
+        e = cudaMemcpyAsync(src, other, bytes, cudaMemcpyDeviceToDevice, l.stream);
         at = src;
     }
-    for (long k = 1; k < nsteps; ++k) {
+    for (long i = 1; i < nsteps && e == cudaSuccess; ++i) {
         void* nxt = at;
         l.src_hi = hi;
-        if (!c->mom_twice) {
+        if (!twice) {
             nxt = at == src ? other : src;
-        } else if (k + 1 == nsteps && (nsteps & 1)) {
+        } else if (i + 1 == nsteps && (nsteps & 1)) {
             nxt = src;
             hi = 0;
         } else {
             hi ^= 1;
         }
         l.dst_hi = hi;
-        LBM_CUDA(c, c->mom->step(l, at, nxt));
+        e = k.step(l, at, nxt);
         at = nxt;
     }
     l.src_hi = hi;
-    LBM_CUDA(c, c->mom->emit(l, at, c->f[to]));
+    return e == cudaSuccess ? k.emit(l, at, f[*to]) : e;
+}
+
+lbm_status step_moments(lbm_ctx* c, long nsteps) {
+    MomentLaunch l = c->mom_launch;
+    l.stream = c->stream;
+    l.args.ref_src = c->ref[c->cur];
+    l.args.ref_dst = c->ref[c->cur ^ int(nsteps & 1)];
+    int to = 0;
+    LBM_CUDA(c, run_moments(*c->mom, l, c->f, c->cur, nsteps, c->mom_bytes, c->mom_twice, &to));
     c->cur = to;
     c->t += nsteps;
     return LBM_OK;
@@ -1301,6 +1309,11 @@ struct lbm_batch {
     BatchBox* boxes_dev = nullptr;
     StepArgs phys{};
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // two-step cycle starting from copy 0 / 1
+    // steps through the moment fields (nullptr: not for these boxes or this operator)
+    const MomentKernels* mom = nullptr;
+    MomentLaunch mom_launch{};
+    BatchBox* mom_boxes_dev = nullptr;
+    bool mom_twice = false;
     char err[512] = {0};
 
     lbm_status fail(lbm_status s, const char* fmt, ...) {
@@ -1375,6 +1388,86 @@ lbm_status batch_configure(lbm_batch* b, int ty, int zc) {
     b->bargs.boxes = b->boxes_dev;
     b->grid = per_sm * b->num_sms < items ? per_sm * b->num_sms : items;
     batch_drop_graphs(b);
+    return LBM_OK;
+}
+
+// The moment kernels' own table of work items (their tiles differ from the
+// population kernels'), where every box's fields fit into its populations.
+lbm_status batch_configure_moments(lbm_batch* b) {
+    const lbm_params& p = b->p;
+    const int coll = b->box[0]->coll;
+    if (p.kernel != 0 || (coll == COLL_SRT && p.tau != 1.0)) return LBM_OK;
+    const MomentKernels* k = moment_kernels(p.storage, coll);
+    if (!k) return LBM_OK;
+    b->mom_twice = true;
+    long long max_rows = 1, max_nz = 1;
+    for (const lbm_ctx* c : b->box) {
+        const lbm_params& q = c->p;
+        const long long fields = (long long)k->fields * moment_cells(q.nx, q.ny, q.nz), pops = (long long)Q * c->n;
+        if (q.nx < 4 || fields > pops) return LBM_OK;
+        if (2 * fields > pops) b->mom_twice = false;
+        const long long rows = (long long)q.ny * q.nz;
+        if (rows > max_rows) max_rows = rows;
+        if (q.nz > max_nz) max_nz = q.nz;
+    }
+    const int per_sm = k->prepare(true);
+    if (per_sm < 1) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    const long long grid = (long long)per_sm * b->num_sms;
+    auto tiles_of = [&](const lbm_params& q) {
+        return ((q.nx + k->tile_x - 1) / k->tile_x) * ((q.ny + k->tile_y - 1) / k->tile_y);
+    };
+    // The chunk that puts the fewest planes on the busiest block (each item also goes through ~4 planes that
+    // are not its own), items dealt round-robin in box order.
+    int zc = 1;
+    long long best = -1;
+    std::vector<long long> load(grid);
+    for (int z = int(max_nz < 96 ? max_nz : 96); z >= 1; z = z > 24 ? z - 4 : z - 1) {
+        std::fill(load.begin(), load.end(), 0);
+        long long item = 0;
+        for (const lbm_ctx* c : b->box) {
+            const int tiles = tiles_of(c->p);
+            for (int zs = 0; zs < c->p.nz; zs += z)
+                for (int t = 0; t < tiles; ++t) load[item++ % grid] += (z < c->p.nz - zs ? z : c->p.nz - zs) + 4;
+        }
+        const long long worst = *std::max_element(load.begin(), load.end());
+        if (best < 0 || worst < best) {
+            best = worst;
+            zc = z;
+        }
+    }
+    std::vector<BatchBox> boxes(b->count);
+    int items = 0;
+    for (int i = 0; i < b->count; ++i) {
+        const lbm_params& q = b->box[i]->p;
+        BatchBox& bx = boxes[i];
+        bx.nx = q.nx;
+        bx.ny = q.ny;
+        bx.nz = q.nz;
+        bx.tiles_x = (q.nx + k->tile_x - 1) / k->tile_x;
+        bx.n_tiles = tiles_of(q);
+        bx.zchunk = zc < q.nz ? zc : q.nz;
+        bx.item_begin = items;
+        bx.base = b->base[i];
+        bx.n = b->box[i]->n;
+        items += bx.n_tiles * ((q.nz + bx.zchunk - 1) / bx.zchunk);
+    }
+    if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
+    LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
+                                b->stream));
+    LBM_CUDA(b, cudaStreamSynchronize(b->stream));
+    MomentLaunch& l = b->mom_launch;
+    l = MomentLaunch{};
+    l.args = b->phys;
+    l.batch.nbox = b->count;
+    l.batch.n_items = items;
+    l.batch.boxes = b->mom_boxes_dev;
+    l.grid = int(grid < items ? grid : items);
+    const long long want = (max_rows + 7) / 8, cap = 1 + 16LL * b->num_sms / b->count;
+    l.gather_grid = int(want < cap ? want : cap);
+    b->mom = k;
     return LBM_OK;
 }
 
@@ -1481,6 +1574,7 @@ lbm_status lbm_batch_create(const lbm_params* p, int count, const int* dims, lbm
     const int ty = p->tile_y ? p->tile_y : (p->collision == LBM_MRT_GUO ? 4 : 8);
     const int zc = p->zchunk ? p->zchunk : 32;
     lbm_status st = batch_configure(b, ty, zc);
+    if (st == LBM_OK) st = batch_configure_moments(b);
     if (st != LBM_OK) {
         snprintf(g_create_err, sizeof(g_create_err), "%s", b->err);
         lbm_batch_destroy(b);
@@ -1503,6 +1597,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->f[0]);
     cudaFree(b->f[1]);
     cudaFree(b->boxes_dev);
+    cudaFree(b->mom_boxes_dev);
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
 }
@@ -1519,6 +1614,19 @@ lbm_status lbm_batch_box(lbm_batch* b, int i, lbm_ctx** view) {
 lbm_status lbm_batch_step(lbm_batch* b, long n) {
     if (!b) return LBM_EINVAL;
     if (n < 0) return b->fail(LBM_EINVAL, "lbm_batch_step: n must be >= 0");
+    if (n >= 2 && b->mom) {
+        MomentLaunch l = b->mom_launch;
+        l.stream = b->stream;
+        int to = 0;
+        LBM_CUDA(b, run_moments(*b->mom, l, b->f, b->cur, n, b->bytes, b->mom_twice, &to));
+        b->cur = to;
+        b->t += n;
+        for (lbm_ctx* c : b->box) {
+            c->cur = to;
+            c->t += n;
+        }
+        return LBM_OK;
+    }
     while (n >= 2) {
         if (!b->graph[b->cur]) {
             lbm_status st = batch_build_graph(b, b->cur);

@@ -118,6 +118,10 @@ struct StepKernels {
 // storage: LBM_F64 .. LBM_BF16_LOCAL (0..5); coll: COLL_SRT .. COLL_MRT_SHEAR.
 const StepKernels& step_kernels(int storage, int coll);
 
+// Row length of the moment fields, and the floats of one field.
+__host__ __device__ inline int moment_pitch(int nx) { return ((nx + 3) & ~3) + 4; }
+inline long long moment_cells(int nx, int ny, int nz) { return (long long)moment_pitch(nx) * ny * nz; }
+
 // Launch description of the moment kernels (step_moment.cuh).  args.tiles_x,
 // n_tiles, n_items and zchunk are those of the moment kernel's tiles; boxes:
 // the batch's box table (nbox > 0) with work items of the same tiles.

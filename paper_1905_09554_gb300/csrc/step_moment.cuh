@@ -40,8 +40,6 @@
 
 namespace lbm {
 
-__host__ __device__ inline int moment_pitch(int nx) { return ((nx + 3) & ~3) + 4; }
-
 template <int NV> struct VecOf;
 template <> struct VecOf<1> { using V = float; };
 template <> struct VecOf<2> { using V = F2; };

@@ -44,3 +44,23 @@ def test_many_steps_at_once_equal_single_steps(box, op):
         got, copy2, t2 = _state(box, 0, calls, **OPS[op])
         assert (copy, t) == (copy2, t2)
         assert np.array_equal(got, want), (calls, np.abs(got - want).max())
+
+
+@pytest.mark.parametrize("op", list(OPS))
+def test_batches_at_once_equal_single_steps(op):
+    """Every box of a batch against the same box alone on the register-staged kernel; one box has rows too
+    short for two sets of fields in a population copy."""
+    dims = [(32, 26, 33), (5, 3, 2), (64, 14, 20), (97, 31, 21), (48, 48, 7)]
+    rho = [inputs.random_density(*d, seed=30 + k, lo=0.3, hi=1.9) for k, d in enumerate(dims)]
+    with lbm.Batch(dims, G=-5.5, storage="f32", **OPS[op]) as B:
+        for v, r in zip(B.boxes, rho):
+            v.set_density(r)
+        for n in (1, 4, 3):
+            B.step(n)
+        got = [v.get_populations() for v in B.boxes]
+    for d, r, f in zip(dims, rho, got):
+        with lbm.Lattice(*d, G=-5.5, storage="f32", kernel=1, **OPS[op]) as L:
+            L.set_density(r)
+            for _ in range(8):
+                L.step(1)
+            assert np.array_equal(f, L.get_populations()), d
