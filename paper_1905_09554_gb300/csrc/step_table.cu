@@ -38,11 +38,27 @@ extern const MomentKernels kMoment_f32_srt;
 extern const MomentKernels kMoment_f32_mrts;
 extern const MomentKernels kMoment_f32_mrtu;
 extern const MomentKernels kMoment_f32_mrtsh;
+extern const MomentKernels kMoment_f16_srt;
+extern const MomentKernels kMoment_f16_mrtu;
+extern const MomentKernels kMoment_bf16_srt;
+extern const MomentKernels kMoment_bf16_mrtu;
+extern const MomentKernels kMoment_f16l_srt;
+extern const MomentKernels kMoment_f16l_mrtu;
+extern const MomentKernels kMoment_bf16l_srt;
+extern const MomentKernels kMoment_bf16l_mrtu;
 
+// 9 or 10 float moments (36 or 40 B) would not be less than 19 16-bit
+// populations (38 B): there only the operators with 4.
 const MomentKernels* moment_kernels(int storage, int coll) {
-    static const MomentKernels* f32[COLL_COUNT] = {&kMoment_f32_srt, nullptr, &kMoment_f32_mrts, &kMoment_f32_mrtu,
-                                                   &kMoment_f32_mrtsh};
-    return storage == 1 ? f32[coll] : nullptr;
+    static const MomentKernels* table[6][COLL_COUNT] = {
+        {},
+        {&kMoment_f32_srt, nullptr, &kMoment_f32_mrts, &kMoment_f32_mrtu, &kMoment_f32_mrtsh},
+        {&kMoment_f16_srt, nullptr, nullptr, &kMoment_f16_mrtu, nullptr},
+        {&kMoment_bf16_srt, nullptr, nullptr, &kMoment_bf16_mrtu, nullptr},
+        {&kMoment_f16l_srt, nullptr, nullptr, &kMoment_f16l_mrtu, nullptr},
+        {&kMoment_bf16l_srt, nullptr, nullptr, &kMoment_bf16l_mrtu, nullptr},
+    };
+    return table[storage][coll];
 }
 
 const StepKernels& step_kernels(int storage, int coll) {

@@ -46,6 +46,17 @@ def test_many_steps_at_once_equal_single_steps(box, op):
         assert np.array_equal(got, want), (calls, np.abs(got - want).max())
 
 
+@pytest.mark.parametrize("storage", ["f16", "bf16", "f16l", "bf16l"])
+@pytest.mark.parametrize("op", ["srt", "unit"])
+def test_16_bit_storage_is_rounded_at_every_step(storage, op):
+    """The populations between the steps of one call go through the storage's rounding too: same bits."""
+    for box in ((32, 26, 33), (6, 14, 9), (65, 15, 7), (130, 9, 5)):
+        for calls in ((2,), (1, 6, 3)):
+            want, _, _ = _state(box, 1, [1] * sum(calls), storage, **OPS[op])
+            got, _, _ = _state(box, 0, calls, storage, **OPS[op])
+            assert np.array_equal(got, want), (box, calls, np.abs(got - want).max())
+
+
 @pytest.mark.parametrize("op", list(OPS))
 def test_batches_at_once_equal_single_steps(op):
     """Every box of a batch against the same box alone on the register-staged kernel; one box has rows too
