@@ -57,6 +57,9 @@ struct lbm_ctx {
     MomentLaunch mom_launch{};
     size_t mom_bytes = 0;             // one set of moment fields
     bool mom_twice = false;           // two sets fit into one population copy
+    // FP64 steps in two kernels (step_split.cuh); in place where the moments
+    // are all a collision needs of the populations it overwrites.
+    bool split = false, split_in_place = false;
     char err[512] = {0};
     lbm_batch* batch = nullptr;       // set when the context is a view of a batch box
     // discrete adjoint (allocated by lbm_adjoint_forward)
@@ -365,6 +368,17 @@ cudaError_t launch_step(const lbm_ctx* c, const void* src, void* dst, void* psi_
     return step_kernels(c->p.storage, c->coll).launch(l, src, dst);
 }
 
+// One step src -> dst by the context's way of stepping.  keep_src: src is not
+// one of the context's own copies (a checkpoint, a recomputed state) and stays
+// as it is; psi_out then receives its psi where the step computes it.
+cudaError_t step_once(const lbm_ctx* c, void* src, void* dst, bool keep_src = false, void* psi_out = nullptr) {
+    if (!c->split) return launch_step(c, src, dst, psi_out);
+    void* psi = psi_out ? psi_out : c->psi_ws;
+    if (!keep_src && c->split_in_place) psi = nullptr;
+    SplitLaunch l{c->args, BatchArgs{}, unsigned(c->n), c->stream};
+    return split_step_f64(l, c->coll, src, dst, psi);
+}
+
 // Tensor maps of the two population copies for the tensor-copy kernel:
 // 4-D (x, y, z, population), FP32, box 32 x tile_y x 1 x 19.
 lbm_status encode_tensor_maps(lbm_ctx* c) {
@@ -467,6 +481,8 @@ long long busiest_block_planes(long long nz, long long tiles, long long grid, lo
     }
     return worst;
 }
+
+constexpr long long kSplitPad = 1024;  // block rounding of the two-kernel step's 32-bit cell index
 
 int auto_zchunk(const lbm_ctx* c) {
     const long long xy_blocks = (long long)((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y);
@@ -883,7 +899,11 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     round_params(a);
     c->coll = collision_kernel(*p, a.s);
-    if (p->G2 != 0.0) {  // psi of the whole box; the step runs without it, slower, where there is no room
+    // FP64 steps in two kernels unless one particular kernel was asked for
+    c->split = p->storage == LBM_F64 && p->kernel == 0 && p->G2 == 0.0 && n <= 0xffffffffLL - kSplitPad;
+    c->split_in_place = c->split && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p->tau != 1.0);
+    if (p->G2 != 0.0 || (c->split && !c->split_in_place)) {
+        // psi of the whole box; where there is no room the step runs without it, slower
         const size_t pbytes = (size_t)n * (p->storage == LBM_F64 ? 8 : 4);
         if (cudaMalloc(&c->psi_ws, pbytes) == cudaSuccess) {
             c->own_bytes += (long long)pbytes;
@@ -891,7 +911,8 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
             c->psi_ws = nullptr;
             cudaGetLastError();
         }
-        a.psi_ws = c->psi_ws;
+        if (p->G2 != 0.0) a.psi_ws = c->psi_ws;
+        else c->split = c->psi_ws != nullptr;
     }
     a.err = c->dev_err;
     a.test_stall = p->test_stall ? 1 : 0;
@@ -1191,7 +1212,7 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_step: this context is a box of a batch; use lbm_batch_step");
     if (nsteps >= 2 && c->mom) return step_moments(c, nsteps);
     for (long k = 0; k < nsteps; ++k) {
-        cudaError_t e = launch_step(c, c->f[c->cur], c->f[c->cur ^ 1]);
+        cudaError_t e = step_once(c, c->f[c->cur], c->f[c->cur ^ 1]);
         if (e != cudaSuccess) return c->fail(LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));
         c->cur ^= 1;
         ++c->t;
@@ -1314,6 +1335,9 @@ struct lbm_batch {
     MomentLaunch mom_launch{};
     BatchBox* mom_boxes_dev = nullptr;
     bool mom_twice = false;
+    // FP64 steps in two kernels over every box, where they run in place
+    bool split = false;
+    unsigned max_cells = 0;
     char err[512] = {0};
 
     lbm_status fail(lbm_status s, const char* fmt, ...) {
@@ -1339,6 +1363,10 @@ StepLaunch batch_launch(const lbm_batch* b) {
 }
 
 cudaError_t batch_launch_step(const lbm_batch* b, int from) {
+    if (b->split) {
+        SplitLaunch l{b->phys, b->bargs, b->max_cells, b->stream};
+        return split_step_f64(l, b->box[0]->coll, b->f[from], b->f[from ^ 1], nullptr);
+    }
     const StepLaunch l = batch_launch(b);
     return step_kernels(b->p.storage, l.coll).batch(l, b->bargs, b->f[from], b->f[from ^ 1]);
 }
@@ -1571,6 +1599,10 @@ lbm_status lbm_batch_create(const lbm_params* p, int count, const int* dims, lbm
         b->box[i] = c;
     }
     b->phys = b->box[0]->args;
+    const int coll = b->box[0]->coll;
+    b->split = p->storage == LBM_F64 && p->kernel == 0 && count <= 65535 && coll != COLL_MRT &&
+               !(coll == COLL_SRT && p->tau != 1.0);
+    for (const lbm_ctx* c : b->box) b->max_cells = std::max(b->max_cells, unsigned(c->n));
     const int ty = p->tile_y ? p->tile_y : (p->collision == LBM_MRT_GUO ? 4 : 8);
     const int zc = p->zchunk ? p->zchunk : 32;
     lbm_status st = batch_configure(b, ty, zc);
@@ -1810,7 +1842,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     // psi of every state of a segment: written by the step kernel during the
     // recomputation where it supports that (kernels 1 and 3, and 5 whose
     // recomputation runs kernel 3), else computed by the reverse step
-    const bool psi_fused = c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
+    const bool psi_fused = c->split || c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
     const size_t psi_bytes = (size_t)c->n * c->elem;
     if (A.psi && A.psi_bytes < (size_t)A.every * psi_bytes) {
         cudaStreamSynchronize(c->stream);
@@ -1847,8 +1879,8 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
                                     cudaMemcpyDeviceToDevice, c->stream));
         char* psi = static_cast<char*>(A.psi);
         for (long t = t0; t + 1 < t1; ++t) {
-            cudaError_t e = launch_step(c, seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state,
-                                        psi_fused ? psi + (size_t)(t - t0) * psi_bytes : nullptr);
+            cudaError_t e = step_once(c, seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state, true,
+                                      psi_fused ? psi + (size_t)(t - t0) * psi_bytes : nullptr);
             if (e != cudaSuccess) return c->fail(LBM_ECUDA, "adjoint recompute: %s", cudaGetErrorString(e));
         }
         for (long t = t1 - 1; t >= t0; --t) {

@@ -57,67 +57,72 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
     R ps[9], pd[9];
     static_for<0, 9>([&](auto pc) {
         constexpr int p = decltype(pc)::value, q = 2 * p + 1;
-        ps[p] = f[q] + f[q + 1];
-        pd[p] = f[q] - f[q + 1];
+        ps[p] = vadd(f[q], f[q + 1]);
+        pd[p] = vsub(f[q], f[q + 1]);
     });
+    // acc + c v, single rounded operations as in collide.cuh
+    auto add = [](auto cc, R v, R acc) {
+        constexpr int c = decltype(cc)::value;
+        if constexpr (c == 1) return vadd(acc, v);
+        else if constexpr (c == -1) return vsub(acc, v);
+        else if constexpr (c != 0) return vfma(v, R(c), acc);
+        else return acc;
+    };
     R m[Q];
     static_for<0, Q>([&](auto kc) {
         constexpr int k = decltype(kc)::value;
         constexpr bool odd = mrt_moment_is_odd(k);
         R acc = R(0);
-        if constexpr (!odd) {
-            constexpr int c0 = mrt_coef(k, 0);
-            if constexpr (c0 != 0) acc = R(c0) * f[0];
-        }
+        if constexpr (!odd) acc = vmul(R(mrt_coef(k, 0)), f[0]);
         static_for<0, 9>([&](auto pc) {
-            constexpr int p = decltype(pc)::value, q = 2 * p + 1;
-            constexpr int c = mrt_coef(k, q);
-            const R v = odd ? pd[p] : ps[p];
-            if constexpr (c == 1) acc += v;
-            else if constexpr (c == -1) acc -= v;
-            else if constexpr (c != 0) acc += R(c) * v;
+            constexpr int p = decltype(pc)::value;
+            acc = add(std::integral_constant<int, mrt_coef(k, 2 * p + 1)>{}, odd ? pd[p] : ps[p], acc);
         });
         m[k] = acc;
     });
     const R rho = m[0];
     const R inv_rho = recip(rho);
-    const R ux = (m[3] + R(0.5) * Fx) * inv_rho;
-    const R uy = (m[5] + R(0.5) * Fy) * inv_rho;
-    const R uz = (m[7] + R(0.5) * Fz) * inv_rho;
-    const R ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
-    const R u2 = ux2 + uy2 + uz2;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-    const R pxx = R(2) * ux2 - uy2 - uz2, pww = uy2 - uz2;
-    const R gxx = R(2) * ux * Fx - uy * Fy - uz * Fz, gww = uy * Fy - uz * Fz;
+    const R half = R(0.5);
+    const R ux = vmul(vfma(half, Fx, m[3]), inv_rho);
+    const R uy = vmul(vfma(half, Fy, m[5]), inv_rho);
+    const R uz = vmul(vfma(half, Fz, m[7]), inv_rho);
+    const R ux2 = vmul(ux, ux), uy2 = vmul(uy, uy), uz2 = vmul(uz, uz);
+    const R yz2 = vadd(uy2, uz2), u2 = vadd(ux2, yz2);
+    const R gx = vmul(ux, Fx), gy = vmul(uy, Fy), gz = vmul(uz, Fz);
+    const R gyz = vadd(gy, gz), uF = vadd(gx, gyz);
+    const R pxx = vsub(vadd(ux2, ux2), yz2), pww = vsub(uy2, uz2);
+    const R gxx = vsub(vadd(gx, gx), gyz), gww = vsub(gy, gz);
+    const R nr = vmul(R(-0.5), rho), q23 = vmul(R(-2.0 / 3.0), rho);
 
     R meq[Q], sg[Q];
-    meq[1] = rho * (R(-11) + R(19) * u2);         sg[1] = R(38) * uF;
-    meq[2] = rho * (R(3) - R(5.5) * u2);          sg[2] = R(-11) * uF;
-    meq[4] = R(-2.0 / 3.0) * rho * ux;            sg[4] = R(-2.0 / 3.0) * Fx;
-    meq[6] = R(-2.0 / 3.0) * rho * uy;            sg[6] = R(-2.0 / 3.0) * Fy;
-    meq[8] = R(-2.0 / 3.0) * rho * uz;            sg[8] = R(-2.0 / 3.0) * Fz;
-    meq[9] = rho * pxx;                           sg[9] = R(2) * gxx;
-    meq[10] = R(-0.5) * rho * pxx;                sg[10] = -gxx;
-    meq[11] = rho * pww;                          sg[11] = R(2) * gww;
-    meq[12] = R(-0.5) * rho * pww;                sg[12] = -gww;
-    meq[13] = rho * ux * uy;                      sg[13] = ux * Fy + uy * Fx;
-    meq[14] = rho * uy * uz;                      sg[14] = uy * Fz + uz * Fy;
-    meq[15] = rho * ux * uz;                      sg[15] = ux * Fz + uz * Fx;
-    meq[16] = R(0);                               sg[16] = R(0);
-    meq[17] = R(0);                               sg[17] = R(0);
-    meq[18] = R(0);                               sg[18] = R(0);
+    meq[1] = vmul(rho, vfma(R(19), u2, R(-11)));  sg[1] = vmul(R(38), uF);
+    meq[2] = vmul(rho, vfma(R(-5.5), u2, R(3)));  sg[2] = vmul(R(-11), uF);
+    meq[4] = vmul(q23, ux);                       sg[4] = vmul(R(-2.0 / 3.0), Fx);
+    meq[6] = vmul(q23, uy);                       sg[6] = vmul(R(-2.0 / 3.0), Fy);
+    meq[8] = vmul(q23, uz);                       sg[8] = vmul(R(-2.0 / 3.0), Fz);
+    meq[9] = vmul(rho, pxx);                      sg[9] = vadd(gxx, gxx);
+    meq[10] = vmul(nr, pxx);                      sg[10] = -gxx;
+    meq[11] = vmul(rho, pww);                     sg[11] = vadd(gww, gww);
+    meq[12] = vmul(nr, pww);                      sg[12] = -gww;
+    meq[13] = vmul(vmul(rho, ux), uy);            sg[13] = vfma(ux, Fy, vmul(uy, Fx));
+    meq[14] = vmul(vmul(rho, uy), uz);            sg[14] = vfma(uy, Fz, vmul(uz, Fy));
+    meq[15] = vmul(vmul(rho, ux), uz);            sg[15] = vfma(ux, Fz, vmul(uz, Fx));
+    meq[16] = meq[17] = meq[18] = R(0);
+    sg[16] = sg[17] = sg[18] = R(0);
 
     // d[k] = (Lambda (m - m_eq) - (I - Lambda/2) S)_k / norm_k
     R d[Q];
     d[0] = R(0);
-    d[3] = -Fx * R(1.0 / mrt_norm(3));
-    d[5] = -Fy * R(1.0 / mrt_norm(5));
-    d[7] = -Fz * R(1.0 / mrt_norm(7));
+    d[3] = vmul(Fx, R(-1.0 / mrt_norm(3)));
+    d[5] = vmul(Fy, R(-1.0 / mrt_norm(5)));
+    d[7] = vmul(Fz, R(-1.0 / mrt_norm(7)));
     static_for<0, Q>([&](auto kc) {
         constexpr int k = decltype(kc)::value;
         if constexpr (k != 0 && k != 3 && k != 5 && k != 7) {
             const R sk = s[k];
-            d[k] = (sk * (m[k] - meq[k]) - (R(1) - R(0.5) * sk) * sg[k]) * R(1.0 / mrt_norm(k));
+            R t = vmul(sk, vsub(m[k], meq[k]));
+            if constexpr (k < 16) t = vfnma(vfnma(half, sk, R(1)), sg[k], t);
+            d[k] = vmul(t, R(1.0 / mrt_norm(k)));
         }
     });
     // f* = f - M^T d: the even moments give the common part E of a velocity
@@ -127,10 +132,9 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
         R e0 = R(0);
         static_for<1, Q>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
-            constexpr int c = mrt_coef(k, 0);
-            if constexpr (c != 0) e0 += R(c) * d[k];
+            e0 = add(std::integral_constant<int, mrt_coef(k, 0)>{}, d[k], e0);
         });
-        f[0] -= e0;
+        f[0] = vsub(f[0], e0);
     }
     static_for<0, 9>([&](auto pc) {
         constexpr int q = 2 * decltype(pc)::value + 1;
@@ -138,21 +142,11 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
         static_for<1, Q>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
             constexpr int c = mrt_coef(k, q);
-            constexpr bool odd = mrt_coef(k, q + 1) == -c && c != 0;
-            if constexpr (c != 0) {
-                if constexpr (odd) {
-                    if constexpr (c == 1) O += d[k];
-                    else if constexpr (c == -1) O -= d[k];
-                    else O += R(c) * d[k];
-                } else {
-                    if constexpr (c == 1) E += d[k];
-                    else if constexpr (c == -1) E -= d[k];
-                    else E += R(c) * d[k];
-                }
-            }
+            if constexpr (c != 0 && mrt_coef(k, q + 1) == -c) O = add(std::integral_constant<int, c>{}, d[k], O);
+            else E = add(std::integral_constant<int, c>{}, d[k], E);
         });
-        f[q] -= E + O;
-        f[q + 1] -= E - O;
+        f[q] = vsub(f[q], vadd(E, O));
+        f[q + 1] = vsub(f[q + 1], vsub(E, O));
     });
 }
 

@@ -75,3 +75,27 @@ def test_batches_at_once_equal_single_steps(op):
             for _ in range(8):
                 L.step(1)
             assert np.array_equal(f, L.get_populations()), d
+
+
+@pytest.mark.parametrize("op", ["srt", "unit", "paper", "shear", "srt09", "general"])
+def test_two_kernel_fp64_step_is_bit_identical(op):
+    """FP64 steps in two kernels (in place where the moments suffice, through a psi field otherwise) against
+    the register-staged kernel, single lattices and batches."""
+    more = {"srt09": dict(collision="srt", tau=0.9),
+            "general": dict(collision="mrt", tau=0.9, rates=[0.8 + 0.04 * ((7 * k) % 19) for k in range(19)])}
+    kw = dict(OPS, **more)[op]
+    boxes = [(1, 1, 5), (2, 3, 2), (33, 13, 5), (65, 15, 7), (32, 32, 64)]
+    want = []
+    for box in boxes:
+        f, copy, t = _state(box, 1, [1] * 7, "f64", **kw)
+        got, copy2, t2 = _state(box, 0, (2, 5), "f64", **kw)
+        assert (copy, t) == (copy2, t2)
+        assert np.array_equal(got, f), box
+        want.append(f)
+    with lbm.Batch(boxes, G=-5.5, storage="f64", **kw) as B:
+        for v, d in zip(B.boxes, boxes):
+            v.set_density(inputs.random_density(*d, seed=7, lo=0.3, hi=1.9))
+        for n in (3, 4):
+            B.step(n)
+        for v, f in zip(B.boxes, want):
+            assert np.array_equal(v.get_populations(), f), v.shape
