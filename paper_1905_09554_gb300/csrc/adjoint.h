@@ -9,8 +9,10 @@ struct AdjointArgs {
     int nx, ny, nz;
     long long n;
     double G, tau, omega, rho0;
-    float Gf, tauf, omegaf, rho0f;  // rounded on the host for the FP32 kernels
+    double gw;                      // -G/36
+    float Gf, tauf, omegaf, rho0f, gwf;  // rounded on the host for the FP32 kernels
     int grid;  // blocks of adjoint_threads() threads (grid-stride loops)
+    bool tau1; // tau = 1: lam holds four values a cell {A, B}, lam_a = A + c_a.B, and gr is not used
 };
 
 int adjoint_threads();
@@ -23,7 +25,8 @@ int adjoint_rows_per_block();  // the step kernels walk x rows, this many per bl
 // forward state f; this step's dJ/dG and dJ/dtau are added to the per-block
 // running sums in `partials` (2 * grid doubles, zeroed before the first
 // step), which adjoint_reduce adds into acc[0..1] once after the last step.
-// psi (n) and gF (4n: psi gF and S.gF, see adj_collide_kernel) are scratch;
+// psi (n) and gF (4n: {psi gF, S.gF} per cell, see adj_collide_kernel) are
+// scratch; lam and gF are 16-byte aligned;
 // acc is not touched here.  Needs nx*ny*nz < 2^32 (32-bit cell indices).
 // psi_ready: psi already holds psi of f (the step kernel wrote it during the
 // recomputation); otherwise it is computed first.

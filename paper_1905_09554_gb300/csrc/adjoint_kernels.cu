@@ -18,6 +18,12 @@
 //      and the gather reads only V of the 18 neighbours.
 // Parameter gradients are summed in float64 per block and reduced in a fixed
 // order (deterministic).
+//
+// At tau = 1 the collision forgets the populations, so their adjoint is
+// lam_a(y) = A(y) + c_a.B(y): four values a cell instead of 20 (lam and gr).
+// adj_collide1_kernel and adj_force_kernel then keep {A, B} as one 16- or
+// 32-byte vector per cell: one vector load per neighbour where the general
+// form loads two values, and 128 + 40 B a cell and step instead of 250 + 40.
 #include <cuda_runtime.h>
 
 #include "adjoint.h"
@@ -59,6 +65,43 @@ __device__ __forceinline__ unsigned nb_of(const Row& w, const unsigned (&xs)[3],
     return w.zo[dz + 1] + w.yo[dy + 1] + xs[dx + 1];
 }
 
+// psi of a cell's neighbours in the plane at offset zo.
+template <class R>
+struct RowPsi {
+    const R* psi;
+    unsigned zo;
+    const Row& w;
+    const unsigned (&xs)[3];
+    template <class DX, class DY>
+    __device__ __forceinline__ R operator()(DX, DY) const {
+        return __ldg(psi + (zo + w.yo[DY::value + 1] + xs[DX::value + 1]));
+    }
+};
+// The step's force of cell xs[1] of row w (collide.cuh).
+template <class R>
+__device__ __forceinline__ Force<R> row_force(const R* psi, const Row& w, const unsigned (&xs)[3], R gw) {
+    PsiView<R> v[3];
+    static_for<0, 3>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const RowPsi<R> at{psi, w.zo[k], w, xs};
+        v[k].c = __ldg(psi + (w.zo[k] + w.yo[1] + xs[1]));
+        psi_axis(v[k], at);
+        if constexpr (k == 1) psi_diag(v[k], at);
+    });
+    return force_of(v[0], v[1], v[2], gw);
+}
+
+// c_q . (x, y, z)
+template <int q, class R>
+__device__ __forceinline__ R dot_c(R x, R y, R z) {
+    R s = R(0);
+    if constexpr (cx(q) != 0) s = cx(q) > 0 ? x : -x;
+    if constexpr (cy(q) != 0) s = cx(q) != 0 ? (cy(q) > 0 ? s + y : s - y) : (cy(q) > 0 ? y : -y);
+    if constexpr (cz(q) != 0)
+        s = (cx(q) != 0 || cy(q) != 0) ? (cz(q) > 0 ? s + z : s - z) : (cz(q) > 0 ? z : -z);
+    return s;
+}
+
 template <class F>
 __device__ __forceinline__ void for_each_cell(int nx, int ny, int nz, F&& body) {
     const unsigned rows = unsigned(ny) * unsigned(nz);
@@ -71,6 +114,27 @@ __device__ __forceinline__ void for_each_cell(int nx, int ny, int nz, F&& body) 
     }
 }
 
+// Four values of one cell, loaded and stored whole.
+template <class R>
+struct alignas(16) Vec4 {
+    R x, y, z, w;
+};
+__device__ __forceinline__ Vec4<float> load4(const Vec4<float>* p) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Vec4<double> load4(const Vec4<double>* p) {
+    const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    return {a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ void store4(Vec4<float>* p, const Vec4<float>& v) {
+    *reinterpret_cast<float4*>(p) = make_float4(v.x, v.y, v.z, v.w);
+}
+__device__ __forceinline__ void store4(Vec4<double>* p, const Vec4<double>& v) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(v.x, v.y);
+    reinterpret_cast<double2*>(p)[1] = make_double2(v.z, v.w);
+}
+
 template <class R>
 __global__ void __launch_bounds__(kThreads) adj_psi_kernel(const R* __restrict__ f, R* __restrict__ psi, unsigned n,
                                                            R rho0, R inv_rho0) {
@@ -81,95 +145,94 @@ __global__ void __launch_bounds__(kThreads) adj_psi_kernel(const R* __restrict__
 }
 
 // Sum of (a, b) over the block, added to out2[0..1] (the block's running
-// sums over the reverse steps); fixed order.
+// sums over the reverse steps); fixed order: a tree within each warp, then
+// the warps in turn.
 __device__ __forceinline__ void block_sum2(double a, double b, double* out2) {
-    __shared__ double red[2][kThreads];
-    const int tid = threadIdx.y * kRowThreads + threadIdx.x;
-    red[0][tid] = a;
-    red[1][tid] = b;
-    __syncthreads();
-    for (int s = kThreads / 2; s > 0; s >>= 1) {
-        if (tid < s) {
-            red[0][tid] += red[0][tid + s];
-            red[1][tid] += red[1][tid + s];
-        }
-        __syncthreads();
+    __shared__ double red[2][kRows];
+    for (int s = 16; s > 0; s >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, s);
+        b += __shfl_down_sync(0xffffffffu, b, s);
     }
-    if (tid == 0) {
-        out2[0] += red[0][0];
-        out2[1] += red[1][0];
+    if (threadIdx.x == 0) {
+        red[0][threadIdx.y] = a;
+        red[1][threadIdx.y] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 && threadIdx.y == 0) {
+        double s = red[threadIdx.x][0];
+        for (int k = 1; k < kRows; ++k) s += red[threadIdx.x][k];
+        out2[threadIdx.x] += s;
     }
 }
 
 // Collision adjoint.  Besides lam_out it writes, per cell, the two pieces of
 // the force adjoint that the gather of adj_force_kernel needs:
-//   fa[0..2n) = V = psi gF (the cell's force sensitivity weighted by its psi)
-//   fa[3n..4n) = T = S . gF (S = sum_a w_a psi(x + c_a) c_a, known here).
+//   V = psi gF (the cell's force sensitivity weighted by its psi)
+//   T = S . gF (S = sum_a w_a psi(x + c_a) c_a, known here),
+// one vector {V, T} per cell.
 template <class R>
 __global__ void __launch_bounds__(kThreads)
 adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* __restrict__ lam_next,
-                   const R* __restrict__ gr_next, R* __restrict__ lam_out, R* __restrict__ fa,
+                   const R* __restrict__ gr_next, R* __restrict__ lam_out, Vec4<R>* __restrict__ fa,
                    double* __restrict__ partials, AdjointArgs a) {
     const unsigned n = unsigned(a.n);
-    const R G = par<R>(a.G, a.Gf), tau = par<R>(a.tau, a.tauf), omega = par<R>(a.omega, a.omegaf);
+    const R tau = par<R>(a.tau, a.tauf), omega = par<R>(a.omega, a.omegaf);
     double accG = 0.0, accT = 0.0;
     for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
         R fv[Q], ls[Q];
-        R rho = R(0), jx = R(0), jy = R(0), jz = R(0), sx = R(0), sy = R(0), sz = R(0);
         static_for<0, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             fv[q] = f[size_t(q) * n + i];
-            rho += fv[q];
-            jx += R(cx(q)) * fv[q];
-            jy += R(cy(q)) * fv[q];
-            jz += R(cz(q)) * fv[q];
             const unsigned nb = nb_of(w, xs, cx(q), cy(q), cz(q));
             ls[q] = lam_next[size_t(q) * n + nb] + gr_next[nb];  // streaming adjoint: pull from x + c_q
-            if constexpr (q != 0) {
-                const R pn = psi[nb];
-                sx += R(wq(q) * cx(q)) * pn;
-                sy += R(wq(q) * cy(q)) * pn;
-                sz += R(wq(q) * cz(q)) * pn;
-            }
         });
+        R m[4];
+        moments_of<COLL_SRT, R>(fv, m);
+        const R rho = m[0];
+        const Force<R> F = row_force(psi, w, xs, par<R>(a.gw, a.gwf));
+        const R Fx = F.g * F.sx, Fy = F.g * F.sy, Fz = F.g * F.sz;
+        const R sx = R(1.0 / 36.0) * F.sx, sy = R(1.0 / 36.0) * F.sy, sz = R(1.0 / 36.0) * F.sz;
         const R ps = psi[i];
-        const R Fx = -G * ps * sx, Fy = -G * ps * sy, Fz = -G * ps * sz;
-        const R inv_rho = R(1) / rho;
-        const R ux = (jx + tau * Fx) * inv_rho, uy = (jy + tau * Fy) * inv_rho, uz = (jz + tau * Fz) * inv_rho;
+        const R inv_rho = recip(rho);
+        const R ux = (m[1] + tau * Fx) * inv_rho, uy = (m[2] + tau * Fy) * inv_rho, uz = (m[3] + tau * Fz) * inv_rho;
         const R u2 = ux * ux + uy * uy + uz * uz;
         // adjoint of f* = (1 - omega) f + omega f_eq(rho, u')
         R g_rho = R(0), gux = R(0), guy = R(0), guz = R(0), g_tau = R(0);
         // w_a rho with the rest weight from sum_a w_a = 1, as the step forms it: with the rounded weights
         // (their sum is 1 + 3e-8 in float) the adjoint field grew by 3e-8 a step, 1e-5 over 500 steps.
         const R r2 = R(1.0 / 36.0) * rho, r1 = r2 + r2, r0 = fma(R(-24), r2, rho);
+        R s_mw = R(0);
         static_for<0, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
-            const R cu = R(cx(q)) * ux + R(cy(q)) * uy + R(cz(q)) * uz;
+            const R cu = dot_c<q>(ux, uy, uz);
             const R wr = q == 0 ? r0 : (q < 7 ? r1 : r2);
-            const R feq = wr * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * u2);
-            const R mu = omega * ls[q];
-            g_rho += mu * feq * inv_rho;
+            const R feq = wr * (R(1) - R(1.5) * u2 + cu * (R(3) + R(4.5) * cu));
+            const R mu = omega * ls[q], mw = mu * wr;
+            g_rho += mu * feq;
             // d f_eq / d u' = w rho (3 c + 9 (c.u') c - 3 u')
-            const R k = R(3) + R(9) * cu;
-            gux += mu * wr * (k * R(cx(q)) - R(3) * ux);
-            guy += mu * wr * (k * R(cy(q)) - R(3) * uy);
-            guz += mu * wr * (k * R(cz(q)) - R(3) * uz);
-            g_tau -= ls[q] * (feq - fv[q]) * (omega * omega);  // d omega / d tau = -1/tau^2
+            const R k = mw * (R(3) + R(9) * cu);
+            if constexpr (cx(q) != 0) gux += R(cx(q)) * k;
+            if constexpr (cy(q) != 0) guy += R(cy(q)) * k;
+            if constexpr (cz(q) != 0) guz += R(cz(q)) * k;
+            s_mw += mw;
+            g_tau -= ls[q] * (feq - fv[q]);
         });
+        gux -= R(3) * s_mw * ux;
+        guy -= R(3) * s_mw * uy;
+        guz -= R(3) * s_mw * uz;
+        g_tau *= omega * omega;  // d omega / d tau = -1/tau^2
         // u' = (j + tau F)/rho
         const R gjx = gux * inv_rho, gjy = guy * inv_rho, gjz = guz * inv_rho;
-        g_rho -= (gux * ux + guy * uy + guz * uz) * inv_rho;
+        g_rho = (g_rho - (gux * ux + guy * uy + guz * uz)) * inv_rho;
         g_tau += (gux * Fx + guy * Fy + guz * Fz) * inv_rho;
         const R gFx = tau * gjx, gFy = tau * gjy, gFz = tau * gjz;
         static_for<0, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
-            lam_out[size_t(q) * n + i] =
-                (R(1) - omega) * ls[q] + g_rho + R(cx(q)) * gjx + R(cy(q)) * gjy + R(cz(q)) * gjz;
+            R v = (R(1) - omega) * ls[q] + g_rho;
+            if constexpr (q != 0) v += dot_c<q>(gjx, gjy, gjz);
+            lam_out[size_t(q) * n + i] = v;
         });
-        fa[i] = ps * gFx;
-        fa[n + i] = ps * gFy;
-        fa[2 * size_t(n) + i] = ps * gFz;
-        fa[3 * size_t(n) + i] = sx * gFx + sy * gFy + sz * gFz;
+        store4(fa + i, Vec4<R>{ps * gFx, ps * gFy, ps * gFz, sx * gFx + sy * gFy + sz * gFz});
         // dF/dG = -psi S
         accG += double(-(ps * sx) * gFx - (ps * sy) * gFy - (ps * sz) * gFz);
         accT += double(g_tau);
@@ -177,34 +240,103 @@ adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* 
     block_sum2(accG, accT, partials + 2 * blockIdx.x);
 }
 
-// Force adjoint: g_psi(y) = -G [ T(y) + sum_a w_a c_a . V(y - c_a) ] and the
-// density term gr(y) = g_psi(y) psi'(rho(y)), psi' = 1 - psi/rho0.
+// The same at tau = 1, from lam_a(y) = A(y) + c_a.B(y) kept as {A, B}: the
+// pulled value of velocity q is A + c_q.B of the neighbour x + c_q.  Opposite
+// velocities share the even part e and odd part o of f_eq = e +/- o.  Writes
+// {g_rho, B} (adj_force_kernel adds the force's part of A) and {V, T}.
 template <class R>
-__global__ void __launch_bounds__(kThreads)
-adj_force_kernel(const R* __restrict__ psi, const R* __restrict__ fa, R* __restrict__ gr, AdjointArgs a) {
+__global__ void __launch_bounds__(kThreads, 2)
+adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Vec4<R>* __restrict__ lam_next,
+                    Vec4<R>* __restrict__ lam_out, Vec4<R>* __restrict__ fa, double* __restrict__ partials,
+                    AdjointArgs a) {
     const unsigned n = unsigned(a.n);
-    const R G = par<R>(a.G, a.Gf), rho0 = par<R>(a.rho0, a.rho0f);
-    const R* __restrict__ Vx = fa;
-    const R* __restrict__ Vy = fa + n;
-    const R* __restrict__ Vz = fa + 2 * size_t(n);
-    const R* __restrict__ T = fa + 3 * size_t(n);
+    double accG = 0.0, accT = 0.0;
     for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
-        R term = T[i];
+        R fv[Q];
+        static_for<0, Q>([&](auto qc) {
+            constexpr int q = decltype(qc)::value;
+            fv[q] = f[size_t(q) * n + i];
+        });
+        R m[4];
+        moments_of<COLL_SRT, R>(fv, m);
+        const R rho = m[0];
+        const Force<R> F = row_force(psi, w, xs, par<R>(a.gw, a.gwf));
+        const R Fx = F.g * F.sx, Fy = F.g * F.sy, Fz = F.g * F.sz;
+        const R ps = psi[i], inv_rho = recip(rho);
+        const R ux = (m[1] + Fx) * inv_rho, uy = (m[2] + Fy) * inv_rho, uz = (m[3] + Fz) * inv_rho;
+        const R base = R(1) - R(1.5) * (ux * ux + uy * uy + uz * uz);
+        const R r2 = R(1.0 / 36.0) * rho, r1 = r2 + r2, r0 = fma(R(-24), r2, rho);
+
+        const R l0 = load4(lam_next + i).x;
+        R s_feq = r0 * base * l0;          // sum_q ls_q f_eq_q
+        R s_f = (r0 * base - fv[0]) * l0;  // sum_q ls_q (f_eq_q - f_q)
+        R s_w1 = R(0), s_w2 = R(0);        // sums of ls over the axis and the edge velocities
+        R gx = R(0), gy = R(0), gz = R(0);
+        static_for<0, 9>([&](auto pc) {
+            constexpr int q = 2 * decltype(pc)::value + 1;
+            const Vec4<R> p = load4(lam_next + nb_of(w, xs, cx(q), cy(q), cz(q)));
+            const Vec4<R> o = load4(lam_next + nb_of(w, xs, -cx(q), -cy(q), -cz(q)));
+            // streaming adjoint: pull from x + c_q
+            const R lp = p.x + dot_c<q>(p.y, p.z, p.w), lm = o.x - dot_c<q>(o.y, o.z, o.w);
+            const R sl = lp + lm, dl = lp - lm;
+            const R cu = dot_c<q>(ux, uy, uz);
+            const R wr = q < 7 ? r1 : r2;
+            const R e = wr * (base + R(4.5) * cu * cu), od = wr * (R(3) * cu);
+            s_feq += e * sl + od * dl;
+            s_f += ((e + od) - fv[q]) * lp + ((e - od) - fv[q + 1]) * lm;
+            if constexpr (q < 7) s_w1 += sl;
+            else s_w2 += sl;
+            // d f_eq / d u' = w rho (3 c + 9 (c.u') c - 3 u')
+            const R k = wr * (R(3) * dl + R(9) * cu * sl);
+            if constexpr (cx(q) != 0) gx += R(cx(q)) * k;
+            if constexpr (cy(q) != 0) gy += R(cy(q)) * k;
+            if constexpr (cz(q) != 0) gz += R(cz(q)) * k;
+        });
+        const R s3 = R(-3) * (r0 * l0 + r1 * s_w1 + r2 * s_w2);
+        gx += s3 * ux;
+        gy += s3 * uy;
+        gz += s3 * uz;
+        // u' = (j + F)/rho at tau = 1
+        const R gjx = gx * inv_rho, gjy = gy * inv_rho, gjz = gz * inv_rho;
+        const R g_rho = (s_feq - (gx * ux + gy * uy + gz * uz)) * inv_rho;
+        store4(lam_out + i, Vec4<R>{g_rho, gjx, gjy, gjz});
+        const R sg = R(1.0 / 36.0) * (F.sx * gjx + F.sy * gjy + F.sz * gjz);
+        store4(fa + i, Vec4<R>{ps * gjx, ps * gjy, ps * gjz, sg});
+        accG += double(-ps * sg);                                        // dF/dG = -psi S
+        accT += double((gjx * Fx + gjy * Fy + gjz * Fz) - s_f);          // d omega / d tau = -1
+    });
+    block_sum2(accG, accT, partials + 2 * blockIdx.x);
+}
+
+// Force adjoint: g_psi(y) = -G [ T(y) + sum_a w_a c_a . V(y - c_a) ] and the
+// density term g_psi(y) psi'(rho(y)), psi' = 1 - psi/rho0.  It is the same for
+// every population: kept in gr and added where it is read, or (TAU1) added to
+// the A of {A, B}.
+template <class R, bool TAU1>
+__global__ void __launch_bounds__(kThreads)
+adj_force_kernel(const R* __restrict__ psi, const Vec4<R>* __restrict__ fa, R* __restrict__ gr, AdjointArgs a) {
+    const R G = par<R>(a.G, a.Gf), inv_rho0 = R(1.0 / a.rho0);
+    for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
+        R axis = R(0), edge = R(0);
         static_for<1, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
-            const unsigned dn = nb_of(w, xs, -cx(q), -cy(q), -cz(q));  // y - c_q
-            R cv = R(0);
-            if constexpr (cx(q) != 0) cv += R(cx(q)) * Vx[dn];
-            if constexpr (cy(q) != 0) cv += R(cy(q)) * Vy[dn];
-            if constexpr (cz(q) != 0) cv += R(cz(q)) * Vz[dn];
-            term += R(wq(q)) * cv;
+            const Vec4<R> v = load4(fa + nb_of(w, xs, -cx(q), -cy(q), -cz(q)));  // y - c_q
+            if constexpr (q < 7) axis += dot_c<q>(v.x, v.y, v.z);
+            else edge += dot_c<q>(v.x, v.y, v.z);
         });
-        // the same for every population: stored once, added where it is read
-        gr[i] = -G * term * (R(1) - psi[i] / rho0);
+        const R term = load4(fa + i).w + (R(1.0 / 18.0) * axis + R(1.0 / 36.0) * edge);
+        const R g = -G * term * (R(1) - psi[i] * inv_rho0);
+        if constexpr (TAU1) gr[4 * size_t(i)] += g;
+        else gr[i] = g;
     });
 }
 
 // lam_a(x, T) = dJ/drho(x) for every a (rho = sum_a f_a); no force term yet.
+template <class R>
+__global__ void adj_seed1_kernel(const double* __restrict__ g, Vec4<R>* __restrict__ lam, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        store4(lam + i, Vec4<R>{R(g[i]), R(0), R(0), R(0)});
+}
 template <class R>
 __global__ void adj_seed_kernel(const double* __restrict__ g, R* __restrict__ lam, R* __restrict__ gr, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -230,6 +362,13 @@ __global__ void adj_rho0_kernel(const R* __restrict__ lam, const R* __restrict__
         });
         out[i] = s;
     }
+}
+
+// At tau = 1 the sum is A: sum_a w_a (A + c_a.B) = A.
+template <class R>
+__global__ void adj_rho01_kernel(const Vec4<R>* __restrict__ lam, double* __restrict__ out, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = double(load4(lam + i).x);
 }
 
 // Fixed-order sum of the per-block partials into acc[0..1]: each of 256
@@ -267,11 +406,18 @@ cudaError_t run_adjoint_step(const AdjointArgs& a, const void* f, void* psi, boo
     if (!psi_ready)
         adj_psi_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(f), static_cast<R*>(psi), unsigned(a.n),
                                                   par<R>(a.rho0, a.rho0f), R(1.0 / a.rho0));
+    Vec4<R>* const v = static_cast<Vec4<R>*>(gF);
+    if (a.tau1) {
+        adj_collide1_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(f), static_cast<const R*>(psi),
+                                                       static_cast<const Vec4<R>*>(lam_next),
+                                                       static_cast<Vec4<R>*>(lam_out), v, partials, a);
+        adj_force_kernel<R, true><<<grid, block, 0, st>>>(static_cast<const R*>(psi), v, static_cast<R*>(lam_out), a);
+        return cudaGetLastError();
+    }
     adj_collide_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(f), static_cast<const R*>(psi),
                                                   static_cast<const R*>(lam_next), static_cast<const R*>(gr_next),
-                                                  static_cast<R*>(lam_out), static_cast<R*>(gF), partials, a);
-    adj_force_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(psi), static_cast<const R*>(gF),
-                                                static_cast<R*>(gr_out), a);
+                                                  static_cast<R*>(lam_out), v, partials, a);
+    adj_force_kernel<R, false><<<grid, block, 0, st>>>(static_cast<const R*>(psi), v, static_cast<R*>(gr_out), a);
     (void)acc;  // the per-block sums stay in `partials` until adjoint_reduce
     return cudaGetLastError();
 }
@@ -288,6 +434,11 @@ cudaError_t adjoint_step(const AdjointArgs& a, bool f64, const void* f, void* ps
 }
 
 cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, void* lam, void* gr, cudaStream_t st) {
+    if (a.tau1) {
+        if (f64) adj_seed1_kernel<double><<<a.grid, kThreads, 0, st>>>(dJdrho, static_cast<Vec4<double>*>(lam), a.n);
+        else adj_seed1_kernel<float><<<a.grid, kThreads, 0, st>>>(dJdrho, static_cast<Vec4<float>*>(lam), a.n);
+        return cudaGetLastError();
+    }
     if (f64)
         adj_seed_kernel<double><<<a.grid, kThreads, 0, st>>>(dJdrho, static_cast<double*>(lam),
                                                              static_cast<double*>(gr), a.n);
@@ -299,6 +450,11 @@ cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, v
 
 cudaError_t adjoint_rho0(const AdjointArgs& a, bool f64, const void* lam, const void* gr, double* out,
                          cudaStream_t st) {
+    if (a.tau1) {
+        if (f64) adj_rho01_kernel<double><<<a.grid, kThreads, 0, st>>>(static_cast<const Vec4<double>*>(lam), out, a.n);
+        else adj_rho01_kernel<float><<<a.grid, kThreads, 0, st>>>(static_cast<const Vec4<float>*>(lam), out, a.n);
+        return cudaGetLastError();
+    }
     if (f64)
         adj_rho0_kernel<double><<<a.grid, kThreads, 0, st>>>(static_cast<const double*>(lam),
                                                              static_cast<const double*>(gr), out, a.n);

@@ -1752,10 +1752,15 @@ AdjointArgs adjoint_args(const lbm_ctx* c) {
     a.tauf = float(a.tau);
     a.omegaf = float(a.omega);
     a.rho0f = float(a.rho0);
+    a.gw = c->args.gw;
+    a.gwf = c->args.gwf;
     const long long rows = (long long)c->p.ny * c->p.nz;
     const long long want = (rows + adjoint_rows_per_block() - 1) / adjoint_rows_per_block();
-    const long long cap = 8LL * c->num_sms;
+    // One block per 8 rows as far as the blocks' partial sums stay small: a cap near the resident blocks left
+    // the last of 1440 blocks' worth of rows (64 x 64 x 180) to a second, mostly empty round.
+    const long long cap = 1 << 14;
     a.grid = int(want < cap ? (want < 1 ? 1 : want) : cap);
+    a.tau1 = c->p.tau == 1.0;
     return a;
 }
 
@@ -1808,11 +1813,10 @@ lbm_status lbm_adjoint_forward(lbm_ctx* c, const double* rho0, int on_device, lo
     }
     lbm_status st = lbm_set_density(c, rho0, on_device);
     if (st != LBM_OK) return st;
-    for (long t = 0; t < nsteps; ++t) {
-        if (t % every == 0)
-            LBM_CUDA(c, cudaMemcpyAsync(static_cast<char*>(A.cp) + (size_t)(t / every) * state, c->f[c->cur], state,
-                                        cudaMemcpyDeviceToDevice, c->stream));
-        st = lbm_step(c, 1);
+    for (long t = 0; t < nsteps; t += every) {
+        LBM_CUDA(c, cudaMemcpyAsync(static_cast<char*>(A.cp) + (size_t)(t / every) * state, c->f[c->cur], state,
+                                    cudaMemcpyDeviceToDevice, c->stream));
+        st = lbm_step(c, t + every < nsteps ? every : nsteps - t);
         if (st != LBM_OK) return st;
     }
     A.T = nsteps;
