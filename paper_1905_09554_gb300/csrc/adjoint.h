@@ -33,6 +33,12 @@ int adjoint_rows_per_block();  // the step kernels walk x rows, this many per bl
 cudaError_t adjoint_step(const AdjointArgs& a, bool f64, const void* f, void* psi, bool psi_ready,
                          const void* lam_next, const void* gr_next, void* lam_out, void* gr_out, void* gF,
                          double* partials, double* acc, cudaStream_t st);
+// The same at tau = 1 in FP32 from a state's moment fields (step_moment.cuh,
+// 4 fields).  lam_next2: lam of two steps on, nullptr in the last step; first:
+// step 0, from a state at rest.
+cudaError_t adjoint_step_moments(const AdjointArgs& a, const float* moments, float* psi, bool psi_ready,
+                                 const void* lam_next, const void* lam_next2, void* lam_out, void* gF,
+                                 double* partials, bool first, cudaStream_t st);
 cudaError_t adjoint_reduce(const AdjointArgs& a, const double* partials, double* acc, cudaStream_t st);
 // lam_a = dJ/drho (every a), gr = 0.
 cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, void* lam, void* gr, cudaStream_t st);

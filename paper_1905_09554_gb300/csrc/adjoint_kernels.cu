@@ -42,6 +42,7 @@ constexpr int kRowThreads = 32, kRows = kThreads / kRowThreads;  // (32, 8) bloc
 // consecutive x of a row, so the neighbour gathers stay coalesced and no
 // cell index is ever divided.
 struct Row {
+    unsigned row;           // its number, y + ny z
     unsigned zo[3], yo[3];  // offsets of planes z-1, z, z+1 and rows y-1, y, y+1
 };
 
@@ -51,6 +52,7 @@ __device__ __forceinline__ Row row_of(unsigned r, int nx, int ny, int nz) {
     const int zm = z == 0 ? nz - 1 : z - 1, zp = z + 1 == nz ? 0 : z + 1;
     const unsigned plane = unsigned(nx) * unsigned(ny);
     Row w;
+    w.row = r;
     w.zo[0] = unsigned(zm) * plane;
     w.zo[1] = unsigned(z) * plane;
     w.zo[2] = unsigned(zp) * plane;
@@ -142,6 +144,17 @@ __global__ void __launch_bounds__(kThreads) adj_psi_kernel(const R* __restrict__
         const R r = density_of<R>([&](auto qc) { return f[size_t(decltype(qc)::value) * n + i]; });
         psi[i] = psi_of<R>(r, rho0, inv_rho0);
     }
+}
+
+// The same from the moment fields of step_moment.cuh.
+__global__ void __launch_bounds__(kThreads) adj_psi_moments_kernel(const float* __restrict__ moments,
+                                                                   float* __restrict__ psi, AdjointArgs a) {
+    const unsigned pitch = unsigned(moment_pitch(a.nx));
+    const float rho0 = a.rho0f, inv_rho0 = float(1.0 / a.rho0);
+    for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
+        const unsigned o = w.row * pitch + xs[1] + 2;
+        psi[i] = psi_of<float>(moments[o], rho0, inv_rho0);
+    });
 }
 
 // Sum of (a, b) over the block, added to out2[0..1] (the block's running
@@ -244,21 +257,42 @@ adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* 
 // pulled value of velocity q is A + c_q.B of the neighbour x + c_q.  Opposite
 // velocities share the even part e and odd part o of f_eq = e +/- o.  Writes
 // {g_rho, B} (adj_force_kernel adds the force's part of A) and {V, T}.
-template <class R>
+//
+// The gradient with respect to tau, sum_x sum_q ls_q (f_eq_q - f_q), needs the
+// populations before the collision.  FROM_MOMENTS has only a state's moments
+// (as step_moment.cuh stores them: 16 B a cell are kept per state instead of
+// 76).  There f_q(x + c_q, t + 1) = f_eq_q(x, t), so the populations of step
+// t + 1 are weighted here, in step t, with the adjoint two links on:
+//   sum_x sum_q f_eq_q(x, t) [ lam_q(x + c_q, t + 1) - lam_q(x + 2 c_q, t + 2) ],
+// a difference along the velocity that is as small as f_eq - f itself.
+// lam_next2: lam(t + 2), nullptr in the last step; first: step 0, whose
+// populations are at rest, f_q = w_q rho.
+template <class R, bool FROM_MOMENTS>
 __global__ void __launch_bounds__(kThreads, 2)
 adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Vec4<R>* __restrict__ lam_next,
-                    Vec4<R>* __restrict__ lam_out, Vec4<R>* __restrict__ fa, double* __restrict__ partials,
-                    AdjointArgs a) {
+                    const Vec4<R>* __restrict__ lam_next2, Vec4<R>* __restrict__ lam_out, Vec4<R>* __restrict__ fa,
+                    double* __restrict__ partials, bool first, AdjointArgs a) {
     const unsigned n = unsigned(a.n);
+    const int pitch = moment_pitch(a.nx);
+    const long long nf = (long long)pitch * a.ny * a.nz;
     double accG = 0.0, accT = 0.0;
     for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
-        R fv[Q];
-        static_for<0, Q>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            fv[q] = f[size_t(q) * n + i];
-        });
-        R m[4];
-        moments_of<COLL_SRT, R>(fv, m);
+        R fv[Q], m[4];
+        if constexpr (FROM_MOMENTS) {
+            // rows of `pitch` floats from column 2 on; rho, then jx and jy by pairs of cells, then jz
+            const unsigned col = xs[1] + 2, o = w.row * unsigned(pitch) + col;
+            const R* const pj = f + (nf + 2 * (long long)(o - (col & 1)) + (col & 1));
+            m[0] = __ldg(f + o);
+            m[1] = __ldg(pj);
+            m[2] = __ldg(pj + 2);
+            m[3] = __ldg(f + (3 * nf + o));
+        } else {
+            static_for<0, Q>([&](auto qc) {
+                constexpr int q = decltype(qc)::value;
+                fv[q] = f[size_t(q) * n + i];
+            });
+            moments_of<COLL_SRT, R>(fv, m);
+        }
         const R rho = m[0];
         const Force<R> F = row_force(psi, w, xs, par<R>(a.gw, a.gwf));
         const R Fx = F.g * F.sx, Fy = F.g * F.sy, Fz = F.g * F.sz;
@@ -269,9 +303,26 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
 
         const R l0 = load4(lam_next + i).x;
         R s_feq = r0 * base * l0;          // sum_q ls_q f_eq_q
-        R s_f = (r0 * base - fv[0]) * l0;  // sum_q ls_q (f_eq_q - f_q)
+        R s_f;                             // sum_q ls_q (f_eq_q - f_q), or its rearrangement
+        if constexpr (FROM_MOMENTS) s_f = r0 * base * (lam_next2 ? l0 - load4(lam_next2 + i).x : l0);
+        else s_f = (r0 * base - fv[0]) * l0;
         R s_w1 = R(0), s_w2 = R(0);        // sums of ls over the axis and the edge velocities
         R gx = R(0), gy = R(0), gz = R(0);
+        // rows, planes and columns two links away
+        unsigned zo2[3], yo2[3], xs2[3];
+        if constexpr (FROM_MOMENTS) {
+            const unsigned plane = unsigned(a.nx) * unsigned(a.ny), vol = plane * unsigned(a.nz);
+            auto two = [](unsigned lo, unsigned hi, unsigned step, unsigned end, unsigned (&o)[3]) {
+                o[0] = lo == 0 ? end - step : lo - step;
+                o[2] = hi + step == end ? 0 : hi + step;
+            };
+            two(w.zo[0], w.zo[2], plane, vol, zo2);
+            two(w.yo[0], w.yo[2], unsigned(a.nx), plane, yo2);
+            two(xs[0], xs[2], 1u, unsigned(a.nx), xs2);
+            zo2[1] = w.zo[1];
+            yo2[1] = w.yo[1];
+            xs2[1] = xs[1];
+        }
         static_for<0, 9>([&](auto pc) {
             constexpr int q = 2 * decltype(pc)::value + 1;
             const Vec4<R> p = load4(lam_next + nb_of(w, xs, cx(q), cy(q), cz(q)));
@@ -283,7 +334,18 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
             const R wr = q < 7 ? r1 : r2;
             const R e = wr * (base + R(4.5) * cu * cu), od = wr * (R(3) * cu);
             s_feq += e * sl + od * dl;
-            s_f += ((e + od) - fv[q]) * lp + ((e - od) - fv[q + 1]) * lm;
+            if constexpr (FROM_MOMENTS) {
+                R kp = lp, km = lm;
+                if (lam_next2) {
+                    const Vec4<R> p2 = load4(lam_next2 + (zo2[cz(q) + 1] + yo2[cy(q) + 1] + xs2[cx(q) + 1]));
+                    const Vec4<R> o2 = load4(lam_next2 + (zo2[1 - cz(q)] + yo2[1 - cy(q)] + xs2[1 - cx(q)]));
+                    kp -= p2.x + dot_c<q>(p2.y, p2.z, p2.w);
+                    km -= o2.x - dot_c<q>(o2.y, o2.z, o2.w);
+                }
+                s_f += (e + od) * kp + (e - od) * km;
+            } else {
+                s_f += ((e + od) - fv[q]) * lp + ((e - od) - fv[q + 1]) * lm;
+            }
             if constexpr (q < 7) s_w1 += sl;
             else s_w2 += sl;
             // d f_eq / d u' = w rho (3 c + 9 (c.u') c - 3 u')
@@ -292,10 +354,13 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
             if constexpr (cy(q) != 0) gy += R(cy(q)) * k;
             if constexpr (cz(q) != 0) gz += R(cz(q)) * k;
         });
-        const R s3 = R(-3) * (r0 * l0 + r1 * s_w1 + r2 * s_w2);
-        gx += s3 * ux;
-        gy += s3 * uy;
-        gz += s3 * uz;
+        const R s_wr = r0 * l0 + r1 * s_w1 + r2 * s_w2;  // sum_q w_q rho ls_q
+        if constexpr (FROM_MOMENTS) {
+            if (first) s_f -= s_wr;
+        }
+        gx -= R(3) * s_wr * ux;
+        gy -= R(3) * s_wr * uy;
+        gz -= R(3) * s_wr * uz;
         // u' = (j + F)/rho at tau = 1
         const R gjx = gx * inv_rho, gjy = gy * inv_rho, gjz = gz * inv_rho;
         const R g_rho = (s_feq - (gx * ux + gy * uy + gz * uz)) * inv_rho;
@@ -408,9 +473,9 @@ cudaError_t run_adjoint_step(const AdjointArgs& a, const void* f, void* psi, boo
                                                   par<R>(a.rho0, a.rho0f), R(1.0 / a.rho0));
     Vec4<R>* const v = static_cast<Vec4<R>*>(gF);
     if (a.tau1) {
-        adj_collide1_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(f), static_cast<const R*>(psi),
-                                                       static_cast<const Vec4<R>*>(lam_next),
-                                                       static_cast<Vec4<R>*>(lam_out), v, partials, a);
+        adj_collide1_kernel<R, false><<<grid, block, 0, st>>>(
+            static_cast<const R*>(f), static_cast<const R*>(psi), static_cast<const Vec4<R>*>(lam_next), nullptr,
+            static_cast<Vec4<R>*>(lam_out), v, partials, false, a);
         adj_force_kernel<R, true><<<grid, block, 0, st>>>(static_cast<const R*>(psi), v, static_cast<R*>(lam_out), a);
         return cudaGetLastError();
     }
@@ -431,6 +496,19 @@ cudaError_t adjoint_step(const AdjointArgs& a, bool f64, const void* f, void* ps
                                           acc, st)
                : run_adjoint_step<float>(a, f, psi, psi_ready, lam_next, gr_next, lam_out, gr_out, gF, partials,
                                          acc, st);
+}
+
+cudaError_t adjoint_step_moments(const AdjointArgs& a, const float* moments, float* psi, bool psi_ready,
+                                 const void* lam_next, const void* lam_next2, void* lam_out, void* gF,
+                                 double* partials, bool first, cudaStream_t st) {
+    const dim3 block(kRowThreads, kRows);
+    if (!psi_ready) adj_psi_moments_kernel<<<a.grid, block, 0, st>>>(moments, psi, a);
+    Vec4<float>* const v = static_cast<Vec4<float>*>(gF);
+    adj_collide1_kernel<float, true><<<a.grid, block, 0, st>>>(
+        moments, psi, static_cast<const Vec4<float>*>(lam_next), static_cast<const Vec4<float>*>(lam_next2),
+        static_cast<Vec4<float>*>(lam_out), v, partials, first, a);
+    adj_force_kernel<float, true><<<a.grid, block, 0, st>>>(psi, v, static_cast<float*>(lam_out), a);
+    return cudaGetLastError();
 }
 
 cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, void* lam, void* gr, cudaStream_t st) {

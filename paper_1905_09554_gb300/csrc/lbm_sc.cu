@@ -76,6 +76,8 @@ struct lbm_ctx {
         size_t cp_bytes = 0, seg_bytes = 0, psi_bytes = 0;
         long T = -1;                  // steps of the recorded forward run
         int every = 0, ncp = 0;
+        bool moments = false;         // cp and seg hold moment fields instead of populations
+        void* lam3 = nullptr;         // moments: lam of two steps on (the third of three in turn)
     } adj;
 
     lbm_status fail(lbm_status s, const char* fmt, ...) {
@@ -955,6 +957,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->adj.seg);
     cudaFree(c->adj.lam[0]);
     cudaFree(c->adj.lam[1]);
+    cudaFree(c->adj.lam3);
     cudaFree(c->adj.gr[0]);
     cudaFree(c->adj.gr[1]);
     cudaFree(c->adj.psi);
@@ -1787,7 +1790,10 @@ lbm_status lbm_adjoint_forward(lbm_ctx* c, const double* rho0, int on_device, lo
     if (!rho0 || nsteps < 1 || every < 1) return c->fail(LBM_EINVAL, "lbm_adjoint_forward: need rho0, n >= 1, every >= 1");
     if (c->n > 0xffffffffLL) return c->fail(LBM_EUNSUPPORTED, "lbm_adjoint_forward: needs nx*ny*nz < 2^32");
     auto& A = c->adj;
-    const size_t state = (size_t)Q * (size_t)c->n * c->elem;
+    // tau = 1 in FP32: a state's four moments are all the adjoint needs of it
+    A.moments = c->mom && c->p.storage == LBM_F32 && c->p.tau == 1.0;
+    const size_t state = A.moments ? c->mom_bytes : (size_t)Q * (size_t)c->n * c->elem;
+    A.T = -1;  // nothing recorded until the run is complete
     const int ncp = int((nsteps + every - 1) / every);
     if (A.cp && (A.cp_bytes < (size_t)ncp * state)) {
         cudaStreamSynchronize(c->stream);
@@ -1813,6 +1819,24 @@ lbm_status lbm_adjoint_forward(lbm_ctx* c, const double* rho0, int on_device, lo
     }
     lbm_status st = lbm_set_density(c, rho0, on_device);
     if (st != LBM_OK) return st;
+    if (A.moments) {
+        // state t of a checkpoint lies in its slot, the others alternate between two of the segment's
+        MomentLaunch l = c->mom_launch;
+        l.stream = c->stream;
+        auto slot = [&](long t) {
+            return t % every == 0 && t < nsteps ? static_cast<char*>(A.cp) + (size_t)(t / every) * state
+                                                : static_cast<char*>(A.seg) + (size_t)(every > 1 ? t & 1 : 0) * state;
+        };
+        LBM_CUDA(c, c->mom->gather(l, c->f[c->cur], slot(0)));
+        for (long t = 0; t + 1 < nsteps; ++t) LBM_CUDA(c, c->mom->step(l, slot(t), slot(t + 1)));
+        c->cur ^= int(nsteps & 1);
+        LBM_CUDA(c, c->mom->emit(l, slot(nsteps - 1), c->f[c->cur]));
+        c->t += nsteps;
+        A.T = nsteps;
+        A.every = every;
+        A.ncp = ncp;
+        return LBM_OK;
+    }
     for (long t = 0; t < nsteps; t += every) {
         LBM_CUDA(c, cudaMemcpyAsync(static_cast<char*>(A.cp) + (size_t)(t / every) * state, c->f[c->cur], state,
                                     cudaMemcpyDeviceToDevice, c->stream));
@@ -1832,16 +1856,20 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     if (A.T < 1) return c->fail(LBM_EINVAL, "lbm_adjoint_backward: call lbm_adjoint_forward first");
     if (!dJdrho) return c->fail(LBM_EINVAL, "lbm_adjoint_backward: dJdrho is NULL");
     const bool f64 = c->p.storage == LBM_F64;
-    const size_t state = (size_t)Q * (size_t)c->n * c->elem;
+    const size_t state = A.moments ? c->mom_bytes : (size_t)Q * (size_t)c->n * c->elem;
     const AdjointArgs a = adjoint_args(c);
     lbm_status st;
+    const size_t field = (size_t)c->n * c->elem;
     for (void** p : {&A.lam[0], &A.lam[1]}) {
-        st = adj_alloc(c, p, state);
+        st = adj_alloc(c, p, (a.tau1 ? 4 : Q) * field);
         if (st != LBM_OK) return st;
     }
-    for (void** p : {&A.gr[0], &A.gr[1]}) {
-        st = adj_alloc(c, p, (size_t)c->n * c->elem);
-        if (st != LBM_OK) return st;
+    if (A.moments && (st = adj_alloc(c, &A.lam3, 4 * field)) != LBM_OK) return st;
+    if (!a.tau1) {
+        for (void** p : {&A.gr[0], &A.gr[1]}) {
+            st = adj_alloc(c, p, field);
+            if (st != LBM_OK) return st;
+        }
     }
     // psi of every state of a segment: written by the step kernel during the
     // recomputation where it supports that (kernels 1 and 3, and 5 whose
@@ -1874,7 +1902,31 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     LBM_CUDA(c, cudaMemsetAsync(A.partials, 0, sizeof(double) * 2 * (size_t)a.grid, c->stream));
     LBM_CUDA(c, adjoint_seed(a, f64, g, A.lam[0], A.gr[0], c->stream));
     int cur = 0;  // lam[cur] holds dJ/df(t+1)
-    for (int k = A.ncp - 1; k >= 0; --k) {
+    void* lams[3] = {A.lam[0], A.lam[1], A.lam3};  // moments: lams[cur] is lam(t + 1), the one before it lam(t + 2)
+    for (int k = A.ncp - 1; k >= 0 && A.moments; --k) {
+        const long t0 = (long)k * A.every;
+        const long t1 = t0 + A.every < A.T ? t0 + A.every : A.T;
+        auto slot = [&](long t) {
+            return t == t0 ? static_cast<char*>(A.cp) + (size_t)k * state
+                           : static_cast<char*>(A.seg) + (size_t)(t - t0) * state;
+        };
+        auto psi_at = [&](long t) { return reinterpret_cast<float*>(static_cast<char*>(A.psi) + (size_t)(t - t0) * psi_bytes); };
+        MomentLaunch l = c->mom_launch;
+        l.stream = c->stream;
+        for (long t = t0; t + 1 < t1; ++t) {
+            l.args.psi_out = psi_at(t);
+            cudaError_t e = c->mom->step(l, slot(t), slot(t + 1));
+            if (e != cudaSuccess) return c->fail(LBM_ECUDA, "adjoint recompute: %s", cudaGetErrorString(e));
+        }
+        for (long t = t1 - 1; t >= t0; --t) {
+            cudaError_t e = adjoint_step_moments(a, reinterpret_cast<const float*>(slot(t)), psi_at(t), t + 1 < t1,
+                                                 lams[cur], t + 1 < A.T ? lams[(cur + 2) % 3] : nullptr,
+                                                 lams[(cur + 1) % 3], A.gF, A.partials, t == 0, c->stream);
+            if (e != cudaSuccess) return c->fail(LBM_ECUDA, "adjoint step: %s", cudaGetErrorString(e));
+            cur = (cur + 1) % 3;
+        }
+    }
+    for (int k = A.ncp - 1; k >= 0 && !A.moments; --k) {
         const long t0 = (long)k * A.every;
         const long t1 = t0 + A.every < A.T ? t0 + A.every : A.T;
         // recompute the segment's states from its checkpoint
@@ -1900,7 +1952,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     LBM_CUDA(c, adjoint_reduce(a, A.partials, A.acc, c->stream));
     if (dJdrho0) {
         double* out = out_on_device ? dJdrho0 : A.io;
-        LBM_CUDA(c, adjoint_rho0(a, f64, A.lam[cur], A.gr[cur], out, c->stream));
+        LBM_CUDA(c, adjoint_rho0(a, f64, lams[cur], cur < 2 ? A.gr[cur] : nullptr, out, c->stream));
         if (!out_on_device)
             LBM_CUDA(c, cudaMemcpyAsync(dJdrho0, A.io, sizeof(double) * (size_t)c->n, cudaMemcpyDeviceToHost, c->stream));
     }

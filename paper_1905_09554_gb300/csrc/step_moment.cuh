@@ -268,6 +268,15 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             float* const buf = buf0 + (p & 1) * T::BUF + T::EXCH;
             q.w.c = psi_v(rho_of(p));
             put_psi(buf, ps, q.w.c);
+            if constexpr (!EMIT && !BATCH && !HALF && NV == 2) {  // kept for the adjoint
+                if (a.psi_out && own && p >= zs && p < ze) {
+                    float* d = static_cast<float*>(a.psi_out) + ((long long)p * ny + y) * nx + x;
+                    float lo, hi;
+                    unpack2(q.w.c, lo, hi);
+                    d[0] = lo;
+                    if (x + 1 < nx) d[1] = hi;
+                }
+            }
             if (ring)
                 put_psi(buf, hs,
                         psi_v(*reinterpret_cast<const V*>(rho_st + (p & 7) * T::RHO + NV * (tid + T::NT))));
