@@ -28,6 +28,7 @@
 
 #include "adjoint.h"
 #include "collide.cuh"
+#include "launch.cuh"
 #include "lattice.cuh"
 
 namespace lbm {
@@ -189,6 +190,7 @@ adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* 
                    const R* __restrict__ gr_next, R* __restrict__ lam_out, Vec4<R>* __restrict__ fa,
                    double* __restrict__ partials, AdjointArgs a) {
     const unsigned n = unsigned(a.n);
+    chain_begin();
     const R tau = par<R>(a.tau, a.tauf), omega = par<R>(a.omega, a.omegaf);
     double accG = 0.0, accT = 0.0;
     for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
@@ -250,6 +252,7 @@ adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* 
         accG += double(-(ps * sx) * gFx - (ps * sy) * gFy - (ps * sz) * gFz);
         accT += double(g_tau);
     });
+    chain_end();
     block_sum2(accG, accT, partials + 2 * blockIdx.x);
 }
 
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Vec4<R>* __restrict__ lam_next,
                     const Vec4<R>* __restrict__ lam_next2, Vec4<R>* __restrict__ lam_out, Vec4<R>* __restrict__ fa,
                     double* __restrict__ partials, bool first, AdjointArgs a) {
+    chain_begin();
     const unsigned n = unsigned(a.n);
     const int pitch = moment_pitch(a.nx);
     const long long nf = (long long)pitch * a.ny * a.nz;
@@ -370,6 +374,7 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
         accG += double(-ps * sg);                                        // dF/dG = -psi S
         accT += double((gjx * Fx + gjy * Fy + gjz * Fz) - s_f);          // d omega / d tau = -1
     });
+    chain_end();
     block_sum2(accG, accT, partials + 2 * blockIdx.x);
 }
 
@@ -380,6 +385,7 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
 template <class R, bool TAU1>
 __global__ void __launch_bounds__(kThreads)
 adj_force_kernel(const R* __restrict__ psi, const Vec4<R>* __restrict__ fa, R* __restrict__ gr, AdjointArgs a) {
+    chain_begin();
     const R G = par<R>(a.G, a.Gf), inv_rho0 = R(1.0 / a.rho0);
     for_each_cell(a.nx, a.ny, a.nz, [&](const Row& w, const unsigned (&xs)[3], unsigned i) {
         R axis = R(0), edge = R(0);
@@ -473,18 +479,21 @@ cudaError_t run_adjoint_step(const AdjointArgs& a, const void* f, void* psi, boo
                                                   par<R>(a.rho0, a.rho0f), R(1.0 / a.rho0));
     Vec4<R>* const v = static_cast<Vec4<R>*>(gF);
     if (a.tau1) {
-        adj_collide1_kernel<R, false><<<grid, block, 0, st>>>(
-            static_cast<const R*>(f), static_cast<const R*>(psi), static_cast<const Vec4<R>*>(lam_next), nullptr,
-            static_cast<Vec4<R>*>(lam_out), v, partials, false, a);
-        adj_force_kernel<R, true><<<grid, block, 0, st>>>(static_cast<const R*>(psi), v, static_cast<R*>(lam_out), a);
-        return cudaGetLastError();
+        cudaError_t e = launch_chained(a.n <= 1500000, adj_collide1_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(f),
+                                       static_cast<const R*>(psi), static_cast<const Vec4<R>*>(lam_next), nullptr,
+                                       static_cast<Vec4<R>*>(lam_out), v, partials, false, a);
+        if (e != cudaSuccess) return e;
+        return launch_chained(a.n <= 1500000, adj_force_kernel<R, true>, grid, block, 0, st, static_cast<const R*>(psi), v,
+                              static_cast<R*>(lam_out), a);
     }
-    adj_collide_kernel<R><<<grid, block, 0, st>>>(static_cast<const R*>(f), static_cast<const R*>(psi),
-                                                  static_cast<const R*>(lam_next), static_cast<const R*>(gr_next),
-                                                  static_cast<R*>(lam_out), v, partials, a);
-    adj_force_kernel<R, false><<<grid, block, 0, st>>>(static_cast<const R*>(psi), v, static_cast<R*>(gr_out), a);
+    cudaError_t e = launch_chained(a.n <= 1500000, adj_collide_kernel<R>, grid, block, 0, st, static_cast<const R*>(f),
+                                   static_cast<const R*>(psi), static_cast<const R*>(lam_next),
+                                   static_cast<const R*>(gr_next), static_cast<R*>(lam_out), v, partials, a);
+    if (e != cudaSuccess) return e;
+    e = launch_chained(a.n <= 1500000, adj_force_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(psi), v,
+                       static_cast<R*>(gr_out), a);
     (void)acc;  // the per-block sums stay in `partials` until adjoint_reduce
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace
@@ -504,11 +513,11 @@ cudaError_t adjoint_step_moments(const AdjointArgs& a, const float* moments, flo
     const dim3 block(kRowThreads, kRows);
     if (!psi_ready) adj_psi_moments_kernel<<<a.grid, block, 0, st>>>(moments, psi, a);
     Vec4<float>* const v = static_cast<Vec4<float>*>(gF);
-    adj_collide1_kernel<float, true><<<a.grid, block, 0, st>>>(
-        moments, psi, static_cast<const Vec4<float>*>(lam_next), static_cast<const Vec4<float>*>(lam_next2),
-        static_cast<Vec4<float>*>(lam_out), v, partials, first, a);
-    adj_force_kernel<float, true><<<a.grid, block, 0, st>>>(psi, v, static_cast<float*>(lam_out), a);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(
+        a.n <= 1500000, adj_collide1_kernel<float, true>, a.grid, block, 0, st, moments, psi, static_cast<const Vec4<float>*>(lam_next),
+        static_cast<const Vec4<float>*>(lam_next2), static_cast<Vec4<float>*>(lam_out), v, partials, first, a);
+    if (e != cudaSuccess) return e;
+    return launch_chained(a.n <= 1500000, adj_force_kernel<float, true>, a.grid, block, 0, st, psi, v, static_cast<float*>(lam_out), a);
 }
 
 cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, void* lam, void* gr, cudaStream_t st) {

@@ -57,8 +57,8 @@ struct lbm_ctx {
     MomentLaunch mom_launch{};
     size_t mom_bytes = 0;             // one set of moment fields
     bool mom_twice = false;           // two sets fit into one population copy
-    // FP64 steps in two kernels (step_split.cuh); in place where the moments
-    // are all a collision needs of the populations it overwrites.
+    // Steps in two kernels (step_split.cuh); in place where the moments are all
+    // a collision needs of the populations it overwrites.
     bool split = false, split_in_place = false;
     char err[512] = {0};
     lbm_batch* batch = nullptr;       // set when the context is a view of a batch box
@@ -378,7 +378,12 @@ cudaError_t step_once(const lbm_ctx* c, void* src, void* dst, bool keep_src = fa
     void* psi = psi_out ? psi_out : c->psi_ws;
     if (!keep_src && c->split_in_place) psi = nullptr;
     SplitLaunch l{c->args, BatchArgs{}, unsigned(c->n), c->stream};
-    return split_step_f64(l, c->coll, src, dst, psi);
+    if (c->ref[0]) {  // local-reference storage: the density fields follow their population copies
+        const int k = src == c->f[0] ? 0 : 1;
+        l.args.ref_src = c->ref[k];
+        l.args.ref_dst = c->ref[k ^ 1];
+    }
+    return split_step(l, c->p.storage, c->coll, src, dst, psi);
 }
 
 // Tensor maps of the two population copies for the tensor-copy kernel:
@@ -482,6 +487,19 @@ long long busiest_block_planes(long long nz, long long tiles, long long grid, lo
         if (load > worst) worst = load;
     }
     return worst;
+}
+
+// Largest box that 32- and 16-bit storage steps in two kernels, measured on
+// GB300 (us a step, marching kernel / two kernels, single steps):
+//   FP32, SRT tau = 0.83: 221 k cells 20.6 / 10.7, 524 k 20.6 / 20.8, 1.02 M 41.1 / 42.3
+//   FP32 in place (tau = 1): 1.02 M 41.1 / 33.4, 1.77 M 60.4 / 67.1
+//   FP16 from one reference: 524 k 22.7 / 21.6, 1.02 M 47.2 / 37.0, 1.77 M 67.7 / 59.7, 4.2 M 117 / 135
+//   FP16 from local references: 221 k 14.5 / 13.2, 524 k 22.6 / 25.0
+//   odd rows (no pipelined kernel): FP16 1.08 M 48.7 / 37.0, 19.6 M 738 / 583
+long long split_cells(const lbm_params& p, bool in_place) {
+    if (p.storage >= LBM_F16_DEV && p.nx % 2 != 0) return 1LL << 40;
+    if (p.storage == LBM_F32) return in_place ? 1200000 : 400000;
+    return p.storage >= LBM_F16_LOCAL ? 250000 : 2000000;
 }
 
 constexpr long long kSplitPad = 1024;  // block rounding of the two-kernel step's 32-bit cell index
@@ -674,6 +692,10 @@ void configure_moments(lbm_ctx* c) {
             l.args.zchunk = z;
         }
     }
+    // Small boxes: a turn of the moment kernel (one plane of the busiest block) takes about 1.5 us however few
+    // blocks there are, two kernels 29 ps a cell and 4 us at least (24x24x48: 10.4 / 4.2 us a step; 64x64x128: 14.7
+    // / 20.5; MRT with the paper's rates 48x48x96: 20.9 / 10.9, 80x80x160: 52.4 / 41.1, 96x96x192: 55.6 / 77).
+    if (c->split && 2.5 + 1.5 * double(best) > 4.0 + 29e-6 * double(c->n)) return;
     l.args.n_items = l.args.n_tiles * ((p.nz + l.args.zchunk - 1) / l.args.zchunk);
     l.grid = int(grid < l.args.n_items ? grid : l.args.n_items);
     const long long rows = ((long long)p.ny * p.nz + 7) / 8;
@@ -901,9 +923,11 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     round_params(a);
     c->coll = collision_kernel(*p, a.s);
-    // FP64 steps in two kernels unless one particular kernel was asked for
-    c->split = p->storage == LBM_F64 && p->kernel == 0 && p->G2 == 0.0 && n <= 0xffffffffLL - kSplitPad;
-    c->split_in_place = c->split && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p->tau != 1.0);
+    // Steps in two kernels, unless one particular kernel was asked for: FP64, small boxes, odd 16-bit rows
+    const bool in_place = p->storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p->tau != 1.0);
+    c->split = p->kernel == 0 && p->G2 == 0.0 && n <= 0xffffffffLL - kSplitPad &&
+               (p->storage == LBM_F64 || n <= split_cells(*p, in_place));
+    c->split_in_place = c->split && in_place;
     if (p->G2 != 0.0 || (c->split && !c->split_in_place)) {
         // psi of the whole box; where there is no room the step runs without it, slower
         const size_t pbytes = (size_t)n * (p->storage == LBM_F64 ? 8 : 4);
@@ -1368,7 +1392,7 @@ StepLaunch batch_launch(const lbm_batch* b) {
 cudaError_t batch_launch_step(const lbm_batch* b, int from) {
     if (b->split) {
         SplitLaunch l{b->phys, b->bargs, b->max_cells, b->stream};
-        return split_step_f64(l, b->box[0]->coll, b->f[from], b->f[from ^ 1], nullptr);
+        return split_step(l, b->p.storage, b->box[0]->coll, b->f[from], b->f[from ^ 1], nullptr);
     }
     const StepLaunch l = batch_launch(b);
     return step_kernels(b->p.storage, l.coll).batch(l, b->bargs, b->f[from], b->f[from ^ 1]);

@@ -148,16 +148,16 @@ struct MomentKernels {
 // nullptr where the collision (or the storage) has no moment form.
 const MomentKernels* moment_kernels(int storage, int coll);
 
-// The FP64 step in two kernels (step_split.cuh), of one lattice or of a
-// batch's boxes (batch.nbox > 0).  psi: a field of its own for psi of `src`,
-// which is then left as it is; without one (not for general MRT rates, and SRT
-// only at tau = 1) the source populations are overwritten.
+// The step in two kernels (step_split.cuh), of one lattice or of a batch's
+// boxes (batch.nbox > 0).  psi: a field of its own for psi of `src`, which is
+// then left as it is; without one (FP64 and FP32; not for general MRT rates,
+// and SRT only at tau = 1) the source populations are overwritten.
 struct SplitLaunch {
     StepArgs args;
     BatchArgs batch;
     unsigned max_cells;   // of the largest box
     cudaStream_t stream;
 };
-cudaError_t split_step_f64(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step(const SplitLaunch& l, int storage, int coll, void* src, void* dst, void* psi);
 
 }  // namespace lbm

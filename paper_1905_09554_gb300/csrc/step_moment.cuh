@@ -36,6 +36,7 @@
 // 3 stores for 4 fields, 5 or 6 for 9 or 10.
 #pragma once
 #include "collide.cuh"
+#include "launch.cuh"
 #include "step_kernel.cuh"
 
 namespace lbm {
@@ -177,6 +178,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
     float* const rho_st = buf0 + 2 * T::BUF;       // [8][RHO]
     float* const rest_st = rho_st + 8 * T::RHO;    // [4][REST]
 
+    chain_begin();
     const float rho0 = a.rho0f, inv_rho0 = a.inv_rho0f;
     const DevParams& dev = a.dev;
     auto psi_v = [&](V r) { return vmap(r, [&](float x) { return psi_of<float>(x, rho0, inv_rho0); }); };
@@ -539,6 +541,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             if (p + 2 <= ze + 2) turn(pc, pa, pb, p + 2);
         }
     }
+    chain_end();
 }
 
 // Populations -> moment fields (all the operators above read of a state).
@@ -548,6 +551,7 @@ __global__ void __launch_bounds__(256)
 sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
     using S = typename Codec::S;
     constexpr int NF = kMoments<COLL>;
+    chain_begin();
     int nx = a.nx, ny = a.ny, nz = a.nz;
     long long base = 0;
     if constexpr (BATCH) {
@@ -593,13 +597,15 @@ sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, 
 template <int COLL>
 constexpr int kCells = kMoments<COLL> == 4 ? 2 : 1;
 
+// Small boxes (a step under ~30 us) chain their kernels.
+inline bool moment_chain(const MomentLaunch& l) { return !l.batch.nbox && l.args.n <= 1500000; }
+
 template <class Codec, int COLL, bool EMIT, bool BATCH>
 cudaError_t moment_launch(const MomentLaunch& l, const void* src, void* dst) {
     using T = MomentTile<kCells<COLL>>;
-    sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH>
-        <<<l.grid, T::NT, T::bytes(kMoments<COLL>), l.stream>>>(src, dst, l.args, l.batch,
-                                                                MomentArgs{l.src_hi, l.dst_hi});
-    return cudaGetLastError();
+    return launch_chained(moment_chain(l), sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH>, l.grid, T::NT,
+                          T::bytes(kMoments<COLL>), l.stream, src, dst, l.args, l.batch,
+                          MomentArgs{l.src_hi, l.dst_hi});
 }
 
 template <class Codec, int COLL, bool EMIT>
@@ -614,14 +620,12 @@ template <class Codec, int COLL>
 cudaError_t moment_gather(const MomentLaunch& l, const void* src, void* dst) {
     constexpr int NV = kCells<COLL>;
     if constexpr (sizeof(typename Codec::S) == 4) {
-        if (l.batch.nbox) {
-            sc_moments_kernel<Codec, COLL, NV, true><<<dim3(l.gather_grid, l.batch.nbox), 256, 0, l.stream>>>(
-                src, dst, l.args, l.batch);
-            return cudaGetLastError();
-        }
+        if (l.batch.nbox)
+            return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, NV, true>, dim3(l.gather_grid, l.batch.nbox), 256, 0,
+                                  l.stream, src, dst, l.args, l.batch);
     }
-    sc_moments_kernel<Codec, COLL, NV, false><<<l.gather_grid, 256, 0, l.stream>>>(src, dst, l.args, l.batch);
-    return cudaGetLastError();
+    return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, NV, false>, l.gather_grid, 256, 0, l.stream, src, dst, l.args,
+                          l.batch);
 }
 
 template <class Codec, int COLL, bool EMIT, bool BATCH>

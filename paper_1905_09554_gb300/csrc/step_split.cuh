@@ -1,31 +1,47 @@
-// The FP64 step in two kernels without any redundant arithmetic.
+// The step in two kernels without any redundant arithmetic.
 //
-// GB300 issues FP64 at 2 lanes an SM and clock, so an FP64 step is bound by
-// its ~150 FP64 operations a cell (150 / (152 x 2 x 2.07 GHz) = 0.24 ns) while
-// HBM would deliver 1600 bytes in that time.  The one-kernel steps compute psi
-// of their tiles' rims again (19 additions, an exponential and a division's
-// worth of work per rim cell; 0.6 rim cells per cell on the 32 x 4 tiles that
-// FP64 needs) and the density twice.  Here
 //   sc_fields_kernel  forms psi of every cell once, from its populations; where
 //       the collision needs no more than the moments (collide.cuh), it leaves
 //       those and psi in the first slots of the cell's own populations,
 //   sc_push_kernel    reads psi of the 18 neighbours (through L1) and the
 //       moments or populations, collides and pushes.
-// The extra traffic (72 to 88 B a cell) hides behind the FP64 pipe.  Cells are dealt
-// linearly to 64-thread blocks, so that small boxes fill the chip too.
+// Cells are dealt linearly to small blocks: no tile, rim, chunk or barrier.
+//
+// FP64: GB300 issues FP64 at 2 lanes an SM and clock, so a step is bound by its
+// ~150 FP64 operations a cell (150 / (152 x 2 x 2.07 GHz) = 0.24 ns) while HBM
+// would deliver 1600 bytes in that time.  The one-kernel steps compute psi of
+// their tiles' rims again (19 additions and an exponential per rim cell, 0.6
+// rim cells per cell on the 32 x 4 tiles that FP64 needs) and the density
+// twice; the 72 to 88 B a cell that the second kernel adds hide behind the
+// FP64 pipe.
+//
+// 32- and 16-bit storage: the extra passes cost bytes, so large boxes keep the
+// marching kernels.  Boxes that live in L2 are bound by the marching kernels'
+// latency instead (a few planes per block, one barrier each), and 16-bit
+// storage with odd rows has no pipelined kernel at all.
 #pragma once
 #include "collide.cuh"
+#include "launch.cuh"
 #include "step_kernel.cuh"
 
 namespace lbm {
 
 constexpr int kSplitThreads = 64;
 
-// psi in slot kMoments<COLL> behind the moments (IN_PLACE), or in its own field.
-template <int COLL, bool IN_PLACE>
+// Element k of cell i of a field array with n cells each.
+template <class S>
+__device__ __forceinline__ S* cell_at(S* p, int k, unsigned n, unsigned i) {
+    return p + (k * (long long)n + i);
+}
+
+// psi in slot kMoments<COLL> behind the moments (IN_PLACE), or in its own
+// field.  Local-reference storage: the density goes to ref_dst as well.
+template <class Codec, int COLL, bool IN_PLACE>
 __global__ void __launch_bounds__(kSplitThreads)
-sc_fields_kernel(double* f_all, double* psi_all, const StepArgs a, const BatchArgs b) {
+sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const StepArgs a, const BatchArgs b) {
+    using R = typename Codec::R;
     constexpr int NF = kMoments<COLL>;
+    chain_begin();
     unsigned n = unsigned(a.n);
     long long base = 0;
     if (b.nbox) {
@@ -35,43 +51,51 @@ sc_fields_kernel(double* f_all, double* psi_all, const StepArgs a, const BatchAr
     }
     const unsigned i = blockIdx.x * kSplitThreads + threadIdx.x;
     if (i >= n) return;
-    double* const f = f_all + base;
-    double v[Q];
+    typename Codec::S* const f = f_all + base;
+    float ref = 0.0f;
+    if constexpr (Codec::kLocal) ref = __ldg(a.ref_src + i);
+    R v[Q], m[NF];
     static_for<0, Q>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        v[q] = f[q * (long long)n + i];
+        const typename Codec::S s = *cell_at(f, q, n, i);
+        if constexpr (Codec::kLocal) v[q] = Codec::template decode_ref<q>(s, ref, a.dev);
+        else v[q] = Codec::template decode<q>(s, a.dev);
     });
+    moments_of<COLL, R>(v, m);  // (the sums that are not needed fall away)
+    const R p = psi_of<R>(m[0], par<R>(a.rho0, a.rho0f), par<R>(a.inv_rho0, a.inv_rho0f));
+    chain_end();
     if constexpr (IN_PLACE) {
-        double m[NF];
-        moments_of<COLL, double>(v, m);
         static_for<0, NF>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
-            f[k * (long long)n + i] = m[k];
+            *cell_at(f, k, n, i) = m[k];
         });
-        f[NF * (long long)n + i] = psi_of<double>(m[0], a.rho0, a.inv_rho0);
+        *cell_at(f, NF, n, i) = p;
     } else {
-        double m[NF];
-        moments_of<COLL, double>(v, m);  // (the sums that the density does not need fall away)
-        psi_all[i] = psi_of<double>(m[0], a.rho0, a.inv_rho0);
+        psi_all[i] = p;
+        if constexpr (Codec::kLocal) a.ref_dst[i] = m[0];
     }
 }
 
 // psi of a cell's neighbours in one plane; yo, xo: offsets of its rows and columns -1, 0, +1.
+template <class R>
 struct NeighbourPsi {
-    const double* plane;
+    const R* plane;
     const unsigned (&yo)[3];
     const unsigned (&xo)[3];
     template <class DX, class DY>
-    __device__ __forceinline__ double operator()(DX, DY) const {
+    __device__ __forceinline__ R operator()(DX, DY) const {
         return __ldg(plane + (yo[DY::value + 1] + xo[DX::value + 1]));
     }
 };
 
-template <int COLL, bool IN_PLACE>
+template <class Codec, int COLL, bool IN_PLACE>
 __global__ void __launch_bounds__(kSplitThreads)
-sc_push_kernel(const double* __restrict__ src_all, const double* __restrict__ psi_all, double* __restrict__ dst_all,
-               const StepArgs a, const BatchArgs b) {
+sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Codec::R* __restrict__ psi_all,
+               typename Codec::S* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
+    using R = typename Codec::R;
+    using S = typename Codec::S;
     constexpr int NF = kMoments<COLL>;
+    chain_begin();
     int nx = a.nx, ny = a.ny, nz = a.nz;
     long long base = 0;
     if (b.nbox) {
@@ -84,9 +108,10 @@ sc_push_kernel(const double* __restrict__ src_all, const double* __restrict__ ps
     const unsigned plane = unsigned(nx) * unsigned(ny), n = plane * unsigned(nz);
     const unsigned i = blockIdx.x * kSplitThreads + threadIdx.x;
     if (i >= n) return;
-    const double* __restrict__ src = src_all + base;
-    double* __restrict__ dst = dst_all + base;
-    const double* __restrict__ psi = IN_PLACE ? src + NF * (long long)n : psi_all;
+    const S* __restrict__ src = src_all + base;
+    S* __restrict__ dst = dst_all + base;
+    const R* __restrict__ psi = psi_all;
+    if constexpr (IN_PLACE) psi = src + NF * (long long)n;
     const int z = int(i / plane), y = int((i - unsigned(z) * plane) / unsigned(nx)),
               x = int(i - unsigned(z) * plane - unsigned(y) * unsigned(nx));
     const unsigned zo[3] = {unsigned(z == 0 ? nz - 1 : z - 1) * plane, unsigned(z) * plane,
@@ -95,57 +120,87 @@ sc_push_kernel(const double* __restrict__ src_all, const double* __restrict__ ps
                             unsigned(y + 1 == ny ? 0 : y + 1) * nx};
     const unsigned xo[3] = {unsigned(x == 0 ? nx - 1 : x - 1), unsigned(x), unsigned(x + 1 == nx ? 0 : x + 1)};
 
-    PsiView<double> w[3];
+    R f[Q], m[NF];
+    if constexpr (IN_PLACE) {
+        static_for<0, NF>([&](auto kc) {
+            constexpr int k = decltype(kc)::value;
+            m[k] = __ldg(cell_at(src, k, n, i));
+        });
+    } else {
+        float ref = 0.0f;
+        if constexpr (Codec::kLocal) ref = __ldg(a.ref_src + i);
+        static_for<0, Q>([&](auto qc) {
+            constexpr int q = decltype(qc)::value;
+            if constexpr (Codec::kLocal) f[q] = Codec::template load_ref<q>(cell_at(src, q, n, i), ref, a.dev);
+            else f[q] = Codec::template load<q>(cell_at(src, q, n, i), a.dev);
+        });
+    }
+    PsiView<R> w[3];
     static_for<0, 3>([&](auto kc) {
         constexpr int k = decltype(kc)::value;
-        const NeighbourPsi at{psi + zo[k], yo, xo};
+        const NeighbourPsi<R> at{psi + zo[k], yo, xo};
         w[k].c = __ldg(psi + (zo[k] + yo[1] + xo[1]));
         psi_axis(w[k], at);
         if constexpr (k == 1) psi_diag(w[k], at);
     });
-    const Force<double> F = force_of(w[0], w[1], w[2], a.gw);
-    double f[Q];
+    const Force<R> F = force_of(w[0], w[1], w[2], par<R>(a.gw, a.gwf));
     if constexpr (IN_PLACE) {
-        double m[NF];
-        static_for<0, NF>([&](auto kc) {
-            constexpr int k = decltype(kc)::value;
-            m[k] = __ldg(src + (k * (long long)n + i));
-        });
-        collide_moments<COLL, double, true>(m, F, a, [&](auto qc, double v) {
+        collide_moments<COLL, R, true>(m, F, a, [&](auto qc, R v) {
             constexpr int q = decltype(qc)::value;
             f[q] = v;
         });
     } else {
-        static_for<0, Q>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            f[q] = __ldg(src + (q * (long long)n + i));
-        });
-        collide<COLL, double>(f, F, a);
+        collide<COLL, R>(f, F, a);
     }
+    chain_end();
     // Eq. LBE streaming: f_a(x + c_a, t + 1) = f*_a(x, t).
     static_for<0, Q>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        dst[q * (long long)n + (zo[cz(q) + 1] + yo[cy(q) + 1] + xo[cx(q) + 1])] = f[q];
+        const unsigned to = zo[cz(q) + 1] + yo[cy(q) + 1] + xo[cx(q) + 1];
+        S* const d = cell_at(dst, q, n, to);
+        if constexpr (Codec::kLocal) {
+            // deviation from the rest equilibrium at the destination's density (written by the first kernel)
+            Codec::template store_ref<q>(d, f[q], __ldg(a.ref_dst + to), a.dev);
+        } else {
+            Codec::template store<q>(d, f[q], a.dev);
+        }
     });
 }
 
-template <int COLL>
+template <class Codec, int COLL>
 cudaError_t split_step(const SplitLaunch& l, void* src, void* dst, void* psi) {
+    using S = typename Codec::S;
+    using R = typename Codec::R;
     const dim3 grid((l.max_cells + kSplitThreads - 1) / kSplitThreads, l.batch.nbox ? l.batch.nbox : 1);
-    double* const s = static_cast<double*>(src);
-    double* const d = static_cast<double*>(dst);
-    double* const p = static_cast<double*>(psi);
-    if constexpr (COLL != COLL_MRT) {
-        if (!psi) {
-            sc_fields_kernel<COLL, true><<<grid, kSplitThreads, 0, l.stream>>>(s, nullptr, l.args, l.batch);
-            sc_push_kernel<COLL, true><<<grid, kSplitThreads, 0, l.stream>>>(s, nullptr, d, l.args, l.batch);
-            return cudaGetLastError();
-        }
+    S* const s = static_cast<S*>(src);
+    S* const d = static_cast<S*>(dst);
+    R* const p = static_cast<R*>(psi);
+    const bool chain = (long long)grid.x * grid.y * kSplitThreads <= 400000;
+    auto both = [&](auto in_place) {
+        constexpr bool IN = decltype(in_place)::value;
+        cudaError_t e = launch_chained(chain, sc_fields_kernel<Codec, COLL, IN>, grid, kSplitThreads, 0, l.stream, s, p, l.args,
+                                       l.batch);
+        if (e == cudaSuccess)
+            e = launch_chained(chain, sc_push_kernel<Codec, COLL, IN>, grid, kSplitThreads, 0, l.stream, s, p, d, l.args,
+                               l.batch);
+        return e;
+    };
+    if constexpr (COLL != COLL_MRT && sizeof(S) == sizeof(R)) {
+        if (!psi) return both(std::true_type{});
     }
     if (!psi || l.batch.nbox) return cudaErrorInvalidValue;
-    sc_fields_kernel<COLL, false><<<grid, kSplitThreads, 0, l.stream>>>(s, p, l.args, l.batch);
-    sc_push_kernel<COLL, false><<<grid, kSplitThreads, 0, l.stream>>>(s, p, d, l.args, l.batch);
-    return cudaGetLastError();
+    return both(std::false_type{});
+}
+
+template <class Codec>
+cudaError_t split_collisions(const SplitLaunch& l, int coll, void* src, void* dst, void* psi) {
+    switch (coll) {
+        case COLL_SRT: return split_step<Codec, COLL_SRT>(l, src, dst, psi);
+        case COLL_MRT: return split_step<Codec, COLL_MRT>(l, src, dst, psi);
+        case COLL_MRT_SPARSE: return split_step<Codec, COLL_MRT_SPARSE>(l, src, dst, psi);
+        case COLL_MRT_UNIT: return split_step<Codec, COLL_MRT_UNIT>(l, src, dst, psi);
+        default: return split_step<Codec, COLL_MRT_SHEAR>(l, src, dst, psi);
+    }
 }
 
 }  // namespace lbm

@@ -1,0 +1,10 @@
+// The two-kernel step of every collision for CodecBF16Local storage.
+#include "step_split.cuh"
+
+namespace lbm {
+
+cudaError_t split_step_bf16l(const SplitLaunch& l, int coll, void* src, void* dst, void* psi) {
+    return split_collisions<CodecBF16Local>(l, coll, src, dst, psi);
+}
+
+}  // namespace lbm

@@ -61,6 +61,19 @@ const MomentKernels* moment_kernels(int storage, int coll) {
     return table[storage][coll];
 }
 
+cudaError_t split_step_f64(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step_f32(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step_f16(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step_bf16(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step_f16l(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+cudaError_t split_step_bf16l(const SplitLaunch& l, int coll, void* src, void* dst, void* psi);
+
+cudaError_t split_step(const SplitLaunch& l, int storage, int coll, void* src, void* dst, void* psi) {
+    static constexpr decltype(&split_step_f64) table[6] = {split_step_f64,  split_step_f32,  split_step_f16,
+                                                           split_step_bf16, split_step_f16l, split_step_bf16l};
+    return table[storage](l, coll, src, dst, psi);
+}
+
 const StepKernels& step_kernels(int storage, int coll) {
     static const StepKernels* table[6][COLL_COUNT] = {
         {&kStep_f64_srt, &kStep_f64_mrt, &kStep_f64_mrts, &kStep_f64_mrtu, &kStep_f64_mrtsh},
