@@ -38,20 +38,22 @@ __device__ __forceinline__ void diag_cell(const typename Codec::S* __restrict__ 
     jz = az;
 }
 
-// Cells first, first + stride, ... < count of the slice whose populations
-// start at fz (population stride n; refz: the slice's reference densities for
+// Cells first, first + stride, ... < count (in runs of kRun of them; with
+// parts > 1 only every parts-th run from the part-th on, so that several
+// blocks share a slice without changing what a run sums) of the slice whose
+// populations start at fz (population stride n; refz: the slice's reference densities for
 // the local-reference codecs).  acc: mass, jx, jy, jz, liquid area, max rho,
 // cells with rho <= 0 / NaN / Inf.
 template <class Codec>
 __device__ __forceinline__ void diag_accumulate(const typename Codec::S* __restrict__ fz, long long n,
                                                 long long count, long long first, int stride, const DevParams& dev,
                                                 double rho_v, double inv, const float* __restrict__ refz,
-                                                double (&acc)[7]) {
+                                                double (&acc)[7], int part = 0, int parts = 1) {
     using R = typename Codec::R;
     constexpr int kRun = 8;
     for (int k = 0; k < 7; ++k) acc[k] = 0.0;
     const R rv = R(rho_v), iv = R(inv);
-    for (long long i = first; i < count; i += (long long)kRun * stride) {
+    for (long long i = first + (long long)part * kRun * stride; i < count; i += (long long)parts * kRun * stride) {
         R m = R(0), jx = R(0), jy = R(0), jz = R(0), area = R(0), mx = R(0);
         int bad = 0;
 #pragma unroll

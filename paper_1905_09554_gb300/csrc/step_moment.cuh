@@ -139,7 +139,7 @@ __device__ __forceinline__ void store_ends(float* d, long long nf, unsigned od, 
     }
 }
 
-template <class Codec, int COLL, int NV, bool EMIT, bool BATCH>
+template <class Codec, int COLL, int NV, bool EMIT, bool BATCH, bool KEEP_PSI = false>
 __global__ void __launch_bounds__(512, 1)
 sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, const StepArgs a, const BatchArgs b,
                  const MomentArgs ma) {
@@ -270,8 +270,9 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             float* const buf = buf0 + (p & 1) * T::BUF + T::EXCH;
             q.w.c = psi_v(rho_of(p));
             put_psi(buf, ps, q.w.c);
-            if constexpr (!EMIT && !BATCH && !HALF && NV == 2) {  // kept for the adjoint
-                if (a.psi_out && own && p >= zs && p < ze) {
+            if constexpr (KEEP_PSI) {  // for the adjoint
+                static_assert(NV == 2);
+                if (own && p >= zs && p < ze) {
                     float* d = static_cast<float*>(a.psi_out) + ((long long)p * ny + y) * nx + x;
                     float lo, hi;
                     unpack2(q.w.c, lo, hi);
@@ -603,9 +604,18 @@ inline bool moment_chain(const MomentLaunch& l) { return !l.batch.nbox && l.args
 template <class Codec, int COLL, bool EMIT, bool BATCH>
 cudaError_t moment_launch(const MomentLaunch& l, const void* src, void* dst) {
     using T = MomentTile<kCells<COLL>>;
+    const int sm = (int)T::bytes(kMoments<COLL>);
+    if constexpr (COLL == COLL_SRT && !EMIT && !BATCH && std::is_same_v<Codec, CodecF32>) {
+        if (l.args.psi_out) {
+            auto kern = sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH, true>;
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            if (e != cudaSuccess) return e;
+            return launch_chained(moment_chain(l), kern, l.grid, T::NT, sm, l.stream, src, dst, l.args, l.batch,
+                                  MomentArgs{l.src_hi, l.dst_hi});
+        }
+    }
     return launch_chained(moment_chain(l), sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH>, l.grid, T::NT,
-                          T::bytes(kMoments<COLL>), l.stream, src, dst, l.args, l.batch,
-                          MomentArgs{l.src_hi, l.dst_hi});
+                          sm, l.stream, src, dst, l.args, l.batch, MomentArgs{l.src_hi, l.dst_hi});
 }
 
 template <class Codec, int COLL, bool EMIT>
