@@ -177,21 +177,22 @@ __global__ void ligament_kernel(typename Codec::S* __restrict__ f, int nx, int n
     }
 }
 
-// Element i of `f` belongs to population q0 + i / n.
+// n cells of populations q0, q0 + 1, ..., one after the other in `f` and the
+// float64 array: one row of blocks (blockIdx.y) each.
 template <class Codec>
-__global__ void decode_kernel(double* __restrict__ out, const typename Codec::S* __restrict__ f,
-                              long long count, long long n, int q0, DevParams dev, const float* ref) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x)
-        out[i] = dec<Codec>(f + i, q0 + int(i / n), ref, i % n, dev);
+__global__ void decode_kernel(double* __restrict__ out, const typename Codec::S* __restrict__ f, long long n, int q0,
+                              DevParams dev, const float* ref) {
+    const long long at = blockIdx.y * n;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[at + i] = dec<Codec>(f + at + i, q0 + int(blockIdx.y), ref, i, dev);
 }
 
 template <class Codec>
-__global__ void encode_kernel(typename Codec::S* __restrict__ f, const double* __restrict__ in,
-                              long long count, long long n, int q0, DevParams dev, const float* ref) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x)
-        enc<Codec>(f + i, q0 + int(i / n), in[i], ref, i % n, dev);
+__global__ void encode_kernel(typename Codec::S* __restrict__ f, const double* __restrict__ in, long long n, int q0,
+                              DevParams dev, const float* ref) {
+    const long long at = blockIdx.y * n;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        enc<Codec>(f + at + i, q0 + int(blockIdx.y), in[at + i], ref, i, dev);
 }
 
 // Local-reference codecs: the reference density of a cell given all its
@@ -214,14 +215,16 @@ __global__ void ref_sum_kernel(float* __restrict__ ref, double* __restrict__ acc
 }
 
 template <class Codec>
-__global__ void density_kernel(double* __restrict__ rho, const typename Codec::S* __restrict__ f,
-                               long long n, DevParams dev, const float* ref) {
+__global__ void density_kernel(double* __restrict__ rho, double* __restrict__ psi,
+                               const typename Codec::S* __restrict__ f, long long n, double rho0, DevParams dev,
+                               const float* ref) {
     // rho summed in the storage's arithmetic type, as the step kernel does
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         typename Codec::R r, jx, jy, jz;
         diag_cell<Codec>(f + i, n, dev, Codec::kLocal ? ref[i] : 0.0f, r, jx, jy, jz);
         rho[i] = double(r);
+        if (psi) psi[i] = rho0 * (1.0 - exp(-double(r) / rho0));
     }
 }
 
@@ -234,15 +237,28 @@ __device__ __forceinline__ int wrap_periodic(int i, int n) {  // periodic index,
 
 template <class Codec>
 __global__ void velocity_kernel(double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ uz,
-                                const double* __restrict__ rho, const typename Codec::S* __restrict__ f,
+                                const double* __restrict__ rho, const double* __restrict__ psi,
+                                const typename Codec::S* __restrict__ f,
                                 int nx, int ny, int nz, double G, double G2, double rho0, DevParams dev,
                                 const float* ref) {
     const long long n = (long long)nx * ny * nz;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        const int x = int(i % nx);
-        const int y = int((i / nx) % ny);
-        const int z = int(i / ((long long)nx * ny));
+        int x, y, z;
+        if (n <= 0xffffffffLL) {
+            const unsigned row = unsigned(i) / unsigned(nx);
+            z = int(row / unsigned(ny));
+            y = int(row - unsigned(z) * unsigned(ny));
+            x = int(unsigned(i) - row * unsigned(nx));
+        } else {
+            x = int(i % nx);
+            y = int((i / nx) % ny);
+            z = int(i / ((long long)nx * ny));
+        }
+        // psi of a cell: from its field, or (no memory for one) from its density
+        auto psi_at = [&](long long cell) {
+            return psi ? __ldg(psi + cell) : rho0 * (1.0 - exp(-rho[cell] / rho0));
+        };
         double jx = 0, jy = 0, jz = 0, sx = 0, sy = 0, sz = 0;
         static_for<0, Q>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
@@ -255,8 +271,7 @@ __global__ void velocity_kernel(double* __restrict__ ux, double* __restrict__ uy
                 xx = xx < 0 ? nx - 1 : (xx == nx ? 0 : xx);
                 yy = yy < 0 ? ny - 1 : (yy == ny ? 0 : yy);
                 zz = zz < 0 ? nz - 1 : (zz == nz ? 0 : zz);
-                const double rn = rho[((long long)zz * ny + yy) * nx + xx];
-                const double psn = rho0 * (1.0 - exp(-rn / rho0));
+                const double psn = psi_at(((long long)zz * ny + yy) * nx + xx);
                 sx += wq(q) * cx(q) * psn;
                 sy += wq(q) * cy(q) * psn;
                 sz += wq(q) * cz(q) * psn;
@@ -271,15 +286,14 @@ __global__ void velocity_kernel(double* __restrict__ ux, double* __restrict__ uy
                 constexpr double pw = mr::p_e8(e.x * e.x + e.y * e.y + e.z * e.z) / 3.0;
                 const int xx = wrap_periodic(x + e.x, nx), yy = wrap_periodic(y + e.y, ny),
                           zz = wrap_periodic(z + e.z, nz);
-                const double rn = rho[((long long)zz * ny + yy) * nx + xx];
-                const double psn = G2 * pw * rho0 * (1.0 - exp(-rn / rho0));
+                const double psn = G2 * pw * psi_at(((long long)zz * ny + yy) * nx + xx);
                 if constexpr (e.x != 0) sx += e.x * psn;
                 if constexpr (e.y != 0) sy += e.y * psn;
                 if constexpr (e.z != 0) sz += e.z * psn;
             });
         }
         const double r = rho[i];
-        const double g = -rho0 * (1.0 - exp(-r / rho0));
+        const double g = -psi_at(i);
         if (ux) ux[i] = (jx + 0.5 * g * sx) / r;
         if (uy) uy[i] = (jy + 0.5 * g * sy) / r;
         if (uz) uz[i] = (jz + 0.5 * g * sz) / r;
@@ -1194,8 +1208,8 @@ lbm_status lbm_set_populations(lbm_ctx* c, const double* f, int on_device) {
         if (ref) ref_sum_kernel<<<blocks, 256, 0, c->stream>>>(ref, nullptr, f, c->n, Q, 0);
         with_codec(c, [&](auto codec) {
             using C = decltype(codec);
-            encode_kernel<C><<<grid_for((long long)Q * c->n, 256, c->num_sms), 256, 0, c->stream>>>(
-                static_cast<typename C::S*>(c->f[c->cur]), f, (long long)Q * c->n, c->n, 0, c->args.dev, ref);
+            encode_kernel<C><<<dim3(blocks, Q), 256, 0, c->stream>>>(static_cast<typename C::S*>(c->f[c->cur]), f,
+                                                                     c->n, 0, c->args.dev, ref);
             return 0;
         });
         LBM_LAUNCHED(c, "encode_kernel");
@@ -1220,8 +1234,8 @@ lbm_status lbm_set_populations(lbm_ctx* c, const double* f, int on_device) {
             with_codec(c, [&](auto codec) {
                 using C = decltype(codec);
                 encode_kernel<C><<<blocks, 256, 0, c->stream>>>(
-                    static_cast<typename C::S*>(c->f[c->cur]) + (size_t)q * c->n, c->scratch, c->n, c->n, q,
-                    c->args.dev, ref);
+                    static_cast<typename C::S*>(c->f[c->cur]) + (size_t)q * c->n, c->scratch, c->n, q, c->args.dev,
+                    ref);
                 return 0;
             });
             LBM_LAUNCHED(c, "encode_kernel");
@@ -1239,9 +1253,8 @@ lbm_status lbm_get_populations(lbm_ctx* c, double* f, int on_device) {
     if (on_device) {
         with_codec(c, [&](auto codec) {
             using C = decltype(codec);
-            decode_kernel<C><<<grid_for((long long)Q * c->n, 256, c->num_sms), 256, 0, c->stream>>>(
-                f, static_cast<const typename C::S*>(c->f[c->cur]), (long long)Q * c->n, c->n, 0, c->args.dev,
-                c->ref[c->cur]);
+            decode_kernel<C><<<dim3(grid_for(c->n, 256, c->num_sms), Q), 256, 0, c->stream>>>(
+                f, static_cast<const typename C::S*>(c->f[c->cur]), c->n, 0, c->args.dev, c->ref[c->cur]);
             return 0;
         });
         LBM_LAUNCHED(c, "decode_kernel");
@@ -1254,8 +1267,8 @@ lbm_status lbm_get_populations(lbm_ctx* c, double* f, int on_device) {
         with_codec(c, [&](auto codec) {
             using C = decltype(codec);
             decode_kernel<C><<<blocks, 256, 0, c->stream>>>(
-                c->scratch, static_cast<const typename C::S*>(c->f[c->cur]) + (size_t)q * c->n, c->n, c->n, q,
-                c->args.dev, c->ref[c->cur]);
+                c->scratch, static_cast<const typename C::S*>(c->f[c->cur]) + (size_t)q * c->n, c->n, q, c->args.dev,
+                c->ref[c->cur]);
             return 0;
         });
         LBM_LAUNCHED(c, "decode_kernel");
@@ -1284,36 +1297,39 @@ lbm_status lbm_moments(lbm_ctx* c, double* rho, double* ux, double* uy, double* 
     if (!c) return LBM_EINVAL;
     if (lbm_status st = check_device_error(c); st != LBM_OK) return st;
     const size_t nb = sizeof(double) * (size_t)c->n;
-    double *d_rho, *d_ux, *d_uy, *d_uz;
-    if (on_device) {
-        lbm_status s = rho ? LBM_OK : ensure_scratch(c, nb);
+    const bool vel = ux || uy || uz;
+    // staging for the requested host fields (rho always: u needs it) and, with a velocity, psi of every cell (18
+    // neighbours would each need an exponential in FP64: 1.0 of 1.9 ms at 80 x 72 x 200); without room for
+    // psi the velocity kernel forms it from the densities
+    const size_t fields = on_device ? (rho ? 0 : 1) : 1 + (ux ? 1 : 0) + (uy ? 1 : 0) + (uz ? 1 : 0);
+    bool with_psi = vel;
+    if (fields + vel) {
+        lbm_status s = ensure_scratch(c, (fields + vel) * nb);
+        if (s == LBM_ENOMEM && vel) {
+            with_psi = false;
+            s = fields ? ensure_scratch(c, fields * nb) : LBM_OK;
+        }
         if (s != LBM_OK) return s;
-        d_rho = rho ? rho : c->scratch;
-        d_ux = ux;
-        d_uy = uy;
-        d_uz = uz;
-    } else {
-        // staging for the requested fields only (rho always: u needs it)
-        const int nf = 1 + (ux ? 1 : 0) + (uy ? 1 : 0) + (uz ? 1 : 0);
-        lbm_status s = ensure_scratch(c, nf * nb);
-        if (s != LBM_OK) return s;
-        double* next = c->scratch;
-        d_rho = next;
-        next += c->n;
-        d_ux = ux ? next : nullptr;
-        next += ux ? c->n : 0;
-        d_uy = uy ? next : nullptr;
-        next += uy ? c->n : 0;
-        d_uz = uz ? next : nullptr;
     }
+    double* next = c->scratch;
+    auto take = [&](bool wanted) {
+        double* const at = wanted ? next : nullptr;
+        if (wanted) next += c->n;
+        return at;
+    };
+    double* const d_rho = on_device && rho ? rho : take(true);
+    double* const d_ux = on_device ? ux : take(ux != nullptr);
+    double* const d_uy = on_device ? uy : take(uy != nullptr);
+    double* const d_uz = on_device ? uz : take(uz != nullptr);
+    double* const d_psi = take(with_psi);
     const int blocks = grid_for(c->n, 256, c->num_sms);
     const auto& p = c->p;
     with_codec(c, [&](auto codec) {
         using C = decltype(codec);
         const auto* f = static_cast<const typename C::S*>(c->f[c->cur]);
-        density_kernel<C><<<blocks, 256, 0, c->stream>>>(d_rho, f, c->n, c->args.dev, c->ref[c->cur]);
-        if (d_ux || d_uy || d_uz)
-            velocity_kernel<C><<<blocks, 256, 0, c->stream>>>(d_ux, d_uy, d_uz, d_rho, f, p.nx, p.ny, p.nz, p.G, p.G2,
+        density_kernel<C><<<blocks, 256, 0, c->stream>>>(d_rho, d_psi, f, c->n, p.rho0, c->args.dev, c->ref[c->cur]);
+        if (vel)
+            velocity_kernel<C><<<blocks, 256, 0, c->stream>>>(d_ux, d_uy, d_uz, d_rho, d_psi, f, p.nx, p.ny, p.nz, p.G, p.G2,
                                                               p.rho0, c->args.dev, c->ref[c->cur]);
         return 0;
     });
