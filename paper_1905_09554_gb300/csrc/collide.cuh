@@ -91,6 +91,13 @@ __device__ __forceinline__ V vmulc(S c, V a) {
     using R = typename VecTraits<V>::R;
     return vmap(a, [&](R x) { return vmul(x, R(c)); });
 }
+// -a, and 2 a + b (doubling is exact: one rounding either way).
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ F2 vneg(F2 a) { return vmulc(-1.0f, a); }
+__device__ __forceinline__ float vtwice(float a, float b) { return vfma(2.0f, a, b); }
+__device__ __forceinline__ double vtwice(double a, double b) { return vfma(2.0, a, b); }
+__device__ __forceinline__ F2 vtwice(F2 a, F2 b) { return vadd(vadd(a, a), b); }
 __device__ __forceinline__ float vmul1(float a, float b) { return vmul(a, b); }
 __device__ __forceinline__ double vmul1(double a, double b) { return vmul(a, b); }
 __device__ __forceinline__ F2 vmul1(F2 a, F2 b) {
@@ -122,11 +129,54 @@ __device__ __forceinline__ V vfmac(S c, V a, T b) {  // b a number, too
 // rounded expf, whose range reduction costs about eight more instructions per
 // call.  Subnormal arguments and results are flushed (psi rounds to the same
 // value), which saves the scaling around them.
+//
+// FP64: the table-driven method of Tang (ACM Trans. Math. Softw. 15, 1989) with
+// 64 entries, 10 FP64 operations where exp takes 16: with
+// a = n ln2/64 + r, |r| <= ln2/128, and n = 64 m + j,
+//   e^a = 2^m 2^(j/64) e^r,  e^r - 1 = r + r^2/2 + ... + r^5/120  (r^6/720 < 4e-17).
+// The entries are 2^(j/64) rounded to double; ln2/64 is split so that n times
+// its upper part is exact.  Below the range of normal results, and for NaN and
+// infinities, exp itself is called.
+__device__ const double kExp2Table[64] = {
+    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
+    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
+    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
+    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
+    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
+    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
+    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
+    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
+    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
+    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0};
+
+__device__ __forceinline__ double exp_table(double a) {
+    if (!(fabs(a) < 700.0)) return exp(a);
+    const double shift = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer in the low bits
+    const double t = __fma_rn(a, 0x1.71547652b82fep+6, shift);
+    const int n = __double2loint(t);
+    const double k = __dsub_rn(t, shift);
+    double r = __fma_rn(k, -0x1.62e4200000000p-7, a);
+    r = __fma_rn(k, -0x1.fdf473de6af28p-28, r);
+    double p = __fma_rn(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = __fma_rn(r, p, 1.0 / 6.0);
+    p = __fma_rn(r, p, 0.5);
+    p = __fma_rn(__dmul_rn(r, r), p, r);
+    const double s = __ldg(kExp2Table + (n & 63));
+    const double e = __fma_rn(s, p, s);
+    return __hiloint2double(__double2hiint(e) + ((n >> 6) << 20), __double2loint(e));
+}
+
 template <class R>
 __device__ __forceinline__ R psi_of(R rho, R rho0, R inv_rho0);
 template <>
 __device__ __forceinline__ double psi_of<double>(double rho, double rho0, double inv_rho0) {
-    return rho0 * (1.0 - exp(-rho * inv_rho0));
+    return __dmul_rn(rho0, __dsub_rn(1.0, exp_table(__dmul_rn(-rho, inv_rho0))));
 }
 template <>
 __device__ __forceinline__ float psi_of<float>(float rho, float rho0, float inv_rho0) {
@@ -135,13 +185,21 @@ __device__ __forceinline__ float psi_of<float>(float rho, float rho0, float inv_
     return __fmul_rn(rho0, __fsub_rn(1.0f, e));
 }
 
-// 1/rho.  Float arithmetic uses the hardware reciprocal (within 1 ulp) instead
+// 1/rho.  FP64: from the hardware's 20-bit approximation y by one third-order
+// step of Householder's iteration, y (1 + e + e^2) with e = 1 - rho y (e^3 is
+// below the rounding), 3 FP64 operations; 0, infinities and subnormals take
+// the division.  Float arithmetic uses the hardware reciprocal (within 1 ulp) instead
 // of the IEEE division, whose special-case check adds a branch per cell.
 template <class R>
 __device__ __forceinline__ R recip(R x);
 template <>
 __device__ __forceinline__ double recip<double>(double x) {
-    return 1.0 / x;
+    const unsigned expo = (unsigned(__double2hiint(x)) >> 20) & 2047u;
+    if (expo - 64u > 1900u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-x, y, 1.0);
+    return __fma_rn(__fma_rn(e, e, e), y, y);
 }
 template <>
 __device__ __forceinline__ float recip<float>(float x) {
@@ -322,9 +380,9 @@ __device__ __forceinline__ Force<V> force_of(const PsiView<V>& lo, const PsiView
     Force<V> F;
     F.g = vmulc(gw, mid.c);
     const V dc = vsub(hi.c, lo.c);
-    F.sx = vadd(vadd(mid.ex, mid.ex), vadd(mid.dx, vadd(lo.ex, hi.ex)));
-    F.sy = vadd(vadd(mid.ey, mid.ey), vadd(mid.dy, vadd(lo.ey, hi.ey)));
-    F.sz = vadd(vadd(dc, dc), vsub(hi.s4, lo.s4));
+    F.sx = vtwice(mid.ex, vadd(mid.dx, vadd(lo.ex, hi.ex)));
+    F.sy = vtwice(mid.ey, vadd(mid.dy, vadd(lo.ey, hi.ey)));
+    F.sz = vtwice(dc, vsub(hi.s4, lo.s4));
     return F;
 }
 
@@ -415,8 +473,8 @@ __device__ __forceinline__ void collide_moments(const V (&m)[kMoments<COLL>], co
         ky = vsub(B, A);
         kxy = vadd(A, B);
         kxz = vsub(A, B);
-        kz = vmulc(R(-1), kxy);
-        kyz = vmulc(R(-1), kx);
+        kz = vneg(kxy);
+        kyz = vneg(kx);
         if constexpr (COLL == COLL_MRT_SPARSE) {
             // e = 19 tr N; coefficients -30, -11, 8 at rest, axis and edge velocities
             const V tr = vsub(vadd(vadd(m[4], m[5]), m[6]), rho);
@@ -435,7 +493,7 @@ __device__ __forceinline__ void collide_moments(const V (&m)[kMoments<COLL>], co
         r0 = vmulc(om, r0);
         r2 = vmulc(om, r2);
     }
-    const V r1 = vadd(r2, r2), h2 = vmulc(R(0.5), r2), n2 = vmulc(R(-1), r2), n1 = vadd(n2, n2);
+    const V r1 = vadd(r2, r2), h2 = vmulc(R(0.5), r2), n2 = vneg(r2), n1 = vneg(r1);
     const V& h1 = r2;
 
     {
