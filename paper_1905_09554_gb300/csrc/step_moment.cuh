@@ -13,9 +13,12 @@
 // of the population kernels (for 16-bit storage through its rounding too), so
 // n steps at once and n calls of one step give the same bits.
 //
-// One block marches along z with the cells of a 34 x 15 region (one per
-// thread; pairs along x with NV = 2, in packed arithmetic) around an output
-// tile of 32 x 13.  Per plane p, after one barrier, a thread
+// One block marches along z with the cells of a 68 x 15 region (pairs along x,
+// one pair per thread, in packed arithmetic) around an output tile of 64 x 13
+// (9 or 10 fields: 68 x 11 around 64 x 9, 384 threads of up to 168 registers,
+// where 512 of 128 spill and single cells take twice the instructions: 97 and
+// 76 against 67 ms for 20 steps of 384 x 384 x 1024).  Per plane p, after one
+// barrier, a thread
 //   * takes the populations of plane p - 2 that stream in from its
 //     neighbours out of shared memory and adds them to the sums of planes
 //     p - 3 (complete: written), p - 2 and p - 1,
@@ -25,7 +28,7 @@
 //     memory for the next turn,
 //   * turns the density of plane p + 1, loaded one turn earlier, into psi.
 // The region's rim is computed twice (by the neighbouring tiles as well):
-// 416 of 512 threads own an output cell.  The rim columns sit in one warp of
+// 416 of 512 threads own output cells.  The rim columns sit in one warp of
 // their own, so that all other warps load and store whole rows.
 //
 // Layout of the fields: rows of nx (rounded up to a multiple of 4) + 4 cells,
@@ -41,112 +44,97 @@
 
 namespace lbm {
 
-template <int NV> struct VecOf;
-template <> struct VecOf<1> { using V = float; };
-template <> struct VecOf<2> { using V = F2; };
-
-template <int NV>
+template <int NF>
 struct MomentTile {
-    static constexpr int ROWS = 15, OUT = 13, NT = 512;
-    static constexpr int TXO = 32 * NV;
+    static constexpr int ROWS = NF == 4 ? 15 : 11, OUT = ROWS - 2, NT = 32 * (ROWS + 1);
+    static constexpr int TXO = 64;
     static constexpr int XP = 35;               // exchange pitch, in region columns
     static constexpr int SLOTS = ROWS * XP;
-    static constexpr int NS = NV == 1 ? 16 : 14;  // scalar exchange arrays
-    static constexpr int NP = NV == 1 ? 0 : 6;    // pair exchange arrays
+    static constexpr int NS = 14;               // scalar exchange arrays
+    static constexpr int NP = 6;                // pair exchange arrays
     static constexpr int EXCH = SLOTS * (NS + 2 * NP);  // floats per exchange buffer
-    // psi: rows -1 .. 15; NV = 1: columns -1 .. 34; NV = 2: even and odd cells apart
-    static constexpr int PP = NV == 1 ? 37 : 35;
+    // psi: rows -1 .. ROWS, even and odd cells apart
+    static constexpr int PP = 35;
     static constexpr int PSI = (ROWS + 2) * PP + 2;
-    static constexpr int NPSI = NV;
-    static constexpr int NRING = NV == 1 ? 2 * 36 + 2 * ROWS : 2 * 34;
+    static constexpr int NRING = 2 * 34;
     // Two turns' buffers (exchange arrays and psi), then the moments in flight:
-    // the density of 8 planes (with the ring cells'), the others of 4, each
+    // the density of 8 planes (with the ring cells'), the others of 3 or 4, each
     // thread's in slots of its own.
-    static constexpr int BUF = (EXCH + NPSI * PSI + 3) / 4 * 4;
-    static constexpr int RHO = NV * (NT + 104);
-    static constexpr int rest(int nf) { return NV * NT * (nf - 1); }
-    static constexpr size_t bytes(int nf) { return sizeof(float) * (size_t)(2 * BUF + 8 * RHO + 4 * rest(nf)); }
-    static_assert(NRING <= 104, "slots of the ring cells");
+    static constexpr int BUF = (EXCH + 2 * PSI + 3) / 4 * 4;
+    static constexpr int RHO = 2 * (NT + NRING);
+    static constexpr int REST = 2 * NT * (NF - 1);
+    // slot of plane p >= -1 in the ring of the other moments (4 where they fit: a mask instead of a remainder)
+    static constexpr int STAGES = NF == 4 ? 4 : 3;
+    static constexpr size_t bytes = sizeof(float) * (size_t)(2 * BUF + 8 * RHO + STAGES * REST);
+    __device__ static unsigned stage(int p) { return NF == 4 ? unsigned(p) & 3u : unsigned(p + 3) % 3u; }
+    static_assert(bytes <= 227 * 1024, "shared memory of one block");
 };
 
-// Scalar exchange array of a population that crosses to another column, or
-// the row-wise ones for NV = 1; -1 where it has none.
-template <int NV>
+// Exchange arrays of a population that changes column: scalar arrays for those
+// moving along x (1, 11, 13 / 2, 14, 12; the value that leaves the pair) and,
+// two each, along the diagonals; pair arrays for those moving along y only.
 __host__ __device__ constexpr int exch_index(int q) {
-    constexpr int one[Q] = {-1, 0, 3, 6, 9, -1, -1, 12, 13, 14, 15, 1, 5, 2, 4, 7, 11, 8, 10};
-    // NV = 2: crossing x: 1, 11, 13 / 2, 14, 12; diagonals take two arrays each; rows: index of the pair array
-    constexpr int two[Q] = {-1, 0, 3, 0, 1, -1, -1, 6, 8, 10, 12, 1, 5, 2, 4, 2, 5, 3, 4};
-    return NV == 1 ? one[q] : two[q];
+    constexpr int t[Q] = {-1, 0, 3, 0, 1, -1, -1, 6, 8, 10, 12, 1, 5, 2, 4, 2, 5, 3, 4};
+    return t[q];
 }
 
 struct MomentArgs {
     int src_hi, dst_hi;  // the buffer's second set of moment fields (0: its first)
 };
 
-// The moments of a thread's cell or pair at float offset od of a field.
-template <int NV, int NF, class V>
-__device__ __forceinline__ void store_moments(float* d, long long nf, unsigned od, const V (&o)[NF]) {
+// The moments of a thread's pair at float offset od of a field.
+template <int NF>
+__device__ __forceinline__ void store_moments(float* d, long long nf, unsigned od, const F2 (&o)[NF]) {
     static_for<0, (NF + 2) / 2>([&](auto gc) {
         constexpr int g = decltype(gc)::value, k = g == 0 ? 0 : 2 * g - 1;
-        if constexpr (k > 0 && k + 1 < NF) {
-            float* p = d + k * nf + 2 * (long long)od;
-            if constexpr (NV == 1) *reinterpret_cast<float2*>(p) = make_float2(o[k], o[k + 1]);
-            else *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(o[k].v, o[k + 1].v);
-        } else if constexpr (k < NF) {
-            float* p = d + k * nf + od;
-            if constexpr (NV == 1) *p = o[k];
-            else *reinterpret_cast<unsigned long long*>(p) = o[k].v;
-        }
+        if constexpr (k > 0 && k + 1 < NF)
+            *reinterpret_cast<ulonglong2*>(d + k * nf + 2 * (long long)od) = make_ulonglong2(o[k].v, o[k + 1].v);
+        else if constexpr (k < NF)
+            *reinterpret_cast<unsigned long long*>(d + k * nf + od) = o[k].v;
     });
 }
-// Field value of cell x (element e of the thread's pair) written to column x + 2 + shift.
-template <int NV, int NF>
+// Field k of the cell in column col (0 .. pitch - 1) of the row that starts at
+// `row`: rho by itself, then two by two, interleaved by pairs of cells.
+template <int NF>
 __device__ __forceinline__ float* moment_at(float* d, long long nf, unsigned row, int col, int k) {
-    // row: offset of the row's first float; fields 1.. are interleaved by two
     const bool two = k > 0 && ((k - 1) / 2) * 2 + 2 < NF;
     if (!two) return d + k * nf + (row + unsigned(col));
     const int k0 = ((k - 1) / 2) * 2 + 1, which = k - k0;
-    return d + k0 * nf + 2 * (long long)(row + unsigned(col / NV * NV)) + which * NV + col % NV;
+    return d + k0 * nf + 2 * (long long)(row + unsigned(col / 2 * 2)) + which * 2 + col % 2;
 }
-// The cells of a thread whose row ends are near: element by element, with the
-// periodic copy of every cell that has one (shift 0: the cells themselves, for
-// the pair that sticks out of an odd row).
-template <int NV, int NF, class V>
-__device__ __forceinline__ void store_ends(float* d, long long nf, unsigned od, const V (&o)[NF], int x, int nx,
+// The pair of a thread near the ends of an odd row: value by value, the
+// periodic copy of every cell that has one (and, for the pair that sticks out
+// of the row, the cell itself).
+template <int NF>
+__device__ __forceinline__ void store_ends(float* d, long long nf, unsigned od, const F2 (&o)[NF], int x, int nx,
                                            bool stick) {
     const unsigned row = od - unsigned(x + 2);
 #pragma unroll 1
-    for (int j = stick ? 0 : NV; j < 2 * NV; ++j) {  // first the cells, then their copies
-        const int e = j % NV, xe = x + e;
+    for (int j = stick ? 0 : 2; j < 4; ++j) {  // first the cells, then their copies
+        const int e = j % 2, xe = x + e;
         if (xe >= nx) continue;
         int col = xe + 2;
-        if (j >= NV) {
+        if (j >= 2) {
             if (xe >= 2 && xe < nx - 2) continue;
             col += xe < 2 ? nx : -nx;
         }
 #pragma unroll
         for (int k = 0; k < NF; ++k) {
-            float v;
-            if constexpr (NV == 1) {
-                v = o[k];
-            } else {
-                float lo, hi;
-                unpack2(o[k], lo, hi);
-                v = e ? hi : lo;
-            }
-            *moment_at<NV, NF>(d, nf, row, col, k) = v;
+            float lo, hi;
+            unpack2(o[k], lo, hi);
+            *moment_at<NF>(d, nf, row, col, k) = e ? hi : lo;
         }
     }
 }
 
-template <class Codec, int COLL, int NV, bool EMIT, bool BATCH, bool KEEP_PSI = false>
-__global__ void __launch_bounds__(512, 1)
+template <class Codec, int COLL, bool EMIT, bool BATCH, bool KEEP_PSI = false>
+__global__ void __launch_bounds__(MomentTile<kMoments<COLL>>::NT, 1)
 sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, const StepArgs a, const BatchArgs b,
                  const MomentArgs ma) {
-    using V = typename VecOf<NV>::V;
+    using V = F2;
     using S = typename Codec::S;
-    using T = MomentTile<NV>;
     constexpr int NF = kMoments<COLL>;
+    using T = MomentTile<NF>;
     constexpr int XP = T::XP, PP = T::PP, ROWS = T::ROWS, SLOTS = T::SLOTS;
     constexpr bool LOCAL = Codec::kLocal, HALF = sizeof(S) == 2;
     static_assert(!BATCH || !HALF, "batches hold 32-bit populations");
@@ -164,19 +152,12 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
     const int ps = (ry + 1) * PP + rp + 1;
     // ring cells (psi only) around the region
     const bool ring = tid < T::NRING;
-    int hp = 0, hy = 0;
-    if (NV == 1) {
-        if (tid < 72) { hp = tid % 36 - 1; hy = tid < 36 ? -1 : ROWS; }
-        else if (ring) { hp = tid < 72 + ROWS ? -1 : 34; hy = (tid - 72) % ROWS; }
-    } else if (ring) {
-        hp = tid % 34;
-        hy = tid < 34 ? -1 : ROWS;
-    }
+    const int hp = tid % 34, hy = tid < 34 ? -1 : ROWS;
     const int hs = (hy + 1) * PP + hp + 1;
 
-    constexpr int REST = T::rest(NF);
+    constexpr int REST = T::REST;
     float* const rho_st = buf0 + 2 * T::BUF;       // [8][RHO]
-    float* const rest_st = rho_st + 8 * T::RHO;    // [4][REST]
+    float* const rest_st = rho_st + 8 * T::RHO;    // [STAGES][REST]
 
     chain_begin();
     const float rho0 = a.rho0f, inv_rho0 = a.inv_rho0f;
@@ -212,24 +193,20 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
         const int tile = local % n_tiles, chunk = local / n_tiles;
         const int x0 = (tile % tiles_x) * T::TXO, y0 = (tile / tiles_x) * T::OUT;
         const int zs = chunk * zchunk, ze = min(zs + zchunk, nz);
-        const int x = x0 + (rp - 1) * NV, y = y0 + ry - 1;
-        const unsigned off = unsigned(wrap_index(y, ny)) * pitch + min(x + 2, pitch - NV);
+        const int x = x0 + (rp - 1) * 2, y = y0 + ry - 1;
+        const unsigned off = unsigned(wrap_index(y, ny)) * pitch + min(x + 2, pitch - 2);
         const unsigned hoff =
-            unsigned(wrap_index(y0 + hy - 1, ny)) * pitch + min(x0 + (hp - 1) * NV + 2, pitch - NV);
+            unsigned(wrap_index(y0 + hy - 1, ny)) * pitch + min(x0 + (hp - 1) * 2 + 2, pitch - 2);
         const bool own = inner && y < ny && x < nx;
         // any cell of this thread with a periodic copy, or a pair that sticks out of an odd row
-        const bool edge = x < 2 || x + NV > nx - 2;
+        const bool edge = x < 2 || x + 2 > nx - 2;
         float* const dst_m = EMIT ? nullptr : static_cast<float*>(dst_all) + base + (ma.dst_hi ? NF * nf : 0);
 
         auto put_psi = [&](float* buf, int slot, V p) {
-            if constexpr (NV == 2) {
-                float e, o;
-                unpack2(p, e, o);
-                buf[slot] = e;
-                buf[T::PSI + slot] = o;
-            } else {
-                buf[slot] = p;
-            }
+            float e, o;
+            unpack2(p, e, o);
+            buf[slot] = e;
+            buf[T::PSI + slot] = o;
         };
 
         // What a thread keeps of three consecutive planes, rotated by the caller.
@@ -237,7 +214,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             PsiView<V> w;
         };
         V own0, own5, own6;          // populations of the last collided plane that stay in the column
-        float kept[6];               // NV = 2: those that move along x within the pair
+        float kept[6];               // those that move along x within the pair
         SumUp<V> up1, upz;           // what plane q sent up (to q + 1), and plane q - 1 (to q)
         V z_r, z_jx, z_jy, z_xx, z_yy, z_xy;  // sums of plane q's cell without what comes from above
 
@@ -246,32 +223,31 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
         int zr = wrap_index(zs - 2, nz), zm = wrap_index(zs - 1, nz);  // planes fetched next
         unsigned rrow = unsigned(zr) * plane, mrow = unsigned(zm) * plane;
         auto fetch_rho = [&](int p) {
-            float* const st = rho_st + (p & 7) * T::RHO + NV * tid;
-            async_copy::copy<4 * NV>(st, src + (rrow + off));
-            if (ring) async_copy::copy<4 * NV>(st + NV * T::NT, src + (rrow + hoff));
+            float* const st = rho_st + (p & 7) * T::RHO + 2 * tid;
+            async_copy::copy<8>(st, src + (rrow + off));
+            if (ring) async_copy::copy<8>(st + 2 * T::NT, src + (rrow + hoff));
             rrow += plane;
             if (++zr == nz) { zr = 0; rrow = 0; }
         };
         auto fetch_rest = [&](int p) {
             const unsigned o = mrow + off;
-            float* const st = rest_st + (p & 3) * REST;
+            float* const st = rest_st + T::stage(p) * REST;
             static_for<0, (NF - 1) / 2>([&](auto gc) {
                 constexpr int k = 2 * decltype(gc)::value + 1;
-                async_copy::copy<8 * NV>(st + (k - 1) * T::NT * NV + 2 * NV * tid, src + k * nf + 2 * (long long)o);
+                async_copy::copy<16>(st + (k - 1) * T::NT * 2 + 4 * tid, src + k * nf + 2 * (long long)o);
             });
             if constexpr (NF % 2 == 0)
-                async_copy::copy<4 * NV>(st + (NF - 2) * T::NT * NV + NV * tid, src + (NF - 1) * nf + o);
+                async_copy::copy<8>(st + (NF - 2) * T::NT * 2 + 2 * tid, src + (NF - 1) * nf + o);
             mrow += plane;
             if (++zm == nz) { zm = 0; mrow = 0; }
         };
-        auto rho_of = [&](int p) -> V { return *reinterpret_cast<const V*>(rho_st + (p & 7) * T::RHO + NV * tid); };
+        auto rho_of = [&](int p) -> V { return *reinterpret_cast<const V*>(rho_st + (p & 7) * T::RHO + 2 * tid); };
         // psi of plane p into its turn's buffer
         auto fill_psi = [&](Plane& q, int p) {
             float* const buf = buf0 + (p & 1) * T::BUF + T::EXCH;
             q.w.c = psi_v(rho_of(p));
             put_psi(buf, ps, q.w.c);
             if constexpr (KEEP_PSI) {  // for the adjoint
-                static_assert(NV == 2);
                 if (own && p >= zs && p < ze) {
                     float* d = static_cast<float*>(a.psi_out) + ((long long)p * ny + y) * nx + x;
                     float lo, hi;
@@ -282,7 +258,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             }
             if (ring)
                 put_psi(buf, hs,
-                        psi_v(*reinterpret_cast<const V*>(rho_st + (p & 7) * T::RHO + NV * (tid + T::NT))));
+                        psi_v(*reinterpret_cast<const V*>(rho_st + (p & 7) * T::RHO + 2 * (tid + T::NT))));
         };
 
         Plane pa, pb, pc;
@@ -318,20 +294,18 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                     if constexpr (q == 0) return own0;
                     else if constexpr (q == 5) return own5;
                     else if constexpr (q == 6) return own6;
-                    else if constexpr (NV == 1) {
-                        return ex_r[exch_index<1>(q) * SLOTS + xs - cx(q) - cy(q) * XP];
-                    } else if constexpr (cx(q) == 0) {
+                    else if constexpr (cx(q) == 0) {
                         F2 r;
-                        r.v = reinterpret_cast<const unsigned long long*>(ex_r)[exch_index<2>(q) * SLOTS + xs -
+                        r.v = reinterpret_cast<const unsigned long long*>(ex_r)[exch_index(q) * SLOTS + xs -
                                                                                  cy(q) * XP];
                         return r;
                     } else {
                         // one cell of the pair receives from the neighbouring pair, the other from this
                         // column: along a diagonal out of shared memory, along x it never left the thread
-                        const float* e = ex_r + 2 * T::NP * SLOTS + exch_index<2>(q) * SLOTS + xs - cy(q) * XP;
+                        const float* e = ex_r + 2 * T::NP * SLOTS + exch_index(q) * SLOTS + xs - cy(q) * XP;
                         const float far = e[-cx(q)];
                         float near;
-                        if constexpr (cy(q) == 0) near = kept[exch_index<2>(q)];
+                        if constexpr (cy(q) == 0) near = kept[exch_index(q)];
                         else near = e[SLOTS];
                         return cx(q) > 0 ? pack2(far, near) : pack2(near, far);
                     }
@@ -340,15 +314,11 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                     constexpr int q = decltype(qc)::value;
                     V v = got(qc);
                     if constexpr (LOCAL && !EMIT) {  // through the 16-bit storage of the destination cell
-                        if constexpr (NV == 2) {
-                            float lo, hi, r0, r1;
-                            unpack2(v, lo, hi);
-                            unpack2(ref, r0, r1);
-                            v = pack2(Codec::template decode_ref<q>(Codec::template encode_ref<q>(lo, r0, dev), r0, dev),
-                                      Codec::template decode_ref<q>(Codec::template encode_ref<q>(hi, r1, dev), r1, dev));
-                        } else {
-                            v = Codec::template decode_ref<q>(Codec::template encode_ref<q>(v, ref, dev), ref, dev);
-                        }
+                        float lo, hi, r0, r1;
+                        unpack2(v, lo, hi);
+                        unpack2(ref, r0, r1);
+                        v = pack2(Codec::template decode_ref<q>(Codec::template encode_ref<q>(lo, r0, dev), r0, dev),
+                                  Codec::template decode_ref<q>(Codec::template encode_ref<q>(hi, r1, dev), r1, dev));
                     }
                     return v;
                 };
@@ -356,10 +326,10 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                 // and one from a neighbour, in opposite cells: added cell by cell, no register is moved.
                 auto both = [&](auto qpc, auto qmc, V ref) -> Opp<V> {
                     constexpr int qp = decltype(qpc)::value, qm = decltype(qmc)::value;
-                    if constexpr (NV == 2 && !LOCAL && cx(qp) == 1 && cy(qp) == 0) {
+                    if constexpr (!LOCAL && cx(qp) == 1 && cy(qp) == 0) {
                         const float* e = ex_r + 2 * T::NP * SLOTS + xs;
-                        const float pl = e[exch_index<2>(qp) * SLOTS - 1], mh = e[exch_index<2>(qm) * SLOTS + 1];
-                        const float ph = kept[exch_index<2>(qp)], ml = kept[exch_index<2>(qm)];
+                        const float pl = e[exch_index(qp) * SLOTS - 1], mh = e[exch_index(qm) * SLOTS + 1];
+                        const float ph = kept[exch_index(qp)], ml = kept[exch_index(qm)];
                         return {pack2(vadd(pl, ml), vadd(ph, mh)), pack2(vsub(pl, ml), vsub(ph, mh))};
                     } else {
                         return opp(in(qpc, ref), in(qmc, ref));
@@ -375,26 +345,21 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                         if (own && t >= zs && t < ze) {
                             S* d = dst + q * cells + ((long long)t * ny + y) * nx + x;
                             const V v = got(qc);
-                            if constexpr (NV == 1) {
-                                if constexpr (LOCAL) Codec::template store_ref<q>(d, v, ref, dev);
-                                else Codec::template store<q>(d, v, dev);
+                            float lo, hi, r0, r1;
+                            unpack2(v, lo, hi);
+                            unpack2(ref, r0, r1);
+                            const bool two = x + 1 < nx;
+                            if constexpr (LOCAL) {
+                                Codec::template store_ref<q>(d, lo, r0, dev);
+                                if (two) Codec::template store_ref<q>(d + 1, hi, r1, dev);
+                            } else if constexpr (HALF) {
+                                Codec::template store<q>(d, lo, dev);
+                                if (two) Codec::template store<q>(d + 1, hi, dev);
+                            } else if ((nx & 1) == 0) {
+                                *reinterpret_cast<unsigned long long*>(d) = v.v;
                             } else {
-                                float lo, hi, r0, r1;
-                                unpack2(v, lo, hi);
-                                unpack2(ref, r0, r1);
-                                if constexpr (HALF) {
-                                    if constexpr (LOCAL) Codec::template store_ref<q>(d, lo, r0, dev);
-                                    else Codec::template store<q>(d, lo, dev);
-                                    if (x + 1 < nx) {
-                                        if constexpr (LOCAL) Codec::template store_ref<q>(d + 1, hi, r1, dev);
-                                        else Codec::template store<q>(d + 1, hi, dev);
-                                    }
-                                } else if ((nx & 1) == 0) {
-                                    *reinterpret_cast<unsigned long long*>(d) = v.v;
-                                } else {
-                                    d[0] = lo;
-                                    if (x + 1 < nx) d[1] = hi;
-                                }
+                                d[0] = lo;
+                                if (two) d[1] = hi;
                             }
                         }
                     };
@@ -411,14 +376,10 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                     if constexpr (LOCAL) {  // the density before this step: the reference of what the cell holds
                         if (own && q >= zs && q < ze) {
                             float* d = a.ref_dst + ((long long)q * ny + y) * nx + x;
-                            if constexpr (NV == 1) {
-                                *d = ref_fl;
-                            } else {
-                                float lo, hi;
-                                unpack2(ref_fl, lo, hi);
-                                d[0] = lo;
-                                if (x + 1 < nx) d[1] = hi;
-                            }
+                            float lo, hi;
+                            unpack2(ref_fl, lo, hi);
+                            d[0] = lo;
+                            if (x + 1 < nx) d[1] = hi;
                         }
                     }
                 } else {
@@ -431,11 +392,11 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                         moments_from<COLL, V>(upz, z_r, z_jx, z_jy, z_xx, z_yy, z_xy, dn, o);
                         float* const d = dst_m;
                         const unsigned od = unsigned(t) * plane + unsigned(y) * pitch + unsigned(x + 2);
-                        const bool stick = NV == 2 && x + 1 >= nx;
-                        if (!stick) store_moments<NV, NF>(d, nf, od, o);
+                        const bool stick = x + 1 >= nx;
+                        if (!stick) store_moments<NF>(d, nf, od, o);
                         if (edge) {
-                            if (NV == 1 || (nx & 1) == 0) store_moments<NV, NF>(d, nf, od + (x < 2 ? nx : -nx), o);
-                            else store_ends<NV, NF>(d, nf, od, o, x, nx, stick);
+                            if ((nx & 1) == 0) store_moments<NF>(d, nf, od + (x < 2 ? nx : -nx), o);
+                            else store_ends<NF>(d, nf, od, o, x, nx, stick);
                         }
                     }
                     const SumFlat<V> fl = sum_flat(LBM_IN(0, ref_fl), LBM_BOTH(1, 2, ref_fl),
@@ -457,11 +418,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
             }
 
             if (p <= ze + 1) {
-                if constexpr (NV == 1) {
-                    const PsiAt<float, PP> at{psi_r + ps};
-                    psi_axis(nxt.w, at);
-                    psi_diag(nxt.w, at);
-                } else {
+                {
                     // rows y - 1, y, y + 1: left neighbour, the pair, right neighbour; differences along x
                     // are formed cell by cell (they mix the halves of neighbouring pairs)
                     float l[3], e[3], o[3], r[3];
@@ -487,22 +444,16 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                     const Force<V> F = force_of(prev.w, cur.w, nxt.w, a.gwf);
                     V m[NF];
                     m[0] = rho_of(p - 1);
-                    const float* const st = rest_st + ((p - 1) & 3) * REST;
+                    const float* const st = rest_st + T::stage(p - 1) * REST;
                     static_for<0, (NF - 1) / 2>([&](auto gc) {
                         constexpr int k = 2 * decltype(gc)::value + 1;
-                        const float* q = st + (k - 1) * T::NT * NV + 2 * NV * tid;
-                        if constexpr (NV == 2) {
-                            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(q);
-                            m[k].v = v.x;
-                            m[k + 1].v = v.y;
-                        } else {
-                            const float2 v = *reinterpret_cast<const float2*>(q);
-                            m[k] = v.x;
-                            m[k + 1] = v.y;
-                        }
+                        const float* q = st + (k - 1) * T::NT * 2 + 4 * tid;
+                        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(q);
+                        m[k].v = v.x;
+                        m[k + 1].v = v.y;
                     });
                     if constexpr (NF % 2 == 0)
-                        m[NF - 1] = *reinterpret_cast<const V*>(st + (NF - 2) * T::NT * NV + NV * tid);
+                        m[NF - 1] = *reinterpret_cast<const V*>(st + (NF - 2) * T::NT * 2 + 2 * tid);
                     collide_moments<COLL, V, true>(m, F, a, [&](auto qc, V f) {
                         constexpr int q = decltype(qc)::value;
                         if constexpr (HALF && !LOCAL && !EMIT) {  // through the 16-bit storage
@@ -513,18 +464,16 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
                         if constexpr (q == 0) own0 = f;
                         else if constexpr (q == 5) own5 = f;
                         else if constexpr (q == 6) own6 = f;
-                        else if constexpr (NV == 1) {
-                            ex_w[exch_index<1>(q) * SLOTS + xs] = f;
-                        } else {
+                        else {
                             float lo, hi;
                             unpack2(f, lo, hi);
-                            float* e = ex_w + 2 * T::NP * SLOTS + exch_index<2>(q) * SLOTS + xs;
+                            float* e = ex_w + 2 * T::NP * SLOTS + exch_index(q) * SLOTS + xs;
                             if constexpr (cx(q) == 0) {
-                                reinterpret_cast<unsigned long long*>(ex_w)[exch_index<2>(q) * SLOTS + xs] = f.v;
+                                reinterpret_cast<unsigned long long*>(ex_w)[exch_index(q) * SLOTS + xs] = f.v;
                             } else {
                                 const float near = cx(q) > 0 ? lo : hi;
                                 e[0] = cx(q) > 0 ? hi : lo;
-                                if constexpr (cy(q) == 0) kept[exch_index<2>(q)] = near;
+                                if constexpr (cy(q) == 0) kept[exch_index(q)] = near;
                                 else e[SLOTS] = near;
                             }
                         }
@@ -547,7 +496,7 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
 
 // Populations -> moment fields (all the operators above read of a state).
 // One thread per cell along x rows; blockIdx.y: the box of a batch.
-template <class Codec, int COLL, int NV, bool BATCH>
+template <class Codec, int COLL, bool BATCH>
 __global__ void __launch_bounds__(256)
 sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
     using S = typename Codec::S;
@@ -584,37 +533,30 @@ sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, 
             const int g = x < 2 ? nx : (x >= nx - 2 ? -nx : 0);
             static_for<0, NF>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;
-                *moment_at<NV, NF>(dst, nf, row, x + 2, k) = m[k];
-                if (g) *moment_at<NV, NF>(dst, nf, row, x + 2 + g, k) = m[k];
+                *moment_at<NF>(dst, nf, row, x + 2, k) = m[k];
+                if (g) *moment_at<NF>(dst, nf, row, x + 2 + g, k) = m[k];
             });
         }
     }
 }
-
-// Cells per thread: pairs where their state fits the 128 registers of a
-// 512-thread block (4 fields: 45 against 31 GLUPS at 256 x 256 x 575, whole
-// calls of 50 steps), single cells for 9 and 10 fields (pairs spill: 31 against
-// 40 GLUPS at 384 x 384 x 1024, calls of 20 steps).
-template <int COLL>
-constexpr int kCells = kMoments<COLL> == 4 ? 2 : 1;
 
 // Small boxes (a step under ~30 us) chain their kernels.
 inline bool moment_chain(const MomentLaunch& l) { return !l.batch.nbox && l.args.n <= 1500000; }
 
 template <class Codec, int COLL, bool EMIT, bool BATCH>
 cudaError_t moment_launch(const MomentLaunch& l, const void* src, void* dst) {
-    using T = MomentTile<kCells<COLL>>;
-    const int sm = (int)T::bytes(kMoments<COLL>);
+    using T = MomentTile<kMoments<COLL>>;
+    const int sm = (int)T::bytes;
     if constexpr (COLL == COLL_SRT && !EMIT && !BATCH && std::is_same_v<Codec, CodecF32>) {
         if (l.args.psi_out) {
-            auto kern = sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH, true>;
+            auto kern = sc_moment_kernel<Codec, COLL, EMIT, BATCH, true>;
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             if (e != cudaSuccess) return e;
             return launch_chained(moment_chain(l), kern, l.grid, T::NT, sm, l.stream, src, dst, l.args, l.batch,
                                   MomentArgs{l.src_hi, l.dst_hi});
         }
     }
-    return launch_chained(moment_chain(l), sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH>, l.grid, T::NT,
+    return launch_chained(moment_chain(l), sc_moment_kernel<Codec, COLL, EMIT, BATCH>, l.grid, T::NT,
                           sm, l.stream, src, dst, l.args, l.batch, MomentArgs{l.src_hi, l.dst_hi});
 }
 
@@ -628,21 +570,20 @@ cudaError_t moment_dispatch(const MomentLaunch& l, const void* src, void* dst) {
 
 template <class Codec, int COLL>
 cudaError_t moment_gather(const MomentLaunch& l, const void* src, void* dst) {
-    constexpr int NV = kCells<COLL>;
     if constexpr (sizeof(typename Codec::S) == 4) {
         if (l.batch.nbox)
-            return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, NV, true>, dim3(l.gather_grid, l.batch.nbox), 256, 0,
+            return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, true>, dim3(l.gather_grid, l.batch.nbox), 256, 0,
                                   l.stream, src, dst, l.args, l.batch);
     }
-    return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, NV, false>, l.gather_grid, 256, 0, l.stream, src, dst, l.args,
+    return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, false>, l.gather_grid, 256, 0, l.stream, src, dst, l.args,
                           l.batch);
 }
 
 template <class Codec, int COLL, bool EMIT, bool BATCH>
 int moment_prepare_one() {
-    using T = MomentTile<kCells<COLL>>;
-    auto kern = sc_moment_kernel<Codec, COLL, kCells<COLL>, EMIT, BATCH>;
-    const int sm = (int)T::bytes(kMoments<COLL>);
+    using T = MomentTile<kMoments<COLL>>;
+    auto kern = sc_moment_kernel<Codec, COLL, EMIT, BATCH>;
+    const int sm = (int)T::bytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T::NT, sm);
@@ -672,5 +613,6 @@ int moment_prepare(bool batch) {
     extern const MomentKernels kMoment_##NAME = {moment_prepare<CODEC, COLL>, moment_gather<CODEC, COLL>, \
                                                  moment_dispatch<CODEC, COLL, false>,                \
                                                  moment_dispatch<CODEC, COLL, true>, kMoments<COLL>, \
-                                                 32 * kCells<COLL>, MomentTile<1>::OUT};             \
+                                                 MomentTile<kMoments<COLL>>::TXO,                    \
+                                                 MomentTile<kMoments<COLL>>::OUT};     \
     }
