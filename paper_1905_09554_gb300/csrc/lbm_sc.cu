@@ -686,6 +686,21 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
             }
         }
         c->zchunk = int(zc < p->nz ? zc : p->nz);
+    } else if (c->kernel == 6) {
+        // Two-belt kernel: 512 (FP64: 256) threads an SM, and 5 planes per chunk that are not its own: the chunk
+        // with the fewest planes on the busiest SM slot (128 x 128 x 288: 10 chunks of 29 planes are 640 blocks
+        // for 304 places, a third round for the last 32).
+        const long long places = (long long)c->num_sms * (p->storage == LBM_F64 ? 8 : 16) / c->tile_y;
+        const long long tiles = (long long)tiles_x * tiles_y;
+        long long best = -1;
+        c->zchunk = 1;
+        for (int z = p->nz < 128 ? p->nz : 128; z >= 1; --z) {
+            const long long load = busiest_block_planes(p->nz, tiles, places > 0 ? places : 1, z, 5);
+            if (best < 0 || load < best) {
+                best = load;
+                c->zchunk = z;
+            }
+        }
     } else {
         c->zchunk = auto_zchunk(c);
     }
