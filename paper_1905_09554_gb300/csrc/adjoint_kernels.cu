@@ -24,6 +24,10 @@
 // adj_collide1_kernel and adj_force_kernel then keep {A, B} as one 16- or
 // 32-byte vector per cell: one vector load per neighbour where the general
 // form loads two values, and 128 + 40 B a cell and step instead of 250 + 40.
+// 64 x 64 x 180 in FP32, 500 steps back with their recomputation: 64.1 ms with
+// 20 values, 50.2 with {A, B}, 41.4 with the recomputed states kept as moments
+// too, 37.7 with the block shape and block sums below.  Both kernels are bound by the latency of their gathers from L2 (about
+// 39 and 17 us a step from a cold cache).
 #include <cuda_runtime.h>
 
 #include "adjoint.h"
@@ -34,12 +38,13 @@
 namespace lbm {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kRowThreads = 32, kRows = kThreads / kRowThreads;  // (32, 8) blocks: 8 rows at a time
+// 64 x 64 x 180, 500 steps back: 41.3 ms with blocks of 256 threads, 39.8 with 128, 39.7 with 64, 40.3 with 32.
+constexpr int kThreads = 128;
+constexpr int kRowThreads = 32, kRows = kThreads / kRowThreads;  // (32, 4) blocks: 4 rows at a time
 
 // The cells of one x row and the periodic neighbour offsets of the row and
 // of its cells (32-bit: the adjoint needs nx*ny*nz < 2^32).  Blocks of
-// (32, 8) threads walk the ny*nz rows (grid-stride); a warp covers 32
+// (32, 4) threads walk the ny*nz rows (grid-stride); a warp covers 32
 // consecutive x of a row, so the neighbour gathers stay coalesced and no
 // cell index is ever divided.
 struct Row {
@@ -159,23 +164,22 @@ __global__ void __launch_bounds__(kThreads) adj_psi_moments_kernel(const float* 
 }
 
 // Sum of (a, b) over the block, added to out2[0..1] (the block's running
-// sums over the reverse steps); fixed order: a tree within each warp, then
-// the warps in turn.
+// sums over the reverse steps); fixed order.  One warp adds up what all have
+// written, a in its lower and b in its upper lanes: an FP64 instruction holds
+// the pipe of 2 lanes for 16 cycles a warp, and a tree by shuffles in every
+// warp takes 10 of them (64 x 64 x 180, 500 steps back: 39.8 -> 38.5 ms).
 __device__ __forceinline__ void block_sum2(double a, double b, double* out2) {
-    __shared__ double red[2][kRows];
-    for (int s = 16; s > 0; s >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, s);
-        b += __shfl_down_sync(0xffffffffu, b, s);
-    }
-    if (threadIdx.x == 0) {
-        red[0][threadIdx.y] = a;
-        red[1][threadIdx.y] = b;
-    }
+    __shared__ double red[2][kThreads];
+    const int t = threadIdx.y * kRowThreads + threadIdx.x;
+    red[0][t] = a;
+    red[1][t] = b;
     __syncthreads();
-    if (threadIdx.x < 2 && threadIdx.y == 0) {
-        double s = red[threadIdx.x][0];
-        for (int k = 1; k < kRows; ++k) s += red[threadIdx.x][k];
-        out2[threadIdx.x] += s;
+    if (t < 32) {
+        const double* const r = red[t >> 4];
+        double s = r[t & 15];
+        for (int k = 16; k < kThreads; k += 16) s += r[k + (t & 15)];
+        for (int k = 8; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k, 16);
+        if ((t & 15) == 0) out2[t >> 4] += s;
     }
 }
 
@@ -271,7 +275,7 @@ adj_collide_kernel(const R* __restrict__ f, const R* __restrict__ psi, const R* 
 // lam_next2: lam(t + 2), nullptr in the last step; first: step 0, whose
 // populations are at rest, f_q = w_q rho.
 template <class R, bool FROM_MOMENTS>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, 4)
 adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Vec4<R>* __restrict__ lam_next,
                     const Vec4<R>* __restrict__ lam_next2, Vec4<R>* __restrict__ lam_out, Vec4<R>* __restrict__ fa,
                     double* __restrict__ partials, bool first, AdjointArgs a) {
@@ -383,7 +387,7 @@ adj_collide1_kernel(const R* __restrict__ f, const R* __restrict__ psi, const Ve
 // every population: kept in gr and added where it is read, or (TAU1) added to
 // the A of {A, B}.
 template <class R, bool TAU1>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 adj_force_kernel(const R* __restrict__ psi, const Vec4<R>* __restrict__ fa, R* __restrict__ gr, AdjointArgs a) {
     chain_begin();
     const R G = par<R>(a.G, a.Gf), inv_rho0 = R(1.0 / a.rho0);
@@ -442,7 +446,7 @@ __global__ void adj_rho01_kernel(const Vec4<R>* __restrict__ lam, double* __rest
         out[i] = double(load4(lam + i).x);
 }
 
-// Fixed-order sum of the per-block partials into acc[0..1]: each of 256
+// Fixed-order sum of the per-block partials into acc[0..1]: each of 128
 // threads sums a strided subset in block order, then a fixed tree.
 __global__ void __launch_bounds__(kThreads) adj_reduce_kernel(const double* __restrict__ partials, int nblocks,
                                                              double* __restrict__ acc) {
