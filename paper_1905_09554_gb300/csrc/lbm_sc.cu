@@ -57,6 +57,7 @@ struct lbm_ctx {
     // launch shape, or mom == nullptr where only populations will do.
     const MomentKernels* mom = nullptr;
     MomentLaunch mom_launch{};
+    void* mom_plan = nullptr;         // device memory of its plan
     size_t mom_bytes = 0;             // one set of moment fields
     bool mom_twice = false;           // two sets fit into one population copy
     // Steps in two kernels (step_split.cuh); in place where the moments are all
@@ -305,7 +306,8 @@ __global__ void velocity_kernel(double* __restrict__ ux, double* __restrict__ uy
 // part[8 * (gridDim.y * z + blockIdx.y) + k]; the last of them to finish adds
 // the parts in turn into out[8*z + k]: k = 0 mass, 1..3 momentum, 4 liquid
 // area, 5 max rho, 6 count of cells with rho <= 0 or non-finite.  With one
-// block per slice 144 slices of 64 x 64 took 21 us (half the SMs idle, 2.1 TB/s).
+// block per slice 144 slices of 64 x 64 took 21 us (half the SMs idle, 2.1 TB/s);
+// bound by HBM for boxes beyond L2 (76 B a cell in FP32).
 constexpr int DIAG_THREADS = 256;
 constexpr int DIAG_RUN_CELLS = 8 * DIAG_THREADS;  // cells of one run of every thread
 
@@ -591,8 +593,11 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
     // formats run the paired kernel on 64x8 tiles (FP16 SRT 35.6 against 32.7
     // for kernel 3 on 32x4), the local-reference ones kernel 3 on 32x8 tiles
     // (33.2 against 31.1 on 32x4, 29.8 on 32x16, 29.2 paired, 22.9
-    // register-staged); 16-bit storage with nx odd and FP64 run the
-    // register-staged kernel on 32x4 tiles (FP64 is bound by its FP64 pipe).
+    // register-staged); 16-bit storage with nx odd and FP64 are configured for
+    // the register-staged kernel on 32x4 tiles, which runs where there is no
+    // room for the two-kernel step's field (step_split.cuh).  The sides were
+    // measured together, before the collision took fewer instructions; the
+    // chosen ones now run at 34.4 (FP32 SRT), 37.9 (FP16) and 34.9 (FP16 local).
     const bool pipe_default = p->storage == LBM_F32 || (p->storage >= LBM_F16_DEV && p->nx % 2 == 0);
     const bool pair_default = (p->storage == LBM_F16_DEV || p->storage == LBM_BF16_DEV) && p->nx % 2 == 0;
     const bool pipe = kernel == 3 || (kernel == 0 && pipe_default && !pair_default);
@@ -717,6 +722,145 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
 // Launch shape of the moment kernels (step_moment.cuh), where the collision
 // has a moment form and its fields fit into a population copy.  A context
 // created for one particular step kernel keeps to it.
+// The moment kernel's work is laid out once: the pieces (planes of a tile of a
+// box) that each block goes through, in turn.  A piece costs its planes and
+// about 4 more.  Two ways:
+//  * dealt: equal chunks, chunk by chunk and tile by tile, dealt to the blocks in
+//    turn, with the chunk that leaves the busiest block the fewest planes.  The
+//    blocks then work on neighbouring tiles at the same height and read each
+//    other's rims from L2.
+//  * cut: the tiles one after the other as one row of planes, cut into one span
+//    per block: the busiest block has hardly more than the average, but rims
+//    come from HBM where the fields do not stay in L2.
+// Planes of the busiest block dealt / cut (average), and the time: 64 uneven boxes
+// 308 / 255 (243), 50 steps 30.0 / 26.1 ms; 256 x 256 x 575 340 / 309 (303), 50
+// steps 24.5 / 23.1 ms; with 10 fields, 384 x 384 x 1024 1813 / 1749 (1738), 20
+// steps 67.5 / 81.0 ms.
+struct MomentPlan {
+    std::vector<MomentPiece> pieces;
+    std::vector<int> first;  // of each block, and the end
+    long long busiest = 0;   // planes of the busiest block, with the extra ones
+};
+
+struct TileColumns {  // the tiles of a box
+    int tiles, nz;
+};
+
+constexpr int kPieceExtra = 4;
+
+// Cuts with at most `most` planes a block (>= 5); false if that takes more than `grid` blocks.
+bool cut_columns(const std::vector<TileColumns>& boxes, long long grid, long long most, MomentPlan* plan) {
+    constexpr int kExtra = kPieceExtra, kLeast = 4;  // a span does not end with a piece of fewer planes than kLeast
+    long long block = 0, room = most;
+    if (plan) plan->first.assign(1, 0);
+    for (size_t i = 0; i < boxes.size(); ++i) {
+        for (int t = 0; t < boxes[i].tiles; ++t) {
+            for (int z = 0; z < boxes[i].nz;) {
+                const int left = boxes[i].nz - z;
+                if (room < most && room - kExtra < (left < kLeast ? left : kLeast)) {
+                    if (++block == grid) return false;
+                    room = most;
+                    if (plan) plan->first.push_back(int(plan->pieces.size()));
+                }
+                const int take = left < room - kExtra ? left : int(room - kExtra);
+                if (plan) plan->pieces.push_back({int(i), t, z, z + take});
+                z += take;
+                room -= take + kExtra;
+            }
+        }
+    }
+    if (plan) {
+        plan->first.push_back(int(plan->pieces.size()));
+        plan->busiest = most;
+    }
+    return true;
+}
+
+MomentPlan cut_plan(const std::vector<TileColumns>& boxes, long long grid) {
+    long long lo = 5, hi = 5;
+    while (!cut_columns(boxes, grid, hi, nullptr)) {
+        lo = hi + 1;
+        hi *= 2;
+    }
+    while (lo < hi) {
+        const long long mid = (lo + hi) / 2;
+        if (cut_columns(boxes, grid, mid, nullptr)) hi = mid;
+        else lo = mid + 1;
+    }
+    MomentPlan plan;
+    cut_columns(boxes, grid, hi, &plan);
+    return plan;
+}
+
+MomentPlan dealt_plan(const std::vector<TileColumns>& boxes, long long grid) {
+    MomentPlan plan;
+    int max_nz = 1, zc = 1;
+    for (const TileColumns& b : boxes) max_nz = b.nz > max_nz ? b.nz : max_nz;
+    std::vector<long long> load(grid);
+    plan.busiest = -1;
+    const bool many = boxes.size() > 1;
+    for (int z = max_nz < (many ? 96 : 128) ? max_nz : (many ? 96 : 128); z >= 1; z = many && z > 24 ? z - 4 : z - 1) {
+        long long worst = 0;
+        if (!many) {
+            worst = busiest_block_planes(boxes[0].nz, boxes[0].tiles, grid, z, kPieceExtra);
+        } else {
+            std::fill(load.begin(), load.end(), 0);
+            long long item = 0;
+            for (const TileColumns& b : boxes)
+                for (int zs = 0; zs < b.nz; zs += z)
+                    for (int t = 0; t < b.tiles; ++t) load[item++ % grid] += (z < b.nz - zs ? z : b.nz - zs) + kPieceExtra;
+            worst = *std::max_element(load.begin(), load.end());
+        }
+        if (plan.busiest < 0 || worst < plan.busiest) {
+            plan.busiest = worst;
+            zc = z;
+        }
+    }
+    std::vector<MomentPiece> items;
+    for (size_t i = 0; i < boxes.size(); ++i)
+        for (int zs = 0; zs < boxes[i].nz; zs += zc)
+            for (int t = 0; t < boxes[i].tiles; ++t)
+                items.push_back({int(i), t, zs, zc < boxes[i].nz - zs ? zs + zc : boxes[i].nz});
+    for (size_t b = 0; b < size_t(grid) && b < items.size(); ++b) {
+        plan.first.push_back(int(plan.pieces.size()));
+        for (size_t k = b; k < items.size(); k += size_t(grid)) plan.pieces.push_back(items[k]);
+    }
+    plan.first.push_back(int(plan.pieces.size()));
+    return plan;
+}
+
+// bytes: one set of the moment fields of all boxes.  The cut pays for its rims with HBM reads unless the fields
+// stay in L2: dealt / cut planes, and what the cut gained, single boxes:
+//   4 fields: 300x200x100 (91 MB) 1.22, +10%; 160x150x320 (117 MB) 1.04, +3%; 192x192x400 1.07, +2%;
+//     256x256x575 1.10, +7%; 384x384x1024 1.05, -2%; 512x512x1024 1.03, +1%
+//   10 fields: 96x90x200 (65 MB) 1.07, +3%; 300x200x100 (228 MB) 1.16, +4%; 192x192x400 1.09, -7%; 256x256x575
+//     1.07, -11%; 384x384x1024 1.04, -20%
+MomentPlan plan_moments(const std::vector<TileColumns>& boxes, long long grid, int fields, size_t bytes) {
+    const MomentPlan dealt = dealt_plan(boxes, grid), cut = cut_plan(boxes, grid);
+    const double needed = bytes <= (128u << 20) ? 1.0 : (fields == 4 ? 1.05 : 1.25);
+    return double(dealt.busiest) > needed * double(cut.busiest) ? cut : dealt;
+}
+
+// Copies a plan to the device (one allocation in *mem) and enters it into the
+// launch description.
+cudaError_t upload_plan(const MomentPlan& plan, MomentLaunch& l, void** mem, size_t* bytes, cudaStream_t stream) {
+    const size_t np = plan.pieces.size() * sizeof(MomentPiece), nf = plan.first.size() * sizeof(int);
+    cudaError_t e = cudaMalloc(mem, np + nf);
+    if (e != cudaSuccess) {
+        *mem = nullptr;
+        return e;
+    }
+    *bytes = np + nf;
+    char* const at = static_cast<char*>(*mem);
+    e = cudaMemcpyAsync(at, plan.pieces.data(), np, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(at + np, plan.first.data(), nf, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    l.pieces = reinterpret_cast<const MomentPiece*>(at);
+    l.first = reinterpret_cast<const int*>(at + np);
+    l.grid = int(plan.first.size()) - 1;
+    return e;
+}
+
 void configure_moments(lbm_ctx* c) {
     const lbm_params& p = c->p;
     c->mom = nullptr;
@@ -738,22 +882,20 @@ void configure_moments(lbm_ctx* c) {
     }
     l.args = c->args;
     l.args.tiles_x = (p.nx + k->tile_x - 1) / k->tile_x;
-    l.args.n_tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
-    const long long grid = (long long)per_sm * c->num_sms;
-    long long best = -1;
-    for (int z = p.nz < 128 ? p.nz : 128; z >= 1; --z) {
-        const long long load = busiest_block_planes(p.nz, l.args.n_tiles, grid, z, 4);
-        if (best < 0 || load < best) {
-            best = load;
-            l.args.zchunk = z;
-        }
-    }
+    const int tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
+    const MomentPlan plan = plan_moments({{tiles, p.nz}}, (long long)per_sm * c->num_sms, k->fields, c->mom_bytes);
     // Small boxes: a turn of the moment kernel (one plane of the busiest block) takes about 1.5 us however few
     // blocks there are, two kernels 29 ps a cell and 4 us at least (24x24x48: 10.4 / 4.2 us a step; 64x64x128: 14.7
     // / 20.5; MRT with the paper's rates 48x48x96: 20.9 / 10.9, 80x80x160: 52.4 / 41.1, 96x96x192: 55.6 / 77).
-    if (c->split && 2.5 + 1.5 * double(best) > 4.0 + 29e-6 * double(c->n)) return;
-    l.args.n_items = l.args.n_tiles * ((p.nz + l.args.zchunk - 1) / l.args.zchunk);
-    l.grid = int(grid < l.args.n_items ? grid : l.args.n_items);
+    if (c->split && 2.5 + 1.5 * double(plan.busiest) > 4.0 + 29e-6 * double(c->n)) return;
+    size_t bytes = 0;
+    if (upload_plan(plan, l, &c->mom_plan, &bytes, c->stream) != cudaSuccess) {  // no room: step the populations
+        cudaGetLastError();
+        cudaFree(c->mom_plan);
+        c->mom_plan = nullptr;
+        return;
+    }
+    c->own_bytes += (long long)bytes;
     const long long rows = ((long long)p.ny * p.nz + 7) / 8;
     l.gather_grid = int(rows < 8LL * c->num_sms ? rows : 8LL * c->num_sms);
     c->mom = k;
@@ -1037,6 +1179,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->ref[1]);
     cudaFree(c->scratch);
     cudaFree(c->psi_ws);
+    cudaFree(c->mom_plan);
     cudaFree(c->diag);
     cudaFree(c->dev_err);
     cudaFree(c->adj.cp);
@@ -1425,6 +1568,7 @@ struct lbm_batch {
     // steps through the moment fields (nullptr: not for these boxes or this operator)
     const MomentKernels* mom = nullptr;
     MomentLaunch mom_launch{};
+    void* mom_plan = nullptr;         // device memory of its plan
     BatchBox* mom_boxes_dev = nullptr;
     bool mom_twice = false;
     // FP64 steps in two kernels over every box, where they run in place
@@ -1520,60 +1664,37 @@ lbm_status batch_configure_moments(lbm_batch* b) {
     const MomentKernels* k = moment_kernels(p.storage, coll);
     if (!k) return LBM_OK;
     b->mom_twice = true;
-    long long max_rows = 1, max_nz = 1;
+    long long max_rows = 1;
+    size_t bytes_all = 0;
     for (const lbm_ctx* c : b->box) {
         const lbm_params& q = c->p;
         const long long fields = (long long)k->fields * moment_cells(q.nx, q.ny, q.nz), pops = (long long)Q * c->n;
         if (q.nx < 4 || fields > pops) return LBM_OK;
         if (2 * fields > pops) b->mom_twice = false;
+        bytes_all += (size_t)fields * sizeof(float);
         const long long rows = (long long)q.ny * q.nz;
         if (rows > max_rows) max_rows = rows;
-        if (q.nz > max_nz) max_nz = q.nz;
     }
     const int per_sm = k->prepare(true);
     if (per_sm < 1) {
         cudaGetLastError();
         return LBM_OK;
     }
-    const long long grid = (long long)per_sm * b->num_sms;
-    auto tiles_of = [&](const lbm_params& q) {
-        return ((q.nx + k->tile_x - 1) / k->tile_x) * ((q.ny + k->tile_y - 1) / k->tile_y);
-    };
-    // The chunk that puts the fewest planes on the busiest block (each item also goes through ~4 planes that
-    // are not its own), items dealt round-robin in box order.
-    int zc = 1;
-    long long best = -1;
-    std::vector<long long> load(grid);
-    for (int z = int(max_nz < 96 ? max_nz : 96); z >= 1; z = z > 24 ? z - 4 : z - 1) {
-        std::fill(load.begin(), load.end(), 0);
-        long long item = 0;
-        for (const lbm_ctx* c : b->box) {
-            const int tiles = tiles_of(c->p);
-            for (int zs = 0; zs < c->p.nz; zs += z)
-                for (int t = 0; t < tiles; ++t) load[item++ % grid] += (z < c->p.nz - zs ? z : c->p.nz - zs) + 4;
-        }
-        const long long worst = *std::max_element(load.begin(), load.end());
-        if (best < 0 || worst < best) {
-            best = worst;
-            zc = z;
-        }
-    }
     std::vector<BatchBox> boxes(b->count);
-    int items = 0;
+    std::vector<TileColumns> columns(b->count);
     for (int i = 0; i < b->count; ++i) {
         const lbm_params& q = b->box[i]->p;
         BatchBox& bx = boxes[i];
+        bx = BatchBox{};
         bx.nx = q.nx;
         bx.ny = q.ny;
         bx.nz = q.nz;
         bx.tiles_x = (q.nx + k->tile_x - 1) / k->tile_x;
-        bx.n_tiles = tiles_of(q);
-        bx.zchunk = zc < q.nz ? zc : q.nz;
-        bx.item_begin = items;
         bx.base = b->base[i];
         bx.n = b->box[i]->n;
-        items += bx.n_tiles * ((q.nz + bx.zchunk - 1) / bx.zchunk);
+        columns[i] = {bx.tiles_x * ((q.ny + k->tile_y - 1) / k->tile_y), q.nz};
     }
+    const MomentPlan plan = plan_moments(columns, (long long)per_sm * b->num_sms, k->fields, bytes_all);
     if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
     LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
                                 b->stream));
@@ -1582,9 +1703,14 @@ lbm_status batch_configure_moments(lbm_batch* b) {
     l = MomentLaunch{};
     l.args = b->phys;
     l.batch.nbox = b->count;
-    l.batch.n_items = items;
     l.batch.boxes = b->mom_boxes_dev;
-    l.grid = int(grid < items ? grid : items);
+    size_t bytes = 0;
+    if (upload_plan(plan, l, &b->mom_plan, &bytes, b->stream) != cudaSuccess) {  // no room: step the populations
+        cudaGetLastError();
+        cudaFree(b->mom_plan);
+        b->mom_plan = nullptr;
+        return LBM_OK;
+    }
     const long long want = (max_rows + 7) / 8, cap = 1 + 16LL * b->num_sms / b->count;
     l.gather_grid = int(want < cap ? want : cap);
     b->mom = k;
@@ -1722,6 +1848,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->f[1]);
     cudaFree(b->boxes_dev);
     cudaFree(b->mom_boxes_dev);
+    cudaFree(b->mom_plan);
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
 }
@@ -1848,8 +1975,8 @@ AdjointArgs adjoint_args(const lbm_ctx* c) {
     a.gwf = c->args.gwf;
     const long long rows = (long long)c->p.ny * c->p.nz;
     const long long want = (rows + adjoint_rows_per_block() - 1) / adjoint_rows_per_block();
-    // One block per 8 rows as far as the blocks' partial sums stay small: a cap near the resident blocks left
-    // the last of 1440 blocks' worth of rows (64 x 64 x 180) to a second, mostly empty round.
+    // One block per group of rows as far as the blocks' partial sums stay small: a cap near the resident blocks left
+    // the last of the groups (2880 at 64 x 64 x 180) to a last, mostly empty round.
     const long long cap = 1 << 14;
     a.grid = int(want < cap ? (want < 1 ? 1 : want) : cap);
     a.tau1 = c->p.tau == 1.0;

@@ -122,13 +122,19 @@ const StepKernels& step_kernels(int storage, int coll);
 __host__ __device__ inline int moment_pitch(int nx) { return ((nx + 3) & ~3) + 4; }
 inline long long moment_cells(int nx, int ny, int nz) { return (long long)moment_pitch(nx) * ny * nz; }
 
-// Launch description of the moment kernels (step_moment.cuh).  args.tiles_x,
-// n_tiles, n_items and zchunk are those of the moment kernel's tiles; boxes:
-// the batch's box table (nbox > 0) with work items of the same tiles.
+// Planes zs .. ze - 1 of a tile of a box: what a block of the moment kernel goes through at a time.
+struct alignas(16) MomentPiece {
+    int box, tile, zs, ze;
+};
+
+// Launch description of the moment kernels (step_moment.cuh).  args.tiles_x is
+// that of the moment kernel's tiles; boxes: the batch's box table (nbox > 0).
 struct MomentLaunch {
     StepArgs args;
     BatchArgs batch;
-    int grid;             // persistent grid of the step
+    const MomentPiece* pieces;  // device: block b takes pieces first[b] .. first[b + 1] - 1
+    const int* first;
+    int grid;             // blocks of the step
     int gather_grid;      // blocks (per box) of the populations -> moments pass
     int src_hi, dst_hi;   // which of a copy's two sets of moment fields
     cudaStream_t stream;

@@ -31,6 +31,14 @@
 // 416 of 512 threads own output cells.  The rim columns sit in one warp of
 // their own, so that all other warps load and store whole rows.
 //
+// Bound: not HBM (32 B a cell and step at 4 fields is 30% of the copy rate) but,
+// with 4 fields, issue slots and the chain within a plane (224 instructions a
+// cell, 49% of the slots at 16 warps an SM), with 9 and 10 the shared memory their planes in flight take
+// (384 threads an SM).  Measured, one call: SRT tau = 1, 256 x 256 x 575, 50
+// steps 55.9 -> 23.1 ms; FP16 with local references, unit-rate MRT, 20 steps
+// 23.4 -> 12.9 ms; 64 uneven boxes, 50 steps 52.6 -> 26.0 ms; the paper's MRT,
+// 384 x 384 x 1024, 20 steps 100.8 -> 66.8 ms.
+//
 // Layout of the fields: rows of nx (rounded up to a multiple of 4) + 4 cells,
 // two periodic copies of cells at either end, so that no load wraps along x
 // and pairs stay aligned for any nx.  The density comes first by itself; the
@@ -80,6 +88,8 @@ __host__ __device__ constexpr int exch_index(int q) {
 
 struct MomentArgs {
     int src_hi, dst_hi;  // the buffer's second set of moment fields (0: its first)
+    const MomentPiece* pieces;
+    const int* first;
 };
 
 // The moments of a thread's pair at float offset od of a field.
@@ -164,35 +174,26 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
     const DevParams& dev = a.dev;
     auto psi_v = [&](V r) { return vmap(r, [&](float x) { return psi_of<float>(x, rho0, inv_rho0); }); };
 
-    const int n_items = BATCH ? b.n_items : a.n_items;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        int nx, ny, nz, tiles_x, n_tiles, zchunk, local;
+    for (int piece = ma.first[blockIdx.x]; piece < ma.first[blockIdx.x + 1]; ++piece) {
+        const MomentPiece work = ma.pieces[piece];
+        int nx, ny, nz, tiles_x;
         long long base = 0;
         if constexpr (BATCH) {
-            int lo = 0, hi = b.nbox - 1;  // last box with item_begin <= item
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (b.boxes[mid].item_begin <= item) lo = mid;
-                else hi = mid - 1;
-            }
-            const BatchBox& bx = b.boxes[lo];
+            const BatchBox& bx = b.boxes[work.box];
             nx = bx.nx; ny = bx.ny; nz = bx.nz;
-            tiles_x = bx.tiles_x; n_tiles = bx.n_tiles; zchunk = bx.zchunk;
-            local = item - bx.item_begin;
+            tiles_x = bx.tiles_x;
             base = bx.base;
         } else {
             nx = a.nx; ny = a.ny; nz = a.nz;
-            tiles_x = a.tiles_x; n_tiles = a.n_tiles; zchunk = a.zchunk;
-            local = item;
+            tiles_x = a.tiles_x;
         }
         const int pitch = moment_pitch(nx);
         const unsigned plane = unsigned(pitch) * unsigned(ny);
         const long long nf = (long long)plane * nz;
         const float* __restrict__ src = static_cast<const float*>(src_all) + base + (ma.src_hi ? NF * nf : 0);
 
-        const int tile = local % n_tiles, chunk = local / n_tiles;
-        const int x0 = (tile % tiles_x) * T::TXO, y0 = (tile / tiles_x) * T::OUT;
-        const int zs = chunk * zchunk, ze = min(zs + zchunk, nz);
+        const int x0 = (work.tile % tiles_x) * T::TXO, y0 = (work.tile / tiles_x) * T::OUT;
+        const int zs = work.zs, ze = work.ze;
         const int x = x0 + (rp - 1) * 2, y = y0 + ry - 1;
         const unsigned off = unsigned(wrap_index(y, ny)) * pitch + min(x + 2, pitch - 2);
         const unsigned hoff =
@@ -553,11 +554,11 @@ cudaError_t moment_launch(const MomentLaunch& l, const void* src, void* dst) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             if (e != cudaSuccess) return e;
             return launch_chained(moment_chain(l), kern, l.grid, T::NT, sm, l.stream, src, dst, l.args, l.batch,
-                                  MomentArgs{l.src_hi, l.dst_hi});
+                                  MomentArgs{l.src_hi, l.dst_hi, l.pieces, l.first});
         }
     }
     return launch_chained(moment_chain(l), sc_moment_kernel<Codec, COLL, EMIT, BATCH>, l.grid, T::NT,
-                          sm, l.stream, src, dst, l.args, l.batch, MomentArgs{l.src_hi, l.dst_hi});
+                          sm, l.stream, src, dst, l.args, l.batch, MomentArgs{l.src_hi, l.dst_hi, l.pieces, l.first});
 }
 
 template <class Codec, int COLL, bool EMIT>

@@ -15,10 +15,16 @@
 // twice; the 72 to 88 B a cell that the second kernel adds hide behind the
 // FP64 pipe.
 //
+// Measured: 32 x 32 x 64, SRT, 50 steps 8.23 -> 1.10 ms (of that the marching
+// kernel's 32 blocks on 152 SMs cost most); 128 x 128 x 288, MRT, 10 steps
+// 30.7 -> 14.5 ms, 3.25 GLUPS.
+//
 // 32- and 16-bit storage: the extra passes cost bytes, so large boxes keep the
 // marching kernels.  Boxes that live in L2 are bound by the marching kernels'
 // latency instead (a few planes per block, one barrier each), and 16-bit
-// storage with odd rows has no pipelined kernel at all.
+// storage with odd rows has no pipelined kernel at all (bound by latency and the
+// partly filled sectors of its unaligned rows; BF16 97 x 85 x 131, 20 steps:
+// 1.14 -> 0.98 ms).
 #pragma once
 #include "collide.cuh"
 #include "launch.cuh"

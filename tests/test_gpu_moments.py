@@ -99,3 +99,24 @@ def test_two_kernel_fp64_step_is_bit_identical(op):
             B.step(n)
         for v, f in zip(B.boxes, want):
             assert np.array_equal(v.get_populations(), f), v.shape
+
+
+@pytest.mark.parametrize("op", list(OPS))
+def test_spans_that_end_within_tiles_and_boxes(op):
+    """More tiles than the device has blocks: a block's span of planes ends within a tile and goes on in the
+    next one, or in the next box of a batch."""
+    box = (256, 620, 7)
+    want, _, _ = _state(box, 1, [1] * 3, **OPS[op])
+    got, _, _ = _state(box, 0, (3,), **OPS[op])
+    assert np.array_equal(got, want), np.abs(got - want).max()
+    dims = [(70, 27, 3 + k % 7) for k in range(60)]
+    with lbm.Batch(dims, G=-5.5, storage="f32", **OPS[op]) as B:
+        for v, d in zip(B.boxes, dims):
+            v.set_density(inputs.random_density(*d, seed=7, lo=0.3, hi=1.9))
+        B.step(3)
+        got = [v.get_populations() for v in B.boxes]
+    for d in dims[:7]:
+        want, _, _ = _state(d, 1, [1] * 3, **OPS[op])
+        for k, f in enumerate(got):
+            if dims[k] == d:
+                assert np.array_equal(f, want), (k, d)
