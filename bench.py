@@ -5,15 +5,18 @@
 
 Workload (default): the sharp-interface ligament R0 = 64, kR0 = 0.7 in a
 256 x 256 x 575 periodic box (37.7 M cells), G = -5.5, SRT with velocity shift
-at tau = 1, FP32 populations, 5% cosine perturbation.  A step is one fused
-step-kernel launch over the whole box; inputs (2 x 2.86 GB population copies)
-are far larger than L2, so no flush is needed between steps.
+at tau = 1, FP32 populations, 5% cosine perturbation.  A step is one call of
+one step (for FP32 one fused kernel launch over the whole box); inputs (2 x
+2.86 GB population copies) are far larger than L2, so no flush is needed
+between steps.
 
 Prints ONE JSON line (rank 0).  `value` is MLUPS (million lattice updates per
 second) over all ranks, device-timed with CUDA events; `e2e` is the same
 metric through the C ABI with host buffers (initial density uploaded from
 pinned host memory, diagnostics read back every 50 steps, final density read
-back); `roofline` relates the step kernel's algorithmic bytes to the measured
+back); `one_call` is the device time of the same number of steps asked for in
+one call, as a run does between two diagnostics (tau = 1 then keeps only the
+moments between the steps); `roofline` relates the step kernel's algorithmic bytes to the measured
 HBM copy bandwidth; `cpu_baseline` times the FP64 reference implementation on
 a bounded slab of the same workload on the host cores.
 
@@ -42,7 +45,31 @@ BYTES_PER_POP = {"f64": 8, "f32": 4, "f16": 2, "bf16": 2, "f16l": 2, "bf16l": 2}
 EXTRA_BYTES_PER_CELL = {"f16l": 8, "bf16l": 8}
 FALLBACK_HBM_GBS = 6800.0
 KERNEL_NAMES = {1: "sc_step_kernel", 2: "sc_step_async_kernel", 3: "sc_step_pipe_kernel", 4: "sc_step_bulk_kernel",
-                5: "sc_step_tma_kernel", 6: "sc_step_mr_kernel", 7: "sc_step_pair16_kernel"}
+                5: "sc_step_tma_kernel", 6: "sc_psi_kernel + sc_step_mr_kernel", 7: "sc_step_pair16_kernel"}
+
+
+def step_kernels(storage, kernel, info, cells):
+    """Names of the kernels of one single step and how many they are: FP64,
+    odd 16-bit rows and boxes that fit into L2 run in two (unless --kernel
+    asks for one), the two-belt force as well."""
+    name = KERNEL_NAMES.get(info["kernel"], "sc_step_kernel")
+    if info["kernel"] == 6:
+        return name, 2
+    small = {"f32": 1200000, "f16": 2000000, "bf16": 2000000, "f16l": 250000, "bf16l": 250000}.get(storage, 0)
+    if kernel == 0 and (info["kernel"] == 1 or cells <= small):
+        return "sc_fields_kernel + sc_push_kernel", 2
+    return name, 1
+
+
+def run_bytes(storage, steps):
+    """Algorithmic bytes per cell and step of one call of `steps` steps at
+    tau = 1 (SRT): FP32 and 16-bit storage read and write four moments a step
+    and the populations once a call; FP64 leaves four moments and psi in the
+    first populations' place between its two kernels."""
+    pops = 2 * 19 * BYTES_PER_POP[storage] + EXTRA_BYTES_PER_CELL.get(storage, 0)
+    if storage == "f64":
+        return pops + 2 * 5 * 8
+    return 32 + pops / steps if steps >= 2 else pops
 
 
 def parse_args():
@@ -327,7 +354,7 @@ def measure_forms(device, clocks):
     (R0 = 16); the batched form; the adjoint form.  About half a minute."""
     peak = measured_hbm()[0]
     forms = {"rates_workload": "ligament R0=64 kR0=0.7 box 256x256x575, G=-5.5, SRT tau=1 (device time, CUDA "
-                               "events around the step launches)",
+                               "events around one call of 20 (f64) or 100 steps)",
              "accuracy_workload": "ligament R0=16 kR0=0.7 box 64x64x144, G=-5.5, SRT tau=1, 5% perturbation, "
                                   "run to the first pinch-off, diagnostics every 5 steps; errors against the "
                                   "FP64 GPU run of the same case"}
@@ -336,11 +363,12 @@ def measure_forms(device, clocks):
     fpc = rec.get("fp64_flops_per_cell") if rec else None
     pk, src = fp64_peak(device, clocks)
     forms["f64"] = {"glups": f64["glups"], "ms_per_step": f64["ms_per_step"],
-                    "hbm_frac": 304 * f64["glups"] / peak,
+                    "hbm_frac": run_bytes("f64", 20) * f64["glups"] / peak,
                     "fp64_pipe_frac": (fpc * f64["glups"] / 1e3 / pk) if fpc else None,
                     "fp64_flops_per_cell": fpc, "fp64_peak_tflops": pk, "fp64_peak_source": src,
                     "kernel": f64["kernel"]}
-    for st, bpc in (("f16l", 84), ("f16", 76), ("bf16l", 84)):
+    for st in ("f16l", "f16", "bf16l"):
+        bpc = run_bytes(st, 100)
         r = measure_rate(st, steps=100, warmup=5)
         forms[st] = {"glups": r["glups"], "ms_per_step": r["ms_per_step"], "bytes_per_cell": bpc,
                      "hbm_frac": bpc * r["glups"] / peak, "speedup_vs_f64": r["glups"] / f64["glups"],
@@ -484,6 +512,11 @@ def run_ours(args):
     torch.cuda.synchronize()
     clocks = sampler.stop() if sampler else None
     total_ms = t_start.elapsed_time(t_end)
+    t_start.record(stream)
+    L.step(args.steps)
+    t_end.record(stream)
+    torch.cuda.synchronize()
+    call_ms = t_start.elapsed_time(t_end)
     kernel_ms = sum(s.elapsed_time(e) for s, e in ev) / args.steps
     d1 = L.diag(w["rho_l"], w["rho_v"])
     mass_drift = abs(d1["mass"] - d0["mass"]) / d0["mass"]
@@ -525,7 +558,7 @@ def run_ours(args):
 
     peak, src = measured_hbm()
     bpc = 2 * 19 * BYTES_PER_POP[args.storage] + EXTRA_BYTES_PER_CELL.get(args.storage, 0)
-    kname = KERNEL_NAMES.get(L_info["kernel"], "sc_step_kernel")
+    kname, n_kernels = step_kernels(args.storage, args.kernel, L_info, ncell)
     rec = step_record()
     if args.storage == "f64" and rec and rec.get("fp64_flops_per_cell"):
         # FP64 is bound by the FP64 pipe: SMs x 2 FP64 lanes per clock
@@ -570,7 +603,9 @@ def run_ours(args):
                          f"{19 * BYTES_PER_POP[args.storage] * ncell / 1e9:.2f} GB each)",
                    "mass_rel_drift": mass_drift},
         "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-        "gpu_launches": args.steps, "host": host_info(), "forms": forms,
+        "one_call": {"value": ncell * args.steps / (call_ms / 1e3) / 1e6, "unit": "MLUPS", "steps": args.steps,
+                     "ms_per_step": call_ms / args.steps, "ranks": "rank 0"},
+        "gpu_launches": args.steps * n_kernels, "host": host_info(), "forms": forms,
     }
     print(json.dumps(line), flush=True)
     if dist is not None:
@@ -597,7 +632,8 @@ def fp64_peak(device, clocks=None):
     return peak, f"FP64 pipe: {sms} SMs x 2 lanes/clk x {mhz:.0f} MHz ({src}) x 2 flop (derived)"
 
 
-STEP_SOURCES = ("step_kernel.cuh", "codec.cuh", "lattice.cuh", "step_multirange.cuh", "e8.cuh", "step_pair16.cuh")
+STEP_SOURCES = ("step_kernel.cuh", "codec.cuh", "lattice.cuh", "step_multirange.cuh", "e8.cuh", "step_pair16.cuh",
+                "collide.cuh", "step_moment.cuh", "step_split.cuh")
 
 
 def step_record():
@@ -638,7 +674,8 @@ def measure_batched(steps, warmup, trial_steps=3):
     """64 independent ligaments (R0 in {8, 12, 16}, kR0 uniform on [0.2, 1.0)
     from seed 0, box 4R0 x 4R0 x round(2 pi R0 / kR0)), FP32 SRT tau = 1,
     G = -5.5, 3% perturbation, advanced together by one launch per step
-    (pairs of steps from a CUDA graph) after the launch-shape autotuner.
+    (between the first and the last on the moments) after the launch-shape
+    autotuner.
     Returns the device time of `steps` steps and the chosen configuration."""
     import torch
 
@@ -666,7 +703,7 @@ def measure_batched(steps, warmup, trial_steps=3):
     return {"ms": ms, "steps": steps, "cells": cells, "config": cfg, "tune": best,
             "ligaments_per_s": 64.0 / (ms / 1e3 * 3000.0 / steps),
             "aggregate_mlups": cells * steps / (ms / 1e3) / 1e6,
-            "hbm_gbs": 152 * cells / (ms / steps / 1e3) / 1e9}
+            "hbm_gbs": run_bytes("f32", steps) * cells / (ms / steps / 1e3) / 1e9}
 
 
 def run_batched(args):
@@ -690,7 +727,7 @@ def run_batched(args):
         "aggregate_mlups": m["aggregate_mlups"],
         "roofline": {"bound": "hbm", "achieved": m["hbm_gbs"], "peak": peak, "unit": "GB/s",
                      "frac": m["hbm_gbs"] / peak},
-        "gpu_launches": args.steps,
+        "gpu_launches": args.steps + 1 if args.steps >= 2 else args.steps,
     }
     print(json.dumps(line), flush=True)
 
@@ -1028,7 +1065,7 @@ def run_multirange(args):
         "ms_per_step": ms, "higher_is_better": True, "dtype": "f32", "data": "synthetic",
         "config": {"workload": "ligament R0=64 kR0=0.7 box 256x256x575, G1=-7, G2=1.5, SRT tau=1, FP32",
                    "kernel": cfg},
-        "roofline": {"bound": "hbm", "achieved": 152 * nx * ny * nz / (ms / 1e3) / 1e9,
+        "roofline": {"bound": "hbm", "achieved": 160 * nx * ny * nz / (ms / 1e3) / 1e9,
                      "peak": measured_hbm()[0], "unit": "GB/s"},
         "splits": splits}), flush=True)
 

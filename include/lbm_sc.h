@@ -94,18 +94,24 @@ typedef struct {
     void *f_a, *f_b;      /* optional caller-owned device buffers for the two
                              population copies (each 19*nx*ny*nz elements of the
                              storage type, 16-byte aligned); NULL = the library
-                             allocates (and frees them in lbm_destroy).            */
-    int zchunk;           /* step kernel: z planes per work item; 0 = auto (at most
-                             32, and at most 24 MiB of one population's planes
-                             on 32x16 tiles; 8 when one population's plane is
+                             allocates (and frees them in lbm_destroy).  A step
+                             may overwrite both: only the current copy
+                             (lbm_current_copy) holds a state.                      */
+    int zchunk;           /* step kernel: z planes per work item; 0 = auto (the
+                             length that loads the blocks most evenly, at most
+                             96, and at most 24 MiB of one population's planes;
+                             8 on 32x16 tiles when one population's plane is
                              1.5 MiB or more)                                       */
     int tile_y;           /* step kernel: tile height (4, 8 or 16); 0 = auto: 16
-                             for FP32 SRT and unit-rate MRT, 8 for other FP32
-                             MRT and for kernel 7, 4 otherwise                      */
+                             for FP32, 8 for 16-bit storage with nx even and for
+                             kernel 6, 4 otherwise                                  */
     int kernel;           /* step kernel variant: 0 = auto (3 for FP32 and the
                              local-reference formats, 7 for the global-reference
                              16-bit formats, when nx is even for 16-bit storage;
-                             else 1),
+                             else 1; lbm_step then also uses the forms described
+                             there: two kernels a step, or moments between the
+                             steps of one call); any other value = that kernel
+                             for every step,
                              1 = register-staged,
                              2 = cp.async-staged persistent, 3 = pipelined
                              persistent (2: FP64/FP32 storage; 3: also the
@@ -115,7 +121,8 @@ typedef struct {
                              nx % 32 == 0, ny % tile_y == 0; steps on buffers
                              other than the two copies, e.g. the adjoint's
                              recomputation, run kernel 3),
-                             6 = two-belt force (chosen when G2 != 0),
+                             6 = two-belt force (chosen when G2 != 0; psi in a
+                             kernel of its own where there is room for it),
                              7 = paired 16-bit pipeline: two cells per thread
                              along x, 64-cell tile rows, shifted pushes as
                              aligned 32-bit words through warp shuffles (16-bit
@@ -181,7 +188,19 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int on_device);
 /* Advance n >= 0 time steps (Eq. LBE): Shan-Chen force (Eq. SC_force with the
  * psi law, plus the second belt when G2 != 0), SRT with the shifted equilibrium velocity u' = u + tau F / rho
  * (Eq. vel_shift) or MRT with Guo-like forcing at u_b = u + F/(2 rho)
- * (Eq. barycentric), then periodic streaming.  Enqueues n kernel launches. */
+ * (Eq. barycentric), then periodic streaming.
+ *
+ * Enqueues the kernels of n steps and returns.  n steps in one call give the
+ * same bits as n calls of one step, in the same population copy.  With
+ * lbm_params.kernel = 0 and 32- or 16-bit storage, a call of n >= 2 steps of
+ * an operator whose result follows from a few moments (SRT at tau = 1; MRT
+ * with every rate 1; FP32 MRT with its rates at 1 outside e, 3pxx, pww and the
+ * off-diagonal stress) reads the populations once, keeps 4, 9 or 10 moments
+ * between the steps (in the two copies themselves) and writes the populations
+ * at the end: ask for many steps at once where nothing is read in between.
+ * FP64, small boxes and 16-bit storage with nx odd step in two kernels, with a
+ * psi field of n cells of their own where the moments do not suffice; if it
+ * cannot be allocated, in one. */
 lbm_status lbm_step(lbm_ctx *ctx, long n);
 
 /* Steps taken since the last initialisation. */
@@ -258,8 +277,8 @@ long long lbm_device_bytes(const lbm_ctx *ctx);
 /* Launch configuration the context chose for the step kernel: variant
  * (1 register-staged, 2 cp.async-staged, 3 pipelined, 4 bulk-copy, 5 tensor
  * copy, 6 two-belt force, 7 paired 16-bit), tile height, z planes per work
- * item and grid size
- * (blocks).  Any pointer may be NULL. */
+ * item and grid size (blocks).  The two-kernel and the moment form of lbm_step
+ * have shapes of their own, which are not reported.  Any pointer may be NULL. */
 lbm_status lbm_kernel_config(const lbm_ctx *ctx, int *kernel, int *tile_y,
                              int *zchunk, int *grid);
 
@@ -311,7 +330,8 @@ lbm_status lbm_adjoint_forward(lbm_ctx *ctx, const double *rho0, int on_device,
  * NULL), dJ/dG and dJ/dtau (host doubles; may be NULL).  Synchronises the
  * context's stream.  Working memory besides the checkpoints: two adjoint
  * states, `every` psi fields (the recomputation stores psi of each state it
- * steps from, with step kernels 1, 3 and 5) and six more fields. */
+ * steps from) and six more fields.  At tau = 1 an adjoint state is 4 values a
+ * cell (20 otherwise). */
 lbm_status lbm_adjoint_backward(lbm_ctx *ctx, const double *dJdrho,
                                 int in_on_device, double *dJdrho0,
                                 int out_on_device, double *dJdG,
@@ -342,8 +362,10 @@ const char *lbm_batch_last_error(const lbm_batch *b);
 lbm_status lbm_batch_box(lbm_batch *b, int i, lbm_ctx **view);
 
 /* Advance every box n >= 0 steps with one kernel launch per step over the
- * work items (xy tile, z chunk) of all boxes; pairs of steps are replayed
- * from a captured CUDA graph. */
+ * work items (xy tile, z chunk) of all boxes.  FP32 operators whose result
+ * follows from a few moments keep only those between the steps of a call
+ * (lbm_step); otherwise pairs of steps are replayed from a captured CUDA
+ * graph. */
 lbm_status lbm_batch_step(lbm_batch *b, long n);
 
 /* Autotune the launch shape: times trial_steps steps for each tile height in

@@ -26,8 +26,9 @@
 // form loads two values, and 128 + 40 B a cell and step instead of 250 + 40.
 // 64 x 64 x 180 in FP32, 500 steps back with their recomputation: 64.1 ms with
 // 20 values, 50.2 with {A, B}, 41.4 with the recomputed states kept as moments
-// too, 37.7 with the block shape and block sums below.  Both kernels are bound by the latency of their gathers from L2 (about
-// 39 and 17 us a step from a cold cache).
+// too, 37.7 with the block shape and block sums below.  Both kernels are bound
+// by the latency of their gathers from L2 (about 39 and 17 us a step from a
+// cold cache before those two).
 #include <cuda_runtime.h>
 
 #include "adjoint.h"

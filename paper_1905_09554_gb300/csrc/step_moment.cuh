@@ -33,8 +33,8 @@
 //
 // Bound: not HBM (32 B a cell and step at 4 fields is 30% of the copy rate) but,
 // with 4 fields, issue slots and the chain within a plane (224 instructions a
-// cell, 49% of the slots at 16 warps an SM), with 9 and 10 the shared memory their planes in flight take
-// (384 threads an SM).  Measured, one call: SRT tau = 1, 256 x 256 x 575, 50
+// cell, 49% of the slots at 16 warps an SM), with 9 and 10 the shared memory
+// their planes in flight take (384 threads an SM).  Measured, one call: SRT tau = 1, 256 x 256 x 575, 50
 // steps 55.9 -> 23.1 ms; FP16 with local references, unit-rate MRT, 20 steps
 // 23.4 -> 12.9 ms; 64 uneven boxes, 50 steps 52.6 -> 26.0 ms; the paper's MRT,
 // 384 x 384 x 1024, 20 steps 100.8 -> 66.8 ms.
