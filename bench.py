@@ -55,7 +55,7 @@ def step_kernels(storage, kernel, info, cells):
     name = KERNEL_NAMES.get(info["kernel"], "sc_step_kernel")
     if info["kernel"] == 6:
         return name, 2
-    small = {"f32": 1200000, "f16": 2000000, "bf16": 2000000, "f16l": 250000, "bf16l": 250000}.get(storage, 0)
+    small = {"f32": 1200000, "f16": 2000000, "bf16": 2000000, "f16l": 1200000, "bf16l": 1200000}.get(storage, 0)
     if kernel == 0 and (info["kernel"] == 1 or cells <= small):
         return "sc_fields_kernel + sc_push_kernel", 2
     return name, 1

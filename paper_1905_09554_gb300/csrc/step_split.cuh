@@ -24,7 +24,7 @@
 // latency instead (a few planes per block, one barrier each), and 16-bit
 // storage with odd rows has no pipelined kernel at all (bound by latency and the
 // partly filled sectors of its unaligned rows; BF16 97 x 85 x 131, 20 steps:
-// 1.14 -> 0.98 ms).
+// 1.14 -> 0.78 ms).
 #pragma once
 #include "collide.cuh"
 #include "launch.cuh"
@@ -32,7 +32,12 @@
 
 namespace lbm {
 
-constexpr int kSplitThreads = 64;
+// Threads a block.  FP64: 64, so that the few blocks of a small box spread over all SMs (32 x 32 x 64, 50 steps: 1.10 ms
+// with 64, 1.18 with 128, 1.24 with 256).  32- and 16-bit storage: 256, because placing blocks of 64 takes longer than
+// their work (BF16 97 x 85 x 131, 20 steps: 983 us with 64, 824 with 128, 775 with 256; FP32 48 x 48 x 96: 10.4 / 8.6 /
+// 8.4 us a step).
+template <class R>
+constexpr int kSplitThreads = sizeof(R) == 8 ? 64 : 256;
 
 // Element k of cell i of a field array with n cells each.
 template <class S>
@@ -43,7 +48,7 @@ __device__ __forceinline__ S* cell_at(S* p, int k, unsigned n, unsigned i) {
 // psi in slot kMoments<COLL> behind the moments (IN_PLACE), or in its own
 // field.  Local-reference storage: the density goes to ref_dst as well.
 template <class Codec, int COLL, bool IN_PLACE>
-__global__ void __launch_bounds__(kSplitThreads)
+__global__ void __launch_bounds__(kSplitThreads<typename Codec::R>)
 sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const StepArgs a, const BatchArgs b) {
     using R = typename Codec::R;
     constexpr int NF = kMoments<COLL>;
@@ -55,7 +60,7 @@ sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const Ste
         n = unsigned(bx.n);
         base = bx.base;
     }
-    const unsigned i = blockIdx.x * kSplitThreads + threadIdx.x;
+    const unsigned i = blockIdx.x * kSplitThreads<R> + threadIdx.x;
     if (i >= n) return;
     typename Codec::S* const f = f_all + base;
     float ref = 0.0f;
@@ -95,7 +100,7 @@ struct NeighbourPsi {
 };
 
 template <class Codec, int COLL, bool IN_PLACE>
-__global__ void __launch_bounds__(kSplitThreads)
+__global__ void __launch_bounds__(kSplitThreads<typename Codec::R>)
 sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Codec::R* __restrict__ psi_all,
                typename Codec::S* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
     using R = typename Codec::R;
@@ -112,7 +117,7 @@ sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Cod
         base = bx.base;
     }
     const unsigned plane = unsigned(nx) * unsigned(ny), n = plane * unsigned(nz);
-    const unsigned i = blockIdx.x * kSplitThreads + threadIdx.x;
+    const unsigned i = blockIdx.x * kSplitThreads<R> + threadIdx.x;
     if (i >= n) return;
     const S* __restrict__ src = src_all + base;
     S* __restrict__ dst = dst_all + base;
@@ -177,17 +182,17 @@ template <class Codec, int COLL>
 cudaError_t split_step(const SplitLaunch& l, void* src, void* dst, void* psi) {
     using S = typename Codec::S;
     using R = typename Codec::R;
-    const dim3 grid((l.max_cells + kSplitThreads - 1) / kSplitThreads, l.batch.nbox ? l.batch.nbox : 1);
+    const dim3 grid((l.max_cells + kSplitThreads<R> - 1) / kSplitThreads<R>, l.batch.nbox ? l.batch.nbox : 1);
     S* const s = static_cast<S*>(src);
     S* const d = static_cast<S*>(dst);
     R* const p = static_cast<R*>(psi);
-    const bool chain = (long long)grid.x * grid.y * kSplitThreads <= 400000;
+    const bool chain = (long long)grid.x * grid.y * kSplitThreads<R> <= 400000;
     auto both = [&](auto in_place) {
         constexpr bool IN = decltype(in_place)::value;
-        cudaError_t e = launch_chained(chain, sc_fields_kernel<Codec, COLL, IN>, grid, kSplitThreads, 0, l.stream, s, p, l.args,
+        cudaError_t e = launch_chained(chain, sc_fields_kernel<Codec, COLL, IN>, grid, kSplitThreads<R>, 0, l.stream, s, p, l.args,
                                        l.batch);
         if (e == cudaSuccess)
-            e = launch_chained(chain, sc_push_kernel<Codec, COLL, IN>, grid, kSplitThreads, 0, l.stream, s, p, d, l.args,
+            e = launch_chained(chain, sc_push_kernel<Codec, COLL, IN>, grid, kSplitThreads<R>, 0, l.stream, s, p, d, l.args,
                                l.batch);
         return e;
     };

@@ -120,3 +120,18 @@ def test_spans_that_end_within_tiles_and_boxes(op):
         for k, f in enumerate(got):
             if dims[k] == d:
                 assert np.array_equal(f, want), (k, d)
+
+
+@pytest.mark.parametrize("storage,op", [("f32", "srt09"), ("f32", "general"), ("f32", "srt"), ("f16", "srt09"),
+                                        ("bf16", "general"), ("f16l", "srt09"), ("bf16l", "paper")])
+def test_two_kernel_step_of_small_boxes_is_bit_identical(storage, op):
+    """FP32 and 16-bit boxes that step in two kernels, against the register-staged kernel: fewer cells than a
+    block has threads, one more, a last block that is nearly empty, odd and even rows."""
+    more = {"srt09": dict(collision="srt", tau=0.9),
+            "general": dict(collision="mrt", tau=0.9, rates=[0.8 + 0.04 * ((7 * k) % 19) for k in range(19)])}
+    kw = dict(OPS, **more)[op]
+    for box in ((1, 3, 5), (257, 1, 1), (32, 8, 2), (33, 13, 5), (64, 50, 31), (101, 99, 97)):
+        want, copy, t = _state(box, 1, [1] * 3, storage, **kw)
+        got, copy2, t2 = _state(box, 0, [1] * 3, storage, **kw)
+        assert (copy, t) == (copy2, t2)
+        assert np.array_equal(got, want), (box, np.abs(got - want).max())
