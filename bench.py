@@ -48,14 +48,16 @@ KERNEL_NAMES = {1: "sc_step_kernel", 2: "sc_step_async_kernel", 3: "sc_step_pipe
                 5: "sc_step_tma_kernel", 6: "sc_psi_kernel + sc_step_mr_kernel", 7: "sc_step_pair16_kernel"}
 
 
-def step_kernels(storage, kernel, info, cells):
+def step_kernels(storage, kernel, info, cells, in_place):
     """Names of the kernels of one single step and how many they are: FP64,
     odd 16-bit rows and boxes that fit into L2 run in two (unless --kernel
-    asks for one), the two-belt force as well."""
+    asks for one), the two-belt force as well.  in_place: the collision needs
+    only a few moments."""
     name = KERNEL_NAMES.get(info["kernel"], "sc_step_kernel")
     if info["kernel"] == 6:
         return name, 2
-    small = {"f32": 1200000, "f16": 2000000, "bf16": 2000000, "f16l": 1200000, "bf16l": 1200000}.get(storage, 0)
+    small = {"f32": 1200000 if in_place else 400000, "f16": 2000000, "bf16": 2000000, "f16l": 250000,
+             "bf16l": 250000}.get(storage, 0)
     if kernel == 0 and (info["kernel"] == 1 or cells <= small):
         return "sc_fields_kernel + sc_push_kernel", 2
     return name, 1
@@ -558,7 +560,8 @@ def run_ours(args):
 
     peak, src = measured_hbm()
     bpc = 2 * 19 * BYTES_PER_POP[args.storage] + EXTRA_BYTES_PER_CELL.get(args.storage, 0)
-    kname, n_kernels = step_kernels(args.storage, args.kernel, L_info, ncell)
+    kname, n_kernels = step_kernels(args.storage, args.kernel, L_info, ncell,
+                                    args.collision == "mrt" or args.tau == 1.0)
     rec = step_record()
     if args.storage == "f64" and rec and rec.get("fp64_flops_per_cell"):
         # FP64 is bound by the FP64 pipe: SMs x 2 FP64 lanes per clock

@@ -534,14 +534,16 @@ long long busiest_block_planes(long long nz, long long tiles, long long grid, lo
 
 // Largest box that 32- and 16-bit storage steps in two kernels, measured on
 // GB300 (us a step, marching kernel / two kernels, single steps):
-//   FP32, SRT tau = 0.83: 223 k cells 20.6 / 9.1, 800 k 32.9 / 30.8, 1.0 M 47.2 / 41.1, 1.79 M 67.6 / 78.2
+//   FP32, SRT tau = 0.83: 223 k cells 20.6 / 9.1, 518 k 24.8 / 20.6, 1.0 M 47.2 / 41.1, 1.79 M 67.6 / 78.2; but
+//     64 x 64 x 180 (737 k), whose tiles fill the blocks evenly, 26 / 30
 //   FP32 in place (tau = 1): 223 k 20.7 / 9.0, 1.0 M 47.2 / 32.9, 1.79 M 67.5 / 68.7, 2.46 M 82.3 / 89.2
 //   FP16 from one reference: 223 k 24.2 / 8.9, 1.0 M 43.3 / 32.3, 1.79 M 64.4 / 60.4, 2.46 M 72.3 / 86.3
-//   FP16 from local references: 223 k 14.4 / 9.9, 1.0 M 45.1 / 35.8, 1.79 M 65.7 / 70.5
+//   FP16 from local references: 223 k 14.4 / 9.9, 518 k 25.2 / 22.6, 800 k 30.9 / 30.8, 1.79 M 65.7 / 70.5
 //   odd rows (no pipelined kernel): FP16 1.08 M 48.7 / 35.0, 19.6 M 738 / 583
-long long split_cells(const lbm_params& p) {
+long long split_cells(const lbm_params& p, bool in_place) {
     if (p.storage >= LBM_F16_DEV && p.nx % 2 != 0) return 1LL << 40;
-    return p.storage == LBM_F16_DEV || p.storage == LBM_BF16_DEV ? 2000000 : 1200000;
+    if (p.storage == LBM_F32) return in_place ? 1200000 : 400000;
+    return p.storage >= LBM_F16_LOCAL ? 250000 : 2000000;
 }
 
 constexpr long long kSplitPad = 1024;  // block rounding of the two-kernel step's 32-bit cell index
@@ -1129,7 +1131,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     // Steps in two kernels, unless one particular kernel was asked for: FP64, small boxes, odd 16-bit rows
     const bool in_place = p->storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p->tau != 1.0);
     c->split = p->kernel == 0 && p->G2 == 0.0 && n <= 0xffffffffLL - kSplitPad &&
-               (p->storage == LBM_F64 || n <= split_cells(*p));
+               (p->storage == LBM_F64 || n <= split_cells(*p, in_place));
     c->split_in_place = c->split && in_place;
     if (p->G2 != 0.0 || (c->split && !c->split_in_place)) {
         // psi of the whole box; where there is no room the step runs without it, slower
