@@ -143,7 +143,8 @@ __device__ __forceinline__ V vfmac(S c, V a, T b) {  // b a number, too
 // Below the range of normal results, and for NaN and infinities, exp itself is
 // called.
 // Worst error over 500 k arguments in [-4.6, 0]: 0.52 ulp (exp: 0.86; with entries
-// of one double and the plain series 1.25, for one operation less).
+// of one double and the plain series 1.25, two operations fewer a step: 14.51
+// against 14.77 ms for 10 steps of 128 x 128 x 288, the division below included).
 __device__ const double2 kExp2Table[64] = {
     {0x1.0000000000000p+0, 0x0.0p+0}, {0x1.02c9a3e778061p+0, -0x1.19083535b085dp-56},
     {0x1.059b0d3158574p+0, 0x1.d73e2a475b465p-55}, {0x1.0874518759bc8p+0, 0x1.186be4bb284ffp-57},
@@ -208,21 +209,14 @@ __device__ __forceinline__ float psi_of<float>(float rho, float rho0, float inv_
     return __fmul_rn(rho0, __fsub_rn(1.0f, e));
 }
 
-// 1/rho.  FP64: from the hardware's 20-bit approximation y by one third-order
-// step of Householder's iteration, y (1 + e + e^2) with e = 1 - rho y (e^3 is
-// below the rounding), 3 FP64 operations; 0, infinities and subnormals take
-// the division.  Float arithmetic uses the hardware reciprocal (within 1 ulp) instead
-// of the IEEE division, whose special-case check adds a branch per cell.
+// 1/rho.  FP64 divides.  Float arithmetic uses the hardware reciprocal (within 1
+// ulp) instead of the IEEE division, whose special-case check adds a branch per
+// cell.
 template <class R>
 __device__ __forceinline__ R recip(R x);
 template <>
 __device__ __forceinline__ double recip<double>(double x) {
-    const unsigned expo = (unsigned(__double2hiint(x)) >> 20) & 2047u;
-    if (expo - 64u > 1900u) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-x, y, 1.0);
-    return __fma_rn(__fma_rn(e, e, e), y, y);
+    return 1.0 / x;
 }
 template <>
 __device__ __forceinline__ float recip<float>(float x) {

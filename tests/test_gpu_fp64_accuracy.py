@@ -1,10 +1,11 @@
-"""The FP64 exponential of the step (csrc/collide.cuh) against
+"""The FP64 exponential and reciprocal of the step (csrc/collide.cuh) against
 64-bit-mantissa (or wider) values, argument by argument: a small program that
-calls the device function, compiled here.
+calls the two device functions, compiled here.
 
 The exponential's last operation is one rounded sum of a table entry and a
 term below 0.011, whose own roundings, the polynomial's and the tables' second
-words add less than 0.03 ulp: 0.55 ulp.  It may not be worse than exp either."""
+words add less than 0.03 ulp: 0.55 ulp.  It may not be worse than exp either.
+The reciprocal has the bits of the division."""
 
 import ctypes
 import os
@@ -24,14 +25,16 @@ from paper_1905_09554_gb300 import build  # noqa: E402
 
 SOURCE = r"""
 #include "collide.cuh"
-__global__ void values(const double* a, double* out, int n) {
+__global__ void values(const double* a, const double* x, double* out, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     out[i] = lbm::exp_table(a[i]);
     out[n + i] = exp(a[i]);
+    out[2 * n + i] = lbm::recip<double>(x[i]);
+    out[3 * n + i] = 1.0 / x[i];
 }
-extern "C" int run(const double* a, double* out, int n) {
-    values<<<(n + 255) / 256, 256>>>(a, out, n);
+extern "C" int run(const double* a, const double* x, double* out, int n) {
+    values<<<(n + 255) / 256, 256>>>(a, x, out, n);
     return cudaDeviceSynchronize();
 }
 """
@@ -50,13 +53,13 @@ def values(tmp_path_factory):
                     str(d / "values.cu")], check=True)
     run = ctypes.CDLL(lib).run
 
-    def call(a):
+    def call(a, x):
         n = len(a)
-        ta = torch.tensor(a, dtype=torch.float64, device="cuda")
-        out = torch.empty(2 * n, dtype=torch.float64, device="cuda")
+        ta, tx = (torch.tensor(v, dtype=torch.float64, device="cuda") for v in (a, x))
+        out = torch.empty(4 * n, dtype=torch.float64, device="cuda")
         torch.cuda.synchronize()
-        assert run(*(ctypes.c_void_p(t.data_ptr()) for t in (ta, out)), n) == 0
-        return out.cpu().numpy().reshape(2, n)
+        assert run(*(ctypes.c_void_p(t.data_ptr()) for t in (ta, tx, out)), n) == 0
+        return out.cpu().numpy().reshape(4, n)
 
     return call
 
@@ -73,7 +76,7 @@ def test_exponential_rounds_as_well_as_exp(values):
     a = np.concatenate([-4.6 * rng.random(n), 1380.0 * rng.random(n) - 690.0,
                         (k + 0.5) * np.log(2.0) / 64 * (1 + 1e-12 * rng.standard_normal(n)),
                         k * np.log(2.0) / 64 - 1e-9 * rng.random(n)])
-    got, ref = values(a)
+    got, ref = values(a, np.ones_like(a))[:2]
     want = np.exp(a.astype(np.longdouble))
     assert _ulps(got, want).max() <= 0.55
     assert _ulps(got, want).max() <= _ulps(ref, want).max()
@@ -82,8 +85,17 @@ def test_exponential_rounds_as_well_as_exp(values):
 def test_ends_of_the_exponentials_fast_range(values):
     a = np.array([0.0, -0.0, -699.9999, -700.0, -700.0001, -745.2, -1e5, 699.9999, 700.0, 709.0, 1e4, np.inf, -np.inf,
                   np.nan])
-    got, ref = values(a)
+    got, ref = values(a, np.ones_like(a))[:2]
     with np.errstate(over="ignore", under="ignore"):
         near = np.nextafter(ref, np.inf), ref, np.nextafter(ref, -np.inf)
     assert all(any(np.array_equal([g], [v], equal_nan=True) for v in row) for g, row in zip(got, zip(*near)))
 
+
+def test_reciprocal_has_the_bits_of_the_division(values):
+    rng = np.random.default_rng(6)
+    n = 1 << 17
+    x = np.concatenate([0.02 + 3.0 * rng.random(n), np.ldexp(1.0 + rng.random(n), rng.integers(-300, 300, n)),
+                        [0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, 1e-310, 2.0 ** -1022, 1.7976931348623157e308, 1.0,
+                         -3.0, 2.0 - 2.0 ** -52, 1.0 + 2.0 ** -52, -1e-300]])
+    inv, div = values(np.zeros_like(x), x)[2:]
+    assert np.array_equal(inv, div, equal_nan=True)
