@@ -19,6 +19,12 @@
 // Parameter gradients are summed in float64 per block and reduced in a fixed
 // order (deterministic).
 //
+// psi and 1/rho are the step's own functions (psi_of, recip), also where FP32
+// takes the hardware's approximations: psi of a state that no step recomputed is
+// then the same wherever the checkpoints lie, and the equilibrium is the one the
+// step took.  With expf and the division the error of the three gradients of
+// 64 x 64 x 180, 500 steps, grew from 4.3e-6 to 4.7e-6 (and 38.0 to 39.1 ms).
+//
 // At tau = 1 the collision forgets the populations, so their adjoint is
 // lam_a(y) = A(y) + c_a.B(y): four values a cell instead of 20 (lam and gr).
 // adj_collide1_kernel and adj_force_kernel then keep {A, B} as one 16- or
