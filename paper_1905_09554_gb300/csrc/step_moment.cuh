@@ -496,48 +496,55 @@ sc_moment_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, c
 }
 
 // Populations -> moment fields (all the operators above read of a state).
-// One thread per cell along x rows; blockIdx.y: the box of a batch.
+// One thread per cell along x rows; of a batch, blockIdx.y takes every
+// gridDim.y-th box (a grid has at most 65,535 rows of blocks, a batch has no
+// such limit).
+constexpr int kMomentGatherRows = 65535;
+
 template <class Codec, int COLL, bool BATCH>
 __global__ void __launch_bounds__(256)
 sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
     using S = typename Codec::S;
     constexpr int NF = kMoments<COLL>;
     chain_begin();
-    int nx = a.nx, ny = a.ny, nz = a.nz;
-    long long base = 0;
-    if constexpr (BATCH) {
-        const BatchBox& bx = b.boxes[blockIdx.y];
-        nx = bx.nx; ny = bx.ny; nz = bx.nz;
-        base = bx.base;
-    }
-    const long long n = (long long)nx * ny * nz;
-    const int pitch = moment_pitch(nx);
-    const unsigned rows = unsigned(ny) * unsigned(nz);
-    const long long nf = (long long)pitch * rows;
-    const S* __restrict__ src = static_cast<const S*>(src_all) + base;
-    float* dst = static_cast<float*>(dst_all) + base;
     const DevParams& dev = a.dev;
-    for (unsigned r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
-        for (int x = threadIdx.x & 31; x < nx; x += 32) {
-            const long long cell = (long long)r * nx + x;
-            float f[Q], m[NF];
-            float ref = 0.0f;
-            if constexpr (Codec::kLocal) ref = __ldg(a.ref_src + cell);
-            static_for<0, Q>([&](auto qc) {
-                constexpr int q = decltype(qc)::value;
-                const S* p = src + (q * n + cell);
-                if constexpr (Codec::kLocal) f[q] = Codec::template load_ref<q>(p, ref, dev);
-                else f[q] = Codec::template load<q>(p, dev);
-            });
-            moments_of<COLL, float>(f, m);
-            const unsigned row = r * unsigned(pitch);
-            const int g = x < 2 ? nx : (x >= nx - 2 ? -nx : 0);
-            static_for<0, NF>([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                *moment_at<NF>(dst, nf, row, x + 2, k) = m[k];
-                if (g) *moment_at<NF>(dst, nf, row, x + 2 + g, k) = m[k];
-            });
+    auto gather = [&](int nx, int ny, int nz, long long base) {
+        const long long n = (long long)nx * ny * nz;
+        const int pitch = moment_pitch(nx);
+        const unsigned rows = unsigned(ny) * unsigned(nz);
+        const long long nf = (long long)pitch * rows;
+        const S* __restrict__ src = static_cast<const S*>(src_all) + base;
+        float* dst = static_cast<float*>(dst_all) + base;
+        for (unsigned r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
+            for (int x = threadIdx.x & 31; x < nx; x += 32) {
+                const long long cell = (long long)r * nx + x;
+                float f[Q], m[NF];
+                float ref = 0.0f;
+                if constexpr (Codec::kLocal) ref = __ldg(a.ref_src + cell);
+                static_for<0, Q>([&](auto qc) {
+                    constexpr int q = decltype(qc)::value;
+                    const S* p = src + (q * n + cell);
+                    if constexpr (Codec::kLocal) f[q] = Codec::template load_ref<q>(p, ref, dev);
+                    else f[q] = Codec::template load<q>(p, dev);
+                });
+                moments_of<COLL, float>(f, m);
+                const unsigned row = r * unsigned(pitch);
+                const int g = x < 2 ? nx : (x >= nx - 2 ? -nx : 0);
+                static_for<0, NF>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    *moment_at<NF>(dst, nf, row, x + 2, k) = m[k];
+                    if (g) *moment_at<NF>(dst, nf, row, x + 2 + g, k) = m[k];
+                });
+            }
         }
+    };
+    if constexpr (BATCH) {
+        for (int i = int(blockIdx.y); i < b.nbox; i += int(gridDim.y)) {
+            const BatchBox& bx = b.boxes[i];
+            gather(bx.nx, bx.ny, bx.nz, bx.base);
+        }
+    } else {
+        gather(a.nx, a.ny, a.nz, 0);
     }
 }
 
@@ -573,8 +580,9 @@ template <class Codec, int COLL>
 cudaError_t moment_gather(const MomentLaunch& l, const void* src, void* dst) {
     if constexpr (sizeof(typename Codec::S) == 4) {
         if (l.batch.nbox)
-            return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, true>, dim3(l.gather_grid, l.batch.nbox), 256, 0,
-                                  l.stream, src, dst, l.args, l.batch);
+            return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, true>,
+                                  dim3(l.gather_grid, l.batch.nbox < kMomentGatherRows ? l.batch.nbox : kMomentGatherRows),
+                                  256, 0, l.stream, src, dst, l.args, l.batch);
     }
     return launch_chained(moment_chain(l), sc_moments_kernel<Codec, COLL, false>, l.gather_grid, 256, 0, l.stream, src, dst, l.args,
                           l.batch);
