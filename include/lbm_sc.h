@@ -58,6 +58,11 @@ enum { LBM_F64 = 0,                            /* populations stored as double  
                                                   reference density, float arithmetic */
        LBM_BF16_LOCAL = 5 };                   /* bf16 deviations from a per-cell
                                                   reference density, float arithmetic */
+/* How a call steps (lbm_step, lbm_set_step_forms); every form gives the same bits. */
+enum { LBM_FORM_AUTO = 0,
+       LBM_FORM_ONE_KERNEL = 1,                /* the kernel and launch shape of lbm_kernel_config */
+       LBM_FORM_TWO_KERNELS = 2,               /* psi (and moments) first, then collision and push */
+       LBM_FORM_MOMENTS = 3 };                 /* calls of n >= 2: moments between the steps      */
 
 typedef struct {
     int lattice;          /* LBM_D3Q19                                              */
@@ -97,6 +102,9 @@ typedef struct {
                              allocates (and frees them in lbm_destroy).  A step
                              may overwrite both: only the current copy
                              (lbm_current_copy) holds a state.                      */
+                          /* zchunk, tile_y, kernel: any of them given makes every
+                             call step by the one kernel of that shape; with all
+                             three 0 lbm_step chooses its form too                  */
     int zchunk;           /* step kernel: z planes per work item; 0 = auto (the
                              length that loads the blocks most evenly, at most
                              96, and at most 24 MiB of one population's planes;
@@ -108,10 +116,7 @@ typedef struct {
     int kernel;           /* step kernel variant: 0 = auto (3 for FP32 and the
                              local-reference formats, 7 for the global-reference
                              16-bit formats, when nx is even for 16-bit storage;
-                             else 1; lbm_step then also uses the forms described
-                             there: two kernels a step, or moments between the
-                             steps of one call); any other value = that kernel
-                             for every step,
+                             else 1); any other value = that kernel,
                              1 = register-staged,
                              2 = cp.async-staged persistent, 3 = pipelined
                              persistent (2: FP64/FP32 storage; 3: also the
@@ -191,17 +196,28 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int on_device);
  * (Eq. barycentric), then periodic streaming.
  *
  * Enqueues the kernels of n steps and returns.  n steps in one call give the
- * same bits as n calls of one step, in the same population copy.  With
- * lbm_params.kernel = 0 and 32- or 16-bit storage, a call of n >= 2 steps of
- * an operator whose result follows from a few moments (SRT at tau = 1; MRT
+ * same bits as n calls of one step, in the same population copy.  Unless a
+ * kernel or a launch shape was asked for, and with 32- or 16-bit storage, a
+ * call of n >= 2 steps of an operator whose result follows from a few moments (SRT at tau = 1; MRT
  * with every rate 1; FP32 MRT with its rates at 1 outside e, 3pxx, pww and the
  * off-diagonal stress) reads the populations once, keeps 4, 9 or 10 moments
  * between the steps (in the two copies themselves) and writes the populations
  * at the end: ask for many steps at once where nothing is read in between.
  * FP64, small boxes and 16-bit storage with nx odd step in two kernels, with a
  * psi field of n cells of their own where the moments do not suffice; if it
- * cannot be allocated, in one. */
+ * cannot be allocated, in one.  lbm_step_form tells which form a call takes. */
 lbm_status lbm_step(lbm_ctx *ctx, long n);
+
+/* The form (LBM_FORM_*, never LBM_FORM_AUTO) that lbm_step(ctx, n) takes; 0 for
+ * a NULL context or n < 1. */
+int lbm_step_form(const lbm_ctx *ctx, long n);
+
+/* Choose the forms of later calls: single for n = 1 (LBM_FORM_AUTO,
+ * LBM_FORM_ONE_KERNEL or LBM_FORM_TWO_KERNELS), several for n >= 2 (any).  May
+ * allocate what a form needs.  LBM_EINVAL for an unknown form or a box of a
+ * batch, LBM_EUNSUPPORTED for a form that cannot serve this lattice (or has no
+ * room); the forms are then unchanged. */
+lbm_status lbm_set_step_forms(lbm_ctx *ctx, int single, int several);
 
 /* Steps taken since the last initialisation. */
 long lbm_time(const lbm_ctx *ctx);
@@ -277,8 +293,9 @@ long long lbm_device_bytes(const lbm_ctx *ctx);
 /* Launch configuration the context chose for the step kernel: variant
  * (1 register-staged, 2 cp.async-staged, 3 pipelined, 4 bulk-copy, 5 tensor
  * copy, 6 two-belt force, 7 paired 16-bit), tile height, z planes per work
- * item and grid size (blocks).  The two-kernel and the moment form of lbm_step
- * have shapes of their own, which are not reported.  Any pointer may be NULL. */
+ * item and grid size (blocks).  It is what steps when lbm_step_form gives
+ * LBM_FORM_ONE_KERNEL; the other forms have shapes of their own, which are not
+ * reported.  Any pointer may be NULL. */
 lbm_status lbm_kernel_config(const lbm_ctx *ctx, int *kernel, int *tile_y,
                              int *zchunk, int *grid);
 
@@ -287,7 +304,8 @@ long long lbm_params_sizeof(void);
 
 /* Change the step kernel's launch shape: variant, tile height and z planes
  * per work item (0 = automatic for each), with the same rules as the
- * lbm_params fields of those names.  Returns LBM_EINVAL (launch shape
+ * lbm_params fields of those names: later calls step by that kernel, or, with
+ * all three 0, in the forms that lbm_step chooses.  Returns LBM_EINVAL (launch shape
  * unchanged) for a shape that cannot serve this lattice, LBM_ECUDA if it
  * cannot be configured on this device.  Not for a box of a batch. */
 lbm_status lbm_set_kernel_config(lbm_ctx *ctx, int kernel, int tile_y,

@@ -53,16 +53,20 @@ struct lbm_ctx {
     int grid3 = 0;                    // kernel 5: grid of the pipelined kernel used for other buffers
     int coll = COLL_SRT;              // collision kernel (COLL_*)
     int grid = 0;                     // persistent grid size (kernels 2, 3)
+    // How a call of one step, and one of several, steps (LBM_FORM_*).
+    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};
     // Calls of several steps through the moment fields (step_moment.cuh):
-    // launch shape, or mom == nullptr where only populations will do.
+    // launch shape, or mom == nullptr where that is not set up or only
+    // populations will do.
     const MomentKernels* mom = nullptr;
     MomentLaunch mom_launch{};
     void* mom_plan = nullptr;         // device memory of its plan
+    long long mom_busiest = 0;        // planes of its busiest block
     size_t mom_bytes = 0;             // one set of moment fields
     bool mom_twice = false;           // two sets fit into one population copy
-    // Steps in two kernels (step_split.cuh); in place where the moments are all
-    // a collision needs of the populations it overwrites.
-    bool split = false, split_in_place = false;
+    // Steps in two kernels (step_split.cuh) go in place where the moments are
+    // all a collision needs of the populations it overwrites.
+    bool split_in_place = false;
     char err[512] = {0};
     lbm_batch* batch = nullptr;       // set when the context is a view of a batch box
     // discrete adjoint (allocated by lbm_adjoint_forward)
@@ -409,11 +413,12 @@ cudaError_t launch_step(const lbm_ctx* c, const void* src, void* dst, void* psi_
     return step_kernels(c->p.storage, c->coll).launch(l, src, dst);
 }
 
-// One step src -> dst by the context's way of stepping.  keep_src: src is not
+// One step src -> dst in one or two kernels.  keep_src: src is not
 // one of the context's own copies (a checkpoint, a recomputed state) and stays
 // as it is; psi_out then receives its psi where the step computes it.
-cudaError_t step_once(const lbm_ctx* c, void* src, void* dst, bool keep_src = false, void* psi_out = nullptr) {
-    if (!c->split) return launch_step(c, src, dst, psi_out);
+cudaError_t step_once(const lbm_ctx* c, int form, void* src, void* dst, bool keep_src = false,
+                      void* psi_out = nullptr) {
+    if (form != LBM_FORM_TWO_KERNELS) return launch_step(c, src, dst, psi_out);
     void* psi = psi_out ? psi_out : c->psi_ws;
     if (!keep_src && c->split_in_place) psi = nullptr;
     SplitLaunch l{c->args, BatchArgs{}, unsigned(c->n), c->stream};
@@ -547,6 +552,19 @@ long long split_cells(const lbm_params& p, bool in_place) {
 }
 
 constexpr long long kSplitPad = 1024;  // block rounding of the two-kernel step's 32-bit cell index
+
+// The field that psi of the whole box goes through, where the step needs one; false without room.
+bool alloc_psi(lbm_ctx* c) {
+    if (c->psi_ws) return true;
+    const size_t bytes = (size_t)c->n * (c->p.storage == LBM_F64 ? 8 : 4);
+    if (cudaMalloc(&c->psi_ws, bytes) != cudaSuccess) {
+        c->psi_ws = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    c->own_bytes += (long long)bytes;
+    return true;
+}
 
 int auto_zchunk(const lbm_ctx* c) {
     const long long xy_blocks = (long long)((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y);
@@ -720,9 +738,6 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
     return LBM_OK;
 }
 
-// Launch shape of the moment kernels (step_moment.cuh), where the collision
-// has a moment form and its fields fit into a population copy.  A context
-// created for one particular step kernel keeps to it.
 // The moment kernel's work is laid out once: the pieces (planes of a tile of a
 // box) that each block goes through, in turn.  A piece costs its planes and
 // about 4 more.  Two ways:
@@ -862,44 +877,74 @@ cudaError_t upload_plan(const MomentPlan& plan, MomentLaunch& l, void** mem, siz
     return e;
 }
 
-void configure_moments(lbm_ctx* c) {
+// Sets up the two-kernel step; false where it cannot serve (the two-belt force,
+// too many cells for its 32-bit index, no room for its psi field).
+bool prepare_split(lbm_ctx* c) {
     const lbm_params& p = c->p;
-    c->mom = nullptr;
-    if (p.kernel != 0 || p.G2 != 0.0 || p.nx < 4) return;
-    if (c->coll == COLL_SRT && p.tau != 1.0) return;  // keeps (1 - omega) f: all 19 populations
+    if (p.G2 != 0.0 || c->n > 0xffffffffLL - kSplitPad) return false;
+    c->split_in_place = p.storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p.tau != 1.0);
+    return c->split_in_place || alloc_psi(c);
+}
+
+// Launch shape of the moment kernels (step_moment.cuh), where the collision
+// has a moment form and its fields fit into a population copy; false elsewhere,
+// and (rival: the box can step in two kernels) where two kernels are expected to
+// be faster: a turn of the moment kernel (one plane of the busiest block) takes
+// about 1.5 us however few blocks there are, two kernels 29 ps a cell and 4 us at
+// least (24x24x48: 10.4 / 4.2 us a step; 64x64x128: 14.7 / 20.5; MRT with the
+// paper's rates 48x48x96: 20.9 / 10.9, 80x80x160: 52.4 / 41.1, 96x96x192: 55.6 / 77).
+bool prepare_moments(lbm_ctx* c, bool rival) {
+    auto slower = [&](long long busiest) {
+        return rival && 2.5 + 1.5 * double(busiest) > 4.0 + 29e-6 * double(c->n);
+    };
+    if (c->mom) return !slower(c->mom_busiest);
+    const lbm_params& p = c->p;
+    if (p.G2 != 0.0 || p.nx < 4) return false;
+    if (c->coll == COLL_SRT && p.tau != 1.0) return false;  // keeps (1 - omega) f: all 19 populations
     const MomentKernels* k = moment_kernels(p.storage, c->coll);
-    if (!k) return;
+    if (!k) return false;
     const long long cells = moment_cells(p.nx, p.ny, p.nz);
     c->mom_bytes = (size_t)k->fields * (size_t)cells * sizeof(float);
     const size_t copy = (size_t)Q * (size_t)c->n * c->elem;
-    if (cells > 0xffffffffLL || c->mom_bytes > copy) return;
+    if (cells > 0xffffffffLL || c->mom_bytes > copy) return false;
     c->mom_twice = 2 * c->mom_bytes <= copy;
     MomentLaunch& l = c->mom_launch;
     l = MomentLaunch{};
     const int per_sm = k->prepare(false);
     if (per_sm < 1) {
         cudaGetLastError();
-        return;
+        return false;
     }
     l.args = c->args;
     l.args.tiles_x = (p.nx + k->tile_x - 1) / k->tile_x;
     const int tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
     const MomentPlan plan = plan_moments({{tiles, p.nz}}, (long long)per_sm * c->num_sms, k->fields, c->mom_bytes);
-    // Small boxes: a turn of the moment kernel (one plane of the busiest block) takes about 1.5 us however few
-    // blocks there are, two kernels 29 ps a cell and 4 us at least (24x24x48: 10.4 / 4.2 us a step; 64x64x128: 14.7
-    // / 20.5; MRT with the paper's rates 48x48x96: 20.9 / 10.9, 80x80x160: 52.4 / 41.1, 96x96x192: 55.6 / 77).
-    if (c->split && 2.5 + 1.5 * double(plan.busiest) > 4.0 + 29e-6 * double(c->n)) return;
+    if (slower(plan.busiest)) return false;
+    c->mom_busiest = plan.busiest;
     size_t bytes = 0;
     if (upload_plan(plan, l, &c->mom_plan, &bytes, c->stream) != cudaSuccess) {  // no room: step the populations
         cudaGetLastError();
         cudaFree(c->mom_plan);
         c->mom_plan = nullptr;
-        return;
+        return false;
     }
     c->own_bytes += (long long)bytes;
     const long long rows = ((long long)p.ny * p.nz + 7) / 8;
     l.gather_grid = int(rows < 8LL * c->num_sms ? rows : 8LL * c->num_sms);
     c->mom = k;
+    return true;
+}
+
+// The forms of a context for which no particular kernel or launch shape was
+// asked.
+void choose_forms(lbm_ctx* c, int (&form)[2]) {
+    const lbm_params& p = c->p;
+    form[0] = form[1] = LBM_FORM_ONE_KERNEL;
+    if (p.G2 != 0.0) return;
+    const bool in_place = p.storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p.tau != 1.0);
+    if ((p.storage == LBM_F64 || c->n <= split_cells(p, in_place)) && prepare_split(c))
+        form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+    if (prepare_moments(c, form[1] == LBM_FORM_TWO_KERNELS)) form[1] = LBM_FORM_MOMENTS;
 }
 
 // n >= 2 steps from the populations in f[from] through the moment fields.  The
@@ -938,11 +983,16 @@ cudaError_t run_moments(const MomentKernels& k, MomentLaunch l, void* const (&f)
     return e == cudaSuccess ? k.emit(l, at, f[*to]) : e;
 }
 
-lbm_status step_moments(lbm_ctx* c, long nsteps) {
+MomentLaunch moment_launch_of(const lbm_ctx* c, long nsteps) {
     MomentLaunch l = c->mom_launch;
     l.stream = c->stream;
     l.args.ref_src = c->ref[c->cur];
     l.args.ref_dst = c->ref[c->cur ^ int(nsteps & 1)];
+    return l;
+}
+
+lbm_status step_moments(lbm_ctx* c, long nsteps) {
+    MomentLaunch l = moment_launch_of(c, nsteps);
     int to = 0;
     LBM_CUDA(c, run_moments(*c->mom, l, c->f, c->cur, nsteps, c->mom_bytes, c->mom_twice, &to));
     c->cur = to;
@@ -1128,23 +1178,8 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     round_params(a);
     c->coll = collision_kernel(*p, a.s);
-    // Steps in two kernels, unless one particular kernel was asked for: FP64, small boxes, odd 16-bit rows
-    const bool in_place = p->storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p->tau != 1.0);
-    c->split = p->kernel == 0 && p->G2 == 0.0 && n <= 0xffffffffLL - kSplitPad &&
-               (p->storage == LBM_F64 || n <= split_cells(*p, in_place));
-    c->split_in_place = c->split && in_place;
-    if (p->G2 != 0.0 || (c->split && !c->split_in_place)) {
-        // psi of the whole box; where there is no room the step runs without it, slower
-        const size_t pbytes = (size_t)n * (p->storage == LBM_F64 ? 8 : 4);
-        if (cudaMalloc(&c->psi_ws, pbytes) == cudaSuccess) {
-            c->own_bytes += (long long)pbytes;
-        } else {
-            c->psi_ws = nullptr;
-            cudaGetLastError();
-        }
-        if (p->G2 != 0.0) a.psi_ws = c->psi_ws;
-        else c->split = c->psi_ws != nullptr;
-    }
+    // two-belt force: where there is no room for psi of the whole box the step runs without it, slower
+    if (p->G2 != 0.0 && alloc_psi(c)) a.psi_ws = c->psi_ws;
     a.err = c->dev_err;
     a.test_stall = p->test_stall ? 1 : 0;
     a.dev = make_dev_params(p->rho_ref, p->dev_scale);
@@ -1157,7 +1192,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
         }
     }
 
-    configure_moments(c);
+    if (p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) choose_forms(c, c->form);
 
     e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1244,6 +1279,29 @@ lbm_status lbm_set_kernel_config(lbm_ctx* c, int kernel, int tile_y, int zchunk)
         configure_step(c, k0, t0, z0, ignored, sizeof(ignored));  // the previous shape worked
         return c->fail(st, "lbm_set_kernel_config: %s", why);
     }
+    // a kernel or shape that was asked for is the one that steps
+    if (kernel || tile_y || zchunk) c->form[0] = c->form[1] = LBM_FORM_ONE_KERNEL;
+    else choose_forms(c, c->form);
+    return LBM_OK;
+}
+
+int lbm_step_form(const lbm_ctx* c, long n) { return c && n >= 1 ? c->form[n >= 2] : 0; }
+
+lbm_status lbm_set_step_forms(lbm_ctx* c, int single, int several) {
+    if (!c) return LBM_EINVAL;
+    if (c->batch) return c->fail(LBM_EINVAL, "lbm_set_step_forms: this context is a box of a batch");
+    if (single < LBM_FORM_AUTO || single > LBM_FORM_TWO_KERNELS || several < LBM_FORM_AUTO || several > LBM_FORM_MOMENTS)
+        return c->fail(LBM_EINVAL, "lbm_set_step_forms: unknown form (%d, %d)", single, several);
+    int form[2];
+    choose_forms(c, form);
+    if (single != LBM_FORM_AUTO) form[0] = single;
+    if (several != LBM_FORM_AUTO) form[1] = several;
+    if ((form[0] == LBM_FORM_TWO_KERNELS || form[1] == LBM_FORM_TWO_KERNELS) && !prepare_split(c))
+        return c->fail(LBM_EUNSUPPORTED, "lbm_set_step_forms: this lattice cannot step in two kernels");
+    if (form[1] == LBM_FORM_MOMENTS && !prepare_moments(c, false))
+        return c->fail(LBM_EUNSUPPORTED, "lbm_set_step_forms: this lattice cannot step through moment fields");
+    c->form[0] = form[0];
+    c->form[1] = form[1];
     return LBM_OK;
 }
 
@@ -1442,9 +1500,10 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (!c) return LBM_EINVAL;
     if (nsteps < 0) return c->fail(LBM_EINVAL, "lbm_step: n must be >= 0");
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_step: this context is a box of a batch; use lbm_batch_step");
-    if (nsteps >= 2 && c->mom) return step_moments(c, nsteps);
+    const int form = c->form[nsteps >= 2];
+    if (form == LBM_FORM_MOMENTS) return step_moments(c, nsteps);
     for (long k = 0; k < nsteps; ++k) {
-        cudaError_t e = step_once(c, c->f[c->cur], c->f[c->cur ^ 1]);
+        cudaError_t e = step_once(c, form, c->f[c->cur], c->f[c->cur ^ 1]);
         if (e != cudaSuccess) return c->fail(LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));
         c->cur ^= 1;
         ++c->t;
@@ -2008,7 +2067,7 @@ lbm_status lbm_adjoint_forward(lbm_ctx* c, const double* rho0, int on_device, lo
     if (c->n > 0xffffffffLL) return c->fail(LBM_EUNSUPPORTED, "lbm_adjoint_forward: needs nx*ny*nz < 2^32");
     auto& A = c->adj;
     // tau = 1 in FP32: a state's four moments are all the adjoint needs of it
-    A.moments = c->mom && c->p.storage == LBM_F32 && c->p.tau == 1.0;
+    A.moments = c->form[1] == LBM_FORM_MOMENTS && c->p.storage == LBM_F32 && c->p.tau == 1.0;
     const size_t state = A.moments ? c->mom_bytes : (size_t)Q * (size_t)c->n * c->elem;
     A.T = -1;  // nothing recorded until the run is complete
     const int ncp = int((nsteps + every - 1) / every);
@@ -2091,7 +2150,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     // psi of every state of a segment: written by the step kernel during the
     // recomputation where it supports that (kernels 1 and 3, and 5 whose
     // recomputation runs kernel 3), else computed by the reverse step
-    const bool psi_fused = c->split || c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
+    const bool psi_fused = c->form[0] == LBM_FORM_TWO_KERNELS || c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
     const size_t psi_bytes = (size_t)c->n * c->elem;
     if (A.psi && A.psi_bytes < (size_t)A.every * psi_bytes) {
         cudaStreamSynchronize(c->stream);
@@ -2152,7 +2211,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
                                     cudaMemcpyDeviceToDevice, c->stream));
         char* psi = static_cast<char*>(A.psi);
         for (long t = t0; t + 1 < t1; ++t) {
-            cudaError_t e = step_once(c, seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state, true,
+            cudaError_t e = step_once(c, c->form[0], seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state, true,
                                       psi_fused ? psi + (size_t)(t - t0) * psi_bytes : nullptr);
             if (e != cudaSuccess) return c->fail(LBM_ECUDA, "adjoint recompute: %s", cudaGetErrorString(e));
         }

@@ -33,6 +33,8 @@ STORAGE = {"f64": LBM_F64, "f32": LBM_F32, "f16": LBM_F16_DEV, "bf16": LBM_BF16_
            "f16l": LBM_F16_LOCAL, "bf16l": LBM_BF16_LOCAL}
 STORAGE_BYTES = {LBM_F64: 8, LBM_F32: 4, LBM_F16_DEV: 2, LBM_BF16_DEV: 2, LBM_F16_LOCAL: 2, LBM_BF16_LOCAL: 2}
 COLLISION = {"srt": LBM_SRT_SHIFT, "mrt": LBM_MRT_GUO}
+LBM_FORM_AUTO, LBM_FORM_ONE_KERNEL, LBM_FORM_TWO_KERNELS, LBM_FORM_MOMENTS = 0, 1, 2, 3
+FORM_NAMES = ["auto", "one", "two", "moments"]  # by LBM_FORM_*
 
 
 class lbm_params(ctypes.Structure):
@@ -89,6 +91,8 @@ _SIGNATURES = {
     "lbm_kernel_config": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                          ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "lbm_set_kernel_config": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
+    "lbm_step_form": (ctypes.c_int, [_P, ctypes.c_long]),
+    "lbm_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
     "lbm_tune": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                 ctypes.POINTER(ctypes.c_int), _D]),
     "lbm_batch_create": (ctypes.c_int, [ctypes.POINTER(lbm_params), ctypes.c_int, ctypes.POINTER(ctypes.c_int),
@@ -306,6 +310,14 @@ def lbm_kernel_config(ctx):
 # ------------------------------------------------------------ object wrapper
 def lbm_set_kernel_config(ctx, kernel, tile_y, zchunk):
     return load().lbm_set_kernel_config(ctx, int(kernel), int(tile_y), int(zchunk))
+
+
+def lbm_step_form(ctx, n):
+    return load().lbm_step_form(ctx, int(n))
+
+
+def lbm_set_step_forms(ctx, single, several):
+    return load().lbm_set_step_forms(ctx, int(single), int(several))
 
 
 def lbm_tune(ctx, trial_steps):
@@ -551,6 +563,15 @@ class Lattice:
 
     def set_kernel_config(self, kernel=0, tile_y=0, zchunk=0):
         self._check(lbm_set_kernel_config(self.ctx, kernel, tile_y, zchunk))
+
+    def step_form(self, n=1):
+        """How step(n) steps: 'one', 'two' (kernels a step) or 'moments'
+        (lbm_step_form)."""
+        return FORM_NAMES[lbm_step_form(self.ctx, n)]
+
+    def set_step_forms(self, single="auto", several="auto"):
+        """Choose how step(1) and step(n >= 2) step (lbm_set_step_forms)."""
+        self._check(lbm_set_step_forms(self.ctx, FORM_NAMES.index(single), FORM_NAMES.index(several)))
 
     def tune(self, trial_steps=3, cache=None):
         """Pick the step's launch shape (kernel variant, tile height, z chunk)

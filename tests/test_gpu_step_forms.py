@@ -1,0 +1,76 @@
+"""The forms a call of lbm_step takes (one kernel, two kernels, moments between
+the steps): a kernel or launch shape that was asked for is the one that steps."""
+
+import numpy as np
+import pytest
+
+from paper_1905_09554_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - CUDA device only
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1905_09554_gb300 import lbm  # noqa: E402
+
+# (storage, box, tau, automatic forms of step(1) and step(n))
+CASES = [("f64", (33, 20, 12), 0.8, ("two", "two")), ("f64", (32, 32, 64), 1.0, ("two", "two")),
+         ("f32", (64, 40, 30), 0.8, ("two", "two")), ("f32", (64, 64, 144), 1.0, ("two", "moments")),
+         ("f32", (128, 128, 130), 1.0, ("one", "moments")), ("f32", (128, 128, 130), 0.8, ("one", "one")),
+         ("f16", (97, 85, 31), 0.9, ("two", "two")), ("f16l", (48, 36, 20), 0.8, ("two", "two"))]
+
+
+def _populations(L, rho, calls=(1, 4, 1)):
+    L.set_density(rho)
+    for n in calls:
+        L.step(n)
+    return L.get_populations()
+
+
+def _forms(L):
+    return L.step_form(1), L.step_form(5)
+
+
+@pytest.mark.parametrize("storage,box,tau,forms", CASES)
+def test_a_shape_that_was_asked_for_steps(storage, box, tau, forms):
+    rho = inputs.random_density(*box, seed=9, lo=0.3, hi=1.9)
+    kw = dict(storage=storage, tau=tau, G=-5.5)
+    with lbm.Lattice(*box, kernel=1, **kw) as L:
+        assert _forms(L) == ("one", "one")
+        want = _populations(L, rho)
+    with lbm.Lattice(*box, **kw) as L:
+        assert _forms(L) == forms
+        assert np.array_equal(_populations(L, rho), want)
+        kernel = L.kernel_config()["kernel"]
+        L.set_kernel_config(kernel, 8, 4)
+        assert _forms(L) == ("one", "one")
+        assert L.kernel_config()["tile_y"] == 8
+        assert np.array_equal(_populations(L, rho), want)
+        L.set_kernel_config()
+        assert _forms(L) == forms
+    for shape in (dict(tile_y=8), dict(zchunk=5)):
+        with lbm.Lattice(*box, **shape, **kw) as L:
+            assert _forms(L) == ("one", "one")
+            assert np.array_equal(_populations(L, rho), want)
+
+
+def test_forms_that_cannot_serve_are_refused():
+    with lbm.Lattice(16, 8, 8, tau=0.8, storage="f32") as L:
+        before = _forms(L)
+        with pytest.raises(lbm.LbmError, match="LBM_EUNSUPPORTED"):
+            L.set_step_forms("one", "moments")  # SRT off tau = 1 keeps all populations
+        assert lbm.lbm_set_step_forms(L.ctx, 3, 0) == lbm.LBM_EINVAL  # moments between the steps of one step
+        assert lbm.lbm_set_step_forms(L.ctx, 0, 4) == lbm.LBM_EINVAL
+        assert _forms(L) == before
+        assert lbm.lbm_step_form(L.ctx, 0) == 0
+    with lbm.Lattice(3, 8, 8, storage="f32") as L:
+        with pytest.raises(lbm.LbmError, match="LBM_EUNSUPPORTED"):
+            L.set_step_forms("auto", "moments")  # rows of fewer than 4 cells
+    with lbm.Lattice(16, 8, 8, G=-7.0, G2=1.5, storage="f32") as L:
+        assert _forms(L) == ("one", "one")
+        with pytest.raises(lbm.LbmError, match="LBM_EUNSUPPORTED"):
+            L.set_step_forms("two", "two")
+    with lbm.Batch([(8, 8, 8)], storage="f32") as B:
+        with pytest.raises(lbm.LbmError, match="LBM_EINVAL"):
+            B.boxes[0].set_step_forms("one", "one")
