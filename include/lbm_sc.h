@@ -320,9 +320,12 @@ lbm_status lbm_set_kernel_config(lbm_ctx *ctx, int kernel, int tile_y,
  * FP32), 7 (paired 16-bit words), each on 32x4, 32x8 and 32x16 tiles
  * (64-wide for kernel 7); kernel 6 on 32x8 / 32x16 when G2 != 0.  The trial
  * steps advance whatever state the context holds (its step counter does not
- * change): tune before setting the initial state.  Outputs (any may be NULL):
- * the chosen kernel, tile height, z chunk and its time per step in ms.
- * Returns LBM_ECUDA if no candidate ran. */
+ * change): tune before setting the initial state.  Then the two-kernel step
+ * (where lbm_step would choose it) is timed against the fastest shape, and the
+ * moment form (trial_steps steps a call, at least 8) against the faster of the
+ * two, and what is faster stays (lbm_step_form).  Outputs (any may be NULL):
+ * the chosen kernel, tile height and z chunk, and the time per step in ms of a
+ * call of one step.  Returns LBM_ECUDA if no candidate ran. */
 lbm_status lbm_tune(lbm_ctx *ctx, int trial_steps, int *kernel, int *tile_y,
                     int *zchunk, double *ms_per_step);
 

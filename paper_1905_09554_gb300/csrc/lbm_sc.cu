@@ -1356,6 +1356,41 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
             pick = sh;
         }
     }
+    // the other forms, as lbm_step runs them; fewer than 8 steps at once would time the moment form's ends
+    const int cur = c->cur;
+    auto timed = [&](int n, auto&& run) {
+        if (run(2) != cudaSuccess) return -1.0f;  // warm-up
+        cudaEventRecord(e0, c->stream);
+        const bool ok = run(n) == cudaSuccess;
+        cudaEventRecord(e1, c->stream);
+        if (!ok || cudaEventSynchronize(e1) != cudaSuccess) return -1.0f;
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        return ms / n;
+    };
+    int form[2], automatic[2];
+    form[0] = form[1] = LBM_FORM_ONE_KERNEL;
+    choose_forms(c, automatic);
+    if (automatic[0] == LBM_FORM_TWO_KERNELS) {
+        const float ms = timed(steps, [&](int n) {
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < n && e == cudaSuccess; ++k)
+                e = step_once(c, LBM_FORM_TWO_KERNELS, c->f[cur ^ (k & 1)], c->f[cur ^ (~k & 1)]);
+            return e;
+        });
+        if (ms >= 0.0f && (best < 0.0f || ms < best)) {
+            best = ms;
+            form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+        }
+    }
+    if (prepare_moments(c, false)) {
+        const float ms = timed(steps < 8 ? 8 : steps, [&](int n) {
+            MomentLaunch l = moment_launch_of(c, n);
+            int to = 0;
+            return run_moments(*c->mom, l, c->f, cur, n, c->mom_bytes, c->mom_twice, &to);
+        });
+        if (ms >= 0.0f && best >= 0.0f && ms < best) form[1] = LBM_FORM_MOMENTS;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaGetLastError();  // a shape that failed to launch is skipped, not an error
@@ -1367,6 +1402,8 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
         return c->fail(st, "lbm_tune: %s", why);
     }
     if (best < 0.0f) return c->fail(LBM_ECUDA, "lbm_tune: no launch shape ran");
+    c->form[0] = form[0];
+    c->form[1] = form[1];
     if (kernel) *kernel = c->kernel;
     if (tile_y) *tile_y = c->tile_y;
     if (zchunk) *zchunk = c->zchunk;

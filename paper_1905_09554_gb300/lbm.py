@@ -324,7 +324,8 @@ def lbm_tune(ctx, trial_steps):
     k, t, z = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     ms = ctypes.c_double()
     st = load().lbm_tune(ctx, int(trial_steps), ctypes.byref(k), ctypes.byref(t), ctypes.byref(z), ctypes.byref(ms))
-    return st, {"kernel": k.value, "tile_y": t.value, "zchunk": z.value, "ms_per_step": ms.value}
+    return st, {"kernel": k.value, "tile_y": t.value, "zchunk": z.value, "ms_per_step": ms.value,
+                "forms": [FORM_NAMES[lbm_step_form(ctx, n)] for n in (1, 2)]}
 
 
 def _host_ptr(a: np.ndarray):
@@ -579,7 +580,8 @@ class Lattice:
         setting the initial state, since the trial steps advance it.  With
         `cache` (a JSON file path) a pick stored for the same box, parameters
         and GPU model is applied without timing, and a new pick is stored.
-        Returns the pick (kernel, tile_y, zchunk, ms_per_step, cached)."""
+        Returns the pick (kernel, tile_y, zchunk, ms_per_step, the forms of
+        step(1) and step(n >= 2), cached)."""
         key = None
         if cache is not None:
             p = self.params
@@ -589,6 +591,9 @@ class Lattice:
             hit = _read_tune_cache(cache).get(key)
             if hit:
                 self.set_kernel_config(hit["kernel"], hit["tile_y"], hit["zchunk"])
+                # (no forms stored, or no room for them any more: one kernel a step)
+                if "forms" in hit:
+                    lbm_set_step_forms(self.ctx, *(FORM_NAMES.index(v) for v in hit["forms"]))
                 return dict(hit, cached=True)
         st, pick = lbm_tune(self.ctx, trial_steps)
         self._check(st)

@@ -1,5 +1,8 @@
 """The forms a call of lbm_step takes (one kernel, two kernels, moments between
-the steps): a kernel or launch shape that was asked for is the one that steps."""
+the steps): a kernel or launch shape that was asked for is the one that steps,
+the tuner times what steps and keeps the fastest, and its cache restores it."""
+
+import json
 
 import numpy as np
 import pytest
@@ -53,6 +56,38 @@ def test_a_shape_that_was_asked_for_steps(storage, box, tau, forms):
         with lbm.Lattice(*box, **shape, **kw) as L:
             assert _forms(L) == ("one", "one")
             assert np.array_equal(_populations(L, rho), want)
+
+
+@pytest.mark.parametrize("storage,box,tau,forms", CASES)
+def test_the_tuner_times_the_forms_and_its_cache_restores_them(storage, box, tau, forms, tmp_path):
+    rho = inputs.random_density(*box, seed=9, lo=0.3, hi=1.9)
+    kw = dict(storage=storage, tau=tau, G=-5.5)
+    path = str(tmp_path / "tune.json")
+    with lbm.Lattice(*box, kernel=1, **kw) as L:
+        want = _populations(L, rho)
+    with lbm.Lattice(*box, **kw) as L:
+        pick = L.tune(trial_steps=2, cache=path)
+        assert tuple(pick["forms"]) == _forms(L)
+        assert np.array_equal(_populations(L, rho), want)
+        L.set_step_forms("one", "one")  # the shape that was found fastest, whatever won
+        assert np.array_equal(_populations(L, rho), want)
+    with lbm.Lattice(*box, **kw) as L:
+        again = L.tune(trial_steps=2, cache=path)
+        assert again["cached"] and tuple(pick["forms"]) == _forms(L)
+    data = json.load(open(path))
+    for entry in data.values():  # as stored before there were forms
+        del entry["forms"]
+    json.dump(data, open(path, "w"))
+    with lbm.Lattice(*box, **kw) as L:
+        assert L.tune(trial_steps=2, cache=path)["cached"]
+        assert _forms(L) == ("one", "one")
+
+
+def test_the_tuner_finds_two_kernels_and_moments_where_they_are_several_times_faster():
+    with lbm.Lattice(32, 32, 64, storage="f64") as L:  # 8.1 against 1.1 ms per 50 steps
+        assert L.tune()["forms"] == ["two", "two"]
+    with lbm.Lattice(256, 256, 300, storage="f32") as L:  # 56 against 23 ms per 50 steps of twice the box
+        assert L.tune()["forms"] == ["one", "moments"]
 
 
 def test_forms_that_cannot_serve_are_refused():
