@@ -367,7 +367,8 @@ typedef struct lbm_batch lbm_batch;
 
 /* Create `count` boxes sharing the physics of *p (G, collision, tau, rates,
  * psi, storage: FP32 or FP64; p->nx/ny/nz are ignored; p->tile_y / zchunk
- * choose the initial launch shape, 0 = default).  dims[3*i + 0..2] are box
+ * choose the launch shape of the one-kernel step, 0 = default; any of kernel,
+ * tile_y and zchunk given makes every call step by that kernel).  dims[3*i + 0..2] are box
  * i's nx, ny, nz (each box needs 19 * cells < 2^31).  One allocation per
  * population copy holds every box (256-byte aligned per box).  If p->stream
  * is NULL the batch creates its own stream (needed to capture the step graph).
@@ -382,17 +383,26 @@ const char *lbm_batch_last_error(const lbm_batch *b);
  * it alone (lbm_step) returns LBM_EINVAL; lbm_destroy ignores it. */
 lbm_status lbm_batch_box(lbm_batch *b, int i, lbm_ctx **view);
 
-/* Advance every box n >= 0 steps with one kernel launch per step over the
- * work items (xy tile, z chunk) of all boxes.  FP32 operators whose result
- * follows from a few moments keep only those between the steps of a call
- * (lbm_step); otherwise pairs of steps are replayed from a captured CUDA
+/* Advance every box n >= 0 steps with the same launches for all boxes.  Unless
+ * a kernel or a launch shape was asked for, FP32 operators whose result
+ * follows from a few moments keep only those between the steps of a call and
+ * FP64 ones step in two kernels (lbm_step); steps of one kernel go over the
+ * work items (xy tile, z chunk) of all boxes.  Except in the moment form, pairs of steps are replayed from a captured CUDA
  * graph. */
 lbm_status lbm_batch_step(lbm_batch *b, long n);
 
-/* Autotune the launch shape: times trial_steps steps for each tile height in
- * {4, 8, 16} and z chunk in {8, 16, 24, 32, 48, 64}, keeps the fastest and reports it
- * (any pointer may be NULL).  The trial steps overwrite the populations:
- * tune first, then initialise the boxes. */
+/* The form (LBM_FORM_*) that lbm_batch_step(b, n) takes, and the choice of it,
+ * as lbm_step_form and lbm_set_step_forms for one lattice. */
+int lbm_batch_step_form(const lbm_batch *b, long n);
+lbm_status lbm_batch_set_step_forms(lbm_batch *b, int single, int several);
+
+/* Autotune the launch shape: times trial_steps steps of the one-kernel form for
+ * each tile height in {4, 8, 16} and z chunk in {8, 16, 24, 32, 48, 64} and
+ * keeps the fastest; then the two-kernel form (FP64) against it and the moment
+ * form (trial_steps steps a call, at least 8) against the faster of the two, and
+ * keeps what is faster (lbm_batch_step_form).  Reports the shape and the time
+ * per step of a call of one step (any pointer may be NULL).  The trial steps
+ * overwrite the populations: tune first, then initialise the boxes. */
 lbm_status lbm_batch_tune(lbm_batch *b, int trial_steps, int *tile_y,
                           int *zchunk, double *ms_per_step);
 

@@ -1668,8 +1668,7 @@ struct lbm_batch {
     void* mom_plan = nullptr;         // device memory of its plan
     BatchBox* mom_boxes_dev = nullptr;
     bool mom_twice = false;
-    // FP64 steps in two kernels over every box, where they run in place
-    bool split = false;
+    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};  // of calls of one and of several steps
     unsigned max_cells = 0;
     char err[512] = {0};
 
@@ -1695,8 +1694,8 @@ StepLaunch batch_launch(const lbm_batch* b) {
     return l;
 }
 
-cudaError_t batch_launch_step(const lbm_batch* b, int from) {
-    if (b->split) {
+cudaError_t batch_launch_step(const lbm_batch* b, int form, int from) {
+    if (form == LBM_FORM_TWO_KERNELS) {
         SplitLaunch l{b->phys, b->bargs, b->max_cells, b->stream};
         return split_step(l, b->p.storage, b->box[0]->coll, b->f[from], b->f[from ^ 1], nullptr);
     }
@@ -1752,12 +1751,19 @@ lbm_status batch_configure(lbm_batch* b, int ty, int zc) {
     return LBM_OK;
 }
 
+// FP64 steps in two kernels over every box, where they run in place; a grid has at most 65,535 rows of blocks.
+bool batch_can_split(const lbm_batch* b) {
+    const int coll = b->box[0]->coll;
+    return b->p.storage == LBM_F64 && b->count <= 65535 && coll != COLL_MRT && !(coll == COLL_SRT && b->p.tau != 1.0);
+}
+
 // The moment kernels' own table of work items (their tiles differ from the
-// population kernels'), where every box's fields fit into its populations.
+// population kernels'), where every box's fields fit into its populations;
+// b->mom stays nullptr elsewhere.
 lbm_status batch_configure_moments(lbm_batch* b) {
     const lbm_params& p = b->p;
     const int coll = b->box[0]->coll;
-    if (p.kernel != 0 || (coll == COLL_SRT && p.tau != 1.0)) return LBM_OK;
+    if (b->mom || (coll == COLL_SRT && p.tau != 1.0)) return LBM_OK;
     const MomentKernels* k = moment_kernels(p.storage, coll);
     if (!k) return LBM_OK;
     b->mom_twice = true;
@@ -1814,11 +1820,25 @@ lbm_status batch_configure_moments(lbm_batch* b) {
     return LBM_OK;
 }
 
+// The forms of a batch for which no particular kernel or launch shape was asked.
+lbm_status batch_choose_forms(lbm_batch* b, int (&form)[2]) {
+    form[0] = form[1] = batch_can_split(b) ? LBM_FORM_TWO_KERNELS : LBM_FORM_ONE_KERNEL;
+    const lbm_status st = batch_configure_moments(b);
+    if (b->mom) form[1] = LBM_FORM_MOMENTS;
+    return st;
+}
+
+void batch_set_forms(lbm_batch* b, const int (&form)[2]) {
+    if (form[1] != b->form[1]) batch_drop_graphs(b);  // they hold steps of that form
+    b->form[0] = form[0];
+    b->form[1] = form[1];
+}
+
 lbm_status batch_build_graph(lbm_batch* b, int from) {
     cudaGraph_t g = nullptr;
     LBM_CUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e1 = batch_launch_step(b, from);
-    cudaError_t e2 = batch_launch_step(b, from ^ 1);
+    cudaError_t e1 = batch_launch_step(b, b->form[1], from);
+    cudaError_t e2 = batch_launch_step(b, b->form[1], from ^ 1);
     cudaError_t e3 = cudaStreamEndCapture(b->stream, &g);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -1914,14 +1934,11 @@ lbm_status lbm_batch_create(const lbm_params* p, int count, const int* dims, lbm
         b->box[i] = c;
     }
     b->phys = b->box[0]->args;
-    const int coll = b->box[0]->coll;
-    b->split = p->storage == LBM_F64 && p->kernel == 0 && count <= 65535 && coll != COLL_MRT &&
-               !(coll == COLL_SRT && p->tau != 1.0);
     for (const lbm_ctx* c : b->box) b->max_cells = std::max(b->max_cells, unsigned(c->n));
     const int ty = p->tile_y ? p->tile_y : (p->collision == LBM_MRT_GUO ? 4 : 8);
     const int zc = p->zchunk ? p->zchunk : 32;
     lbm_status st = batch_configure(b, ty, zc);
-    if (st == LBM_OK) st = batch_configure_moments(b);
+    if (st == LBM_OK && p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) st = batch_choose_forms(b, b->form);
     if (st != LBM_OK) {
         snprintf(g_create_err, sizeof(g_create_err), "%s", b->err);
         lbm_batch_destroy(b);
@@ -1962,7 +1979,8 @@ lbm_status lbm_batch_box(lbm_batch* b, int i, lbm_ctx** view) {
 lbm_status lbm_batch_step(lbm_batch* b, long n) {
     if (!b) return LBM_EINVAL;
     if (n < 0) return b->fail(LBM_EINVAL, "lbm_batch_step: n must be >= 0");
-    if (n >= 2 && b->mom) {
+    const int form = b->form[n >= 2];
+    if (form == LBM_FORM_MOMENTS) {
         MomentLaunch l = b->mom_launch;
         l.stream = b->stream;
         int to = 0;
@@ -1986,7 +2004,7 @@ lbm_status lbm_batch_step(lbm_batch* b, long n) {
         for (lbm_ctx* c : b->box) c->t += 2;
     }
     if (n == 1) {
-        cudaError_t e = batch_launch_step(b, b->cur);
+        cudaError_t e = batch_launch_step(b, form, b->cur);
         if (e != cudaSuccess) return b->fail(LBM_ECUDA, "batch step launch failed: %s", cudaGetErrorString(e));
         b->cur ^= 1;
         ++b->t;
@@ -1995,6 +2013,24 @@ lbm_status lbm_batch_step(lbm_batch* b, long n) {
             ++c->t;
         }
     }
+    return LBM_OK;
+}
+
+int lbm_batch_step_form(const lbm_batch* b, long n) { return b && n >= 1 ? b->form[n >= 2] : 0; }
+
+lbm_status lbm_batch_set_step_forms(lbm_batch* b, int single, int several) {
+    if (!b) return LBM_EINVAL;
+    if (single < LBM_FORM_AUTO || single > LBM_FORM_TWO_KERNELS || several < LBM_FORM_AUTO || several > LBM_FORM_MOMENTS)
+        return b->fail(LBM_EINVAL, "lbm_batch_set_step_forms: unknown form (%d, %d)", single, several);
+    int form[2];
+    if (const lbm_status st = batch_choose_forms(b, form); st != LBM_OK) return st;
+    if (single != LBM_FORM_AUTO) form[0] = single;
+    if (several != LBM_FORM_AUTO) form[1] = several;
+    if ((form[0] == LBM_FORM_TWO_KERNELS || form[1] == LBM_FORM_TWO_KERNELS) && !batch_can_split(b))
+        return b->fail(LBM_EUNSUPPORTED, "lbm_batch_set_step_forms: these boxes cannot step in two kernels");
+    if (form[1] == LBM_FORM_MOMENTS && !b->mom)
+        return b->fail(LBM_EUNSUPPORTED, "lbm_batch_set_step_forms: these boxes cannot step through moment fields");
+    batch_set_forms(b, form);
     return LBM_OK;
 }
 
@@ -2011,9 +2047,9 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
     for (int ty : tys) {
         for (int zc : zcs) {
             if (batch_configure(b, ty, zc) != LBM_OK) continue;
-            if (batch_launch_step(b, 0) != cudaSuccess) continue;  // warm-up
+            if (batch_launch_step(b, LBM_FORM_ONE_KERNEL, 0) != cudaSuccess) continue;  // warm-up
             cudaEventRecord(e0, b->stream);
-            for (int k = 0; k < trial_steps; ++k) batch_launch_step(b, k & 1);
+            for (int k = 0; k < trial_steps; ++k) batch_launch_step(b, LBM_FORM_ONE_KERNEL, k & 1);
             cudaEventRecord(e1, b->stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) continue;
             float ms = 0.0f;
@@ -2026,12 +2062,45 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
             }
         }
     }
+    // the other forms, as lbm_batch_step runs them; fewer than 8 steps at once would time the moment form's ends
+    auto timed = [&](int n, auto&& run) {
+        if (run(2) != cudaSuccess) return -1.0f;  // warm-up
+        cudaEventRecord(e0, b->stream);
+        const bool ok = run(n) == cudaSuccess;
+        cudaEventRecord(e1, b->stream);
+        if (!ok || cudaEventSynchronize(e1) != cudaSuccess) return -1.0f;
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        return ms / n;
+    };
+    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};
+    if (batch_can_split(b)) {
+        const float ms = timed(trial_steps, [&](int n) {
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < n && e == cudaSuccess; ++k) e = batch_launch_step(b, LBM_FORM_TWO_KERNELS, k & 1);
+            return e;
+        });
+        if (ms >= 0.0f && (best < 0.0f || ms < best)) {
+            best = ms;
+            form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+        }
+    }
+    if (batch_configure_moments(b) == LBM_OK && b->mom) {
+        MomentLaunch l = b->mom_launch;
+        l.stream = b->stream;
+        const float ms = timed(trial_steps < 8 ? 8 : trial_steps, [&](int n) {
+            int to = 0;
+            return run_moments(*b->mom, l, b->f, 0, n, b->bytes, b->mom_twice, &to);
+        });
+        if (ms >= 0.0f && best >= 0.0f && ms < best) form[1] = LBM_FORM_MOMENTS;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return b->fail(LBM_ECUDA, "lbm_batch_tune: %s", cudaGetErrorString(e));
     lbm_status st = batch_configure(b, best_ty, best_zc);
     if (st != LBM_OK) return st;
+    if (best >= 0.0f) batch_set_forms(b, form);
     if (tile_y) *tile_y = best_ty;
     if (zchunk) *zchunk = best_zc;
     if (ms_per_step) *ms_per_step = best;

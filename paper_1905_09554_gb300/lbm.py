@@ -101,6 +101,8 @@ _SIGNATURES = {
     "lbm_batch_last_error": (ctypes.c_char_p, [_P]),
     "lbm_batch_box": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(_P)]),
     "lbm_batch_step": (ctypes.c_int, [_P, ctypes.c_long]),
+    "lbm_batch_step_form": (ctypes.c_int, [_P, ctypes.c_long]),
+    "lbm_batch_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
     "lbm_batch_tune": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                       _D]),
     "lbm_batch_config": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
@@ -280,10 +282,19 @@ def lbm_batch_step(b, n):
     return load().lbm_batch_step(b, n)
 
 
+def lbm_batch_step_form(b, n):
+    return load().lbm_batch_step_form(b, int(n))
+
+
+def lbm_batch_set_step_forms(b, single, several):
+    return load().lbm_batch_set_step_forms(b, int(single), int(several))
+
+
 def lbm_batch_tune(b, trial_steps):
     ty, zc, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_double()
     st = load().lbm_batch_tune(b, trial_steps, ctypes.byref(ty), ctypes.byref(zc), ctypes.byref(ms))
-    return st, dict(tile_y=ty.value, zchunk=zc.value, ms_per_step=ms.value)
+    return st, dict(tile_y=ty.value, zchunk=zc.value, ms_per_step=ms.value,
+                    forms=[FORM_NAMES[lbm_batch_step_form(b, n)] for n in (1, 2)])
 
 
 def lbm_batch_config(b):
@@ -618,6 +629,9 @@ class _BoxView(Lattice):
     def close(self):
         self.ctx = None  # owned by the batch
 
+    def step_form(self, n=1):
+        return self._batch.step_form(n)  # boxes step with their batch
+
     def step(self, n=1):
         raise LbmError(LBM_EINVAL, "boxes of a batch are stepped together with Batch.step")
 
@@ -661,8 +675,8 @@ class Batch:
     together; the physics keywords are those of Lattice (FP32/FP64 only).
 
     tune_cache: path of a JSON file of launch-shape picks.  When given (and
-    neither tile_y nor zchunk is), a pick stored for the same boxes, physics
-    and GPU model is used; otherwise the batch is autotuned once at creation
+    neither tile_y nor zchunk is), a pick (launch shape and forms) stored for
+    the same boxes, physics and GPU model is used; otherwise the batch is autotuned once at creation
     (lbm_batch_tune, before any state is set) and its pick stored."""
 
     def __init__(self, dims, stream=None, tune_cache=None, trial_steps=3, **kw):
@@ -691,10 +705,13 @@ class Batch:
             st, v = lbm_batch_box(b, i)
             self._check(st)
             self.boxes.append(_BoxView(self, i, v, (nz, ny, nx)))
+        # (no forms stored, or no room for them any more: one kernel a step)
+        if cached and "forms" in cached:
+            lbm_batch_set_step_forms(self.b, *(FORM_NAMES.index(v) for v in cached["forms"]))
         if key is not None and not cached:
             best = self.tune(trial_steps)
             data = _read_tune_cache(tune_cache)
-            data[key] = {"tile_y": best["tile_y"], "zchunk": best["zchunk"], "ms_per_step": best["ms_per_step"]}
+            data[key] = {k: best[k] for k in ("tile_y", "zchunk", "ms_per_step", "forms") if k in best}
             _write_tune_cache(tune_cache, data)
 
     def _check(self, st):
@@ -703,6 +720,14 @@ class Batch:
 
     def step(self, n=1):
         self._check(lbm_batch_step(self.b, int(n)))
+
+    def step_form(self, n=1):
+        """How step(n) steps: 'one', 'two' (kernels a step) or 'moments'."""
+        return FORM_NAMES[lbm_batch_step_form(self.b, n)]
+
+    def set_step_forms(self, single="auto", several="auto"):
+        """Choose how step(1) and step(n >= 2) step (lbm_batch_set_step_forms)."""
+        self._check(lbm_batch_set_step_forms(self.b, FORM_NAMES.index(single), FORM_NAMES.index(several)))
 
     def tune(self, trial_steps=3):
         st, r = lbm_batch_tune(self.b, int(trial_steps))

@@ -109,3 +109,45 @@ def test_forms_that_cannot_serve_are_refused():
     with lbm.Batch([(8, 8, 8)], storage="f32") as B:
         with pytest.raises(lbm.LbmError, match="LBM_EINVAL"):
             B.boxes[0].set_step_forms("one", "one")
+
+
+DIMS = [(32, 32, 50), (20, 17, 33), (48, 48, 75), (33, 40, 9), (64, 64, 101)]
+
+
+@pytest.mark.parametrize("storage,tau,forms", [("f64", 1.0, ("two", "two")), ("f64", 0.9, ("one", "one")),
+                                               ("f32", 1.0, ("one", "moments")), ("f32", 0.9, ("one", "one"))])
+def test_batches_step_by_a_shape_that_was_asked_for_and_their_tuner_times_the_forms(storage, tau, forms, tmp_path):
+    rho = [inputs.random_density(*d, seed=30 + k, lo=0.3, hi=1.9) for k, d in enumerate(DIMS)]
+    path = str(tmp_path / "tune.json")
+
+    def populations(B):
+        for v, r in zip(B.boxes, rho):
+            v.set_density(r)
+        for n in (1, 4, 3, 2):
+            B.step(n)
+        return [v.get_populations() for v in B.boxes]
+
+    kw = dict(storage=storage, tau=tau, G=-5.5)
+    with lbm.Batch(DIMS, tile_y=8, zchunk=16, **kw) as B:
+        assert (B.step_form(1), B.step_form(2)) == ("one", "one") == (B.boxes[0].step_form(1), B.boxes[0].step_form(2))
+        want = populations(B)
+    with lbm.Batch(DIMS, **kw) as B:
+        assert (B.step_form(1), B.step_form(2)) == forms
+        assert all(np.array_equal(a, b) for a, b in zip(populations(B), want))
+        B.set_step_forms("one", "one")  # the graphs of the other form are gone
+        assert all(np.array_equal(a, b) for a, b in zip(populations(B), want))
+        B.set_step_forms()
+        assert (B.step_form(1), B.step_form(2)) == forms
+        if forms[1] != "moments":
+            with pytest.raises(lbm.LbmError, match="LBM_EUNSUPPORTED"):
+                B.set_step_forms("auto", "moments")
+    with lbm.Batch(DIMS, tune_cache=path, **kw) as B:
+        tuned = B.step_form(1), B.step_form(2)
+        assert all(np.array_equal(a, b) for a, b in zip(populations(B), want))
+    if storage == "f64":  # several times faster wherever it can run
+        assert tuned == forms
+    entry, = json.load(open(path)).values()
+    assert tuple(entry["forms"]) == tuned
+    with lbm.Batch(DIMS, tune_cache=path, **kw) as B:
+        assert (B.step_form(1), B.step_form(2)) == tuned
+        assert all(np.array_equal(a, b) for a, b in zip(populations(B), want))
