@@ -99,9 +99,11 @@ typedef struct {
     void *f_a, *f_b;      /* optional caller-owned device buffers for the two
                              population copies (each 19*nx*ny*nz elements of the
                              storage type, 16-byte aligned); NULL = the library
-                             allocates (and frees them in lbm_destroy).  A step
-                             may overwrite both: only the current copy
-                             (lbm_current_copy) holds a state.                      */
+                             allocates (and frees them in lbm_destroy).  The
+                             current copy (lbm_current_copy) holds the state;
+                             after a call of one step the other one holds the
+                             state before it, a call of several steps may
+                             overwrite both.                                        */
                           /* zchunk, tile_y, kernel: any of them given makes every
                              call step by the one kernel of that shape; with all
                              three 0 lbm_step chooses its form too                  */
@@ -205,7 +207,10 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int on_device);
  * at the end: ask for many steps at once where nothing is read in between.
  * FP64, small boxes and 16-bit storage with nx odd step in two kernels, with a
  * psi field of n cells of their own where the moments do not suffice; if it
- * cannot be allocated, in one.  lbm_step_form tells which form a call takes. */
+ * cannot be allocated, in one.  lbm_step_form tells which form a call takes.
+ * Where the moments suffice, a call of one step on copies that the caller owns
+ * keeps the state before it and leaves its moments in fields of their own (5, 10
+ * or 11 of n cells), allocated by the first such call. */
 lbm_status lbm_step(lbm_ctx *ctx, long n);
 
 /* The form (LBM_FORM_*, never LBM_FORM_AUTO) that lbm_step(ctx, n) takes; 0 for

@@ -279,14 +279,8 @@ __device__ __forceinline__ SumFlat<V> sum_flat(V f0, const Opp<V>& a, const Opp<
     return s;
 }
 
-// Moments that an operator reads before the collision: rho, jx, jy, jz, then
-// the second moments whose rates differ from 1.
-//   SRT at tau = 1, MRT with every rate 1:      4
-//   MRT, shear rule: 2 xx - yy - zz, yy - zz, xy, yz, xz:  9
-//   MRT, paper's rule: xx, yy, zz, xy, yz, xz:  10
-// (SRT at another tau and MRT with general rates need all 19 populations.)
 template <int COLL>
-constexpr int kMoments = COLL == COLL_MRT_SHEAR ? 9 : (COLL == COLL_MRT_SPARSE ? 10 : 4);
+constexpr int kMoments = moments_of_operator(COLL);
 
 template <int COLL, class V>
 __device__ __forceinline__ void moments_from(const SumUp<V>& up, const V& rho_uf, const V& jx_uf, const V& jy_uf,

@@ -42,7 +42,8 @@ struct lbm_ctx {
     double* diag = nullptr;           // diagnostics: 8 per slice, 8 per slice and part, a counter per slice
     int diag_parts = 1;               // blocks per slice
     mutable bool waits = false;       // a kernel with bounded waits ran since its error word was last read
-    void* psi_ws = nullptr;           // two-belt force: psi of the state being stepped
+    void* psi_ws = nullptr;           // two-belt force and two-kernel step: psi of the state being stepped
+    bool ws_moments = false;          // two-kernel step: the moments are in front of it
     int* dev_err = nullptr;           // device error word of the bounded waits
     std::vector<double> diag_host;
     long long own_bytes = 0;
@@ -413,15 +414,15 @@ cudaError_t launch_step(const lbm_ctx* c, const void* src, void* dst, void* psi_
     return step_kernels(c->p.storage, c->coll).launch(l, src, dst);
 }
 
-// One step src -> dst in one or two kernels.  keep_src: src is not
-// one of the context's own copies (a checkpoint, a recomputed state) and stays
-// as it is; psi_out then receives its psi where the step computes it.
+// One step src -> dst in one or two kernels.  keep_src: src stays as it is (the
+// caller may read it, or it is a checkpoint or a recomputed state); psi_out then
+// receives its psi where the step computes it.
 cudaError_t step_once(const lbm_ctx* c, int form, void* src, void* dst, bool keep_src = false,
                       void* psi_out = nullptr) {
     if (form != LBM_FORM_TWO_KERNELS) return launch_step(c, src, dst, psi_out);
     void* psi = psi_out ? psi_out : c->psi_ws;
-    if (!keep_src && c->split_in_place) psi = nullptr;
     SplitLaunch l{c->args, BatchArgs{}, unsigned(c->n), c->stream};
+    if (c->split_in_place && !psi_out) l.moments = !keep_src ? src : (c->ws_moments ? c->psi_ws : nullptr);
     if (c->ref[0]) {  // local-reference storage: the density fields follow their population copies
         const int k = src == c->f[0] ? 0 : 1;
         l.args.ref_src = c->ref[k];
@@ -553,10 +554,10 @@ long long split_cells(const lbm_params& p, bool in_place) {
 
 constexpr long long kSplitPad = 1024;  // block rounding of the two-kernel step's 32-bit cell index
 
-// The field that psi of the whole box goes through, where the step needs one; false without room.
-bool alloc_psi(lbm_ctx* c) {
+// Fields of n cells in the arithmetic type for the two-kernel step or the two-belt force; false without room.
+bool alloc_psi(lbm_ctx* c, int fields = 1) {
     if (c->psi_ws) return true;
-    const size_t bytes = (size_t)c->n * (c->p.storage == LBM_F64 ? 8 : 4);
+    const size_t bytes = (size_t)fields * (size_t)c->n * (c->p.storage == LBM_F64 ? 8 : 4);
     if (cudaMalloc(&c->psi_ws, bytes) != cudaSuccess) {
         c->psi_ws = nullptr;
         cudaGetLastError();
@@ -877,13 +878,39 @@ cudaError_t upload_plan(const MomentPlan& plan, MomentLaunch& l, void** mem, siz
     return e;
 }
 
+// Operators and storages whose two-kernel step needs only the moments.
+bool split_by_moments(const lbm_ctx* c) {
+    return c->p.storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && c->p.tau != 1.0);
+}
+
 // Sets up the two-kernel step; false where it cannot serve (the two-belt force,
 // too many cells for its 32-bit index, no room for its psi field).
 bool prepare_split(lbm_ctx* c) {
-    const lbm_params& p = c->p;
-    if (p.G2 != 0.0 || c->n > 0xffffffffLL - kSplitPad) return false;
-    c->split_in_place = p.storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p.tau != 1.0);
+    if (c->p.G2 != 0.0 || c->n > 0xffffffffLL - kSplitPad) return false;
+    c->split_in_place = split_by_moments(c);
     return c->split_in_place || alloc_psi(c);
+}
+
+// A caller who holds the copies may read the state before a call of one step
+// (also a difference of two states is taken that way), so such a call does not
+// go in place: its moments go into fields of their own, allocated by the first
+// one, or psi alone does where there is no room for them (the second kernel then
+// sums the moments again: FP64 128 x 128 x 288 1561 us against 1218).  False
+// without room for either.
+bool prepare_split_once(lbm_ctx* c) {
+    if (!c->split_in_place || c->own_f || c->psi_ws) return true;
+    // (also while a stream is captured, here or in another thread)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    c->ws_moments = alloc_psi(c, moments_of_operator(c->coll) + 1);
+    const bool ok = c->ws_moments || alloc_psi(c);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return ok;
+}
+
+// Whether the two-kernel step is expected to be faster than the one-kernel step.
+bool split_wanted(const lbm_ctx* c) {
+    return c->p.storage == LBM_F64 || c->n <= split_cells(c->p, split_by_moments(c));
 }
 
 // Launch shape of the moment kernels (step_moment.cuh), where the collision
@@ -938,12 +965,9 @@ bool prepare_moments(lbm_ctx* c, bool rival) {
 // The forms of a context for which no particular kernel or launch shape was
 // asked.
 void choose_forms(lbm_ctx* c, int (&form)[2]) {
-    const lbm_params& p = c->p;
     form[0] = form[1] = LBM_FORM_ONE_KERNEL;
-    if (p.G2 != 0.0) return;
-    const bool in_place = p.storage <= LBM_F32 && c->coll != COLL_MRT && !(c->coll == COLL_SRT && p.tau != 1.0);
-    if ((p.storage == LBM_F64 || c->n <= split_cells(p, in_place)) && prepare_split(c))
-        form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+    if (c->p.G2 != 0.0) return;
+    if (split_wanted(c) && prepare_split(c)) form[0] = form[1] = LBM_FORM_TWO_KERNELS;
     if (prepare_moments(c, form[1] == LBM_FORM_TWO_KERNELS)) form[1] = LBM_FORM_MOMENTS;
 }
 
@@ -1371,16 +1395,19 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
     int form[2], automatic[2];
     form[0] = form[1] = LBM_FORM_ONE_KERNEL;
     choose_forms(c, automatic);
-    if (automatic[0] == LBM_FORM_TWO_KERNELS) {
+    float several = best;
+    for (int many = 0; many < 2; ++many) {  // calls of one step and of several
+        if (automatic[0] == LBM_FORM_ONE_KERNEL || (!many && !prepare_split_once(c))) continue;
         const float ms = timed(steps, [&](int n) {
             cudaError_t e = cudaSuccess;
             for (int k = 0; k < n && e == cudaSuccess; ++k)
-                e = step_once(c, LBM_FORM_TWO_KERNELS, c->f[cur ^ (k & 1)], c->f[cur ^ (~k & 1)]);
+                e = step_once(c, LBM_FORM_TWO_KERNELS, c->f[cur ^ (k & 1)], c->f[cur ^ (~k & 1)], !many && !c->own_f);
             return e;
         });
-        if (ms >= 0.0f && (best < 0.0f || ms < best)) {
-            best = ms;
-            form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+        float& rival = many ? several : best;
+        if (ms >= 0.0f && (rival < 0.0f || ms < rival)) {
+            rival = ms;
+            form[many] = LBM_FORM_TWO_KERNELS;
         }
     }
     if (prepare_moments(c, false)) {
@@ -1389,7 +1416,7 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
             int to = 0;
             return run_moments(*c->mom, l, c->f, cur, n, c->mom_bytes, c->mom_twice, &to);
         });
-        if (ms >= 0.0f && best >= 0.0f && ms < best) form[1] = LBM_FORM_MOMENTS;
+        if (ms >= 0.0f && several >= 0.0f && ms < several) form[1] = LBM_FORM_MOMENTS;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1537,10 +1564,12 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (!c) return LBM_EINVAL;
     if (nsteps < 0) return c->fail(LBM_EINVAL, "lbm_step: n must be >= 0");
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_step: this context is a box of a batch; use lbm_batch_step");
-    const int form = c->form[nsteps >= 2];
+    int form = c->form[nsteps >= 2];
     if (form == LBM_FORM_MOMENTS) return step_moments(c, nsteps);
+    if (nsteps == 1 && form == LBM_FORM_TWO_KERNELS && !prepare_split_once(c)) form = LBM_FORM_ONE_KERNEL;
+    const bool keep = nsteps == 1 && !c->own_f;
     for (long k = 0; k < nsteps; ++k) {
-        cudaError_t e = step_once(c, form, c->f[c->cur], c->f[c->cur ^ 1]);
+        cudaError_t e = step_once(c, form, c->f[c->cur], c->f[c->cur ^ 1], keep);
         if (e != cudaSuccess) return c->fail(LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));
         c->cur ^= 1;
         ++c->t;
@@ -1696,7 +1725,7 @@ StepLaunch batch_launch(const lbm_batch* b) {
 
 cudaError_t batch_launch_step(const lbm_batch* b, int form, int from) {
     if (form == LBM_FORM_TWO_KERNELS) {
-        SplitLaunch l{b->phys, b->bargs, b->max_cells, b->stream};
+        SplitLaunch l{b->phys, b->bargs, b->max_cells, b->stream, b->f[from]};
         return split_step(l, b->p.storage, b->box[0]->coll, b->f[from], b->f[from ^ 1], nullptr);
     }
     const StepLaunch l = batch_launch(b);

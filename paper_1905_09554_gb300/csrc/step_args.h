@@ -15,6 +15,16 @@ namespace lbm {
 // rates outside {3pxx, pww, pxy, pyz, pxz} are 1 (the shear rule).
 enum { COLL_SRT = 0, COLL_MRT = 1, COLL_MRT_SPARSE = 2, COLL_MRT_UNIT = 3, COLL_MRT_SHEAR = 4, COLL_COUNT = 5 };
 
+// Moments that an operator reads before the collision: rho, jx, jy, jz, then
+// the second moments whose rates differ from 1.
+//   SRT at tau = 1, MRT with every rate 1:      4
+//   MRT, shear rule: 2 xx - yy - zz, yy - zz, xy, yz, xz:  9
+//   MRT, paper's rule: xx, yy, zz, xy, yz, xz:  10
+// (SRT at another tau and MRT with general rates need all 19 populations.)
+__host__ __device__ constexpr int moments_of_operator(int coll) {
+    return coll == COLL_MRT_SHEAR ? 9 : (coll == COLL_MRT_SPARSE ? 10 : 4);
+}
+
 struct StepArgs {
     int nx, ny, nz;
     int zchunk;           // planes per block (work item) along z
@@ -155,14 +165,17 @@ struct MomentKernels {
 const MomentKernels* moment_kernels(int storage, int coll);
 
 // The step in two kernels (step_split.cuh), of one lattice or of a batch's
-// boxes (batch.nbox > 0).  psi: a field of its own for psi of `src`, which is
-// then left as it is; without one (FP64 and FP32; not for general MRT rates,
-// and SRT only at tau = 1) the source populations are overwritten.
+// boxes (batch.nbox > 0).  Its first kernel leaves, for the second, either
+//  * moments != nullptr (FP64 and FP32; not for general MRT rates, and SRT only
+//    at tau = 1): the moments and psi there, fields of n cells each; this may be
+//    `src`, whose populations are then overwritten; or
+//  * psi of `src` in the field `psi` (not for batches).
 struct SplitLaunch {
     StepArgs args;
     BatchArgs batch;
     unsigned max_cells;   // of the largest box
     cudaStream_t stream;
+    void* moments = nullptr;
 };
 cudaError_t split_step(const SplitLaunch& l, int storage, int coll, void* src, void* dst, void* psi);
 

@@ -2,7 +2,8 @@
 //
 //   sc_fields_kernel  forms psi of every cell once, from its populations; where
 //       the collision needs no more than the moments (collide.cuh), it leaves
-//       those and psi in the first slots of the cell's own populations,
+//       those and psi in the first slots of the cell's own populations, or in
+//       fields of their own where the populations have to stay,
 //   sc_push_kernel    reads psi of the 18 neighbours (through L1) and the
 //       moments or populations, collides and pushes.
 // Cells are dealt linearly to small blocks: no tile, rim, chunk or barrier.
@@ -45,11 +46,12 @@ __device__ __forceinline__ S* cell_at(S* p, int k, unsigned n, unsigned i) {
     return p + (k * (long long)n + i);
 }
 
-// psi in slot kMoments<COLL> behind the moments (IN_PLACE), or in its own
-// field.  Local-reference storage: the density goes to ref_dst as well.
-template <class Codec, int COLL, bool IN_PLACE>
+// MOMENTS: `fields` receives the moments and, behind them, psi (it may be f_all);
+// otherwise psi alone.  Local-reference storage: the density goes to ref_dst as
+// well.
+template <class Codec, int COLL, bool MOMENTS>
 __global__ void __launch_bounds__(kSplitThreads<typename Codec::R>)
-sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const StepArgs a, const BatchArgs b) {
+sc_fields_kernel(const typename Codec::S* f_all, typename Codec::R* fields, const StepArgs a, const BatchArgs b) {
     using R = typename Codec::R;
     constexpr int NF = kMoments<COLL>;
     chain_begin();
@@ -62,7 +64,7 @@ sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const Ste
     }
     const unsigned i = blockIdx.x * kSplitThreads<R> + threadIdx.x;
     if (i >= n) return;
-    typename Codec::S* const f = f_all + base;
+    const typename Codec::S* const f = f_all + base;
     float ref = 0.0f;
     if constexpr (Codec::kLocal) ref = __ldg(a.ref_src + i);
     R v[Q], m[NF];
@@ -75,14 +77,14 @@ sc_fields_kernel(typename Codec::S* f_all, typename Codec::R* psi_all, const Ste
     moments_of<COLL, R>(v, m);  // (the sums that are not needed fall away)
     const R p = psi_of<R>(m[0], par<R>(a.rho0, a.rho0f), par<R>(a.inv_rho0, a.inv_rho0f));
     chain_end();
-    if constexpr (IN_PLACE) {
+    if constexpr (MOMENTS) {
         static_for<0, NF>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
-            *cell_at(f, k, n, i) = m[k];
+            *cell_at(fields + base, k, n, i) = m[k];
         });
-        *cell_at(f, NF, n, i) = p;
+        *cell_at(fields + base, NF, n, i) = p;
     } else {
-        psi_all[i] = p;
+        fields[i] = p;
         if constexpr (Codec::kLocal) a.ref_dst[i] = m[0];
     }
 }
@@ -99,9 +101,9 @@ struct NeighbourPsi {
     }
 };
 
-template <class Codec, int COLL, bool IN_PLACE>
+template <class Codec, int COLL, bool MOMENTS>
 __global__ void __launch_bounds__(kSplitThreads<typename Codec::R>)
-sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Codec::R* __restrict__ psi_all,
+sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Codec::R* __restrict__ fields,
                typename Codec::S* __restrict__ dst_all, const StepArgs a, const BatchArgs b) {
     using R = typename Codec::R;
     using S = typename Codec::S;
@@ -121,8 +123,8 @@ sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Cod
     if (i >= n) return;
     const S* __restrict__ src = src_all + base;
     S* __restrict__ dst = dst_all + base;
-    const R* __restrict__ psi = psi_all;
-    if constexpr (IN_PLACE) psi = src + NF * (long long)n;
+    const R* __restrict__ psi = fields;
+    if constexpr (MOMENTS) psi += base + NF * (long long)n;
     const int z = int(i / plane), y = int((i - unsigned(z) * plane) / unsigned(nx)),
               x = int(i - unsigned(z) * plane - unsigned(y) * unsigned(nx));
     const unsigned zo[3] = {unsigned(z == 0 ? nz - 1 : z - 1) * plane, unsigned(z) * plane,
@@ -132,10 +134,10 @@ sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Cod
     const unsigned xo[3] = {unsigned(x == 0 ? nx - 1 : x - 1), unsigned(x), unsigned(x + 1 == nx ? 0 : x + 1)};
 
     R f[Q], m[NF];
-    if constexpr (IN_PLACE) {
+    if constexpr (MOMENTS) {
         static_for<0, NF>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
-            m[k] = __ldg(cell_at(src, k, n, i));
+            m[k] = __ldg(cell_at(fields + base, k, n, i));
         });
     } else {
         float ref = 0.0f;
@@ -155,7 +157,7 @@ sc_push_kernel(const typename Codec::S* __restrict__ src_all, const typename Cod
         if constexpr (k == 1) psi_diag(w[k], at);
     });
     const Force<R> F = force_of(w[0], w[1], w[2], par<R>(a.gw, a.gwf));
-    if constexpr (IN_PLACE) {
+    if constexpr (MOMENTS) {
         collide_moments<COLL, R, true>(m, F, a, [&](auto qc, R v) {
             constexpr int q = decltype(qc)::value;
             f[q] = v;
@@ -185,22 +187,22 @@ cudaError_t split_step(const SplitLaunch& l, void* src, void* dst, void* psi) {
     const dim3 grid((l.max_cells + kSplitThreads<R> - 1) / kSplitThreads<R>, l.batch.nbox ? l.batch.nbox : 1);
     S* const s = static_cast<S*>(src);
     S* const d = static_cast<S*>(dst);
-    R* const p = static_cast<R*>(psi);
     const bool chain = (long long)grid.x * grid.y * kSplitThreads<R> <= 400000;
-    auto both = [&](auto in_place) {
-        constexpr bool IN = decltype(in_place)::value;
-        cudaError_t e = launch_chained(chain, sc_fields_kernel<Codec, COLL, IN>, grid, kSplitThreads<R>, 0, l.stream, s, p, l.args,
+    auto both = [&](auto with_moments, void* fields) {
+        constexpr bool M = decltype(with_moments)::value;
+        R* const p = static_cast<R*>(fields);
+        cudaError_t e = launch_chained(chain, sc_fields_kernel<Codec, COLL, M>, grid, kSplitThreads<R>, 0, l.stream, s, p, l.args,
                                        l.batch);
         if (e == cudaSuccess)
-            e = launch_chained(chain, sc_push_kernel<Codec, COLL, IN>, grid, kSplitThreads<R>, 0, l.stream, s, p, d, l.args,
+            e = launch_chained(chain, sc_push_kernel<Codec, COLL, M>, grid, kSplitThreads<R>, 0, l.stream, s, p, d, l.args,
                                l.batch);
         return e;
     };
     if constexpr (COLL != COLL_MRT && sizeof(S) == sizeof(R)) {
-        if (!psi) return both(std::true_type{});
+        if (l.moments) return both(std::true_type{}, l.moments);
     }
     if (!psi || l.batch.nbox) return cudaErrorInvalidValue;
-    return both(std::false_type{});
+    return both(std::false_type{}, psi);
 }
 
 template <class Codec>

@@ -458,7 +458,9 @@ class Lattice:
     def stored_populations(self):
         """The torch uint8 buffer that holds the current state exactly as
         stored (19 * nx * ny * nz elements of the storage type, library
-        velocity order); only with torch_buffers=True."""
+        velocity order); only with torch_buffers=True.  After step(1) the
+        buffer returned before it still holds the state before the step;
+        step(n) with n >= 2 may overwrite both buffers."""
         if self._bufs is None:
             raise LbmError(LBM_EINVAL, "stored_populations: the population copies are not torch buffers")
         return self._bufs[lbm_current_copy(self.ctx)]
