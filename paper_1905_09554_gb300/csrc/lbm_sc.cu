@@ -41,7 +41,7 @@ struct lbm_ctx {
     size_t scratch_bytes = 0;
     double* diag = nullptr;           // diagnostics: 8 per slice, 8 per slice and part, a counter per slice
     int diag_parts = 1;               // blocks per slice
-    mutable bool waits = false;       // a kernel with bounded waits ran since its error word was last read
+    mutable bool waits = false;       // a kernel with bounded waits was launched (or captured: a graph may run it again)
     void* psi_ws = nullptr;           // two-belt force and two-kernel step: psi of the state being stepped
     bool ws_moments = false;          // two-kernel step: the moments are in front of it
     int* dev_err = nullptr;           // device error word of the bounded waits
@@ -505,14 +505,13 @@ lbm_status ensure_scratch(lbm_ctx* c, size_t bytes) {
 
 // Read and clear the device error word: a bounded device wait that timed out
 // leaves the populations invalid.
-// Only the bulk- and tensor-copy kernels wait; without one since the last
-// reading there is nothing to read and nothing to wait for.
+// Only the bulk- and tensor-copy kernels wait; a context that never launched
+// one has nothing to read and nothing to wait for.
 lbm_status check_device_error(lbm_ctx* c) {
     if (!c->waits) return LBM_OK;
     int e = 0;
     LBM_CUDA(c, cudaMemcpyAsync(&e, c->dev_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-    c->waits = false;
     if (e) {
         LBM_CUDA(c, cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream));
         return c->fail(LBM_ETIMEOUT, "a bounded device wait of the step kernel timed out; the populations are invalid");
