@@ -1,5 +1,5 @@
-// Per-thread part of the ligament diagnostics, shared by lbm_diag and
-// lbm_diag_noalloc so that both give the same numbers.
+// The sums of the ligament diagnostics, shared by lbm_diag and
+// lbm_diag_noalloc so that both give the same numbers, to the last bit.
 //
 // Each cell's rho and j come from its 19 populations in the codec's
 // arithmetic type (float for 32- and 16-bit storage, double for FP64).  The
@@ -10,6 +10,8 @@
 // GPU issues at a small fraction of the FP32 rate and bounded the per-cell
 // form.  The order of all sums is fixed, so results are deterministic.
 #pragma once
+#include <algorithm>
+
 #include "codec.cuh"
 #include "lattice.cuh"
 
@@ -38,6 +40,20 @@ __device__ __forceinline__ void diag_cell(const typename Codec::S* __restrict__ 
     jz = az;
 }
 
+constexpr int kDiagThreads = 256;
+constexpr int kDiagRun = 8;
+constexpr int kDiagRunCells = kDiagRun * kDiagThreads;  // cells of one run of every thread
+
+// Parts that a slice is summed in, one block each: about 8 blocks an SM over all
+// slices, at least one run of cells a part, and, for more than one part, at most
+// kDiagMaxParts in all (152 SMs ask for 2430 at most).
+constexpr int kDiagMaxParts = 4096;
+inline int diag_parts(long long plane, int nz, int num_sms) {
+    const long long runs = (plane + kDiagRunCells - 1) / kDiagRunCells, want = (8LL * num_sms + nz - 1) / nz;
+    const long long most = nz < kDiagMaxParts ? kDiagMaxParts / nz : 1;
+    return int(std::min(std::min(want, runs), most));
+}
+
 // Cells first, first + stride, ... < count (in runs of kRun of them; with
 // parts > 1 only every parts-th run from the part-th on, so that several
 // blocks share a slice without changing what a run sums) of the slice whose
@@ -50,7 +66,7 @@ __device__ __forceinline__ void diag_accumulate(const typename Codec::S* __restr
                                                 double rho_v, double inv, const float* __restrict__ refz,
                                                 double (&acc)[7], int part = 0, int parts = 1) {
     using R = typename Codec::R;
-    constexpr int kRun = 8;
+    constexpr int kRun = kDiagRun;
     for (int k = 0; k < 7; ++k) acc[k] = 0.0;
     const R rv = R(rho_v), iv = R(inv);
     for (long long i = first + (long long)part * kRun * stride; i < count; i += (long long)parts * kRun * stride) {
@@ -81,6 +97,33 @@ __device__ __forceinline__ void diag_accumulate(const typename Codec::S* __restr
         acc[5] = fmax(acc[5], double(mx));
         acc[6] += double(bad);
     }
+}
+
+__device__ __forceinline__ double diag_join(int k, double a, double b) { return k == 5 ? fmax(a, b) : a + b; }
+
+// One block's sum of a part of a slice, by a fixed tree: threads 0 .. 6 return
+// quantity threadIdx.x of `acc`'s order.
+template <class Codec>
+__device__ __forceinline__ double diag_part(const typename Codec::S* __restrict__ fz, long long n, long long plane,
+                                            const DevParams& dev, double rho_l, double rho_v,
+                                            const float* __restrict__ refz, int part, int parts) {
+    __shared__ double red[7][kDiagThreads / 32];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double acc[7];
+    diag_accumulate<Codec>(fz, n, plane, threadIdx.x, kDiagThreads, dev, rho_v, 1.0 / (rho_l - rho_v), refz, acc, part,
+                           parts);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        for (int s = 16; s > 0; s >>= 1) acc[k] = diag_join(k, acc[k], __shfl_down_sync(0xffffffffu, acc[k], s));
+        if (lane == 0) red[k][warp] = acc[k];
+    }
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < 7) {
+        v = red[threadIdx.x][0];
+        for (int w = 1; w < kDiagThreads / 32; ++w) v = diag_join(threadIdx.x, v, red[threadIdx.x][w]);
+    }
+    return v;
 }
 
 }  // namespace lbm

@@ -27,66 +27,58 @@ using namespace lbm;
 namespace {
 
 constexpr int kMaxNz = LBM_NOALLOC_MAX_NZ;
-constexpr int kThreads = 256;
 constexpr int kMaxDevices = 64;
 
-// Per-slice partials, quantity-major: slot k*kMaxNz + z with k = 0 mass,
-// 1..3 momentum, 4 liquid area, 5 max rho, 6 bad cells; then the 4 totals
+// Per-slice sums, quantity-major: row k*kMaxNz with k = 0 mass,
+// 1..3 momentum, 4 liquid area, 5 max rho, 6 bad cells (parts of slices and the
+// slices' sums, see below); then the 4 totals
 // (mass, momentum) and the total bad-cell count at 7*kMaxNz.
 static __device__ __align__(256) double g_noalloc_scratch[8 * kMaxNz];
 
 std::mutex g_setup_mutex;
 double* g_scratch_ptr[kMaxDevices] = {nullptr};
 
-// One block per z slice, fixed-order tree reduction in float64 (the same
-// per-slice arithmetic as the context-based diagnostics), written into the
-// quantity-major scratch layout.
+// A z slice in the parts in which the context-based diagnostics sum it, one
+// block each: part i of slice z at slot parts * z + i of the quantity-major
+// scratch layout.
 template <class Codec>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kDiagThreads)
 slice_diag_noalloc_kernel(double* __restrict__ scratch, const typename Codec::S* __restrict__ f, int nx, int ny,
                           long long n, double rho_l, double rho_v, DevParams dev) {
-    __shared__ double red[7][kThreads];
-    const int z = blockIdx.x;
+    const int z = blockIdx.x, parts = gridDim.y;
     const long long plane = (long long)nx * ny;
-    double acc[7];
-    diag_accumulate<Codec>(f + z * plane, n, plane, threadIdx.x, kThreads, dev, rho_v, 1.0 / (rho_l - rho_v),
-                           nullptr, acc);
-    const double m = acc[0], jx = acc[1], jy = acc[2], jz = acc[3], area = acc[4], mx = acc[5], bad = acc[6];
-    red[0][threadIdx.x] = m;
-    red[1][threadIdx.x] = jx;
-    red[2][threadIdx.x] = jy;
-    red[3][threadIdx.x] = jz;
-    red[4][threadIdx.x] = area;
-    red[5][threadIdx.x] = mx;
-    red[6][threadIdx.x] = bad;
-    __syncthreads();
-    for (int s = kThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            for (int k = 0; k < 7; ++k) {
-                if (k == 5) red[k][threadIdx.x] = fmax(red[k][threadIdx.x], red[k][threadIdx.x + s]);
-                else red[k][threadIdx.x] += red[k][threadIdx.x + s];
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 7) scratch[threadIdx.x * kMaxNz + z] = red[threadIdx.x][0];
+    const double sum = diag_part<Codec>(f + z * plane, n, plane, dev, rho_l, rho_v, nullptr, blockIdx.y, parts);
+    if (threadIdx.x < 7) scratch[threadIdx.x * kMaxNz + parts * z + blockIdx.y] = sum;
 }
 
-// Totals over slices, summed in z order by one thread (deterministic), into
-// scratch[7*kMaxNz + 0..4]; optionally copies the per-slice area / max rho and
+// Slices of several parts: their sums, in turn, to slot kJoined + z (both fit:
+// several parts are kDiagMaxParts in all at most).
+constexpr int kJoined = kDiagMaxParts;
+static_assert(2 * kDiagMaxParts <= kMaxNz, "parts and joined slices in one scratch row");
+__global__ void join_parts_noalloc_kernel(double* __restrict__ scratch, int nz, int parts) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 7 * nz; i += gridDim.x * blockDim.x) {
+        const int k = i / nz, z = i - k * nz;
+        const double* const p = scratch + k * kMaxNz + parts * z;
+        double v = p[0];
+        for (int j = 1; j < parts; ++j) v = diag_join(k, v, p[j]);
+        scratch[k * kMaxNz + kJoined + z] = v;
+    }
+}
+
+// Totals over slices (slot z of `rows`), summed in z order by one thread (deterministic), into
+// tot[0..4]; optionally copies the per-slice area / max rho and
 // the totals to caller device arrays.
-__global__ void totals_noalloc_kernel(double* __restrict__ scratch, int nz, double* mass, double* mom,
-                                      double* area_z, double* maxrho_z) {
+__global__ void totals_noalloc_kernel(const double* __restrict__ rows, double* __restrict__ tot, int nz, double* mass,
+                                      double* mom, double* area_z, double* maxrho_z) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         double m = 0, jx = 0, jy = 0, jz = 0, bad = 0;
         for (int z = 0; z < nz; ++z) {
-            m += scratch[0 * kMaxNz + z];
-            jx += scratch[1 * kMaxNz + z];
-            jy += scratch[2 * kMaxNz + z];
-            jz += scratch[3 * kMaxNz + z];
-            bad += scratch[6 * kMaxNz + z];
+            m += rows[0 * kMaxNz + z];
+            jx += rows[1 * kMaxNz + z];
+            jy += rows[2 * kMaxNz + z];
+            jz += rows[3 * kMaxNz + z];
+            bad += rows[6 * kMaxNz + z];
         }
-        double* tot = scratch + 7 * kMaxNz;
         tot[0] = m;
         tot[1] = jx;
         tot[2] = jy;
@@ -100,8 +92,8 @@ __global__ void totals_noalloc_kernel(double* __restrict__ scratch, int nz, doub
         }
     }
     for (int z = blockIdx.x * blockDim.x + threadIdx.x; z < nz; z += gridDim.x * blockDim.x) {
-        if (area_z) area_z[z] = scratch[4 * kMaxNz + z];
-        if (maxrho_z) maxrho_z[z] = scratch[5 * kMaxNz + z];
+        if (area_z) area_z[z] = rows[4 * kMaxNz + z];
+        if (maxrho_z) maxrho_z[z] = rows[5 * kMaxNz + z];
     }
 }
 
@@ -125,9 +117,9 @@ cudaError_t scratch_address(double** out) {
 
 template <class Codec>
 cudaError_t launch_slices(double* scratch, const void* f, int nx, int ny, int nz, double rho_l, double rho_v,
-                          const DevParams& dev, cudaStream_t st) {
-    slice_diag_noalloc_kernel<Codec><<<nz, kThreads, 0, st>>>(scratch, static_cast<const typename Codec::S*>(f),
-                                                              nx, ny, (long long)nx * ny * nz, rho_l, rho_v, dev);
+                          const DevParams& dev, int parts, cudaStream_t st) {
+    slice_diag_noalloc_kernel<Codec><<<dim3(nz, parts), kDiagThreads, 0, st>>>(
+        scratch, static_cast<const typename Codec::S*>(f), nx, ny, (long long)nx * ny * nz, rho_l, rho_v, dev);
     return cudaGetLastError();
 }
 
@@ -146,25 +138,31 @@ extern "C" lbm_status lbm_diag_noalloc(const void* f, int storage, int nx, int n
     double* scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     if (e != cudaSuccess) return LBM_ECUDA;
+    int device = 0, num_sms = 0;
+    e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return LBM_ECUDA;
+    const int parts = diag_parts((long long)nx * ny, nz, num_sms);
     const DevParams dev = make_dev_params(rho_ref, dev_scale > 0 ? dev_scale : 1.0);
     switch (storage) {
-        case LBM_F64: e = launch_slices<CodecF64>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, st); break;
-        case LBM_F32: e = launch_slices<CodecF32>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, st); break;
-        case LBM_F16_DEV: e = launch_slices<CodecF16Dev>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, st); break;
-        default: e = launch_slices<CodecBF16Dev>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, st); break;
+        case LBM_F64: e = launch_slices<CodecF64>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, parts, st); break;
+        case LBM_F32: e = launch_slices<CodecF32>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, parts, st); break;
+        case LBM_F16_DEV: e = launch_slices<CodecF16Dev>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, parts, st); break;
+        default: e = launch_slices<CodecBF16Dev>(scratch, f, nx, ny, nz, rho_l, rho_v, dev, parts, st); break;
     }
     if (e != cudaSuccess) return LBM_ECUDA;
-    const int tb = 256, tg = (nz + tb - 1) / tb;
-    if (on_device) totals_noalloc_kernel<<<tg, tb, 0, st>>>(scratch, nz, mass, mom, area_z, maxrho_z);
-    else totals_noalloc_kernel<<<tg, tb, 0, st>>>(scratch, nz, nullptr, nullptr, nullptr, nullptr);
+    const int tb = 256, tg = (nz + tb - 1) / tb, at = parts > 1 ? kJoined : 0;
+    if (parts > 1) join_parts_noalloc_kernel<<<(7 * nz + tb - 1) / tb, tb, 0, st>>>(scratch, nz, parts);
+    if (on_device) totals_noalloc_kernel<<<tg, tb, 0, st>>>(scratch + at, scratch + 7 * kMaxNz, nz, mass, mom, area_z, maxrho_z);
+    else totals_noalloc_kernel<<<tg, tb, 0, st>>>(scratch + at, scratch + 7 * kMaxNz, nz, nullptr, nullptr, nullptr, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return LBM_ECUDA;
     double tot[5];
     e = cudaMemcpyAsync(tot, scratch + 7 * kMaxNz, sizeof(tot), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess && !on_device) {
-        if (area_z) e = cudaMemcpyAsync(area_z, scratch + 4 * kMaxNz, sizeof(double) * nz, cudaMemcpyDeviceToHost, st);
+        if (area_z) e = cudaMemcpyAsync(area_z, scratch + 4 * kMaxNz + at, sizeof(double) * nz, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess && maxrho_z)
-            e = cudaMemcpyAsync(maxrho_z, scratch + 5 * kMaxNz, sizeof(double) * nz, cudaMemcpyDeviceToHost, st);
+            e = cudaMemcpyAsync(maxrho_z, scratch + 5 * kMaxNz + at, sizeof(double) * nz, cudaMemcpyDeviceToHost, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return LBM_ECUDA;

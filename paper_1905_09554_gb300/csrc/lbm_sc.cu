@@ -313,35 +313,19 @@ __global__ void velocity_kernel(double* __restrict__ ux, double* __restrict__ uy
 // area, 5 max rho, 6 count of cells with rho <= 0 or non-finite.  With one
 // block per slice 144 slices of 64 x 64 took 21 us (half the SMs idle, 2.1 TB/s);
 // bound by HBM for boxes beyond L2 (76 B a cell in FP32).
-constexpr int DIAG_THREADS = 256;
-constexpr int DIAG_RUN_CELLS = 8 * DIAG_THREADS;  // cells of one run of every thread
-
-__device__ __forceinline__ double diag_join(int k, double a, double b) { return k == 5 ? fmax(a, b) : a + b; }
-
 template <class Codec>
-__global__ void __launch_bounds__(DIAG_THREADS)
+__global__ void __launch_bounds__(kDiagThreads)
 diag_kernel(double* __restrict__ out, double* __restrict__ part, unsigned* __restrict__ done,
             const typename Codec::S* __restrict__ f, int nx, int ny, long long n, double rho_l, double rho_v,
             DevParams dev, const float* ref) {
-    __shared__ double red[7][DIAG_THREADS / 32];
     __shared__ bool last;
-    const int z = blockIdx.x, parts = gridDim.y, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int z = blockIdx.x, parts = gridDim.y;
     const long long plane = (long long)nx * ny;
-    double acc[7];
-    diag_accumulate<Codec>(f + z * plane, n, plane, threadIdx.x, DIAG_THREADS, dev, rho_v, 1.0 / (rho_l - rho_v),
-                           Codec::kLocal ? ref + z * plane : nullptr, acc, blockIdx.y, parts);
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        for (int s = 16; s > 0; s >>= 1) acc[k] = diag_join(k, acc[k], __shfl_down_sync(0xffffffffu, acc[k], s));
-        if (lane == 0) red[k][warp] = acc[k];
-    }
-    __syncthreads();
+    const double sum = diag_part<Codec>(f + z * plane, n, plane, dev, rho_l, rho_v,
+                                        Codec::kLocal ? ref + z * plane : nullptr, blockIdx.y, parts);
     if (threadIdx.x < 7) {
-        const int k = threadIdx.x;
-        double v = red[k][0];
-        for (int w = 1; w < DIAG_THREADS / 32; ++w) v = diag_join(k, v, red[k][w]);
-        if (parts == 1) out[8 * z + k] = v;
-        else part[8 * ((long long)parts * z + blockIdx.y) + k] = v;
+        if (parts == 1) out[8 * z + threadIdx.x] = sum;
+        else part[8 * ((long long)parts * z + blockIdx.y) + threadIdx.x] = sum;
     }
     if (parts == 1) return;
     __threadfence();
@@ -1147,11 +1131,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
         }
         c->own_bytes += 2 * (long long)rbytes;
     }
-    {   // about 8 blocks an SM in all, at least one run of cells each
-        const long long plane = (long long)p->nx * p->ny, runs = (plane + DIAG_RUN_CELLS - 1) / DIAG_RUN_CELLS;
-        const long long want = (8LL * c->num_sms + p->nz - 1) / p->nz;
-        c->diag_parts = int(want < runs ? want : runs);
-    }
+    c->diag_parts = diag_parts((long long)p->nx * p->ny, p->nz, c->num_sms);
     e = cudaMalloc(&c->diag, sizeof(double) * diag_doubles(c));
     if (e == cudaSuccess) e = cudaMemsetAsync(c->diag, 0, sizeof(double) * diag_doubles(c), c->stream);
     if (e != cudaSuccess) {
@@ -1635,7 +1615,7 @@ lbm_status lbm_diag(lbm_ctx* c, double rho_l, double rho_v, double* mass, double
     const auto& p = c->p;
     with_codec(c, [&](auto codec) {
         using C = decltype(codec);
-        diag_kernel<C><<<dim3(p.nz, c->diag_parts), DIAG_THREADS, 0, c->stream>>>(
+        diag_kernel<C><<<dim3(p.nz, c->diag_parts), kDiagThreads, 0, c->stream>>>(
             c->diag, c->diag + 8 * (size_t)p.nz, reinterpret_cast<unsigned*>(c->diag + diag_doubles(c) - p.nz),
             static_cast<const typename C::S*>(c->f[c->cur]), p.nx, p.ny, c->n, rho_l, rho_v, c->args.dev,
             c->ref[c->cur]);
