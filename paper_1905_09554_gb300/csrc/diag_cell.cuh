@@ -44,14 +44,18 @@ constexpr int kDiagThreads = 256;
 constexpr int kDiagRun = 8;
 constexpr int kDiagRunCells = kDiagRun * kDiagThreads;  // cells of one run of every thread
 
-// Parts that a slice is summed in, one block each: about 8 blocks an SM over all
-// slices, at least one run of cells a part, and, for more than one part, at most
-// kDiagMaxParts in all (152 SMs ask for 2430 at most).
+// Parts that a slice is summed in, one block each: as many as leave 3.5 blocks an
+// SM over all slices, so that one round of blocks takes them all, at least one run
+// of cells a part, and, for more than one part, at most kDiagMaxParts in all.
+// us a call of lbm_diag with one part / 8 blocks an SM rounded up / this rule:
+//   FP32 64x64x144 48.9 / 41.0 / 42.2, 128x128x288 109.5 / 136.7 / 100.8, 256x256x575 563 / 580 / 544,
+//   300x200x100 230 / 156 / 133, 384x384x300 634 / 652 / 616; FP64 128x128x288 614 / 629 / 603
+// (the one part by a tree in shared memory).
 constexpr int kDiagMaxParts = 4096;
 inline int diag_parts(long long plane, int nz, int num_sms) {
-    const long long runs = (plane + kDiagRunCells - 1) / kDiagRunCells, want = (8LL * num_sms + nz - 1) / nz;
+    const long long runs = (plane + kDiagRunCells - 1) / kDiagRunCells, want = 7LL * num_sms / (2LL * nz);
     const long long most = nz < kDiagMaxParts ? kDiagMaxParts / nz : 1;
-    return int(std::min(std::min(want, runs), most));
+    return int(std::max(1LL, std::min(std::min(want, runs), most)));
 }
 
 // Cells first, first + stride, ... < count (in runs of kRun of them; with
