@@ -62,7 +62,7 @@ enum { LBM_F64 = 0,                            /* populations stored as double  
 enum { LBM_FORM_AUTO = 0,
        LBM_FORM_ONE_KERNEL = 1,                /* the kernel and launch shape of lbm_kernel_config */
        LBM_FORM_TWO_KERNELS = 2,               /* psi (and moments) first, then collision and push */
-       LBM_FORM_MOMENTS = 3 };                 /* calls of n >= 2: moments between the steps      */
+       LBM_FORM_MOMENTS = 3 };                 /* calls of several: moments between the steps     */
 
 typedef struct {
     int lattice;          /* LBM_D3Q19                                              */
@@ -200,7 +200,7 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int on_device);
  * Enqueues the kernels of n steps and returns.  n steps in one call give the
  * same bits as n calls of one step, in the same population copy.  Unless a
  * kernel or a launch shape was asked for, and with 32- or 16-bit storage, a
- * call of n >= 2 steps of an operator whose result follows from a few moments (SRT at tau = 1; MRT
+ * call of enough steps (2 for most boxes at tau = 1) of an operator whose result follows from a few moments (SRT at tau = 1; MRT
  * with every rate 1; FP32 MRT with its rates at 1 outside e, 3pxx, pww and the
  * off-diagonal stress) reads the populations once, keeps 4, 9 or 10 moments
  * between the steps (in the two copies themselves) and writes the populations
@@ -218,11 +218,13 @@ lbm_status lbm_step(lbm_ctx *ctx, long n);
 int lbm_step_form(const lbm_ctx *ctx, long n);
 
 /* Choose the forms of later calls: single for n = 1 (LBM_FORM_AUTO,
- * LBM_FORM_ONE_KERNEL or LBM_FORM_TWO_KERNELS), several for n >= 2 (any).  May
- * allocate what a form needs.  LBM_EINVAL for an unknown form or a box of a
+ * LBM_FORM_ONE_KERNEL or LBM_FORM_TWO_KERNELS), several for n >= 2 (any).
+ * LBM_FORM_MOMENTS holds for n >= moments_from (2 if less), shorter calls then
+ * step in the form of `single`; moments_from is ignored otherwise.  May allocate what a form needs.  LBM_EINVAL for an unknown form or a box of a
  * batch, LBM_EUNSUPPORTED for a form that cannot serve this lattice (or has no
  * room); the forms are then unchanged. */
-lbm_status lbm_set_step_forms(lbm_ctx *ctx, int single, int several);
+lbm_status lbm_set_step_forms(lbm_ctx *ctx, int single, int several,
+                              long moments_from);
 
 /* Steps taken since the last initialisation. */
 long lbm_time(const lbm_ctx *ctx);
@@ -327,8 +329,9 @@ lbm_status lbm_set_kernel_config(lbm_ctx *ctx, int kernel, int tile_y,
  * steps advance whatever state the context holds (its step counter does not
  * change): tune before setting the initial state.  Then the two-kernel step
  * (where lbm_step would choose it) is timed against the fastest shape, and the
- * moment form (trial_steps steps a call, at least 8) against the faster of the
- * two, and what is faster stays (lbm_step_form).  Outputs (any may be NULL):
+ * moment form (calls of trial_steps, at least 8, and of twice as many) against
+ * the faster of the two, and what is faster stays, the moment form from the
+ * number of steps on that makes up for its ends (lbm_step_form).  Outputs (any may be NULL):
  * the chosen kernel, tile height and z chunk, and the time per step in ms of a
  * call of one step.  Returns LBM_ECUDA if no candidate ran. */
 lbm_status lbm_tune(lbm_ctx *ctx, int trial_steps, int *kernel, int *tile_y,
@@ -399,13 +402,14 @@ lbm_status lbm_batch_step(lbm_batch *b, long n);
 /* The form (LBM_FORM_*) that lbm_batch_step(b, n) takes, and the choice of it,
  * as lbm_step_form and lbm_set_step_forms for one lattice. */
 int lbm_batch_step_form(const lbm_batch *b, long n);
-lbm_status lbm_batch_set_step_forms(lbm_batch *b, int single, int several);
+lbm_status lbm_batch_set_step_forms(lbm_batch *b, int single, int several,
+                                    long moments_from);
 
 /* Autotune the launch shape: times trial_steps steps of the one-kernel form for
  * each tile height in {4, 8, 16} and z chunk in {8, 16, 24, 32, 48, 64} and
  * keeps the fastest; then the two-kernel form (FP64) against it and the moment
- * form (trial_steps steps a call, at least 8) against the faster of the two, and
- * keeps what is faster (lbm_batch_step_form).  Reports the shape and the time
+ * form against the faster of the two as lbm_tune does, and keeps what is faster
+ * (lbm_batch_step_form).  Reports the shape and the time
  * per step of a call of one step (any pointer may be NULL).  The trial steps
  * overwrite the populations: tune first, then initialise the boxes. */
 lbm_status lbm_batch_tune(lbm_batch *b, int trial_steps, int *tile_y,

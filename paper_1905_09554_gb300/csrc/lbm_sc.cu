@@ -25,6 +25,15 @@ using namespace lbm;
 
 struct lbm_batch;
 
+// How a call steps (LBM_FORM_*): of one step; of 2 .. from - 1 steps; of at
+// least `from` steps.  The middle one is LBM_FORM_MOMENTS for none.
+struct Forms {
+    int single = LBM_FORM_ONE_KERNEL, few = LBM_FORM_ONE_KERNEL, several = LBM_FORM_ONE_KERNEL;
+    long from = 2;
+    int of(long n) const { return n < 2 ? single : (n < from ? few : several); }
+    static Forms every(int form) { return {form, form, form, 2}; }
+};
+
 struct lbm_ctx {
     lbm_params p;
     cudaStream_t stream = nullptr;
@@ -54,8 +63,7 @@ struct lbm_ctx {
     int grid3 = 0;                    // kernel 5: grid of the pipelined kernel used for other buffers
     int coll = COLL_SRT;              // collision kernel (COLL_*)
     int grid = 0;                     // persistent grid size (kernels 2, 3)
-    // How a call of one step, and one of several, steps (LBM_FORM_*).
-    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};
+    Forms forms;
     // Calls of several steps through the moment fields (step_moment.cuh):
     // launch shape, or mom == nullptr where that is not set up or only
     // populations will do.
@@ -896,18 +904,59 @@ bool split_wanted(const lbm_ctx* c) {
     return c->p.storage == LBM_F64 || c->n <= split_cells(c->p, split_by_moments(c));
 }
 
+// Steps from which on a call through the moment fields is faster than `rival`
+// us a step, or 0 if it never is.  A step of the moment kernel costs its busiest
+// block's planes, the ends (gather, and populations written by the last step
+// instead of moments) their bytes; odd rows cost more in both.  Measured, us:
+//   a plane of the busiest block, 64 x 64 x 128 (9 or 11 planes) to 256 x 256 x 200 (112 or 176): FP32 SRT 1.38 to
+//     1.49, unit-rate MRT 1.50 to 1.59, shear rule 1.58 to 1.81, paper's rule 1.67 to 1.87; 16-bit SRT 1.71 to 1.89,
+//     MRT 1.80 to 1.97; 255 x 255 x 200 1.17 to 1.24 times these; 10 us a launch at least
+//   ends, ps a cell, even / odd rows: FP32 4 fields 16 to 23 / 43, 9 fields 21 / 25, 10 fields 35 / 37; 16-bit 11 to
+//     14 / 25; batches of small boxes 22 to 28, 47 to 80 and 45 to 69
+// so that calls of 2 steps of 256 x 256 x 200 take 607 us for SRT (two steps of one kernel: 780), but 1051 (800) with
+// 10 fields, where 6 steps break even; 24 boxes of 32 x 32 with 10 fields never do (94 us a step, one kernel 80).
+long moments_pay_from(int storage, int coll, long long cells, bool odd, bool batch, long long busiest, double rival) {
+    const bool f32 = storage == LBM_F32;
+    const double plane = !f32 ? (coll == COLL_SRT ? 1.8 : 1.85)
+                              : (coll == COLL_SRT ? 1.45 : (coll == COLL_MRT_UNIT ? 1.55 : (coll == COLL_MRT_SHEAR ? 1.6 : 1.7)));
+    const double batched = !batch ? 1.0 : (moments_of_operator(coll) > 4 ? 2.2 : 1.2);
+    const double end = !f32 ? (odd ? 25.0 : 12.5)
+                            : (coll == COLL_MRT_SHEAR ? (odd ? 25.0 : 21.0) : (coll == COLL_MRT_SPARSE ? (odd ? 37.0 : 35.0) : (odd ? 43.0 : 21.0)));
+    const double step = std::max(10.0, plane * (odd ? 1.2 : 1.0) * double(busiest)), gain = rival - step;
+    if (gain <= 0.0) return 0;
+    const double n = std::ceil(end * batched * 1e-6 * double(cells) / gain);
+    return n > 1e9 ? 0 : (n < 2.0 ? 2 : long(n));
+}
+
+// us of a step in one kernel and in two.  FP32: 2.2 us a plane of the busiest block (256 x 256 x 200 390 us, 128^3
+// 74, 160 x 150 x 200 152); 16-bit storage 31 ps a cell (364 to 388, 65 to 74, 149 to 165), 20 us at least.  Two
+// kernels: up to 400,000 cells (launched without gaps) 24 x 24 x 48 4.2 us, 48 x 48 x 96 7.9; beyond, 64 x 64 x 128
+// 20.6, 96^3 28 to 38, 255 x 255 x 200 in FP16 409 to 431, from local references 458 to 498.
+double one_kernel_us(const lbm_ctx* c) {
+    double us = 31e-6 * double(c->n);
+    if (c->p.storage == LBM_F32 && c->kernel == 3) {
+        const long long tiles = (long long)((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y);
+        us = 2.2 * double(busiest_block_planes(c->p.nz, tiles, c->grid, c->zchunk));
+    }
+    return us < 20.0 ? 20.0 : us;
+}
+double two_kernels_us(const lbm_ctx* c) {
+    const double n = double(c->n);
+    if (n <= 400000) return 3.7 + 19e-6 * n;
+    const bool odd16 = c->p.storage >= LBM_F16_DEV && c->p.nx % 2 != 0;
+    return 4.5 + (!odd16 ? 29.5e-6 : (c->p.storage >= LBM_F16_LOCAL ? 36e-6 : 32e-6)) * n;
+}
+
 // Launch shape of the moment kernels (step_moment.cuh), where the collision
-// has a moment form and its fields fit into a population copy; false elsewhere,
-// and (rival: the box can step in two kernels) where two kernels are expected to
-// be faster: a turn of the moment kernel (one plane of the busiest block) takes
-// about 1.5 us however few blocks there are, two kernels 29 ps a cell and 4 us at
-// least (24x24x48: 10.4 / 4.2 us a step; 64x64x128: 14.7 / 20.5; MRT with the
-// paper's rates 48x48x96: 20.9 / 10.9, 80x80x160: 52.4 / 41.1, 96x96x192: 55.6 / 77).
-bool prepare_moments(lbm_ctx* c, bool rival) {
-    auto slower = [&](long long busiest) {
-        return rival && 2.5 + 1.5 * double(busiest) > 4.0 + 29e-6 * double(c->n);
+// has a moment form and its fields fit into a population copy; false elsewhere.
+// from: set to moments_pay_from() against `rival`, and false where that is 0
+// (nullptr: not asked).
+bool prepare_moments(lbm_ctx* c, double rival = 0.0, long* from = nullptr) {
+    auto pays = [&](long long busiest) {
+        if (from) *from = moments_pay_from(c->p.storage, c->coll, c->n, c->p.nx % 2 != 0, false, busiest, rival);
+        return !from || *from > 0;
     };
-    if (c->mom) return !slower(c->mom_busiest);
+    if (c->mom) return pays(c->mom_busiest);
     const lbm_params& p = c->p;
     if (p.G2 != 0.0 || p.nx < 4) return false;
     if (c->coll == COLL_SRT && p.tau != 1.0) return false;  // keeps (1 - omega) f: all 19 populations
@@ -929,7 +978,7 @@ bool prepare_moments(lbm_ctx* c, bool rival) {
     l.args.tiles_x = (p.nx + k->tile_x - 1) / k->tile_x;
     const int tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
     const MomentPlan plan = plan_moments({{tiles, p.nz}}, (long long)per_sm * c->num_sms, k->fields, c->mom_bytes);
-    if (slower(plan.busiest)) return false;
+    if (!pays(plan.busiest)) return false;
     c->mom_busiest = plan.busiest;
     size_t bytes = 0;
     if (upload_plan(plan, l, &c->mom_plan, &bytes, c->stream) != cudaSuccess) {  // no room: step the populations
@@ -947,11 +996,45 @@ bool prepare_moments(lbm_ctx* c, bool rival) {
 
 // The forms of a context for which no particular kernel or launch shape was
 // asked.
-void choose_forms(lbm_ctx* c, int (&form)[2]) {
-    form[0] = form[1] = LBM_FORM_ONE_KERNEL;
-    if (c->p.G2 != 0.0) return;
-    if (split_wanted(c) && prepare_split(c)) form[0] = form[1] = LBM_FORM_TWO_KERNELS;
-    if (prepare_moments(c, form[1] == LBM_FORM_TWO_KERNELS)) form[1] = LBM_FORM_MOMENTS;
+Forms choose_forms(lbm_ctx* c) {
+    Forms f;
+    if (c->p.G2 != 0.0) return f;
+    if (split_wanted(c) && prepare_split(c)) f = Forms::every(LBM_FORM_TWO_KERNELS);
+    const double rival = f.few == LBM_FORM_TWO_KERNELS ? two_kernels_us(c) : one_kernel_us(c);
+    long from = 0;
+    if (prepare_moments(c, rival, &from)) {
+        f.several = LBM_FORM_MOMENTS;
+        f.from = from;
+    }
+    return f;
+}
+
+// Tuners: the moment form from the calls on that it is faster for, given ms a
+// step of `few` and of calls of n and 2 n steps through the moments (< 0: did
+// not run).
+void moments_from(Forms& f, float few, int n, float short_call, float long_call) {
+    if (short_call < 0.0f || long_call < 0.0f) return;
+    const double step = 2.0 * long_call - short_call, ends = 2.0 * n * (double(short_call) - long_call);
+    if (!(step < few)) return;
+    const double from = std::ceil(ends / (few - step));
+    if (from > 1e6) return;
+    f.several = LBM_FORM_MOMENTS;
+    f.from = from < 2.0 ? 2 : long(from);
+}
+
+// `automatic` with the forms that were asked for; false for an unknown one.
+bool asked_forms(Forms& f, const Forms& automatic, int single, int several, long from) {
+    if (single < LBM_FORM_AUTO || single > LBM_FORM_TWO_KERNELS || several < LBM_FORM_AUTO || several > LBM_FORM_MOMENTS)
+        return false;
+    f = automatic;
+    if (single != LBM_FORM_AUTO) f.single = single;
+    if (several != LBM_FORM_AUTO) {
+        f.several = several;
+        if (several != LBM_FORM_MOMENTS) f.few = several;
+        else if (single != LBM_FORM_AUTO) f.few = single;
+        f.from = several == LBM_FORM_MOMENTS && from > 2 ? from : 2;
+    }
+    return true;
 }
 
 // n >= 2 steps from the populations in f[from] through the moment fields.  The
@@ -1195,7 +1278,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
         }
     }
 
-    if (p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) choose_forms(c, c->form);
+    if (p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) c->forms = choose_forms(c);
 
     e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1283,28 +1366,23 @@ lbm_status lbm_set_kernel_config(lbm_ctx* c, int kernel, int tile_y, int zchunk)
         return c->fail(st, "lbm_set_kernel_config: %s", why);
     }
     // a kernel or shape that was asked for is the one that steps
-    if (kernel || tile_y || zchunk) c->form[0] = c->form[1] = LBM_FORM_ONE_KERNEL;
-    else choose_forms(c, c->form);
+    c->forms = kernel || tile_y || zchunk ? Forms() : choose_forms(c);
     return LBM_OK;
 }
 
-int lbm_step_form(const lbm_ctx* c, long n) { return c && n >= 1 ? c->form[n >= 2] : 0; }
+int lbm_step_form(const lbm_ctx* c, long n) { return c && n >= 1 ? c->forms.of(n) : 0; }
 
-lbm_status lbm_set_step_forms(lbm_ctx* c, int single, int several) {
+lbm_status lbm_set_step_forms(lbm_ctx* c, int single, int several, long moments_from) {
     if (!c) return LBM_EINVAL;
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_set_step_forms: this context is a box of a batch");
-    if (single < LBM_FORM_AUTO || single > LBM_FORM_TWO_KERNELS || several < LBM_FORM_AUTO || several > LBM_FORM_MOMENTS)
+    Forms f;
+    if (!asked_forms(f, choose_forms(c), single, several, moments_from))
         return c->fail(LBM_EINVAL, "lbm_set_step_forms: unknown form (%d, %d)", single, several);
-    int form[2];
-    choose_forms(c, form);
-    if (single != LBM_FORM_AUTO) form[0] = single;
-    if (several != LBM_FORM_AUTO) form[1] = several;
-    if ((form[0] == LBM_FORM_TWO_KERNELS || form[1] == LBM_FORM_TWO_KERNELS) && !prepare_split(c))
+    if ((f.single == LBM_FORM_TWO_KERNELS || f.few == LBM_FORM_TWO_KERNELS) && !prepare_split(c))
         return c->fail(LBM_EUNSUPPORTED, "lbm_set_step_forms: this lattice cannot step in two kernels");
-    if (form[1] == LBM_FORM_MOMENTS && !prepare_moments(c, false))
+    if (f.several == LBM_FORM_MOMENTS && !prepare_moments(c))
         return c->fail(LBM_EUNSUPPORTED, "lbm_set_step_forms: this lattice cannot step through moment fields");
-    c->form[0] = form[0];
-    c->form[1] = form[1];
+    c->forms = f;
     return LBM_OK;
 }
 
@@ -1359,7 +1437,7 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
             pick = sh;
         }
     }
-    // the other forms, as lbm_step runs them; fewer than 8 steps at once would time the moment form's ends
+    // the other forms, as lbm_step runs them
     const int cur = c->cur;
     auto timed = [&](int n, auto&& run) {
         if (run(2) != cudaSuccess) return -1.0f;  // warm-up
@@ -1371,31 +1449,33 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
         cudaEventElapsedTime(&ms, e0, e1);
         return ms / n;
     };
-    int form[2], automatic[2];
-    form[0] = form[1] = LBM_FORM_ONE_KERNEL;
-    choose_forms(c, automatic);
-    float several = best;
-    for (int many = 0; many < 2; ++many) {  // calls of one step and of several
-        if (automatic[0] == LBM_FORM_ONE_KERNEL || (!many && !prepare_split_once(c))) continue;
-        const float ms = timed(steps, [&](int n) {
-            cudaError_t e = cudaSuccess;
-            for (int k = 0; k < n && e == cudaSuccess; ++k)
-                e = step_once(c, LBM_FORM_TWO_KERNELS, c->f[cur ^ (k & 1)], c->f[cur ^ (~k & 1)], !many && !c->own_f);
-            return e;
-        });
-        float& rival = many ? several : best;
-        if (ms >= 0.0f && (rival < 0.0f || ms < rival)) {
-            rival = ms;
-            form[many] = LBM_FORM_TWO_KERNELS;
+    Forms forms;
+    float few = best;
+    if (p.G2 == 0.0 && split_wanted(c) && prepare_split(c)) {
+        for (int many = 0; many < 2; ++many) {  // calls of one step and of several
+            if (!many && !prepare_split_once(c)) continue;
+            const float ms = timed(steps, [&](int n) {
+                cudaError_t e = cudaSuccess;
+                for (int k = 0; k < n && e == cudaSuccess; ++k)
+                    e = step_once(c, LBM_FORM_TWO_KERNELS, c->f[cur ^ (k & 1)], c->f[cur ^ (~k & 1)], !many && !c->own_f);
+                return e;
+            });
+            float& rival = many ? few : best;
+            if (ms >= 0.0f && (rival < 0.0f || ms < rival)) {
+                rival = ms;
+                (many ? forms.few : forms.single) = LBM_FORM_TWO_KERNELS;
+            }
         }
     }
-    if (prepare_moments(c, false)) {
-        const float ms = timed(steps < 8 ? 8 : steps, [&](int n) {
-            MomentLaunch l = moment_launch_of(c, n);
+    forms.several = forms.few;
+    if (few >= 0.0f && prepare_moments(c)) {
+        // two lengths: what a step and what the ends cost
+        auto call = [&](int n) {
             int to = 0;
-            return run_moments(*c->mom, l, c->f, cur, n, c->mom_bytes, c->mom_twice, &to);
-        });
-        if (ms >= 0.0f && several >= 0.0f && ms < several) form[1] = LBM_FORM_MOMENTS;
+            return run_moments(*c->mom, moment_launch_of(c, n), c->f, cur, n, c->mom_bytes, c->mom_twice, &to);
+        };
+        const int n = steps < 8 ? 8 : steps;
+        moments_from(forms, few, n, timed(n, call), timed(2 * n, call));
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1408,8 +1488,7 @@ lbm_status lbm_tune(lbm_ctx* c, int trial_steps, int* kernel, int* tile_y, int* 
         return c->fail(st, "lbm_tune: %s", why);
     }
     if (best < 0.0f) return c->fail(LBM_ECUDA, "lbm_tune: no launch shape ran");
-    c->form[0] = form[0];
-    c->form[1] = form[1];
+    c->forms = forms;
     if (kernel) *kernel = c->kernel;
     if (tile_y) *tile_y = c->tile_y;
     if (zchunk) *zchunk = c->zchunk;
@@ -1543,7 +1622,7 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (!c) return LBM_EINVAL;
     if (nsteps < 0) return c->fail(LBM_EINVAL, "lbm_step: n must be >= 0");
     if (c->batch) return c->fail(LBM_EINVAL, "lbm_step: this context is a box of a batch; use lbm_batch_step");
-    int form = c->form[nsteps >= 2];
+    int form = c->forms.of(nsteps);
     if (form == LBM_FORM_MOMENTS) return step_moments(c, nsteps);
     if (nsteps == 1 && form == LBM_FORM_TWO_KERNELS && !prepare_split_once(c)) form = LBM_FORM_ONE_KERNEL;
     const bool keep = nsteps == 1 && !c->own_f;
@@ -1676,7 +1755,8 @@ struct lbm_batch {
     void* mom_plan = nullptr;         // device memory of its plan
     BatchBox* mom_boxes_dev = nullptr;
     bool mom_twice = false;
-    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};  // of calls of one and of several steps
+    long long mom_busiest = 0;        // planes of its busiest block
+    Forms forms;
     unsigned max_cells = 0;
     char err[512] = {0};
 
@@ -1806,6 +1886,7 @@ lbm_status batch_configure_moments(lbm_batch* b) {
         columns[i] = {bx.tiles_x * ((q.ny + k->tile_y - 1) / k->tile_y), q.nz};
     }
     const MomentPlan plan = plan_moments(columns, (long long)per_sm * b->num_sms, k->fields, bytes_all);
+    b->mom_busiest = plan.busiest;
     if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
     LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
                                 b->stream));
@@ -1829,24 +1910,37 @@ lbm_status batch_configure_moments(lbm_batch* b) {
 }
 
 // The forms of a batch for which no particular kernel or launch shape was asked.
-lbm_status batch_choose_forms(lbm_batch* b, int (&form)[2]) {
-    form[0] = form[1] = batch_can_split(b) ? LBM_FORM_TWO_KERNELS : LBM_FORM_ONE_KERNEL;
+lbm_status batch_choose_forms(lbm_batch* b, Forms& f) {
+    f = Forms::every(batch_can_split(b) ? LBM_FORM_TWO_KERNELS : LBM_FORM_ONE_KERNEL);
     const lbm_status st = batch_configure_moments(b);
-    if (b->mom) form[1] = LBM_FORM_MOMENTS;
+    if (!b->mom) return st;
+    // one kernel: 37 ps a cell of its 32 x 8 tiles, 20 us at least (24 boxes of 32 x 32 69 to 80 us, 16 of 33 .. 48 x 31
+    // 67 to 71)
+    double padded = 0.0;
+    bool odd = false;
+    for (const lbm_ctx* c : b->box) {
+        padded += double((c->p.nx + 31) / 32 * 32) * ((c->p.ny + 7) / 8 * 8) * c->p.nz;
+        odd = odd || c->p.nx % 2 != 0;
+    }
+    const double rival = 37e-6 * padded;
+    const long from = moments_pay_from(b->p.storage, b->box[0]->coll, b->cells, odd, true, b->mom_busiest, rival < 20.0 ? 20.0 : rival);
+    if (from > 0) {
+        f.several = LBM_FORM_MOMENTS;
+        f.from = from;
+    }
     return st;
 }
 
-void batch_set_forms(lbm_batch* b, const int (&form)[2]) {
-    if (form[1] != b->form[1]) batch_drop_graphs(b);  // they hold steps of that form
-    b->form[0] = form[0];
-    b->form[1] = form[1];
+void batch_set_forms(lbm_batch* b, const Forms& f) {
+    if (f.few != b->forms.few) batch_drop_graphs(b);  // they hold steps of that form
+    b->forms = f;
 }
 
 lbm_status batch_build_graph(lbm_batch* b, int from) {
     cudaGraph_t g = nullptr;
     LBM_CUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e1 = batch_launch_step(b, b->form[1], from);
-    cudaError_t e2 = batch_launch_step(b, b->form[1], from ^ 1);
+    cudaError_t e1 = batch_launch_step(b, b->forms.few, from);
+    cudaError_t e2 = batch_launch_step(b, b->forms.few, from ^ 1);
     cudaError_t e3 = cudaStreamEndCapture(b->stream, &g);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -1946,7 +2040,7 @@ lbm_status lbm_batch_create(const lbm_params* p, int count, const int* dims, lbm
     const int ty = p->tile_y ? p->tile_y : (p->collision == LBM_MRT_GUO ? 4 : 8);
     const int zc = p->zchunk ? p->zchunk : 32;
     lbm_status st = batch_configure(b, ty, zc);
-    if (st == LBM_OK && p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) st = batch_choose_forms(b, b->form);
+    if (st == LBM_OK && p->kernel == 0 && p->tile_y == 0 && p->zchunk == 0) st = batch_choose_forms(b, b->forms);
     if (st != LBM_OK) {
         snprintf(g_create_err, sizeof(g_create_err), "%s", b->err);
         lbm_batch_destroy(b);
@@ -1987,7 +2081,7 @@ lbm_status lbm_batch_box(lbm_batch* b, int i, lbm_ctx** view) {
 lbm_status lbm_batch_step(lbm_batch* b, long n) {
     if (!b) return LBM_EINVAL;
     if (n < 0) return b->fail(LBM_EINVAL, "lbm_batch_step: n must be >= 0");
-    const int form = b->form[n >= 2];
+    const int form = b->forms.of(n);
     if (form == LBM_FORM_MOMENTS) {
         MomentLaunch l = b->mom_launch;
         l.stream = b->stream;
@@ -2024,21 +2118,19 @@ lbm_status lbm_batch_step(lbm_batch* b, long n) {
     return LBM_OK;
 }
 
-int lbm_batch_step_form(const lbm_batch* b, long n) { return b && n >= 1 ? b->form[n >= 2] : 0; }
+int lbm_batch_step_form(const lbm_batch* b, long n) { return b && n >= 1 ? b->forms.of(n) : 0; }
 
-lbm_status lbm_batch_set_step_forms(lbm_batch* b, int single, int several) {
+lbm_status lbm_batch_set_step_forms(lbm_batch* b, int single, int several, long moments_from) {
     if (!b) return LBM_EINVAL;
-    if (single < LBM_FORM_AUTO || single > LBM_FORM_TWO_KERNELS || several < LBM_FORM_AUTO || several > LBM_FORM_MOMENTS)
+    Forms automatic, f;
+    if (const lbm_status st = batch_choose_forms(b, automatic); st != LBM_OK) return st;
+    if (!asked_forms(f, automatic, single, several, moments_from))
         return b->fail(LBM_EINVAL, "lbm_batch_set_step_forms: unknown form (%d, %d)", single, several);
-    int form[2];
-    if (const lbm_status st = batch_choose_forms(b, form); st != LBM_OK) return st;
-    if (single != LBM_FORM_AUTO) form[0] = single;
-    if (several != LBM_FORM_AUTO) form[1] = several;
-    if ((form[0] == LBM_FORM_TWO_KERNELS || form[1] == LBM_FORM_TWO_KERNELS) && !batch_can_split(b))
+    if ((f.single == LBM_FORM_TWO_KERNELS || f.few == LBM_FORM_TWO_KERNELS) && !batch_can_split(b))
         return b->fail(LBM_EUNSUPPORTED, "lbm_batch_set_step_forms: these boxes cannot step in two kernels");
-    if (form[1] == LBM_FORM_MOMENTS && !b->mom)
+    if (f.several == LBM_FORM_MOMENTS && !b->mom)
         return b->fail(LBM_EUNSUPPORTED, "lbm_batch_set_step_forms: these boxes cannot step through moment fields");
-    batch_set_forms(b, form);
+    batch_set_forms(b, f);
     return LBM_OK;
 }
 
@@ -2070,7 +2162,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
             }
         }
     }
-    // the other forms, as lbm_batch_step runs them; fewer than 8 steps at once would time the moment form's ends
+    // the other forms, as lbm_batch_step runs them
     auto timed = [&](int n, auto&& run) {
         if (run(2) != cudaSuccess) return -1.0f;  // warm-up
         cudaEventRecord(e0, b->stream);
@@ -2081,7 +2173,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
         cudaEventElapsedTime(&ms, e0, e1);
         return ms / n;
     };
-    int form[2] = {LBM_FORM_ONE_KERNEL, LBM_FORM_ONE_KERNEL};
+    Forms forms;
     if (batch_can_split(b)) {
         const float ms = timed(trial_steps, [&](int n) {
             cudaError_t e = cudaSuccess;
@@ -2090,17 +2182,18 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
         });
         if (ms >= 0.0f && (best < 0.0f || ms < best)) {
             best = ms;
-            form[0] = form[1] = LBM_FORM_TWO_KERNELS;
+            forms = Forms::every(LBM_FORM_TWO_KERNELS);
         }
     }
-    if (batch_configure_moments(b) == LBM_OK && b->mom) {
+    if (best >= 0.0f && batch_configure_moments(b) == LBM_OK && b->mom) {
         MomentLaunch l = b->mom_launch;
         l.stream = b->stream;
-        const float ms = timed(trial_steps < 8 ? 8 : trial_steps, [&](int n) {
+        auto call = [&](int n) {
             int to = 0;
             return run_moments(*b->mom, l, b->f, 0, n, b->bytes, b->mom_twice, &to);
-        });
-        if (ms >= 0.0f && best >= 0.0f && ms < best) form[1] = LBM_FORM_MOMENTS;
+        };
+        const int n = trial_steps < 8 ? 8 : trial_steps;
+        moments_from(forms, best, n, timed(n, call), timed(2 * n, call));
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -2108,7 +2201,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* tile_y, int* zchun
     if (e != cudaSuccess) return b->fail(LBM_ECUDA, "lbm_batch_tune: %s", cudaGetErrorString(e));
     lbm_status st = batch_configure(b, best_ty, best_zc);
     if (st != LBM_OK) return st;
-    if (best >= 0.0f) batch_set_forms(b, form);
+    if (best >= 0.0f) batch_set_forms(b, forms);
     if (tile_y) *tile_y = best_ty;
     if (zchunk) *zchunk = best_zc;
     if (ms_per_step) *ms_per_step = best;
@@ -2181,7 +2274,7 @@ lbm_status lbm_adjoint_forward(lbm_ctx* c, const double* rho0, int on_device, lo
     if (c->n > 0xffffffffLL) return c->fail(LBM_EUNSUPPORTED, "lbm_adjoint_forward: needs nx*ny*nz < 2^32");
     auto& A = c->adj;
     // tau = 1 in FP32: a state's four moments are all the adjoint needs of it
-    A.moments = c->form[1] == LBM_FORM_MOMENTS && c->p.storage == LBM_F32 && c->p.tau == 1.0;
+    A.moments = c->forms.several == LBM_FORM_MOMENTS && c->p.storage == LBM_F32 && c->p.tau == 1.0;
     const size_t state = A.moments ? c->mom_bytes : (size_t)Q * (size_t)c->n * c->elem;
     A.T = -1;  // nothing recorded until the run is complete
     const int ncp = int((nsteps + every - 1) / every);
@@ -2264,7 +2357,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
     // psi of every state of a segment: written by the step kernel during the
     // recomputation where it supports that (kernels 1 and 3, and 5 whose
     // recomputation runs kernel 3), else computed by the reverse step
-    const bool psi_fused = c->form[0] == LBM_FORM_TWO_KERNELS || c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
+    const bool psi_fused = c->forms.few == LBM_FORM_TWO_KERNELS || c->kernel == 1 || c->kernel == 3 || c->kernel == 5;
     const size_t psi_bytes = (size_t)c->n * c->elem;
     if (A.psi && A.psi_bytes < (size_t)A.every * psi_bytes) {
         cudaStreamSynchronize(c->stream);
@@ -2325,7 +2418,7 @@ lbm_status lbm_adjoint_backward(lbm_ctx* c, const double* dJdrho, int in_on_devi
                                     cudaMemcpyDeviceToDevice, c->stream));
         char* psi = static_cast<char*>(A.psi);
         for (long t = t0; t + 1 < t1; ++t) {
-            cudaError_t e = step_once(c, c->form[0], seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state, true,
+            cudaError_t e = step_once(c, c->forms.few, seg + (size_t)(t - t0) * state, seg + (size_t)(t - t0 + 1) * state, true,
                                       psi_fused ? psi + (size_t)(t - t0) * psi_bytes : nullptr);
             if (e != cudaSuccess) return c->fail(LBM_ECUDA, "adjoint recompute: %s", cudaGetErrorString(e));
         }

@@ -92,7 +92,7 @@ _SIGNATURES = {
                                          ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "lbm_set_kernel_config": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "lbm_step_form": (ctypes.c_int, [_P, ctypes.c_long]),
-    "lbm_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
+    "lbm_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_long]),
     "lbm_tune": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                 ctypes.POINTER(ctypes.c_int), _D]),
     "lbm_batch_create": (ctypes.c_int, [ctypes.POINTER(lbm_params), ctypes.c_int, ctypes.POINTER(ctypes.c_int),
@@ -102,7 +102,7 @@ _SIGNATURES = {
     "lbm_batch_box": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(_P)]),
     "lbm_batch_step": (ctypes.c_int, [_P, ctypes.c_long]),
     "lbm_batch_step_form": (ctypes.c_int, [_P, ctypes.c_long]),
-    "lbm_batch_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
+    "lbm_batch_set_step_forms": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_long]),
     "lbm_batch_tune": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                       _D]),
     "lbm_batch_config": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
@@ -286,15 +286,15 @@ def lbm_batch_step_form(b, n):
     return load().lbm_batch_step_form(b, int(n))
 
 
-def lbm_batch_set_step_forms(b, single, several):
-    return load().lbm_batch_set_step_forms(b, int(single), int(several))
+def lbm_batch_set_step_forms(b, single, several, moments_from=2):
+    return load().lbm_batch_set_step_forms(b, int(single), int(several), int(moments_from))
 
 
 def lbm_batch_tune(b, trial_steps):
     ty, zc, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_double()
     st = load().lbm_batch_tune(b, trial_steps, ctypes.byref(ty), ctypes.byref(zc), ctypes.byref(ms))
     return st, dict(tile_y=ty.value, zchunk=zc.value, ms_per_step=ms.value,
-                    forms=[FORM_NAMES[lbm_batch_step_form(b, n)] for n in (1, 2)])
+                    forms=_forms(lambda n: lbm_batch_step_form(b, n)))
 
 
 def lbm_batch_config(b):
@@ -327,8 +327,26 @@ def lbm_step_form(ctx, n):
     return load().lbm_step_form(ctx, int(n))
 
 
-def lbm_set_step_forms(ctx, single, several):
-    return load().lbm_set_step_forms(ctx, int(single), int(several))
+def lbm_set_step_forms(ctx, single, several, moments_from=2):
+    return load().lbm_set_step_forms(ctx, int(single), int(several), int(moments_from))
+
+
+def _forms(step_form):
+    """[form of one step, of many, and the calls from which on that holds], as the tuners' caches keep it;
+    step_form(n): LBM_FORM_* of a call of n steps."""
+    many = step_form(2 ** 31 - 1)
+    lo, hi = 1, 2 ** 21  # the tuners' limit is 1e6 steps
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        if mid > 1 and step_form(mid) == many:
+            hi = mid
+        else:
+            lo = mid
+    return [FORM_NAMES[step_form(1)], FORM_NAMES[many], max(hi, 2)]
+
+
+def _form_args(forms):
+    return FORM_NAMES.index(forms[0]), FORM_NAMES.index(forms[1]), int(forms[2])
 
 
 def lbm_tune(ctx, trial_steps):
@@ -336,7 +354,7 @@ def lbm_tune(ctx, trial_steps):
     ms = ctypes.c_double()
     st = load().lbm_tune(ctx, int(trial_steps), ctypes.byref(k), ctypes.byref(t), ctypes.byref(z), ctypes.byref(ms))
     return st, {"kernel": k.value, "tile_y": t.value, "zchunk": z.value, "ms_per_step": ms.value,
-                "forms": [FORM_NAMES[lbm_step_form(ctx, n)] for n in (1, 2)]}
+                "forms": _forms(lambda n: lbm_step_form(ctx, n))}
 
 
 def _host_ptr(a: np.ndarray):
@@ -583,9 +601,10 @@ class Lattice:
         (lbm_step_form)."""
         return FORM_NAMES[lbm_step_form(self.ctx, n)]
 
-    def set_step_forms(self, single="auto", several="auto"):
-        """Choose how step(1) and step(n >= 2) step (lbm_set_step_forms)."""
-        self._check(lbm_set_step_forms(self.ctx, FORM_NAMES.index(single), FORM_NAMES.index(several)))
+    def set_step_forms(self, single="auto", several="auto", moments_from=2):
+        """Choose how step(1) and step(n >= 2) step (lbm_set_step_forms);
+        'moments' holds for n >= moments_from."""
+        self._check(lbm_set_step_forms(self.ctx, *_form_args((single, several, moments_from))))
 
     def tune(self, trial_steps=3, cache=None):
         """Pick the step's launch shape (kernel variant, tile height, z chunk)
@@ -594,7 +613,7 @@ class Lattice:
         `cache` (a JSON file path) a pick stored for the same box, parameters
         and GPU model is applied without timing, and a new pick is stored.
         Returns the pick (kernel, tile_y, zchunk, ms_per_step, the forms of
-        step(1) and step(n >= 2), cached)."""
+        step(1) and of many steps and from how many on, cached)."""
         key = None
         if cache is not None:
             p = self.params
@@ -606,7 +625,7 @@ class Lattice:
                 self.set_kernel_config(hit["kernel"], hit["tile_y"], hit["zchunk"])
                 # (no forms stored, or no room for them any more: one kernel a step)
                 if "forms" in hit:
-                    lbm_set_step_forms(self.ctx, *(FORM_NAMES.index(v) for v in hit["forms"]))
+                    lbm_set_step_forms(self.ctx, *_form_args(hit["forms"]))
                 return dict(hit, cached=True)
         st, pick = lbm_tune(self.ctx, trial_steps)
         self._check(st)
@@ -709,7 +728,7 @@ class Batch:
             self.boxes.append(_BoxView(self, i, v, (nz, ny, nx)))
         # (no forms stored, or no room for them any more: one kernel a step)
         if cached and "forms" in cached:
-            lbm_batch_set_step_forms(self.b, *(FORM_NAMES.index(v) for v in cached["forms"]))
+            lbm_batch_set_step_forms(self.b, *_form_args(cached["forms"]))
         if key is not None and not cached:
             best = self.tune(trial_steps)
             data = _read_tune_cache(tune_cache)
@@ -727,9 +746,10 @@ class Batch:
         """How step(n) steps: 'one', 'two' (kernels a step) or 'moments'."""
         return FORM_NAMES[lbm_batch_step_form(self.b, n)]
 
-    def set_step_forms(self, single="auto", several="auto"):
-        """Choose how step(1) and step(n >= 2) step (lbm_batch_set_step_forms)."""
-        self._check(lbm_batch_set_step_forms(self.b, FORM_NAMES.index(single), FORM_NAMES.index(several)))
+    def set_step_forms(self, single="auto", several="auto", moments_from=2):
+        """Choose how step(1) and step(n >= 2) step (lbm_batch_set_step_forms);
+        'moments' holds for n >= moments_from."""
+        self._check(lbm_batch_set_step_forms(self.b, *_form_args((single, several, moments_from))))
 
     def tune(self, trial_steps=3):
         st, r = lbm_batch_tune(self.b, int(trial_steps))
