@@ -192,7 +192,11 @@ __global__ void ligament_kernel(typename Codec::S* __restrict__ f, int nx, int n
 }
 
 // n cells of populations q0, q0 + 1, ..., one after the other in `f` and the
-// float64 array: one row of blocks (blockIdx.y) each.
+// float64 array: one row of blocks (blockIdx.y) each.  A thread takes 8 cells
+// where that leaves the SMs enough blocks: with one, placing the blocks takes as
+// long as their work (FP32 64 x 64 x 128 from a device array 40 us, now 21; 128 x
+// 128 x 200 121, 109; 256 x 256 x 300 625 either way).
+constexpr int kConvertCells = 256 * 8;  // of a block
 template <class Codec>
 __global__ void decode_kernel(double* __restrict__ out, const typename Codec::S* __restrict__ f, long long n, int q0,
                               DevParams dev, const float* ref) {
@@ -1547,8 +1551,8 @@ lbm_status lbm_set_populations(lbm_ctx* c, const double* f, int on_device) {
         if (ref) ref_sum_kernel<<<blocks, 256, 0, c->stream>>>(ref, nullptr, f, c->n, Q, 0);
         with_codec(c, [&](auto codec) {
             using C = decltype(codec);
-            encode_kernel<C><<<dim3(blocks, Q), 256, 0, c->stream>>>(static_cast<typename C::S*>(c->f[c->cur]), f,
-                                                                     c->n, 0, c->args.dev, ref);
+            encode_kernel<C><<<dim3(grid_for(c->n, kConvertCells, c->num_sms), Q), 256, 0, c->stream>>>(
+                static_cast<typename C::S*>(c->f[c->cur]), f, c->n, 0, c->args.dev, ref);
             return 0;
         });
         LBM_LAUNCHED(c, "encode_kernel");
@@ -1592,7 +1596,7 @@ lbm_status lbm_get_populations(lbm_ctx* c, double* f, int on_device) {
     if (on_device) {
         with_codec(c, [&](auto codec) {
             using C = decltype(codec);
-            decode_kernel<C><<<dim3(grid_for(c->n, 256, c->num_sms), Q), 256, 0, c->stream>>>(
+            decode_kernel<C><<<dim3(grid_for(c->n, kConvertCells, c->num_sms), Q), 256, 0, c->stream>>>(
                 f, static_cast<const typename C::S*>(c->f[c->cur]), c->n, 0, c->args.dev, c->ref[c->cur]);
             return 0;
         });
