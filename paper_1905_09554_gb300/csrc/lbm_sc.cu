@@ -864,9 +864,9 @@ cudaError_t upload_plan(const MomentPlan& plan, MomentLaunch& l, void** mem, siz
     }
     *bytes = np + nf;
     char* const at = static_cast<char*>(*mem);
+    // (copies from pageable memory return once the source has been read: nothing waits for the stream)
     e = cudaMemcpyAsync(at, plan.pieces.data(), np, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(at + np, plan.first.data(), nf, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     l.pieces = reinterpret_cast<const MomentPiece*>(at);
     l.first = reinterpret_cast<const int*>(at + np);
     l.grid = int(plan.first.size()) - 1;
@@ -1894,7 +1894,6 @@ lbm_status batch_configure_moments(lbm_batch* b) {
     if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
     LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
                                 b->stream));
-    LBM_CUDA(b, cudaStreamSynchronize(b->stream));
     MomentLaunch& l = b->mom_launch;
     l = MomentLaunch{};
     l.args = b->phys;
