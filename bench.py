@@ -48,30 +48,34 @@ KERNEL_NAMES = {1: "sc_step_kernel", 2: "sc_step_async_kernel", 3: "sc_step_pipe
                 5: "sc_step_tma_kernel", 6: "sc_psi_kernel + sc_step_mr_kernel", 7: "sc_step_pair16_kernel"}
 
 
-def step_kernels(storage, kernel, info, cells, in_place):
-    """Names of the kernels of one single step and how many they are: FP64,
-    odd 16-bit rows and boxes that fit into L2 run in two (unless --kernel
-    asks for one), the two-belt force as well.  in_place: the collision needs
-    only a few moments."""
-    name = KERNEL_NAMES.get(info["kernel"], "sc_step_kernel")
-    if info["kernel"] == 6:
-        return name, 2
-    small = {"f32": 1200000 if in_place else 400000, "f16": 2000000, "bf16": 2000000, "f16l": 250000,
-             "bf16l": 250000}.get(storage, 0)
-    if kernel == 0 and (info["kernel"] == 1 or cells <= small):
+def step_kernels(form, info):
+    """Names of the kernels of one step outside the moment form and how many
+    they are, from the form that the library reports and its launch shape; the
+    two-belt force runs in two as well."""
+    if form == "two":
         return "sc_fields_kernel + sc_push_kernel", 2
-    return name, 1
+    return KERNEL_NAMES.get(info["kernel"], "sc_step_kernel"), 2 if info["kernel"] == 6 else 1
 
 
-def run_bytes(storage, steps):
+def ran(L, steps):
+    """What stepped in calls of `steps` steps: the form, its kernels and, in the
+    one-kernel form, the launch shape (the other forms have their own)."""
+    form, info = L.step_form(steps), L.kernel_config()
+    if form == "moments":
+        return {"form": form, "kernels": "sc_moments_kernel + sc_moment_kernel"}
+    got = {"form": form, "kernels": step_kernels(form, info)[0]}
+    return dict(info, **got) if form == "one" else got
+
+
+def run_bytes(storage, steps, form):
     """Algorithmic bytes per cell and step of one call of `steps` steps at
-    tau = 1 (SRT): FP32 and 16-bit storage read and write four moments a step
-    and the populations once a call; FP64 leaves four moments and psi in the
-    first populations' place between its two kernels."""
+    tau = 1 (SRT): the moment form reads and writes four moments a step and the
+    populations once a call; the two-kernel form leaves four moments and psi
+    between its kernels."""
     pops = 2 * 19 * BYTES_PER_POP[storage] + EXTRA_BYTES_PER_CELL.get(storage, 0)
-    if storage == "f64":
-        return pops + 2 * 5 * 8
-    return 32 + pops / steps if steps >= 2 else pops
+    if form == "two":
+        return pops + 2 * 5 * BYTES_PER_POP[storage]
+    return 32 + pops / steps if form == "moments" else pops
 
 
 def parse_args():
@@ -294,8 +298,8 @@ def c_reference_mlups(w, args, slab, steps):
 # ------------------------------------------------------------ other forms
 def measure_rate(storage, steps, warmup, R0=64.0, kR0=0.7, collision="srt", tau=1.0):
     """Device time per step (CUDA events on the lattice's stream around
-    `steps` step launches) of the ligament R0, kR0 with `storage`
-    populations; returns GLUPS, ms per step, cells and the launch shape."""
+    one call of `steps` steps) of the ligament R0, kR0 with `storage`
+    populations; returns GLUPS, ms per step, cells and what ran."""
     import torch
 
     from paper_1905_09554_gb300 import inputs, lbm
@@ -318,9 +322,10 @@ def measure_rate(storage, steps, warmup, R0=64.0, kR0=0.7, collision="srt", tau=
         e1.record(stream)
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / steps
-        cfg = L.kernel_config()
+        shape = ran(L, steps)
     cells = nx * ny * nz
-    return {"glups": cells / (ms / 1e3) / 1e9, "ms_per_step": ms, "cells": cells, "kernel": cfg}
+    return {"glups": cells / (ms / 1e3) / 1e9, "ms_per_step": ms, "cells": cells, "ran": shape,
+            "bytes_per_cell": run_bytes(storage, steps, shape["form"])}
 
 
 def breakup_run_to_pinch(storage, R0=16.0, kR0=0.7, collision="srt", tau=1.0, every=5, max_steps=20000):
@@ -365,16 +370,16 @@ def measure_forms(device, clocks):
     fpc = rec.get("fp64_flops_per_cell") if rec else None
     pk, src = fp64_peak(device, clocks)
     forms["f64"] = {"glups": f64["glups"], "ms_per_step": f64["ms_per_step"],
-                    "hbm_frac": run_bytes("f64", 20) * f64["glups"] / peak,
+                    "hbm_frac": f64["bytes_per_cell"] * f64["glups"] / peak,
                     "fp64_pipe_frac": (fpc * f64["glups"] / 1e3 / pk) if fpc else None,
                     "fp64_flops_per_cell": fpc, "fp64_peak_tflops": pk, "fp64_peak_source": src,
-                    "kernel": f64["kernel"]}
+                    "ran": f64["ran"]}
     for st in ("f16l", "f16", "bf16l"):
-        bpc = run_bytes(st, 100)
         r = measure_rate(st, steps=100, warmup=5)
+        bpc = r["bytes_per_cell"]
         forms[st] = {"glups": r["glups"], "ms_per_step": r["ms_per_step"], "bytes_per_cell": bpc,
                      "hbm_frac": bpc * r["glups"] / peak, "speedup_vs_f64": r["glups"] / f64["glups"],
-                     "kernel": r["kernel"]}
+                     "ran": r["ran"]}
     import numpy as np
     tb64, rho64 = breakup_run_to_pinch("f64")
     forms["f64"]["t_break_steps_R0_16"] = tb64
@@ -387,7 +392,7 @@ def measure_forms(device, clocks):
     b = measure_batched(300, 10)
     forms["batched"] = {"ligaments_per_s": b["ligaments_per_s"], "aggregate_glups": b["aggregate_mlups"] / 1e3,
                         "hbm_frac": b["hbm_gbs"] / peak, "speedup_vs_f64": b["aggregate_mlups"] / 1e3 / f64["glups"],
-                        "cells": b["cells"], "tile_y": b["config"]["tile_y"], "zchunk": b["config"]["zchunk"],
+                        "cells": b["cells"], "ran": b["ran"],
                         "workload": "64 ligaments R0 in {8,12,16}, kR0 ~ U[0.2,1.0) seed 0, FP32 SRT; ligaments/s "
                                     "of 3000-step runs from 300 timed steps"}
     adj = measure_adjoint()
@@ -396,7 +401,7 @@ def measure_forms(device, clocks):
                         "f64_adjoint_steps_per_s": adj["T"] / d["bwd_s"],
                         "f32_forward_with_checkpoints_steps_per_s": adj["T"] / a["fwd_s"],
                         "f32_vs_f64_gradient": adj["fp32_vs_fp64"],
-                        "step_launch_shape": {"f32": adj["f32_tune"], "f64": adj["f64_tune"]},
+                        "forward_steps": {"f32": adj["f32_ran"], "f64": adj["f64_ran"]},
                         "workload": "64x64x180 ligament, neck energy at step 500, checkpoints every 23"}
     return forms
 
@@ -486,7 +491,7 @@ def run_ours(args):
                     storage=args.storage,
                     rates=mrt_rates(args), zchunk=args.zchunk, tile_y=args.tile_y, kernel=args.kernel)
     L.init_ligament(args.R0, 0.05, w["rho_l"], w["rho_v"])
-    L_info = L.kernel_config()
+    L_info, single, one_call = L.kernel_config(), L.step_form(1), ran(L, args.steps)
     stream = torch.cuda.current_stream()
     d0 = L.diag(w["rho_l"], w["rho_v"])
     L.step(args.warmup)
@@ -560,8 +565,9 @@ def run_ours(args):
 
     peak, src = measured_hbm()
     bpc = 2 * 19 * BYTES_PER_POP[args.storage] + EXTRA_BYTES_PER_CELL.get(args.storage, 0)
-    kname, n_kernels = step_kernels(args.storage, args.kernel, L_info, ncell,
-                                    args.collision == "mrt" or args.tau == 1.0)
+    kname, n_kernels = step_kernels(single, L_info)
+    shape = dict(L_info, form=single) if single == "one" else {"form": single}
+    traffic = load_traffic(args, ncell, L_info, (nx, ny, nz)) if single == "one" else None
     rec = step_record()
     if args.storage == "f64" and rec and rec.get("fp64_flops_per_cell"):
         # FP64 is bound by the FP64 pipe: SMs x 2 FP64 lanes per clock
@@ -570,14 +576,14 @@ def run_ours(args):
         achieved = fpc * ncell / (kernel_ms / 1e3) / 1e12
         peak_alu, peak_src = fp64_peak(local, clocks)
         roofline = {"bound": "alu", "achieved": achieved, "peak": peak_alu, "unit": "TFLOP/s",
-                    "frac": achieved / peak_alu, "traffic": load_traffic(args, ncell, L_info, (nx, ny, nz)),
+                    "frac": achieved / peak_alu, "traffic": traffic,
                     "peak_source": peak_src,
                     "kernel": kname, "fp64_flops_per_cell": fpc, "kernel_ms": kernel_ms,
                     "hbm_frac": bpc * ncell / (kernel_ms / 1e3) / 1e9 / peak}
     else:
         achieved = bpc * ncell / (kernel_ms / 1e3) / 1e9
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                    "frac": achieved / peak, "traffic": load_traffic(args, ncell, L_info, (nx, ny, nz)),
+                    "frac": achieved / peak, "traffic": traffic,
                     "peak_source": f"{src} HBM copy bandwidth",
                     "kernel": kname, "algorithmic_bytes_per_cell": bpc, "kernel_ms": kernel_ms}
 
@@ -600,14 +606,13 @@ def run_ours(args):
         "scaling": "weak", "vs_baseline": None, "dtype": args.storage, "data": "synthetic",
         "config": {"workload": w["name"], "cells": ncell, "collision": args.collision,
                    "storage": args.storage, "parallelism": f"replicas x{world}",
-                   "kernel": L_info["kernel"], "zchunk": L_info["zchunk"], "tile_y": L_info["tile_y"],
-                   "grid": L_info["grid"],
+                   **shape,
                    "l2": "inputs larger than L2 (two population copies of "
                          f"{19 * BYTES_PER_POP[args.storage] * ncell / 1e9:.2f} GB each)",
                    "mass_rel_drift": mass_drift},
         "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
         "one_call": {"value": ncell * args.steps / (call_ms / 1e3) / 1e6, "unit": "MLUPS", "steps": args.steps,
-                     "ms_per_step": call_ms / args.steps, "ranks": "rank 0"},
+                     "ms_per_step": call_ms / args.steps, "ranks": "rank 0", "ran": one_call},
         "gpu_launches": args.steps * n_kernels, "host": host_info(), "forms": forms,
     }
     print(json.dumps(line), flush=True)
@@ -677,9 +682,8 @@ def measure_batched(steps, warmup, trial_steps=3):
     """64 independent ligaments (R0 in {8, 12, 16}, kR0 uniform on [0.2, 1.0)
     from seed 0, box 4R0 x 4R0 x round(2 pi R0 / kR0)), FP32 SRT tau = 1,
     G = -5.5, 3% perturbation, advanced together by one launch per step
-    (between the first and the last on the moments) after the launch-shape
-    autotuner.
-    Returns the device time of `steps` steps and the chosen configuration."""
+    (between the first and the last on the moments) after the autotuner.
+    Returns the device time of `steps` steps and what ran."""
     import torch
 
     from paper_1905_09554_gb300 import inputs, lbm
@@ -693,7 +697,8 @@ def measure_batched(steps, warmup, trial_steps=3):
         for box, d in zip(B.boxes, insts):
             box.init_ligament(d["R0"], 0.03, rl, rv)
         B.step(warmup)
-        cfg = B.config()
+        cfg, form = B.config(), B.step_form(steps)
+        shape = dict(cfg, form=form) if form == "one" else {"form": form}
         t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         torch.cuda.synchronize()
         t0.record(stream)
@@ -703,10 +708,10 @@ def measure_batched(steps, warmup, trial_steps=3):
         ms = t0.elapsed_time(t1)
         B.close()
     cells = cfg["cells"]
-    return {"ms": ms, "steps": steps, "cells": cells, "config": cfg, "tune": best,
+    return {"ms": ms, "steps": steps, "cells": cells, "ran": shape, "tune": best,
             "ligaments_per_s": 64.0 / (ms / 1e3 * 3000.0 / steps),
             "aggregate_mlups": cells * steps / (ms / 1e3) / 1e6,
-            "hbm_gbs": run_bytes("f32", steps) * cells / (ms / steps / 1e3) / 1e9}
+            "hbm_gbs": run_bytes("f32", steps, form) * cells / (ms / steps / 1e3) / 1e9}
 
 
 def run_batched(args):
@@ -715,7 +720,6 @@ def run_batched(args):
     import torch
     torch.cuda.set_device(int(os.environ.get("LOCAL_RANK", "0")))
     m = measure_batched(args.steps, args.warmup)
-    cfg = m["config"]
     peak = measured_hbm()[0]
     line = {
         "metric": "batched ligaments/s (64 uneven ligaments, one launch per step)",
@@ -725,12 +729,12 @@ def run_batched(args):
         "dtype": "f32", "data": "synthetic",
         "config": {"workload": "64 ligaments, R0 in {8,12,16}, kR0 ~ U[0.2,1.0) seed 0, boxes 4R0x4R0xround(2piR0/kR0), "
                                "G=-5.5, SRT tau=1, FP32, 3% perturbation",
-                   "cells": m["cells"], "tile_y": cfg["tile_y"], "zchunk": cfg["zchunk"], "grid": cfg["grid"],
-                   "autotune_ms_per_step": m["tune"]["ms_per_step"]},
+                   "cells": m["cells"], "ran": m["ran"],
+                   "autotune_single_step_ms": m["tune"]["ms_per_step"]},
         "aggregate_mlups": m["aggregate_mlups"],
         "roofline": {"bound": "hbm", "achieved": m["hbm_gbs"], "peak": peak, "unit": "GB/s",
                      "frac": m["hbm_gbs"] / peak},
-        "gpu_launches": args.steps + 1 if args.steps >= 2 else args.steps,
+        "gpu_launches": args.steps + 1 if m["ran"]["form"] == "moments" else args.steps,
     }
     print(json.dumps(line), flush=True)
 
@@ -769,8 +773,9 @@ def measure_adjoint(T=500, every=23):
     out = {}
     for storage in ("f32", "f64"):
         with lbm.Lattice(nx, ny, nz, G=-5.5, tau=1.0, storage=storage) as L:
-            # the recomputation steps this small box many times: pick its launch shape
-            out[storage + "_tune"] = L.tune(trial_steps=4)
+            # the recomputation steps this small box many times: pick its launch shape and forms
+            L.tune(trial_steps=4)
+            out[storage + "_ran"] = {"single": ran(L, 1), "checkpoint_to_checkpoint": ran(L, every)}
             torch.cuda.synchronize()
             t0 = time.perf_counter()
             L.adjoint_forward(rho0, T, every)
@@ -808,7 +813,7 @@ def run_adjoint(args):
                                "G=-5.5, SRT tau=1, objective: neck energy at step 500",
                    "checkpoint_every": out["every"], "cells": out["cells"]},
         "forward_with_checkpoints_steps_per_s": T / a["fwd_s"],
-        "step_launch_shape": {"f32": out["f32_tune"], "f64": out["f64_tune"]},
+        "forward_steps": {"f32": out["f32_ran"], "f64": out["f64_ran"]},
         "fp64": {"adjoint_steps_per_s": T / b["bwd_s"], "dJ_dG": b["dG"], "dJ_dtau": b["dtau"], "J": b["J"]},
         "fp32": {"dJ_dG": a["dG"], "dJ_dtau": a["dtau"], "J": a["J"]},
         "fp32_vs_fp64": out["fp32_vs_fp64"],
@@ -846,7 +851,7 @@ def run_precision(args):
             e1.record(stream)
             torch.cuda.synchronize()
             res[f]["mlups_200"] = nx * ny * nz * 200 / (e0.elapsed_time(e1) / 1e3) / 1e6
-            res[f]["kernel"] = L.kernel_config()
+            res[f]["ran"] = ran(L, 200)
             fields[f] = L.moments()
     for f in fmts[1:]:
         res[f]["err200_rho"] = float(np.abs(fields[f][0] - fields["f64"][0]).max())
@@ -948,7 +953,7 @@ def run_paper(args):
                                  checkpoint=ck)
             torch.cuda.synchronize()
             wall = time.perf_counter() - t0
-            cfg = L.kernel_config()
+            shape = ran(L, every)
         tb = res["T_break_over_tcap"]
         cases.append({"collision": coll, "R0": R0, "eps": eps, "box": [nx, ny, nz], "tau": tau, "t_cap": tcap,
                       "rho_l": rl, "rho_v": rv, "steps": res["steps"], "diag_every": every,
@@ -960,7 +965,7 @@ def run_paper(args):
                       "rel_diff": (tb - fig_t) / fig_t if tb is not None and fig_t else None,
                       "resumed_from_step": res["resumed_from_step"], "wall_s": wall,
                       "glups": nx * ny * nz * (res["steps"] - res["resumed_from_step"]) / wall / 1e9,
-                      "kernel": cfg})
+                      "ran": shape})
         if "series" in res:
             cases[-1]["series"] = res["series"]
             print(json.dumps({"collision": coll, "R0": R0, "eps": eps,
@@ -1060,14 +1065,14 @@ def run_multirange(args):
     e1.record(stream)
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / steps
-    cfg = L.kernel_config()
+    shape = ran(L, steps)
     L.close()
     print(json.dumps({
         "metric": "two-belt Shan-Chen force: surface tension at fixed EoS, and step rate",
         "value": nx * ny * nz / (ms / 1e3) / 1e6, "unit": "MLUPS", "n_gpus": 1, "steps": steps,
         "ms_per_step": ms, "higher_is_better": True, "dtype": "f32", "data": "synthetic",
         "config": {"workload": "ligament R0=64 kR0=0.7 box 256x256x575, G1=-7, G2=1.5, SRT tau=1, FP32",
-                   "kernel": cfg},
+                   "ran": shape},
         "roofline": {"bound": "hbm", "achieved": 160 * nx * ny * nz / (ms / 1e3) / 1e9,
                      "peak": measured_hbm()[0], "unit": "GB/s"},
         "splits": splits}), flush=True)
