@@ -243,7 +243,7 @@ lbm_status lbm_moments(lbm_ctx *ctx, double *rho, double *ux, double *uy,
                        double *uz, int on_device);
 
 /* Ligament diagnostics of the current state, accumulated in float64 on the
- * device, one thread block per z slice, deterministic:
+ * device, in a fixed order:
  *   mass     = sum rho                          (host, 1 value)
  *   mom      = sum_a c_a f_a over the box        (host, 3 values)
  *   area_z   = sum_xy clamp((rho - rho_v)/(rho_l - rho_v), 0, 1) per slice

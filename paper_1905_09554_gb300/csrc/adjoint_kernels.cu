@@ -490,18 +490,18 @@ cudaError_t run_adjoint_step(const AdjointArgs& a, const void* f, void* psi, boo
                                                   par<R>(a.rho0, a.rho0f), R(1.0 / a.rho0));
     Vec4<R>* const v = static_cast<Vec4<R>*>(gF);
     if (a.tau1) {
-        cudaError_t e = launch_chained(a.n <= 1500000, adj_collide1_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(f),
+        cudaError_t e = launch_chained(a.n <= kChainCells, adj_collide1_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(f),
                                        static_cast<const R*>(psi), static_cast<const Vec4<R>*>(lam_next), nullptr,
                                        static_cast<Vec4<R>*>(lam_out), v, partials, false, a);
         if (e != cudaSuccess) return e;
-        return launch_chained(a.n <= 1500000, adj_force_kernel<R, true>, grid, block, 0, st, static_cast<const R*>(psi), v,
+        return launch_chained(a.n <= kChainCells, adj_force_kernel<R, true>, grid, block, 0, st, static_cast<const R*>(psi), v,
                               static_cast<R*>(lam_out), a);
     }
-    cudaError_t e = launch_chained(a.n <= 1500000, adj_collide_kernel<R>, grid, block, 0, st, static_cast<const R*>(f),
+    cudaError_t e = launch_chained(a.n <= kChainCells, adj_collide_kernel<R>, grid, block, 0, st, static_cast<const R*>(f),
                                    static_cast<const R*>(psi), static_cast<const R*>(lam_next),
                                    static_cast<const R*>(gr_next), static_cast<R*>(lam_out), v, partials, a);
     if (e != cudaSuccess) return e;
-    e = launch_chained(a.n <= 1500000, adj_force_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(psi), v,
+    e = launch_chained(a.n <= kChainCells, adj_force_kernel<R, false>, grid, block, 0, st, static_cast<const R*>(psi), v,
                        static_cast<R*>(gr_out), a);
     (void)acc;  // the per-block sums stay in `partials` until adjoint_reduce
     return e;
@@ -525,10 +525,10 @@ cudaError_t adjoint_step_moments(const AdjointArgs& a, const float* moments, flo
     if (!psi_ready) adj_psi_moments_kernel<<<a.grid, block, 0, st>>>(moments, psi, a);
     Vec4<float>* const v = static_cast<Vec4<float>*>(gF);
     cudaError_t e = launch_chained(
-        a.n <= 1500000, adj_collide1_kernel<float, true>, a.grid, block, 0, st, moments, psi, static_cast<const Vec4<float>*>(lam_next),
+        a.n <= kChainCells, adj_collide1_kernel<float, true>, a.grid, block, 0, st, moments, psi, static_cast<const Vec4<float>*>(lam_next),
         static_cast<const Vec4<float>*>(lam_next2), static_cast<Vec4<float>*>(lam_out), v, partials, first, a);
     if (e != cudaSuccess) return e;
-    return launch_chained(a.n <= 1500000, adj_force_kernel<float, true>, a.grid, block, 0, st, psi, v, static_cast<float*>(lam_out), a);
+    return launch_chained(a.n <= kChainCells, adj_force_kernel<float, true>, a.grid, block, 0, st, psi, v, static_cast<float*>(lam_out), a);
 }
 
 cudaError_t adjoint_seed(const AdjointArgs& a, bool f64, const double* dJdrho, void* lam, void* gr, cudaStream_t st) {

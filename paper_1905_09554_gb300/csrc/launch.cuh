@@ -19,9 +19,14 @@ __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wai
 // they piled up on some: FP64 32x32x64 1.41 -> 2.38 ms per 50 steps).
 __device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// chain: false launches in plain stream order, which large grids want (their
-// successor's blocks would take places among their last ones: FP32 steps of
-// 19.6 M cells 583 us plain, 712 chained).
+// Cells up to which kernels are chained: of the moment and adjoint kernels,
+// whose launches take some 30 us there, and of the two-kernel step's pair.
+// Beyond, grids are many rounds of blocks long and want plain stream order: their
+// successor's blocks would take places among their last ones (FP32 steps of 19.6 M
+// cells in two kernels 583 us plain, 712 chained).
+constexpr long long kChainCells = 1500000, kChainSplitCells = 400000;
+
+// chain: false launches in plain stream order.
 template <class... P, class... A>
 cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t stream,
                            A&&... args) {

@@ -18,6 +18,7 @@
 #include "diag_cell.cuh"
 #include "e8.cuh"
 #include "lattice.cuh"
+#include "launch.cuh"
 #include "step_args.h"
 #include "adjoint.h"
 
@@ -236,7 +237,7 @@ template <class Codec>
 __global__ void density_kernel(double* __restrict__ rho, double* __restrict__ psi,
                                const typename Codec::S* __restrict__ f, long long n, double rho0, DevParams dev,
                                const float* ref) {
-    // rho summed in the storage's arithmetic type, as the step kernel does
+    // rho in the storage's arithmetic type, in population order (the step sums by planes: the last bits differ)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         typename Codec::R r, jx, jy, jz;
@@ -934,7 +935,7 @@ long moments_pay_from(int storage, int coll, long long cells, bool odd, bool bat
 
 // us of a step in one kernel and in two.  FP32: 2.2 us a plane of the busiest block (256 x 256 x 200 390 us, 128^3
 // 74, 160 x 150 x 200 152); 16-bit storage 31 ps a cell (364 to 388, 65 to 74, 149 to 165), 20 us at least.  Two
-// kernels: up to 400,000 cells (launched without gaps) 24 x 24 x 48 4.2 us, 48 x 48 x 96 7.9; beyond, 64 x 64 x 128
+// kernels: up to kChainSplitCells (launched without gaps) 24 x 24 x 48 4.2 us, 48 x 48 x 96 7.9; beyond, 64 x 64 x 128
 // 20.6, 96^3 28 to 38, 255 x 255 x 200 in FP16 409 to 431, from local references 458 to 498.
 double one_kernel_us(const lbm_ctx* c) {
     double us = 31e-6 * double(c->n);
@@ -946,7 +947,7 @@ double one_kernel_us(const lbm_ctx* c) {
 }
 double two_kernels_us(const lbm_ctx* c) {
     const double n = double(c->n);
-    if (n <= 400000) return 3.7 + 19e-6 * n;
+    if (c->n <= kChainSplitCells) return 3.7 + 19e-6 * n;
     const bool odd16 = c->p.storage >= LBM_F16_DEV && c->p.nx % 2 != 0;
     return 4.5 + (!odd16 ? 29.5e-6 : (c->p.storage >= LBM_F16_LOCAL ? 36e-6 : 32e-6)) * n;
 }

@@ -9,6 +9,9 @@
 
 namespace lbm {
 
+// Blocks of the psi kernel at most: 32 of 256 threads for each of the 152 SMs, which then walk the cells by the grid.
+constexpr long long kPsiBlocks = 152 * 32;
+
 template <class Codec, int COLL, int TY>
 cudaError_t launch_step_t(const StepLaunch& c, const void* src, void* dst) {
     constexpr int TX = 32;
@@ -18,7 +21,7 @@ cudaError_t launch_step_t(const StepLaunch& c, const void* src, void* dst) {
             dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + a.zchunk - 1) / a.zchunk);
             if (a.psi_ws) {
                 const long long blocks = (a.n + 255) / 256;
-                sc_psi_kernel<Codec><<<unsigned(blocks < 152 * 32 ? blocks : 152 * 32), 256, 0, c.stream>>>(
+                sc_psi_kernel<Codec><<<unsigned(blocks < kPsiBlocks ? blocks : kPsiBlocks), 256, 0, c.stream>>>(
                     static_cast<const typename Codec::S*>(src), static_cast<typename Codec::R*>(a.psi_ws), a);
             }
             sc_step_mr_kernel<Codec, COLL, TX, TY><<<grid, TX * TY, 0, c.stream>>>(

@@ -548,8 +548,7 @@ sc_moments_kernel(const void* __restrict__ src_all, void* __restrict__ dst_all, 
     }
 }
 
-// Small boxes (a step under ~30 us) chain their kernels.
-inline bool moment_chain(const MomentLaunch& l) { return !l.batch.nbox && l.args.n <= 1500000; }
+inline bool moment_chain(const MomentLaunch& l) { return !l.batch.nbox && l.args.n <= kChainCells; }
 
 template <class Codec, int COLL, bool EMIT, bool BATCH>
 cudaError_t moment_launch(const MomentLaunch& l, const void* src, void* dst) {

@@ -160,7 +160,7 @@ sc_step_pair16_kernel(const typename Codec::S* __restrict__ src, typename Codec:
             }
             async_copy::commit();
         };
-        // density of one half of a raw word, summed in population order
+        // density of one half of a raw word (in density_of's order)
         auto dens = [&](const uint32_t (&w)[Q], int hi, float ref) {
             return density_of<R>([&](auto qc) {
                 constexpr int q = decltype(qc)::value;

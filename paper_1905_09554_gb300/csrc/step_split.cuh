@@ -187,7 +187,7 @@ cudaError_t split_step(const SplitLaunch& l, void* src, void* dst, void* psi) {
     const dim3 grid((l.max_cells + kSplitThreads<R> - 1) / kSplitThreads<R>, l.batch.nbox ? l.batch.nbox : 1);
     S* const s = static_cast<S*>(src);
     S* const d = static_cast<S*>(dst);
-    const bool chain = (long long)grid.x * grid.y * kSplitThreads<R> <= 400000;
+    const bool chain = (long long)grid.x * grid.y * kSplitThreads<R> <= kChainSplitCells;
     auto both = [&](auto with_moments, void* fields) {
         constexpr bool M = decltype(with_moments)::value;
         R* const p = static_cast<R*>(fields);
