@@ -26,6 +26,13 @@ using namespace lbm;
 
 struct lbm_batch;
 
+// Work of the moment kernel's blocks (plan_moments).
+struct MomentPlan {
+    std::vector<MomentPiece> pieces;
+    std::vector<int> first;  // of each block, and the end
+    long long busiest = 0;   // planes of the busiest block, with the extra ones
+};
+
 // How a call steps (LBM_FORM_*): of one step; of 2 .. from - 1 steps; of at
 // least `from` steps.  The middle one is LBM_FORM_MOMENTS for none.
 struct Forms {
@@ -70,8 +77,8 @@ struct lbm_ctx {
     // populations will do.
     const MomentKernels* mom = nullptr;
     MomentLaunch mom_launch{};
+    MomentPlan mom_host;              // its plan, alive as long as the copy to the device may read it
     void* mom_plan = nullptr;         // device memory of its plan
-    long long mom_busiest = 0;        // planes of its busiest block
     size_t mom_bytes = 0;             // one set of moment fields
     bool mom_twice = false;           // two sets fit into one population copy
     // Steps in two kernels (step_split.cuh) go in place where the moments are
@@ -749,12 +756,6 @@ lbm_status configure_step(lbm_ctx* c, int kernel, int tile_y, int zchunk, char* 
 // 308 / 255 (243), 50 steps 30.0 / 26.1 ms; 256 x 256 x 575 340 / 309 (303), 50
 // steps 24.5 / 23.1 ms; with 10 fields, 384 x 384 x 1024 1813 / 1749 (1738), 20
 // steps 67.5 / 81.0 ms.
-struct MomentPlan {
-    std::vector<MomentPiece> pieces;
-    std::vector<int> first;  // of each block, and the end
-    long long busiest = 0;   // planes of the busiest block, with the extra ones
-};
-
 struct TileColumns {  // the tiles of a box
     int tiles, nz;
 };
@@ -865,7 +866,7 @@ cudaError_t upload_plan(const MomentPlan& plan, MomentLaunch& l, void** mem, siz
     }
     *bytes = np + nf;
     char* const at = static_cast<char*>(*mem);
-    // (copies from pageable memory return once the source has been read: nothing waits for the stream)
+    // (nothing waits for the stream: the caller keeps `plan`)
     e = cudaMemcpyAsync(at, plan.pieces.data(), np, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(at + np, plan.first.data(), nf, cudaMemcpyHostToDevice, stream);
     l.pieces = reinterpret_cast<const MomentPiece*>(at);
@@ -961,7 +962,7 @@ bool prepare_moments(lbm_ctx* c, double rival = 0.0, long* from = nullptr) {
         if (from) *from = moments_pay_from(c->p.storage, c->coll, c->n, c->p.nx % 2 != 0, false, busiest, rival);
         return !from || *from > 0;
     };
-    if (c->mom) return pays(c->mom_busiest);
+    if (c->mom) return pays(c->mom_host.busiest);
     const lbm_params& p = c->p;
     if (p.G2 != 0.0 || p.nx < 4) return false;
     if (c->coll == COLL_SRT && p.tau != 1.0) return false;  // keeps (1 - omega) f: all 19 populations
@@ -982,11 +983,10 @@ bool prepare_moments(lbm_ctx* c, double rival = 0.0, long* from = nullptr) {
     l.args = c->args;
     l.args.tiles_x = (p.nx + k->tile_x - 1) / k->tile_x;
     const int tiles = l.args.tiles_x * ((p.ny + k->tile_y - 1) / k->tile_y);
-    const MomentPlan plan = plan_moments({{tiles, p.nz}}, (long long)per_sm * c->num_sms, k->fields, c->mom_bytes);
-    if (!pays(plan.busiest)) return false;
-    c->mom_busiest = plan.busiest;
+    c->mom_host = plan_moments({{tiles, p.nz}}, (long long)per_sm * c->num_sms, k->fields, c->mom_bytes);
+    if (!pays(c->mom_host.busiest)) return false;
     size_t bytes = 0;
-    if (upload_plan(plan, l, &c->mom_plan, &bytes, c->stream) != cudaSuccess) {  // no room: step the populations
+    if (upload_plan(c->mom_host, l, &c->mom_plan, &bytes, c->stream) != cudaSuccess) {  // no room: step the populations
         cudaGetLastError();
         cudaFree(c->mom_plan);
         c->mom_plan = nullptr;
@@ -1759,8 +1759,9 @@ struct lbm_batch {
     MomentLaunch mom_launch{};
     void* mom_plan = nullptr;         // device memory of its plan
     BatchBox* mom_boxes_dev = nullptr;
+    MomentPlan mom_host;              // the plan and the boxes, alive as long as their copies may read them
+    std::vector<BatchBox> mom_boxes;
     bool mom_twice = false;
-    long long mom_busiest = 0;        // planes of its busiest block
     Forms forms;
     unsigned max_cells = 0;
     char err[512] = {0};
@@ -1876,7 +1877,8 @@ lbm_status batch_configure_moments(lbm_batch* b) {
         cudaGetLastError();
         return LBM_OK;
     }
-    std::vector<BatchBox> boxes(b->count);
+    std::vector<BatchBox>& boxes = b->mom_boxes;
+    boxes.assign(b->count, BatchBox{});
     std::vector<TileColumns> columns(b->count);
     for (int i = 0; i < b->count; ++i) {
         const lbm_params& q = b->box[i]->p;
@@ -1890,8 +1892,7 @@ lbm_status batch_configure_moments(lbm_batch* b) {
         bx.n = b->box[i]->n;
         columns[i] = {bx.tiles_x * ((q.ny + k->tile_y - 1) / k->tile_y), q.nz};
     }
-    const MomentPlan plan = plan_moments(columns, (long long)per_sm * b->num_sms, k->fields, bytes_all);
-    b->mom_busiest = plan.busiest;
+    b->mom_host = plan_moments(columns, (long long)per_sm * b->num_sms, k->fields, bytes_all);
     if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
     LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
                                 b->stream));
@@ -1901,7 +1902,7 @@ lbm_status batch_configure_moments(lbm_batch* b) {
     l.batch.nbox = b->count;
     l.batch.boxes = b->mom_boxes_dev;
     size_t bytes = 0;
-    if (upload_plan(plan, l, &b->mom_plan, &bytes, b->stream) != cudaSuccess) {  // no room: step the populations
+    if (upload_plan(b->mom_host, l, &b->mom_plan, &bytes, b->stream) != cudaSuccess) {  // no room: step the populations
         cudaGetLastError();
         cudaFree(b->mom_plan);
         b->mom_plan = nullptr;
@@ -1927,7 +1928,7 @@ lbm_status batch_choose_forms(lbm_batch* b, Forms& f) {
         odd = odd || c->p.nx % 2 != 0;
     }
     const double rival = 37e-6 * padded;
-    const long from = moments_pay_from(b->p.storage, b->box[0]->coll, b->cells, odd, true, b->mom_busiest, rival < 20.0 ? 20.0 : rival);
+    const long from = moments_pay_from(b->p.storage, b->box[0]->coll, b->cells, odd, true, b->mom_host.busiest, rival < 20.0 ? 20.0 : rival);
     if (from > 0) {
         f.several = LBM_FORM_MOMENTS;
         f.from = from;

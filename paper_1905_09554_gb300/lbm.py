@@ -412,6 +412,8 @@ class Lattice:
     'bf16l' (deviations from a per-cell reference density).  With torch_buffers=True the two population
     copies are torch.cuda tensors owned by this object and all work runs on
     torch's current stream.
+    kernel, tile_y, zchunk: any of them given, every step runs by the one
+    kernel of that launch shape (see step_form).
     """
 
     def __init__(self, nx, ny, nz, G=-5.5, tau=1.0, collision="srt", rates=None,
