@@ -1893,7 +1893,11 @@ lbm_status batch_configure_moments(lbm_batch* b) {
         columns[i] = {bx.tiles_x * ((q.ny + k->tile_y - 1) / k->tile_y), q.nz};
     }
     b->mom_host = plan_moments(columns, (long long)per_sm * b->num_sms, k->fields, bytes_all);
-    if (!b->mom_boxes_dev) LBM_CUDA(b, cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count));
+    if (!b->mom_boxes_dev && cudaMalloc(&b->mom_boxes_dev, sizeof(BatchBox) * b->count) != cudaSuccess) {
+        cudaGetLastError();  // no room: step the populations
+        b->mom_boxes_dev = nullptr;
+        return LBM_OK;
+    }
     LBM_CUDA(b, cudaMemcpyAsync(b->mom_boxes_dev, boxes.data(), sizeof(BatchBox) * b->count, cudaMemcpyHostToDevice,
                                 b->stream));
     MomentLaunch& l = b->mom_launch;
