@@ -9,7 +9,7 @@ struct AdjointArgs {
     int nx, ny, nz;
     long long n;
     double G, tau, omega, rho0;
-    double gw;                      // -G/36
+    double gw;                      // -G (gwf: -G/36), as force_of takes it
     float Gf, tauf, omegaf, rho0f, gwf;  // rounded on the host for the FP32 kernels
     int grid;  // blocks of adjoint_threads() threads (grid-stride loops)
     bool tau1; // tau = 1: lam holds four values a cell {A, B}, lam_a = A + c_a.B, and gr is not used

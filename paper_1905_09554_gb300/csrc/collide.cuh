@@ -384,12 +384,17 @@ template <class V>
 struct Force {
     V g, sx, sy, sz;
 };
-// gw = -G/36.
+// gw: float -G/36, double -G: there the weight 1/36 is a factor of its own, with
+// the same rounding (5.6e-17 low) as in the equilibrium's w rho, so that the two
+// cancel in the balance of pressure and force that sets the densities of the
+// phases.  -G/36 rounded once is off by another amount (8.1e-17 high at G =
+// -5.5): 20 steps then left the vapour's density 4e-16 to 9e-16 low.
 template <class V, class R>
 __device__ __forceinline__ Force<V> force_of(const PsiView<V>& lo, const PsiView<V>& mid, const PsiView<V>& hi,
                                              R gw) {
     Force<V> F;
     F.g = vmulc(gw, mid.c);
+    if constexpr (sizeof(R) == sizeof(double)) F.g = vmul(F.g, 1.0 / 36.0);
     const V dc = vsub(hi.c, lo.c);
     F.sx = vtwice(mid.ex, vadd(mid.dx, vadd(lo.ex, hi.ex)));
     F.sy = vtwice(mid.ey, vadd(mid.dy, vadd(lo.ey, hi.ey)));

@@ -36,7 +36,7 @@ struct StepArgs {
     double tau, omega;    // SRT relaxation time and 1/tau
     double rho0, inv_rho0;
     double s[Q];          // MRT rates, moment order
-    double gw;            // -G/36: the force's strength per edge weight
+    double gw;            // the force's strength as force_of takes it: -G (gwf: -G/36)
     // (1 - s_k)/norm_k of the rows e (times 19), 3pxx, pww, pxy, pyz, pxz
     double kk[6];
     // The same parameters rounded to float once on the host, for the float
@@ -71,8 +71,8 @@ __host__ __device__ __forceinline__ const R (&row_rates(const StepArgs& a))[6] {
 // Fill the derived parameters and the float copies from the double fields.
 inline void round_params(StepArgs& a) {
     constexpr int rows[6] = {1, 9, 11, 13, 14, 15};
-    a.gw = -a.G / 36.0;
-    a.gwf = float(a.gw);
+    a.gw = -a.G;
+    a.gwf = float(-a.G / 36.0);
     for (int i = 0; i < 6; ++i) {
         a.kk[i] = (1.0 - a.s[rows[i]]) / mrt_norm(rows[i]) * (i == 0 ? 19.0 : 1.0);
         a.kkf[i] = float(a.kk[i]);
