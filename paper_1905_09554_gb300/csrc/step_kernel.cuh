@@ -94,21 +94,23 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
     const R gxx = vsub(vadd(gx, gx), gyz), gww = vsub(gy, gz);
     const R nr = vmul(R(-0.5), rho), q23 = vmul(R(-2.0 / 3.0), rho);
 
-    R meq[Q], sg[Q];
-    meq[1] = vmul(rho, vfma(R(19), u2, R(-11)));  sg[1] = vmul(R(38), uF);
-    meq[2] = vmul(rho, vfma(R(-5.5), u2, R(3)));  sg[2] = vmul(R(-11), uF);
-    meq[4] = vmul(q23, ux);                       sg[4] = vmul(R(-2.0 / 3.0), Fx);
-    meq[6] = vmul(q23, uy);                       sg[6] = vmul(R(-2.0 / 3.0), Fy);
-    meq[8] = vmul(q23, uz);                       sg[8] = vmul(R(-2.0 / 3.0), Fz);
-    meq[9] = vmul(rho, pxx);                      sg[9] = vadd(gxx, gxx);
-    meq[10] = vmul(nr, pxx);                      sg[10] = -gxx;
-    meq[11] = vmul(rho, pww);                     sg[11] = vadd(gww, gww);
-    meq[12] = vmul(nr, pww);                      sg[12] = -gww;
-    meq[13] = vmul(vmul(rho, ux), uy);            sg[13] = vfma(ux, Fy, vmul(uy, Fx));
-    meq[14] = vmul(vmul(rho, uy), uz);            sg[14] = vfma(uy, Fz, vmul(uz, Fy));
-    meq[15] = vmul(vmul(rho, ux), uz);            sg[15] = vfma(ux, Fz, vmul(uz, Fx));
-    meq[16] = meq[17] = meq[18] = R(0);
-    sg[16] = sg[17] = sg[18] = R(0);
+    // dm = m - m_eq, the equilibrium's last product not rounded by itself
+    R dm[Q], sg[Q];
+    dm[1] = vfnma(rho, vfma(R(19), u2, R(-11)), m[1]);  sg[1] = vmul(R(38), uF);
+    dm[2] = vfnma(rho, vfma(R(-5.5), u2, R(3)), m[2]);  sg[2] = vmul(R(-11), uF);
+    dm[4] = vfnma(q23, ux, m[4]);                       sg[4] = vmul(R(-2.0 / 3.0), Fx);
+    dm[6] = vfnma(q23, uy, m[6]);                       sg[6] = vmul(R(-2.0 / 3.0), Fy);
+    dm[8] = vfnma(q23, uz, m[8]);                       sg[8] = vmul(R(-2.0 / 3.0), Fz);
+    dm[9] = vfnma(rho, pxx, m[9]);                      sg[9] = vadd(gxx, gxx);
+    dm[10] = vfnma(nr, pxx, m[10]);                     sg[10] = -gxx;
+    dm[11] = vfnma(rho, pww, m[11]);                    sg[11] = vadd(gww, gww);
+    dm[12] = vfnma(nr, pww, m[12]);                     sg[12] = -gww;
+    dm[13] = vfnma(vmul(rho, ux), uy, m[13]);           sg[13] = vfma(ux, Fy, vmul(uy, Fx));
+    dm[14] = vfnma(vmul(rho, uy), uz, m[14]);           sg[14] = vfma(uy, Fz, vmul(uz, Fy));
+    dm[15] = vfnma(vmul(rho, ux), uz, m[15]);           sg[15] = vfma(ux, Fz, vmul(uz, Fx));
+    dm[16] = m[16];
+    dm[17] = m[17];
+    dm[18] = m[18];
 
     // d[k] = (Lambda (m - m_eq) - (I - Lambda/2) S)_k / norm_k
     R d[Q];
@@ -120,7 +122,7 @@ __device__ __forceinline__ void collide_mrt(R (&f)[Q], R Fx, R Fy, R Fz, const R
         constexpr int k = decltype(kc)::value;
         if constexpr (k != 0 && k != 3 && k != 5 && k != 7) {
             const R sk = s[k];
-            R t = vmul(sk, vsub(m[k], meq[k]));
+            R t = vmul(sk, dm[k]);
             if constexpr (k < 16) t = vfnma(vfnma(half, sk, R(1)), sg[k], t);
             d[k] = vmul(t, R(1.0 / mrt_norm(k)));
         }

@@ -18,7 +18,7 @@
 //
 // Measured: 32 x 32 x 64, SRT, 50 steps 8.10 -> 1.12 ms (of that the marching
 // kernel's 32 blocks on 152 SMs cost most); 128 x 128 x 288, MRT, 10 steps
-// 30.7 -> 14.8 ms, 3.19 GLUPS.
+// 30.7 -> 14.8 ms, 3.18 GLUPS.
 //
 // 32- and 16-bit storage: the extra passes cost bytes, so large boxes keep the
 // marching kernels.  Boxes that live in L2 are bound by the marching kernels'
